@@ -199,20 +199,25 @@ void dev_free(gencd_problem* p, void* ptr) {
     cudaFree(ptr);
 }
 
-int ensure_slots(gencd_problem* p, int64_t count) {
-  if (count <= p->slot_cap) return GENCD_OK;
+int ensure_slots(gencd_problem* p, int64_t count, int64_t partitions) {
+  if (count <= p->slot_cap && partitions <= p->slot_cnt_cap) return GENCD_OK;
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
   dev_free(p, p->slot_m);
   dev_free(p, p->slot_d);
   dev_free(p, p->slot_j);
+  dev_free(p, p->slot_cnt);
   p->slot_m = nullptr;
   p->slot_d = nullptr;
   p->slot_j = nullptr;
-  p->slot_cap = 0;
+  p->slot_cnt = nullptr;
+  p->slot_cap = p->slot_cnt_cap = 0;
   GENCD_TRY(dev_alloc(p, &p->slot_m, count));
   GENCD_TRY(dev_alloc(p, &p->slot_d, count));
   GENCD_TRY(dev_alloc(p, &p->slot_j, count));
+  GENCD_TRY(dev_alloc(p, &p->slot_cnt, partitions));
+  GENCD_CUDA_TRY(cudaMemsetAsync(p->slot_cnt, 0, sizeof(unsigned int) * partitions, p->stream));
   p->slot_cap = count;
+  p->slot_cnt_cap = partitions;
   return GENCD_OK;
 }
 
@@ -334,7 +339,7 @@ static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt)
   const int v = p->params.variant;
   if (v == GENCD_THREAD_GREEDY || v == GENCD_GREEDY) {
     const int B = effective_B(p);
-    GENCD_CUDA_TRY(cudaMemsetAsync(p->dscal, 0, sizeof(double), p->stream));  // KKT maximum
+    if (want_kkt) GENCD_CUDA_TRY(cudaMemsetAsync(p->dscal, 0, sizeof(double), p->stream));  // KKT maximum
     GENCD_TRY(launch_propose_all(p, p->u, p->precision == GENCD_F64));  // Propose, all columns
     GENCD_TRY(launch_finalize_accept(p, B, want_kkt));  // step, proxy (+ KKT of the start state); Accept
     GENCD_TRY(launch_merge_accept(p, B));               // accept backoff (groups of partitions), if any
@@ -542,7 +547,7 @@ static void free_problem(gencd_problem* p) {
                   p->delta, p->phi, p->list_j, p->list_d, p->list_m, p->w_start, p->top_buf, p->dscal, p->red, p->perm,
                   p->sort_tmp,
                   p->row_ptr, p->col_idx, p->csr_val, p->color, p->color_ptr, p->cols_by_color,
-                  p->slot_m, p->slot_d, p->slot_j, p->list_off, p->scan_tmp, p->bj, p->w32, p->bj32, p->ib32,
+                  p->slot_m, p->slot_d, p->slot_j, p->slot_cnt, p->list_off, p->scan_tmp, p->bj, p->w32, p->bj32, p->ib32,
                   p->part_lo, p->col_val, p->block_lo, p->block_P};
   if (p->stream) cudaStreamSynchronize(p->stream);
   free_propose_plan(p);

@@ -207,11 +207,13 @@ struct gencd_problem {
   int64_t* part_lo = nullptr;
   int64_t part_B = 0, part_cap = 0;
 
-  // accept candidates of (chunk, partition) pairs when partitions are few
+  // accept candidates of a partition's chunks of columns, and a count per
+  // partition of the chunks done (zero between launches)
   uint64_t* slot_m = nullptr;
   double* slot_d = nullptr;
   int32_t* slot_j = nullptr;
-  int64_t slot_cap = 0;
+  unsigned int* slot_cnt = nullptr;
+  int64_t slot_cap = 0, slot_cnt_cap = 0;
 
   // FP32 mode: float copies of w, beta_j and 1/beta_j for the per-column
   // selection pass (w32[j] is 0 exactly when w[j] is); null in FP64 mode
@@ -285,7 +287,7 @@ int launch_merge_accept(gencd_problem* p, int64_t B);  // keep the best of every
 // Improve delta_j (Algorithm 3): refine the accepted steps D[e] of columns
 // J[e] >= 0 in place (params.improve_steps Eq. 7 steps each; 0: nothing)
 int launch_improve_list(gencd_problem* p, const int32_t* J, double* D, int64_t m);
-int ensure_slots(gencd_problem* p, int64_t count);
+int ensure_slots(gencd_problem* p, int64_t count, int64_t partitions);
 // exclusive prefix sum of m uint32 (in place allowed); tmp holds scan_tmp_words(m)
 int exclusive_scan(gencd_problem* p, const uint32_t* in, uint32_t* out, int64_t m, uint32_t* tmp);
 int64_t scan_tmp_words(int64_t m);

@@ -10,12 +10,16 @@
 //    constant whatever the column lengths (1 ... 50,000 non-zeros).
 //  * k_finalize: g_j = gacc_j / n, the Eq. 7 step, the Eq. 9 proxy and the
 //    KKT violation per column; resets gacc for the next launch.
-//  * k_accept: Thread-Greedy / Greedy accept (Table 2), one CTA per partition,
-//    argmin of phi with ties to the lower column; accepted iff phi < 0.
+//  * k_accept_partitions: the same per-column work and the Thread-Greedy /
+//    Greedy accept (Table 2) in one pass: argmin of phi per partition, ties to
+//    the lower column; accepted iff phi < 0.
 //  * k_propose_list: Algorithm 4 over a selected list J (Shotgun, parity hook),
 //    one warp per column with a shuffle reduction.
 //  * k_objective_*: P(w) of Eq. 1 in FP64 with a fixed-order two-pass sum.
 #include <float.h>
+
+#include <algorithm>
+#include <type_traits>
 
 #include "device_math.cuh"
 #include "gencd_internal.cuh"
@@ -146,22 +150,22 @@ __device__ __forceinline__ bool cand_better(uint64_t ma, int32_t ja, uint64_t mb
   return ma > mb || (ma == mb && ma != 0 && ja < jb);
 }
 
-// block reduction of the best candidate (mag, j, delta) over NT threads;
-// valid in thread 0
-template <int NT = kThreads>
-__device__ __forceinline__ void block_best(uint64_t& m, int32_t& j, double& d) {
-  __shared__ uint64_t s_m[NT / 32];
-  __shared__ double s_d[NT / 32];
-  __shared__ int32_t s_j[NT / 32];
+// block reduction of the best candidate (mag, j, payload) over kThreads
+// threads; valid in thread 0
+template <typename X>
+__device__ __forceinline__ void block_best(uint64_t& m, int32_t& j, X& x) {
+  __shared__ uint64_t s_m[kThreads / 32];
+  __shared__ X s_x[kThreads / 32];
+  __shared__ int32_t s_j[kThreads / 32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
-    const uint64_t xm = __shfl_xor_sync(0xffffffffu, m, o);
-    const int32_t xj = __shfl_xor_sync(0xffffffffu, j, o);
-    const double xd = __shfl_xor_sync(0xffffffffu, d, o);
-    if (cand_better(xm, xj, m, j)) {
-      m = xm;
-      j = xj;
-      d = xd;
+    const uint64_t ym = __shfl_xor_sync(0xffffffffu, m, o);
+    const int32_t yj = __shfl_xor_sync(0xffffffffu, j, o);
+    const X yx = __shfl_xor_sync(0xffffffffu, x, o);
+    if (cand_better(ym, yj, m, j)) {
+      m = ym;
+      j = yj;
+      x = yx;
     }
   }
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -169,15 +173,15 @@ __device__ __forceinline__ void block_best(uint64_t& m, int32_t& j, double& d) {
   if (lane == 0) {
     s_m[wid] = m;
     s_j[wid] = j;
-    s_d[wid] = d;
+    s_x[wid] = x;
   }
   __syncthreads();
   if (threadIdx.x == 0)
-    for (int q = 1; q < NT / 32; ++q)
+    for (int q = 1; q < kThreads / 32; ++q)
       if (cand_better(s_m[q], s_j[q], m, j)) {
         m = s_m[q];
         j = s_j[q];
-        d = s_d[q];
+        x = s_x[q];
       }
 }
 
@@ -194,11 +198,6 @@ __device__ __forceinline__ void block_max_bits_to(double* out, uint64_t v) {
     v = x > v ? x : v;
   }
   if ((threadIdx.x & 31) == 0 && v) atomicMax(reinterpret_cast<unsigned long long*>(out), (unsigned long long)v);
-}
-
-// partition of column j: the b with floor(b k / B) <= j < floor((b+1) k / B)
-__device__ __forceinline__ int64_t partition_of(int64_t j, int64_t k, int64_t B) {
-  return ((j + 1) * B - 1) / k;
 }
 
 // Eq. 7 step and Eq. 9 proxy of an active column from its raw sum
@@ -292,98 +291,12 @@ __global__ void __launch_bounds__(kThreads)
   block_max_bits_to(kkt_out + 7, gmax);  // max |g_j| over the active columns (idle ones have |g_j| <= lambda)
 }
 
-// Thread-Greedy with many partitions: one CTA per partition computes the
-// step and proxy of its columns and accepts the best proxy (Table 2, "greedy
-// per thread"), so delta and phi never reach memory.  want_kkt: also reduce
-// the KKT violation (convergence checks only).  Idle columns (phi = 0) are
-// never accepted and are not queued.
-template <typename G>
-__global__ void __launch_bounds__(kThreads)
-    k_finalize_accept(G* __restrict__ gacc, const double* __restrict__ w, const double* __restrict__ bjs,
-                      const double* __restrict__ ib, int64_t k, double inv_n, double lam, uint64_t lnb64,
-                      uint32_t lnb32, int64_t B, int want_kkt, int32_t* __restrict__ list_j,
-                      double* __restrict__ list_d, uint64_t* __restrict__ list_m, double* __restrict__ kkt_out) {
-  __shared__ int s_n;
-  __shared__ int64_t s_j[kRoundCols];
-  __shared__ double s_g[kRoundCols], s_w[kRoundCols];
-  __shared__ int64_t s_lo, s_hi;
-  uint64_t vmax = 0;
-  for (int64_t b = blockIdx.x; b < B; b += gridDim.x) {
-    // 64-bit divisions run on the FP64 unit, which is small on this GPU:
-    // one thread computes the partition bounds
-    if (threadIdx.x == 0) {
-      s_lo = b * k / B;
-      s_hi = (b + 1) * k / B;
-    }
-    __syncthreads();
-    const int64_t lo = s_lo, hi = s_hi;
-    uint64_t bm = 0;
-    int32_t bj = INT32_MAX;
-    double bd = 0.0;
-    for (int64_t base = lo; base < hi; base += kRoundCols) {  // uniform across the CTA
-      if (threadIdx.x == 0) s_n = 0;
-      __syncthreads();
-      const int na = scan_round(gacc, w, base, hi, lnb64, lnb32, &s_n, s_j, s_g, s_w, (double*)nullptr,
-                                (double*)nullptr);
-      for (int e = threadIdx.x; e < na; e += kThreads) {
-        const int64_t j = s_j[e];
-        double g, d, f;
-        active_step(s_g[e], inv_n, s_w[e], lam, bjs[j], ib[j], g, d, f);
-        if (want_kkt) max_bits(vmax, kkt_violation(g, s_w[e], lam));
-        const uint64_t m = candidate_mag(f);
-        if (cand_better(m, (int32_t)j, bm, bj)) {
-          bm = m;
-          bj = (int32_t)j;
-          bd = d;
-        }
-      }
-      __syncthreads();
-    }
-    block_best(bm, bj, bd);
-    if (threadIdx.x == 0) {
-      list_j[b] = bm ? bj : -1;
-      list_d[b] = bm ? bd : 0.0;
-      list_m[b] = bm;
-    }
-  }
-  if (want_kkt) block_max_bits_to(kkt_out, vmax);
-}
-
 // ---------------------------------------------------------------------------
 // FP32 mode: the per-column pass ranks the columns with Eq. 7 / Eq. 9 in FP32
 // (FP32 sums, the float copies of w, beta_j and 1/beta_j); only the accepted
 // column's step is recomputed in FP64 (eq7_step with the FP64 w), and it is
 // accepted when that proxy is negative.  GB300 runs FP64 at a small fraction
 // of its FP32 rate, so the per-column work stays on the FP32 pipe.
-
-
-// one round of 4 columns per thread of NT: load, zero the sums, integer idle
-// test, queue the active columns (j, raw sum) in shared memory
-template <int NT>
-__device__ __forceinline__ int scan_round_f32(float* __restrict__ gacc, const float* __restrict__ w32, int64_t base,
-                                              int64_t hi, uint32_t lnb32, int* s_n, int32_t* s_j, float* s_g) {
-  float ga[kColsPerThread], wv[kColsPerThread];
-#pragma unroll
-  for (int q = 0; q < kColsPerThread; ++q) {
-    const int64_t j = base + q * NT + threadIdx.x;
-    ga[q] = j < hi ? gacc[j] : 0.0f;
-    wv[q] = j < hi ? w32[j] : 0.0f;
-  }
-#pragma unroll
-  for (int q = 0; q < kColsPerThread; ++q) {
-    const int64_t j = base + q * NT + threadIdx.x;
-    if (j >= hi) continue;
-    gacc[j] = 0.0f;
-    const bool idle = (__float_as_uint(wv[q]) << 1) == 0 && (__float_as_uint(ga[q]) & 0x7fffffffu) <= lnb32;
-    if (!idle) {
-      const int slot = atomicAdd(s_n, 1);
-      s_j[slot] = (int32_t)j;
-      s_g[slot] = ga[q];
-    }
-  }
-  __syncthreads();
-  return *s_n;
-}
 
 // FP64 step and proxy of the ranked winner (raw sum ga): the accepted delta,
 // or no acceptance (false) when that proxy is not negative
@@ -399,226 +312,166 @@ __device__ __forceinline__ uint64_t kkt_bits_f32(uint32_t vmax32) {
   return (uint64_t)__double_as_longlong((double)__uint_as_float(vmax32));
 }
 
-constexpr int kFinThreads = 256;  // small CTAs: every partition of config 2 (3,906 columns, 4 rounds) resident at once
+// the per-column inputs of the Accept, in FP64 and (FP32 mode) as floats
+struct AcceptCols {
+  const double *w, *bj, *ib;
+  const float *w32, *bj32, *ib32;
+  double inv_n, lam;
+  float inv_nf, lamf;  // converted on the host: a conversion runs on the FP64 pipe (16 cycles a warp)
+  uint64_t lnb64;
+  uint32_t lnb32;
+};
 
-__global__ void __launch_bounds__(kFinThreads)
-    k_finalize_accept_f32(float* __restrict__ gacc, const float* __restrict__ w32, const float* __restrict__ bj32,
-                          const float* __restrict__ ib32, const double* __restrict__ w,
-                          const double* __restrict__ bjs, const double* __restrict__ ib, int64_t k, float inv_nf,
-                          float lamf, double inv_n, double lam, uint32_t lnb32, int64_t B,
-                          const int64_t* __restrict__ part_lo, int want_kkt, int32_t* __restrict__ list_j,
-                          double* __restrict__ list_d, uint64_t* __restrict__ list_m, double* __restrict__ kkt_out) {
-  constexpr int ROUND = kColsPerThread * kFinThreads;
-  __shared__ int s_n;
-  __shared__ int32_t s_j[ROUND];
-  __shared__ float s_g[ROUND];
-  uint32_t vmax = 0;
-  for (int64_t b = blockIdx.x; b < B; b += gridDim.x) {
-    const int64_t lo = part_lo[b], hi = part_lo[b + 1];  // precomputed: no 64-bit division here
+// scan_round for FP32 sums and the float copy of w: the queue holds (j, raw sum)
+__device__ __forceinline__ int scan_round_f32(float* __restrict__ gacc, const float* __restrict__ w32, int64_t base,
+                                              int64_t hi, uint32_t lnb32, int* s_n, int32_t* s_j, float* s_g) {
+  float ga[kColsPerThread], wv[kColsPerThread];
+#pragma unroll
+  for (int q = 0; q < kColsPerThread; ++q) {
+    const int64_t j = base + q * kThreads + threadIdx.x;
+    ga[q] = j < hi ? gacc[j] : 0.0f;
+    wv[q] = j < hi ? w32[j] : 0.0f;
+  }
+#pragma unroll
+  for (int q = 0; q < kColsPerThread; ++q) {
+    const int64_t j = base + q * kThreads + threadIdx.x;
+    if (j >= hi) continue;
+    gacc[j] = 0.0f;
+    const bool idle = (__float_as_uint(wv[q]) << 1) == 0 && (__float_as_uint(ga[q]) & 0x7fffffffu) <= lnb32;
+    if (!idle) {
+      const int slot = atomicAdd(s_n, 1);
+      s_j[slot] = (int32_t)j;
+      s_g[slot] = ga[q];
+    }
+  }
+  __syncthreads();
+  return *s_n;
+}
+
+// Thread-Greedy / Greedy Accept (Table 2, "greedy per thread"): the best proxy
+// of every partition, in one launch for any number of partitions, so that
+// delta and phi never reach memory.  A partition is cut into `per` chunks of
+// columns, one CTA each; with more than one chunk the chunk winners go to
+// slots, and the CTA that finishes a partition last (a counter per partition)
+// picks among them.  want_kkt: also reduce the KKT violation (convergence
+// checks only).  Idle columns (phi = 0) are never accepted.
+//
+// Bound: latency (a few dependent loads and block reductions per CTA), so
+// what counts is that every chunk is resident at once and that no thread
+// walks columns one after another: the launcher cuts to about 8 CTAs per SM.
+// Chunks of 4,096 columns, a thread walking its 16 columns serially, and a
+// second launch for the slots took 34.5 + 5.5 us on k = 100,000, B = 1 (25
+// CTAs), 44.7 + 5.7 us on k = 500,000, B = 16 and, in FP64, 62.5 + 4.1 us on
+// k = 400,000, B = 128; this takes 11.1, 11.0 and 21.7 us (ncu, cold caches).
+// One CTA per partition, the many-partitions form, is the same work as before
+// (15 us on k = 4,000,000, B = 1,024).  The active columns are queued: testing
+// and evaluating them in place, four per thread, serialised their loads of
+// beta_j (89 us on k = 4,000,000).
+template <typename G>
+__global__ void __launch_bounds__(kThreads)
+    k_accept_partitions(G* __restrict__ gacc, AcceptCols c, int64_t B, int per, int64_t chunk,
+                        const int64_t* __restrict__ part_lo, int want_kkt, uint64_t* __restrict__ slot_m,
+                        int32_t* __restrict__ slot_j, double* __restrict__ slot_x, unsigned int* __restrict__ slot_cnt,
+                        int32_t* __restrict__ list_j, double* __restrict__ list_d, uint64_t* __restrict__ list_m,
+                        double* __restrict__ kkt_out) {
+  constexpr bool F32 = sizeof(G) == 4;
+  using J = typename std::conditional<F32, int32_t, int64_t>::type;
+  __shared__ int s_n;  // the active columns of a round, processed packed
+  __shared__ J s_j[kRoundCols];
+  __shared__ G s_g[kRoundCols];
+  __shared__ double s_w[F32 ? 1 : kRoundCols];
+  __shared__ bool s_last;
+  uint64_t vmax64 = 0;
+  uint32_t vmax32 = 0;
+  const int64_t items = B * per;
+  for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+    const int64_t b = per == 1 ? it : (int64_t)((uint32_t)it / (uint32_t)per);  // items < 2^32 when per > 1
+    const int64_t lo = part_lo[b] + (it - b * per) * chunk;
+    const int64_t end = part_lo[b + 1];
+    const int64_t hi = per == 1 ? end : (lo + chunk < end ? lo + chunk : end);
     uint64_t bm = 0;
     int32_t bj = INT32_MAX;
-    float bga = 0.0f;
-    for (int64_t base = lo; base < hi; base += ROUND) {  // uniform across the CTA
+    G bx = G(0);  // FP32: the winner's raw sum; FP64: its step
+    for (int64_t base = lo; base < hi; base += kRoundCols) {  // uniform across the CTA
       if (threadIdx.x == 0) s_n = 0;
       __syncthreads();
-      const int na = scan_round_f32<kFinThreads>(gacc, w32, base, hi, lnb32, &s_n, s_j, s_g);
-      for (int e = threadIdx.x; e < na; e += kFinThreads) {
-        const int32_t j = s_j[e];
-        const float g = s_g[e] * inv_nf, wj = w32[j];
-        float d, f;
-        eq7_step_f32(g, wj, lamf, bj32[j], ib32[j], d, f);
-        if (want_kkt) {
-          const uint32_t v = __float_as_uint(kkt_violation_f32(g, wj, lamf));
-          vmax = v > vmax ? v : vmax;
+      int na;
+      if constexpr (F32)
+        na = scan_round_f32(gacc, c.w32, base, hi, c.lnb32, &s_n, s_j, s_g);
+      else
+        na = scan_round(gacc, c.w, base, hi, c.lnb64, c.lnb32, &s_n, s_j, s_g, s_w, (double*)nullptr,
+                        (double*)nullptr);
+      for (int e = threadIdx.x; e < na; e += kThreads) {
+        const int64_t j = s_j[e];
+        uint64_t m;
+        G x;
+        if constexpr (F32) {
+          const float g = s_g[e] * c.inv_nf, wj = c.w32[j];
+          float d, f;
+          eq7_step_f32(g, wj, c.lamf, c.bj32[j], c.ib32[j], d, f);
+          if (want_kkt) {
+            const uint32_t v = __float_as_uint(kkt_violation_f32(g, wj, c.lamf));
+            vmax32 = v > vmax32 ? v : vmax32;
+          }
+          m = candidate_mag32(f);
+          x = s_g[e];
+        } else {
+          double g, d, f;
+          active_step(s_g[e], c.inv_n, s_w[e], c.lam, c.bj[j], c.ib[j], g, d, f);
+          if (want_kkt) max_bits(vmax64, kkt_violation(g, s_w[e], c.lam));
+          m = candidate_mag(f);
+          x = d;
         }
-        const uint64_t m = candidate_mag32(f);
-        if (cand_better(m, j, bm, bj)) {
+        if (cand_better(m, (int32_t)j, bm, bj)) {
           bm = m;
-          bj = j;
-          bga = s_g[e];
+          bj = (int32_t)j;
+          bx = x;
         }
       }
       __syncthreads();
     }
-    double dga = (double)bga;
-    block_best<kFinThreads>(bm, bj, dga);
-    if (threadIdx.x == 0) {
-      double d = 0.0;
-      const bool ok = bm && accept_fp64(dga, bj, inv_n, lam, w, bjs, ib, d);
+    block_best(bm, bj, bx);
+    bool decide = per == 1;
+    if (per > 1) {
+      if (threadIdx.x == 0) {
+        slot_m[it] = bm;
+        slot_j[it] = bj;
+        slot_x[it] = (double)bx;
+        __threadfence();  // the slot is written before the count says so
+        const unsigned int prev = atomicAdd(slot_cnt + b, 1u);
+        s_last = prev == (unsigned int)per - 1u;
+        if (s_last) slot_cnt[b] = 0u;  // for the next launch
+        __threadfence();
+      }
+      __syncthreads();
+      decide = s_last;
+      if (decide) {
+        bm = 0;
+        bj = INT32_MAX;
+        bx = G(0);
+        for (int64_t q = b * per + threadIdx.x; q < (b + 1) * per; q += kThreads) {
+          const uint64_t m = __ldcg(slot_m + q);
+          const int32_t j = __ldcg(slot_j + q);
+          if (cand_better(m, j, bm, bj)) {
+            bm = m;
+            bj = j;
+            bx = (G)__ldcg(slot_x + q);
+          }
+        }
+        block_best(bm, bj, bx);
+      }
+    }
+    if (decide && threadIdx.x == 0) {
+      double d = (double)bx;
+      bool ok = bm != 0;
+      if (F32 && ok) ok = accept_fp64((double)bx, bj, c.inv_n, c.lam, c.w, c.bj, c.ib, d);
       list_j[b] = ok ? bj : -1;
       list_d[b] = ok ? d : 0.0;
       list_m[b] = ok ? bm : 0ull;
     }
-    __syncthreads();  // s_n and the queue are reused by the next partition
+    __syncthreads();  // the reduction buffers and s_last are reused
   }
-  if (want_kkt) block_max_bits_to(kkt_out, kkt_bits_f32(vmax));
-}
-
-// few partitions, stage 1 in FP32 (see k_finalize_chunks); slot_d carries the
-// winner's raw sum, and k_accept_slots computes its FP64 step
-__global__ void __launch_bounds__(kThreads)
-    k_finalize_chunks_f32(float* __restrict__ gacc, const float* __restrict__ w32, const float* __restrict__ bj32,
-                          const float* __restrict__ ib32, int64_t k, float inv_nf, float lamf, uint32_t lnb32,
-                          int64_t B, int64_t S, int64_t nchunks, int want_kkt, uint64_t* __restrict__ slot_m,
-                          int32_t* __restrict__ slot_j, double* __restrict__ slot_d, double* __restrict__ kkt_out) {
-  __shared__ int64_t s_b[3];
-  uint32_t vmax = 0;
-  for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-    const int64_t lo = ch * S, hi = lo + S < k ? lo + S : k;
-    if (threadIdx.x == 0) {  // one thread does the 64-bit divisions
-      s_b[0] = partition_of(lo, k, B);
-      s_b[1] = partition_of(hi - 1, k, B);
-      s_b[2] = (s_b[0] + 1) * k / B;  // first column after partition b0
-    }
-    __syncthreads();
-    const int64_t b0 = s_b[0], b1 = s_b[1], end0 = s_b[2];
-    uint64_t m0 = 0, m1 = 0;
-    int32_t j0 = INT32_MAX, j1 = INT32_MAX;
-    float g0 = 0.0f, g1 = 0.0f;
-    for (int64_t j = lo + threadIdx.x; j < hi; j += blockDim.x) {
-      const float ga = gacc[j];
-      gacc[j] = 0.0f;
-      const float wj = w32[j];
-      if ((__float_as_uint(wj) << 1) == 0 && (__float_as_uint(ga) & 0x7fffffffu) <= lnb32) continue;
-      const float g = ga * inv_nf;
-      float d, f;
-      eq7_step_f32(g, wj, lamf, bj32[j], ib32[j], d, f);
-      if (want_kkt) {
-        const uint32_t v = __float_as_uint(kkt_violation_f32(g, wj, lamf));
-        vmax = v > vmax ? v : vmax;
-      }
-      const uint64_t m = candidate_mag32(f);
-      if (j < end0) {
-        if (cand_better(m, (int32_t)j, m0, j0)) {
-          m0 = m;
-          j0 = (int32_t)j;
-          g0 = ga;
-        }
-      } else if (cand_better(m, (int32_t)j, m1, j1)) {
-        m1 = m;
-        j1 = (int32_t)j;
-        g1 = ga;
-      }
-    }
-    double d0 = (double)g0, d1 = (double)g1;
-    block_best(m0, j0, d0);
-    block_best(m1, j1, d1);
-    if (threadIdx.x == 0) {
-      slot_m[ch + b0] = m0;
-      slot_j[ch + b0] = j0;
-      slot_d[ch + b0] = d0;
-      if (b1 != b0) {
-        slot_m[ch + b1] = m1;
-        slot_j[ch + b1] = j1;
-        slot_d[ch + b1] = d1;
-      }
-    }
-    __syncthreads();
-  }
-  if (want_kkt) block_max_bits_to(kkt_out, kkt_bits_f32(vmax));
-}
-
-// Thread-Greedy with few partitions (Greedy: B = 1), stage 1: one CTA per
-// chunk of S <= floor(k / B) columns, which meets at most two partitions;
-// the best candidate of (chunk c, partition b) goes to slot c + b.
-template <typename G>
-__global__ void __launch_bounds__(kThreads)
-    k_finalize_chunks(G* __restrict__ gacc, const double* __restrict__ w, const double* __restrict__ bjs,
-                      const double* __restrict__ ib, int64_t k, double inv_n, double lam, uint64_t lnb64,
-                      uint32_t lnb32,
-                      int64_t B, int64_t S, int64_t nchunks, int want_kkt, uint64_t* __restrict__ slot_m,
-                      int32_t* __restrict__ slot_j, double* __restrict__ slot_d, double* __restrict__ kkt_out) {
-  __shared__ int64_t s_b[3];
-  uint64_t vmax = 0;
-  for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-    const int64_t lo = ch * S, hi = lo + S < k ? lo + S : k;
-    if (threadIdx.x == 0) {  // one thread does the 64-bit divisions (FP64 unit)
-      s_b[0] = partition_of(lo, k, B);
-      s_b[1] = partition_of(hi - 1, k, B);
-      s_b[2] = (s_b[0] + 1) * k / B;  // first column after partition b0
-    }
-    __syncthreads();
-    const int64_t b0 = s_b[0], b1 = s_b[1], end0 = s_b[2];
-    uint64_t m0 = 0, m1 = 0;
-    int32_t j0 = INT32_MAX, j1 = INT32_MAX;
-    double d0 = 0.0, d1 = 0.0;
-    for (int64_t j = lo + threadIdx.x; j < hi; j += blockDim.x) {
-      const G ga = gacc[j];
-      gacc[j] = G(0);
-      const double wj = w[j];
-      if (idle_raw(ga, wj, lnb64, lnb32)) continue;
-      double g, d, f;
-      active_step((double)ga, inv_n, wj, lam, bjs[j], ib[j], g, d, f);
-      if (want_kkt) max_bits(vmax, kkt_violation(g, wj, lam));
-      const uint64_t m = candidate_mag(f);
-      if (j < end0) {  // partition b0
-        if (cand_better(m, (int32_t)j, m0, j0)) {
-          m0 = m;
-          j0 = (int32_t)j;
-          d0 = d;
-        }
-      } else if (cand_better(m, (int32_t)j, m1, j1)) {
-        m1 = m;
-        j1 = (int32_t)j;
-        d1 = d;
-      }
-    }
-    block_best(m0, j0, d0);
-    block_best(m1, j1, d1);
-    if (threadIdx.x == 0) {
-      slot_m[ch + b0] = m0;
-      slot_j[ch + b0] = j0;
-      slot_d[ch + b0] = d0;
-      if (b1 != b0) {
-        slot_m[ch + b1] = m1;
-        slot_j[ch + b1] = j1;
-        slot_d[ch + b1] = d1;
-      }
-    }
-    __syncthreads();
-  }
-  if (want_kkt) block_max_bits_to(kkt_out, vmax);
-}
-
-// stage 2: partition b reduces its slots c + b for the chunks c it meets
-// (FP32 mode: slot_d holds raw sums and the winner's step is computed here
-// in FP64 from w, bjs, ib; FP64 mode: w is null and slot_d holds the steps)
-__global__ void __launch_bounds__(kThreads)
-    k_accept_slots(const uint64_t* __restrict__ slot_m, const int32_t* __restrict__ slot_j,
-                   const double* __restrict__ slot_d, int64_t k, int64_t B, int64_t S,
-                   int32_t* __restrict__ list_j, double* __restrict__ list_d, uint64_t* __restrict__ list_m,
-                   const double* __restrict__ w, const double* __restrict__ bjs, const double* __restrict__ ib,
-                   double inv_n, double lam) {
-  __shared__ int64_t s_c[2];
-  for (int64_t b = blockIdx.x; b < B; b += gridDim.x) {
-    if (threadIdx.x == 0) {  // one thread does the 64-bit divisions (FP64 unit)
-      s_c[0] = (b * k / B) / S;
-      s_c[1] = ((b + 1) * k / B - 1) / S;
-    }
-    __syncthreads();
-    const int64_t c0 = s_c[0], c1 = s_c[1];
-    uint64_t bm = 0;
-    int32_t bj = INT32_MAX;
-    double bd = 0.0;
-    for (int64_t ch = c0 + threadIdx.x; ch <= c1; ch += blockDim.x) {
-      const uint64_t m = slot_m[ch + b];
-      const int32_t j = slot_j[ch + b];
-      if (cand_better(m, j, bm, bj)) {
-        bm = m;
-        bj = j;
-        bd = slot_d[ch + b];
-      }
-    }
-    block_best(bm, bj, bd);
-    if (threadIdx.x == 0) {
-      bool ok = bm != 0;
-      if (ok && w) ok = accept_fp64(bd, bj, inv_n, lam, w, bjs, ib, bd);
-      list_j[b] = ok ? bj : -1;
-      list_d[b] = ok ? bd : 0.0;
-      list_m[b] = ok ? bm : 0ull;
-    }
-    __syncthreads();
-  }
+  if (want_kkt) block_max_bits_to(kkt_out, F32 ? kkt_bits_f32(vmax32) : vmax64);
 }
 
 template <typename V, typename U>
@@ -834,47 +687,34 @@ static int ensure_part_bounds(gencd_problem* p, int64_t B) {
   return GENCD_OK;
 }
 
+// Chunk size of k_accept_partitions: the smallest of 256, 512, ... columns
+// that keeps the launch within 8 CTAs per SM (all resident at once); a
+// partition that fits one chunk is one CTA and needs no slots.
 int launch_finalize_accept(gencd_problem* p, int64_t B, bool want_kkt) {
-  const double inv_n = 1.0 / (double)p->n;
   uint64_t b64;
   uint32_t b32;
   lambda_bits(p, p->lambda, &b64, &b32);
   const bool f64 = p->precision == GENCD_F64;
+  GENCD_TRY(ensure_part_bounds(p, B));
+  const AcceptCols c{p->w, p->bj, p->ib, p->w32, p->bj32, p->ib32, 1.0 / (double)p->n, p->lambda,
+                     (float)(1.0 / (double)p->n), (float)p->lambda, b64, b32};
+  const int64_t resident = (int64_t)p->num_sms * 8;
+  const int64_t most = (p->k + B - 1) / B;  // columns of the largest partition
+  int64_t chunk = kThreads;
+  while (chunk < most && B * ((most + chunk - 1) / chunk) > resident) chunk *= 2;
+  const int64_t per = (most + chunk - 1) / chunk;
+  if (per > 1) GENCD_TRY(ensure_slots(p, B * per, B));
+  const int grid = (int)std::min<int64_t>(B * per, 2 * resident);
   cudaEvent_t ev = nullptr;
   prof_begin(p, K_FINALIZE, &ev);
-  if (B >= 2LL * p->num_sms) {
-    const int grid = (int)(B < (int64_t)p->num_sms * 16 ? B : (int64_t)p->num_sms * 16);
-    if (f64)
-      k_finalize_accept<double><<<grid, kThreads, 0, p->stream>>>((double*)p->gnat, p->w, p->bj, p->ib, p->k, inv_n,
-                                                                  p->lambda, b64, b32, B, want_kkt ? 1 : 0, p->list_j,
-                                                                  p->list_d, p->list_m, p->dscal + 0);
-    else {
-      GENCD_TRY(ensure_part_bounds(p, B));
-      k_finalize_accept_f32<<<grid, kFinThreads, 0, p->stream>>>(
-          (float*)p->gnat, p->w32, p->bj32, p->ib32, p->w, p->bj, p->ib, p->k, (float)inv_n, (float)p->lambda, inv_n,
-          p->lambda, b32, B, p->part_lo, want_kkt ? 1 : 0, p->list_j, p->list_d, p->list_m, p->dscal + 0);
-    }
-  } else {
-    int64_t S = p->k / B;  // >= 1 since B <= k; a chunk meets at most two partitions
-    if (S > 4096) S = 4096;
-    const int64_t nchunks = (p->k + S - 1) / S;
-    GENCD_TRY(ensure_slots(p, nchunks + B));
-    const int grid = grid_for(nchunks * kThreads, kThreads, blocks_per_sm_cap(p, 8));
-    if (f64)
-      k_finalize_chunks<double><<<grid, kThreads, 0, p->stream>>>((double*)p->gnat, p->w, p->bj, p->ib, p->k, inv_n,
-                                                                  p->lambda, b64, b32, B, S, nchunks, want_kkt ? 1 : 0,
-                                                                  p->slot_m, p->slot_j, p->slot_d, p->dscal + 0);
-    else
-      k_finalize_chunks_f32<<<grid, kThreads, 0, p->stream>>>((float*)p->gnat, p->w32, p->bj32, p->ib32, p->k,
-                                                              (float)inv_n, (float)p->lambda, b32, B, S, nchunks,
-                                                              want_kkt ? 1 : 0, p->slot_m, p->slot_j, p->slot_d,
-                                                              p->dscal + 0);
-    const int g2 = (int)(B < (int64_t)p->num_sms * 16 ? B : (int64_t)p->num_sms * 16);
-    k_accept_slots<<<g2, kThreads, 0, p->stream>>>(p->slot_m, p->slot_j, p->slot_d, p->k, B, S, p->list_j,
-                                                   p->list_d, p->list_m, f64 ? nullptr : p->w, p->bj, p->ib, inv_n,
-                                                   p->lambda);
-    p->prof.launches[K_ACCEPT] += 1;
-  }
+  if (f64)
+    k_accept_partitions<double><<<grid, kThreads, 0, p->stream>>>(
+        (double*)p->gnat, c, B, (int)per, chunk, p->part_lo, want_kkt ? 1 : 0, p->slot_m, p->slot_j, p->slot_d,
+        p->slot_cnt, p->list_j, p->list_d, p->list_m, p->dscal + 0);
+  else
+    k_accept_partitions<float><<<grid, kThreads, 0, p->stream>>>(
+        (float*)p->gnat, c, B, (int)per, chunk, p->part_lo, want_kkt ? 1 : 0, p->slot_m, p->slot_j, p->slot_d,
+        p->slot_cnt, p->list_j, p->list_d, p->list_m, p->dscal + 0);
   prof_end(p, ev);
   GENCD_CUDA_TRY(cudaGetLastError());
   return GENCD_OK;

@@ -782,3 +782,35 @@ def test_config2_at_one_percent_solves_to_a_certified_point(gb, precision, tol_r
     P = o_s.objective(w)
     assert o_s.duality_gap(w) <= (1e-5 if precision == "f64" else 1e-2) * P
     assert r.objective == pytest.approx(P, rel=1e-9)
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+@pytest.mark.parametrize("k,B", [(1, 1), (255, 1), (256, 2), (257, 1), (1025, 1), (1025, 4), (3000, 3000),
+                                 (70_001, 3), (400_003, 1)])
+def test_accept_takes_each_partitions_best_column(gb, precision, k, B):
+    # partitions of one chunk of columns and of many (the last chunk short,
+    # more than one round of a CTA), launched twice: the chunk counts are reset
+    prob = workloads.uniform_problem(400, k, 5, values="lognormal", n_planted=20, loss="logistic", seed=k + B)
+    orc = oracle.Oracle(prob)
+    lam = 0.02 * orc.lambda_max()
+    orc.set_lambda(lam)
+    w = _state(prob, 3, frac=min(0.05, 200 / k), scale=0.3)
+    bounds = (np.arange(B + 1, dtype=np.int64) * k) // B
+    with gb.Problem(prob, precision=precision) as p:
+        p.set_lambda(lam)
+        p.set_params(variant="thread_greedy", blocks=B)
+        p.set_w(w)
+        for _ in range(2):
+            w0 = p.w()
+            _, phi = orc.propose(w0, orc.fitted(w0), np.arange(k, dtype=np.int32))
+            p.iterate(1)
+            moved = np.flatnonzero(p.w() != w0)
+            part = np.searchsorted(bounds, moved, side="right") - 1
+            best = np.minimum.reduceat(phi, bounds[:-1])
+            # FP32 proxies differ from the oracle's by their rounding (1e-4 of
+            # the largest bounds it: sums of 5 terms, proxies of differences)
+            slack = 1e-12 if precision == "f64" else 1e-4
+            assert np.unique(part).size == part.size
+            assert np.isin(np.flatnonzero(best < -slack * abs(phi).max()), part).all()
+            assert (best[part] < (0 if precision == "f64" else slack * abs(phi).max())).all()
+            assert np.all(phi[moved] <= best[part] * (1 - slack) + slack * abs(phi).max())
