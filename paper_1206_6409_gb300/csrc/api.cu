@@ -77,19 +77,6 @@ __global__ void k_inv_beta(const double* __restrict__ c, int64_t k, double beta,
   }
 }
 
-__global__ void k_mirror_w(const double* __restrict__ w, int64_t k, float* __restrict__ w32) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < k; j += stride) w32[j] = w_mirror(w[j]);
-}
-
-int launch_mirror_w(gencd_problem* p) {
-  if (!p->w32) return GENCD_OK;
-  k_mirror_w<<<grid_for(p->k, kThreads, p->num_sms * 8), kThreads, 0, p->stream>>>(p->w, p->k, p->w32);
-  p->prof.launches[K_SETUP] += 1;
-  GENCD_CUDA_TRY(cudaGetLastError());
-  return GENCD_OK;
-}
-
 int launch_inv_beta(gencd_problem* p) {
   if (p->ib_mode == p->params.beta_mode) return GENCD_OK;
   const double beta = p->loss == GENCD_LOSS_SQUARED ? 1.0 : 0.25;
@@ -824,10 +811,7 @@ int solve_advance(gencd_problem* p, SolveRun* S) {
     S->best_kkt = S->best_obj = HUGE_VAL;
     S->stall = 0;
     GENCD_CUDA_TRY(cudaMemcpyAsync(p->w, p->w_start, sizeof(double) * p->k, cudaMemcpyDeviceToDevice, p->stream));
-    GENCD_TRY(launch_mirror_w(p));
-    GENCD_TRY(build_csr(p));
-    GENCD_TRY(launch_csr_spmv(p, p->w, p->z));
-    GENCD_TRY(launch_fill_u(p));
+    GENCD_TRY(launch_state_from_w(p));
     GENCD_TRY(solve_evaluate(p, S));
     return 1;
   }
@@ -1134,12 +1118,7 @@ int gencd_set_w(gencd_problem* p, const double* w, int64_t k, int32_t memory) {
       if (!std::isfinite(w[j])) return fail(GENCD_EINVAL, "w[" + std::to_string(j) + "] is not finite");
   }
   GENCD_CUDA_TRY(cudaMemcpyAsync(p->w, w, sizeof(double) * k, kind_in(memory), p->stream));
-  GENCD_TRY(launch_mirror_w(p));
-  GENCD_TRY(build_csr(p));
-  GENCD_TRY(launch_csr_spmv(p, p->w, p->z));
-  GENCD_TRY(launch_fill_u(p));
-  GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
-  return GENCD_OK;
+  return launch_state_from_w(p);
 }
 
 int gencd_duality_gap(gencd_problem* p, double* gap, double* primal, double* dual) {

@@ -61,6 +61,7 @@ constexpr int kListPlanPer = 4;
 constexpr int64_t kListPlanMax = (int64_t)kListPlanThreads * kListPlanPer;
 constexpr int32_t kMaxShotgunBlocks = 1024;  // column blocks of block Shotgun (one selection CTA)
 constexpr int kScalars = 16;  // device scalars of a problem (dscal / hpin)
+constexpr int kScalFit = 10;  // the first of the two that z = Xw uses
 
 // kernel ids for launch counting / profiling
 enum KernelId {
@@ -225,7 +226,8 @@ struct gencd_problem {
   // [1] objective, [2] loss sum, [3] l1 sum, [4] updates (int64), [5] nnz
   // processed (int64), [6] scratch, [7] max_j |g_j| of the last full
   // evaluation (bits; idle columns count as lambda), [8] the duality gap's
-  // sum of conjugates, [9] the duality gap P(w) - D
+  // sum of conjugates, [9] the duality gap P(w) - D, [10], [11] non-zeros and
+  // segments of the columns that z = Xw scatters (int64)
   double* dscal = nullptr;
   double* red = nullptr;  // per-block partial sums (2 * kRedBlocks)
   double* hpin = nullptr; // pinned host mirror of dscal
@@ -305,14 +307,15 @@ int launch_propose_list(gencd_problem* p, const int32_t* J, int64_t m, double* d
 int launch_objective(gencd_problem* p, bool gap);  // P(w); with gap also the duality gap (after a finalize)
 int launch_col_sumsq(gencd_problem* p);  // gacc_j = sum_i X_ij^2
 int launch_inv_beta(gencd_problem* p);   // ib_j = 1 / beta_j for the current beta_mode
-int launch_mirror_w(gencd_problem* p);   // w32 from w (FP32 mode)
 
 // kernels_update.cu
-int launch_fill_u(gencd_problem* p);
+// u = l'(y, z); with report (pinned host memory), counts[0..1] are copied there and reset
+int launch_fill_u(gencd_problem* p, unsigned long long* counts = nullptr, unsigned long long* report = nullptr);
 int launch_update_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m, bool skip_neg);
 int launch_refresh_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m, bool skip_neg);
 int launch_coloring_iter(gencd_problem* p, int64_t q);
 int launch_csr_spmv(gencd_problem* p, const double* x, double* out);  // out = X x (FP64)
+int launch_state_from_w(gencd_problem* p);  // z, u and w32 from p->w (synchronises the stream)
 
 // kernels_setup.cu
 int launch_col_scale(gencd_problem* p);
