@@ -340,8 +340,8 @@ int gencd_set_propose_schedule(gencd_problem* p, int32_t split);
  * paper has no counterpart; this is a deployment entry point.
  *
  * It allocates nothing: no problem handle, no cudaMalloc/cudaFree, no
- * allocating library call.  Its scratch is a fixed device array of 9.44 MB
- * (9,437,192 bytes; every GPU that loads this library holds it until the
+ * allocating library call.  Its scratch is a fixed device array of 13.1 MB
+ * (13,107,208 bytes; every GPU that loads this library holds it until the
  * process exits), which
  * bounds the input: k <= 524,288 columns and nnz <= 33,554,432 non-zeros;
  * larger inputs, a non-finite or negative lambda return GENCD_EINVAL.  The
@@ -354,7 +354,7 @@ int gencd_set_propose_schedule(gencd_problem* p, int32_t split);
  * satisfy the CSC rules of gencd_create): col_ptr int64[k+1], row_idx
  * int32[nnz], val double[nnz], y double[n], z = Xw double[n], w double[k];
  * loss, lambda >= 0, beta_mode as in gencd_params.  u = l'(y, z) is evaluated
- * on the fly.  Outputs (device): delta, phi double[k], kkt double[1].
+ * into the scratch (n <= 524,288 and n <= nnz) or per non-zero.  Outputs (device): delta, phi double[k], kkt double[1].
  * Work is enqueued on `stream`; the call returns without synchronising.
  */
 int gencd_propose_all_noalloc(int64_t n, int64_t k, int64_t nnz, const int64_t* col_ptr, const int32_t* row_idx,

@@ -172,4 +172,26 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
+// Segmented suffix sums over the lanes, in place: x_L becomes x_L + x_{L+1} +
+// ... + x_M where M is the first lane >= L with stop set (all lanes to 31 when
+// there is none; `ended` reports whether such an M exists), the same for y.
+// FP64: an addition holds the pipe for some 64 cycles a warp, so the steps
+// stop as soon as every lane's run has ended.
+__device__ __forceinline__ void lane_suffix_sum2(double& x, double& y, bool stop, int lane, bool& ended) {
+  bool e = stop;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const bool open = !e && lane + d < 32;
+    if (!__any_sync(0xffffffffu, open)) break;
+    const double xn = __shfl_down_sync(0xffffffffu, x, d), yn = __shfl_down_sync(0xffffffffu, y, d);
+    const bool en = __shfl_down_sync(0xffffffffu, (int)e, d) != 0;
+    if (open) {
+      x += xn;
+      y += yn;
+      e = en;
+    }
+  }
+  ended = e;
+}
+
 }  // namespace gencd

@@ -128,6 +128,36 @@ def test_noalloc_at_its_size_limit_then_on_a_smaller_problem(gb):
     _check_against_oracle(gb, small, lam_s, 0, w_s, calls=2)
 
 
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("n,k,nnz", [(1 << 19, 700, 600_001), ((1 << 19) + 1, 700, 600_001), (5000, 300, 4_999),
+                                     (40, 3, 9), (900, 2000, 16_383)])
+def test_noalloc_with_u_in_the_scratch_or_per_non_zero(gb, n, k, nnz, offset):
+    # both sides of the rows that fit the scratch and of n <= nnz; ragged last
+    # tiles; offset 1: arrays that are not 16-byte aligned (scalar loads)
+    import torch
+
+    prob = workloads.zipf_problem(n, k, nnz, cap=max(4, n // 4), n_planted=3, loss="logistic", seed=n % 97)
+    lam = 0.1 * oracle.Oracle(prob).lambda_max()
+    w = np.where(np.random.default_rng(2).random(prob.k) < 0.2, 0.1, 0.0)
+    orc = oracle.Oracle(prob, lam)
+    z = orc.fitted(w)
+    J = np.arange(prob.k, dtype=np.int32)
+    d_cpu, f_cpu = orc.propose(w, z, J)
+
+    def t(a):
+        buf = torch.zeros(a.size + offset, dtype=torch.from_numpy(a[:1].copy()).dtype, device="cuda")
+        buf[offset:] = torch.from_numpy(np.ascontiguousarray(a)).cuda()
+        return buf[offset:]
+
+    out = [torch.full((prob.k,), float("nan"), dtype=torch.float64, device="cuda") for _ in range(2)]
+    kkt = torch.full((1,), float("nan"), dtype=torch.float64, device="cuda")
+    gb.gencd_propose_all_noalloc(prob.n, prob.k, prob.nnz, t(prob.col_ptr), t(prob.row_idx), t(prob.val), t(prob.y),
+                                 t(z), t(w), prob.loss, lam, 0, *out, kkt)
+    torch.cuda.synchronize()
+    assert_steps_close(prob, z, w, lam, J, out[0].cpu().numpy(), out[1].cpu().numpy(), d_cpu, f_cpu, TOL["f64"])
+    assert kkt.item() == pytest.approx(orc.kkt(w, z), rel=1e-9, abs=1e-15)
+
+
 def test_noalloc_rejects_inputs_beyond_its_scratch(gb):
     import torch
 
