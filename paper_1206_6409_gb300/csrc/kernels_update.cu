@@ -266,6 +266,11 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+__global__ void k_mirror_w(const double* __restrict__ w, int64_t k, float* __restrict__ w32) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < k; j += stride) w32[j] = w_mirror(w[j]);
+}
+
 // z = X w from the columns with w_j != 0, in segments of kSegEntries
 // non-zeros so that a long column is spread over many warps.  Pass 1 lists the
 // segments (writes the float copy of w and zeroes z): a CTA counts its columns'
@@ -498,7 +503,30 @@ int launch_coloring_iter(gencd_problem* p, int64_t q) {
 // columns with w_j != 0, scattered / by rows, on 4.0e7 FP32 non-zeros 48 / 276
 // us at 0.5%, 84 / 276 at 12.5%, 155 / 276 at 40%, 309 / 276 at 100%, and on
 // 2.0e7 FP64 non-zeros 52 / 123, 74 / 123, 116 / 123 and 164 / 123 us.
+//
+// At most kFitRowsNnz non-zeros: always by rows.  Reading all of X takes no
+// longer there than listing w's segments, and the sums have a fixed order, so
+// that equal problems get equal z to the last bit (the scatter's atomic adds
+// do not).
+constexpr int64_t kFitRowsNnz = int64_t(1) << 20;
+
+static int state_by_rows(gencd_problem* p) {
+  GENCD_TRY(build_csr(p));
+  GENCD_TRY(launch_csr_spmv(p, p->w, p->z));
+  GENCD_TRY(launch_fill_u(p));
+  GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
+  return GENCD_OK;
+}
+
 int launch_state_from_w(gencd_problem* p) {
+  if (p->nnz <= kFitRowsNnz) {
+    if (p->w32) {
+      k_mirror_w<<<grid_for(p->k, kThreads, p->num_sms * 8), kThreads, 0, p->stream>>>(p->w, p->k, p->w32);
+      p->prof.launches[K_SETUP] += 1;
+      GENCD_CUDA_TRY(cudaGetLastError());
+    }
+    return state_by_rows(p);
+  }
   unsigned long long* total = reinterpret_cast<unsigned long long*>(p->dscal + kScalFit);  // zero between calls
   unsigned long long* count = total + 1;
   unsigned long long* host = reinterpret_cast<unsigned long long*>(p->hpin + kScalFit);
@@ -518,11 +546,7 @@ int launch_state_from_w(gencd_problem* p) {
   GENCD_TRY(launch_fill_u(p, total, host));
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
   if (host[0] <= limit && host[1] <= (unsigned long long)p->k) return GENCD_OK;
-  GENCD_TRY(build_csr(p));
-  GENCD_TRY(launch_csr_spmv(p, p->w, p->z));
-  GENCD_TRY(launch_fill_u(p));
-  GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
-  return GENCD_OK;
+  return state_by_rows(p);
 }
 
 int launch_csr_spmv(gencd_problem* p, const double* x, double* out) {

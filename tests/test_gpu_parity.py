@@ -818,17 +818,21 @@ def test_accept_takes_each_partitions_best_column(gb, precision, k, B):
 
 @pytest.mark.parametrize("precision", ["f64", "f32"])
 @pytest.mark.parametrize("frac", [0.0, 0.002, 0.3, 0.5, 1.0])
-def test_set_w_fits_sparse_and_dense_coefficients(gb, precision, frac):
-    # on both sides of the line between scattering columns and summing rows,
-    # columns of many segments among them; a second call starts from scratch
-    prob = ragged_problem("squared", 4)
+@pytest.mark.parametrize("large", [False, True])
+def test_set_w_fits_sparse_and_dense_coefficients(gb, precision, frac, large):
+    # below and above the size from which columns are scattered, there on both
+    # sides of the line between scattering columns and summing rows, columns
+    # of many segments among them; a second call starts from scratch
+    prob = (workloads.zipf_problem(60_000, 8_000, 1_200_000, cap=50_000, n_planted=10, loss="squared", seed=4)
+            if large else ragged_problem("squared", 4))
+    longest = int(np.argmax(prob.col_nnz()))
     orc = oracle.Oracle(prob)
     rng = np.random.default_rng(8)
     with gb.Problem(prob, precision=precision) as p:
         for _ in range(2):
             w = np.where(rng.random(prob.k) < frac, rng.normal(0, 0.5, prob.k), 0.0)
             if frac == 0.002:
-                w[16] = 0.7  # the column of 50,000 non-zeros alone is 81% of X
+                w[longest] = 0.7  # a column of 50,000 non-zeros
             p.set_w(w)
             # sums of at most a few hundred terms of size 10 in FP64 (stored values rounded to FP32)
             np.testing.assert_allclose(p.z(), orc.fitted(w), rtol=0, atol=1e-11 if precision == "f64" else 2e-5)
