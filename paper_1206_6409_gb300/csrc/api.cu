@@ -321,6 +321,20 @@ static int launch_top_accept(gencd_problem* p, int64_t B) {
   return GENCD_OK;
 }
 
+// Shotgun's iteration on the selected list J (Jacobi: every proposal from the
+// start state's u)
+static int shotgun_on_list(gencd_problem* p, const int32_t* J, int64_t m) {
+  if (p->params.improve_steps <= 0) {
+    GENCD_TRY(launch_shotgun_step(p, J, m));
+    return launch_refresh_list(p, J, m, false);
+  }
+  GENCD_TRY(launch_propose_list(p, J, m, p->list_d, p->phi));
+  GENCD_TRY(launch_improve_list(p, J, p->list_d, m));  // Improve delta_j: from the start state's z
+  GENCD_TRY(launch_apply_list(p, J, p->list_d, m));
+  GENCD_TRY(launch_update_list(p, J, p->list_d, m));
+  return launch_refresh_list(p, J, m, true);
+}
+
 // one GenCD iteration (Algorithm 1) of the configured variant, enqueued
 static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt) {
   const int v = p->params.variant;
@@ -328,11 +342,16 @@ static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt)
     const int B = effective_B(p);
     if (want_kkt) GENCD_CUDA_TRY(cudaMemsetAsync(p->dscal, 0, sizeof(double), p->stream));  // KKT maximum
     GENCD_TRY(launch_propose_all(p, p->u, p->precision == GENCD_F64));  // Propose, all columns
-    GENCD_TRY(launch_finalize_accept(p, B, want_kkt));  // step, proxy (+ KKT of the start state); Accept
-    GENCD_TRY(launch_merge_accept(p, B));               // accept backoff (groups of partitions), if any
-    GENCD_TRY(launch_improve_list(p, p->list_j, p->list_d, B));  // Improve delta_j (Algorithm 3), if asked
-    GENCD_TRY(launch_update_list(p, p->list_j, p->list_d, B, true));     // Update (atomic z)
-    GENCD_TRY(launch_refresh_list(p, p->list_j, p->list_d, B, true));
+    // the accepted steps go into w at once unless they still change
+    const bool settled = p->accept_group <= 1 && p->params.improve_steps <= 0;
+    GENCD_TRY(launch_finalize_accept(p, B, want_kkt, settled));  // step, proxy (+ KKT of the start state); Accept
+    if (!settled) {
+      GENCD_TRY(launch_merge_accept(p, B));             // accept backoff (groups of partitions), if any
+      GENCD_TRY(launch_improve_list(p, p->list_j, p->list_d, B));  // Improve delta_j (Algorithm 3), if asked
+      GENCD_TRY(launch_apply_list(p, p->list_j, p->list_d, B));
+    }
+    GENCD_TRY(launch_update_list(p, p->list_j, p->list_d, B));  // Update (atomic z)
+    GENCD_TRY(launch_refresh_list(p, p->list_j, B, true));
     *host_nnz += p->nnz;
     p->stat_host_nnz += p->nnz;
   } else if (v == GENCD_TOP_GREEDY) {
@@ -343,8 +362,9 @@ static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt)
     GENCD_TRY(launch_finalize(p, p->lambda, true));    // delta, phi of every column (+ KKT of the start state)
     GENCD_TRY(launch_top_accept(p, B));                 // Accept: the B lowest proxies
     GENCD_TRY(launch_improve_list(p, p->list_j, p->list_d, B));
-    GENCD_TRY(launch_update_list(p, p->list_j, p->list_d, B, true));  // Update (atomic z)
-    GENCD_TRY(launch_refresh_list(p, p->list_j, p->list_d, B, true));
+    GENCD_TRY(launch_apply_list(p, p->list_j, p->list_d, B));
+    GENCD_TRY(launch_update_list(p, p->list_j, p->list_d, B));  // Update (atomic z)
+    GENCD_TRY(launch_refresh_list(p, p->list_j, B, true));
     *host_nnz += p->nnz;
     p->stat_host_nnz += p->nnz;
   } else if (v == GENCD_SHOTGUN) {
@@ -356,10 +376,7 @@ static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt)
     GENCD_TRY(ensure_selection(p, e, p->k));                             // Select, random subset
     const int64_t lo = q * P, m = (lo + P <= p->k ? P : p->k - lo);
     const int32_t* J = p->perm + lo;
-    GENCD_TRY(launch_propose_list(p, J, m, p->list_d, p->phi));          // Propose (Jacobi)
-    GENCD_TRY(launch_improve_list(p, J, p->list_d, m));                  // Improve delta_j, if asked
-    GENCD_TRY(launch_update_list(p, J, p->list_d, m, false));            // Accept all, Update
-    GENCD_TRY(launch_refresh_list(p, J, p->list_d, m, false));
+    GENCD_TRY(shotgun_on_list(p, J, m));                                 // Propose, Accept all, Update
   } else if (v == GENCD_SHOTGUN_BLOCKS) {
     const int32_t B = (int32_t)std::min<int64_t>(p->params.blocks > 0 ? p->params.blocks : 16, p->k);
     GENCD_TRY(compute_block_pstar(p, B));
@@ -379,10 +396,7 @@ static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt)
     k_block_select<<<1, kThreads, 0, p->stream>>>(p->t, B, p->block_lo, p->block_P, p->perm, p->list_j);
     p->prof.launches[K_SETUP] += 1;
     GENCD_CUDA_TRY(cudaGetLastError());
-    GENCD_TRY(launch_propose_list(p, p->list_j, m, p->list_d, p->phi));  // Propose (Jacobi)
-    GENCD_TRY(launch_improve_list(p, p->list_j, p->list_d, m));         // Improve delta_j, if asked
-    GENCD_TRY(launch_update_list(p, p->list_j, p->list_d, m, false));   // Accept all, Update
-    GENCD_TRY(launch_refresh_list(p, p->list_j, p->list_d, m, false));
+    GENCD_TRY(shotgun_on_list(p, p->list_j, m));                        // Propose, Accept all, Update
   } else if (v == GENCD_COLORING) {
     if (!p->color) GENCD_TRY(run_coloring(p));
     const int64_t C = p->ncolors;

@@ -172,6 +172,15 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
+// w_j += d of an accepted column (w32: FP32 mode's copy) and its list entry:
+// the column's length, flagged as applied (kApplied)
+__device__ __forceinline__ uint32_t apply_column(int32_t j, double d, const int64_t* col_ptr, double* w, float* w32) {
+  const double wn = w[j] + d;
+  w[j] = wn;
+  if (w32) w32[j] = w_mirror(wn);
+  return (uint32_t)(col_ptr[j + 1] - col_ptr[j]) | 0x80000000u;
+}
+
 // Segmented suffix sums over the lanes, in place: x_L becomes x_L + x_{L+1} +
 // ... + x_M where M is the first lane >= L with stop set (all lanes to 31 when
 // there is none; `ended` reports whether such an M exists), the same for y.

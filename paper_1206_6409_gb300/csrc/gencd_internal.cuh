@@ -54,11 +54,10 @@ constexpr int kThreads = 256;  // default CTA size
 constexpr int kValPlain = 0;  // the storage precision's values
 constexpr int kValBf16 = 1;   // bfloat16 (GENCD_BF16)
 constexpr int kValNone = 2;   // index only, one value per column (GENCD_BINARY)
-// the single-CTA plan of an update list (lengths, prefix, w) takes lists of at
-// most kListPlanMax entries
-constexpr int kListPlanThreads = 1024;
-constexpr int kListPlanPer = 4;
-constexpr int64_t kListPlanMax = (int64_t)kListPlanThreads * kListPlanPer;
+// the passes over an update list sum its lengths in shared memory when it has
+// at most kListScanMax entries
+constexpr int kListScanMax = 4096;
+constexpr uint32_t kApplied = 0x80000000u;  // list_off entry, before its prefix sum: the column was applied
 constexpr int32_t kMaxShotgunBlocks = 1024;  // column blocks of block Shotgun (one selection CTA)
 constexpr int kScalars = 16;  // device scalars of a problem (dscal / hpin)
 constexpr int kScalFit = 10;  // the first of the two that z = Xw uses
@@ -201,7 +200,7 @@ struct gencd_problem {
   double* w_start = nullptr;    // w at the start of a solve (restarts of the accept backoff)
   int64_t accept_group = 1;     // Thread-Greedy partitions merged per accept group (1: none)
   double* list_d = nullptr;
-  uint32_t* list_off = nullptr;  // exclusive prefix of the listed columns' nnz (k + 2)
+  uint32_t* list_off = nullptr;  // the listed columns' nnz | kApplied, or their exclusive prefix (k + 2)
   uint32_t* scan_tmp = nullptr;  // scratch of the prefix sum
 
   // Thread-Greedy partition bounds floor(b k / B), b = 0..part_B
@@ -284,7 +283,8 @@ int launch_propose_plan(gencd_problem* p, const void* u_vec);
 int tune_propose_plan(gencd_problem* p);  // picks the fastest form of the streaming propose
 void free_propose_plan(gencd_problem* p);
 int launch_finalize(gencd_problem* p, double lambda, bool write_steps);
-int launch_finalize_accept(gencd_problem* p, int64_t B, bool want_kkt);  // Thread-Greedy / Greedy
+// Thread-Greedy / Greedy; apply: the accepted columns' w and list_off too
+int launch_finalize_accept(gencd_problem* p, int64_t B, bool want_kkt, bool apply);
 int launch_merge_accept(gencd_problem* p, int64_t B);  // keep the best of every accept_group partitions
 // Improve delta_j (Algorithm 3): refine the accepted steps D[e] of columns
 // J[e] >= 0 in place (params.improve_steps Eq. 7 steps each; 0: nothing)
@@ -311,8 +311,10 @@ int launch_inv_beta(gencd_problem* p);   // ib_j = 1 / beta_j for the current be
 // kernels_update.cu
 // u = l'(y, z); with report (pinned host memory), counts[0..1] are copied there and reset
 int launch_fill_u(gencd_problem* p, unsigned long long* counts = nullptr, unsigned long long* report = nullptr);
-int launch_update_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m, bool skip_neg);
-int launch_refresh_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m, bool skip_neg);
+int launch_apply_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m);   // w, list_off
+int launch_update_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m);  // z (after w)
+int launch_refresh_list(gencd_problem* p, const int32_t* J, int64_t m, bool counted);    // u (after z)
+int launch_shotgun_step(gencd_problem* p, const int32_t* J, int64_t m);                  // propose, w and z
 int launch_coloring_iter(gencd_problem* p, int64_t q);
 int launch_csr_spmv(gencd_problem* p, const double* x, double* out);  // out = X x (FP64)
 int launch_state_from_w(gencd_problem* p);  // z, u and w32 from p->w (synchronises the stream)

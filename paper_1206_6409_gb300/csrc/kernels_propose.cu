@@ -354,7 +354,8 @@ __device__ __forceinline__ int scan_round_f32(float* __restrict__ gacc, const fl
 // columns, one CTA each; with more than one chunk the chunk winners go to
 // slots, and the CTA that finishes a partition last (a counter per partition)
 // picks among them.  want_kkt: also reduce the KKT violation (convergence
-// checks only).  Idle columns (phi = 0) are never accepted.
+// checks only).  Idle columns (phi = 0) are never accepted.  list_len not
+// null: the accepted step goes into w at once, for the passes that follow.
 //
 // Bound: latency (a few dependent loads and block reductions per CTA), so
 // what counts is that every chunk is resident at once and that no thread
@@ -373,7 +374,8 @@ __global__ void __launch_bounds__(kThreads)
                         const int64_t* __restrict__ part_lo, int want_kkt, uint64_t* __restrict__ slot_m,
                         int32_t* __restrict__ slot_j, double* __restrict__ slot_x, unsigned int* __restrict__ slot_cnt,
                         int32_t* __restrict__ list_j, double* __restrict__ list_d, uint64_t* __restrict__ list_m,
-                        double* __restrict__ kkt_out) {
+                        double* __restrict__ kkt_out, const int64_t* __restrict__ col_ptr, double* w_out,
+                        float* w32_out, uint32_t* __restrict__ list_len) {
   constexpr bool F32 = sizeof(G) == 4;
   using J = typename std::conditional<F32, int32_t, int64_t>::type;
   __shared__ int s_n;  // the active columns of a round, processed packed
@@ -468,6 +470,8 @@ __global__ void __launch_bounds__(kThreads)
       list_j[b] = ok ? bj : -1;
       list_d[b] = ok ? d : 0.0;
       list_m[b] = ok ? bm : 0ull;
+      // apply: no other CTA reads this partition's w any more
+      if (list_len) list_len[b] = ok && d != 0.0 ? apply_column(bj, d, col_ptr, w_out, w32_out) : 0u;
     }
     __syncthreads();  // the reduction buffers and s_last are reused
   }
@@ -690,7 +694,7 @@ static int ensure_part_bounds(gencd_problem* p, int64_t B) {
 // Chunk size of k_accept_partitions: the smallest of 256, 512, ... columns
 // that keeps the launch within 8 CTAs per SM (all resident at once); a
 // partition that fits one chunk is one CTA and needs no slots.
-int launch_finalize_accept(gencd_problem* p, int64_t B, bool want_kkt) {
+int launch_finalize_accept(gencd_problem* p, int64_t B, bool want_kkt, bool apply) {
   uint64_t b64;
   uint32_t b32;
   lambda_bits(p, p->lambda, &b64, &b32);
@@ -710,11 +714,13 @@ int launch_finalize_accept(gencd_problem* p, int64_t B, bool want_kkt) {
   if (f64)
     k_accept_partitions<double><<<grid, kThreads, 0, p->stream>>>(
         (double*)p->gnat, c, B, (int)per, chunk, p->part_lo, want_kkt ? 1 : 0, p->slot_m, p->slot_j, p->slot_d,
-        p->slot_cnt, p->list_j, p->list_d, p->list_m, p->dscal + 0);
+        p->slot_cnt, p->list_j, p->list_d, p->list_m, p->dscal + 0, p->col_ptr, p->w, p->w32,
+        apply ? p->list_off : nullptr);
   else
     k_accept_partitions<float><<<grid, kThreads, 0, p->stream>>>(
         (float*)p->gnat, c, B, (int)per, chunk, p->part_lo, want_kkt ? 1 : 0, p->slot_m, p->slot_j, p->slot_d,
-        p->slot_cnt, p->list_j, p->list_d, p->list_m, p->dscal + 0);
+        p->slot_cnt, p->list_j, p->list_d, p->list_m, p->dscal + 0, p->col_ptr, p->w, p->w32,
+        apply ? p->list_off : nullptr);
   prof_end(p, ev);
   GENCD_CUDA_TRY(cudaGetLastError());
   return GENCD_OK;

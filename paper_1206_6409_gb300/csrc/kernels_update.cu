@@ -1,9 +1,11 @@
 // kernels_update.cu -- the Update step of GenCD (Algorithm 3) on sm_103a.
 //
 //  * k_update_flat: z += delta_j X_j for accepted columns that may share rows
-//    (Shotgun, Thread-Greedy, Greedy), FP64 atomic adds into z (the paper's
-//    OpenMP `atomic`, Section 4.2), work spread evenly over the non-zeros of
-//    all accepted columns; k_apply_w does w_j += delta_j.
+//    (Thread-Greedy, Greedy), FP64 atomic adds into z (the paper's OpenMP
+//    `atomic`, Section 4.2), work spread evenly over the non-zeros of all
+//    accepted columns; w_j += delta_j where the column is accepted, or in
+//    k_apply_list.
+//  * k_shotgun_step: Propose and the Update of w and z for Shotgun's list.
 //  * k_refresh_flat: u_i = l'(y_i, z_i) on the rows of the accepted columns,
 //    launched after every atomic add of the iteration has landed.
 //  * k_coloring_iter: one Coloring iteration fused into a single pass: the
@@ -34,37 +36,35 @@ __global__ void __launch_bounds__(kThreads)
 }
 
 // The applied columns of a list (J[e] >= 0 and D[e] != 0) are laid end to end
-// in a virtual range [0, off[m]) (off = exclusive prefix of their lengths), and
-// threads take equal runs of that range: a 50,000-nnz column is spread over
-// the whole GPU instead of one CTA.
-__global__ void k_list_len(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ J,
-                           const double* __restrict__ D, int64_t m, uint32_t* __restrict__ len) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e <= m; e += stride) {
-    uint32_t l = 0;
-    if (e < m) {
-      const int32_t j = J[e];
-      if (j >= 0 && D[e] != 0.0) l = (uint32_t)(col_ptr[j + 1] - col_ptr[j]);
-    }
-    len[e] = l;
-  }
-}
+// in a virtual range [0, total), and threads take equal parts of that range: a
+// 50,000-nnz column is spread over the whole GPU instead of one CTA.
+// Whoever applies the list writes list[e] = the column's length | kApplied, or
+// 0 for an entry that is not applied; the passes over the range prefix-sum it.
 
-// w_j += delta_j for the applied entries (distinct columns), and the counters
-__global__ void k_apply_w(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ J,
-                          const double* __restrict__ D, int64_t m, double* __restrict__ w, float* __restrict__ w32,
-                          unsigned long long* __restrict__ counters) {
+// w_j += delta_j for the applied entries (distinct columns), and list[e]
+__global__ void k_apply_list(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ J,
+                             const double* __restrict__ D, int64_t m, double* __restrict__ w,
+                             float* __restrict__ w32, uint32_t* __restrict__ list) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  unsigned long long upd = 0, work = 0;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += stride) {
     const int32_t j = J[e];
     const double d = D[e];
-    if (j < 0 || d == 0.0) continue;
-    const double wn = w[j] + d;
-    w[j] = wn;
-    if (w32) w32[j] = w_mirror(wn);
-    upd += 1;
-    work += (unsigned long long)(col_ptr[j + 1] - col_ptr[j]);
+    uint32_t l = 0;
+    if (j >= 0 && d != 0.0) l = apply_column(j, d, col_ptr, w, w32);
+    list[e] = l;
+  }
+}
+
+// A list of more than kListScanMax entries: lengths without the flag (list[m]
+// = 0) for the prefix sum in memory, and the counters
+__global__ void k_list_lengths(uint32_t* __restrict__ list, int64_t m, unsigned long long* __restrict__ counters) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  unsigned long long upd = 0, work = 0;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e <= m; e += stride) {
+    const uint32_t v = e < m ? list[e] : 0u;
+    list[e] = v & ~kApplied;
+    upd += v >> 31;
+    work += v & ~kApplied;
   }
   upd = warp_sum(upd);
   work = warp_sum(work);
@@ -74,70 +74,8 @@ __global__ void k_apply_w(const int64_t* __restrict__ col_ptr, const int32_t* __
   }
 }
 
-// One CTA for lists of at most kListPlanMax entries: lengths of the applied
-// entries, their exclusive prefix (off[0..m]), w_j += delta_j and the counters
-// -- k_list_len, the scan and k_apply_w in one launch.
-
-__global__ void __launch_bounds__(kListPlanThreads)
-    k_list_plan(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ J, const double* __restrict__ D,
-                int64_t m, double* __restrict__ w, float* __restrict__ w32, uint32_t* __restrict__ off,
-                unsigned long long* __restrict__ counters) {
-  __shared__ uint32_t s_warp[kListPlanThreads / 32];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  uint32_t len[kListPlanPer];
-  uint32_t mine = 0, upd = 0;
-#pragma unroll
-  for (int q = 0; q < kListPlanPer; ++q) {
-    const int64_t e = (int64_t)tid * kListPlanPer + q;
-    len[q] = 0;
-    if (e < m) {
-      const int32_t j = J[e];
-      const double d = D[e];
-      if (j >= 0 && d != 0.0) {
-        len[q] = (uint32_t)(col_ptr[j + 1] - col_ptr[j]);
-        const double wn = w[j] + d;  // the entries name distinct columns
-        w[j] = wn;
-        if (w32) w32[j] = w_mirror(wn);
-        ++upd;
-      }
-    }
-    mine += len[q];
-  }
-  // block-wide exclusive prefix of the per-thread sums
-  uint32_t incl = mine;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
-    if (lane >= d) incl += y;
-  }
-  if (lane == 31) s_warp[wid] = incl;
-  __syncthreads();
-  if (wid == 0) {
-    uint32_t v = s_warp[lane];
-#pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, v, d);
-      if (lane >= d) v += y;
-    }
-    s_warp[lane] = v;  // inclusive over warps
-  }
-  __syncthreads();
-  uint32_t run = (wid > 0 ? s_warp[wid - 1] : 0u) + incl - mine;
-#pragma unroll
-  for (int q = 0; q < kListPlanPer; ++q) {
-    const int64_t e = (int64_t)tid * kListPlanPer + q;
-    if (e < m) off[e] = run;
-    run += len[q];
-  }
-  const uint32_t total = s_warp[kListPlanThreads / 32 - 1];
-  if (tid == 0) off[m] = total;
-  const unsigned long long u_all = warp_sum((unsigned long long)upd);
-  if (lane == 0 && u_all) atomicAdd(counters + 0, u_all);
-  if (tid == 0 && total) atomicAdd(counters + 1, (unsigned long long)total);
-}
-
 // last entry e in [0, m) with off[e] <= q
-__device__ __forceinline__ int64_t entry_of(const uint32_t* __restrict__ off, int64_t m, uint32_t q) {
+__device__ __forceinline__ int64_t entry_of(const uint32_t* off, int64_t m, uint32_t q) {
   int64_t lo = 0, hi = m - 1;
   while (lo < hi) {
     const int64_t mid = (lo + hi + 1) >> 1;
@@ -149,55 +87,192 @@ __device__ __forceinline__ int64_t entry_of(const uint32_t* __restrict__ off, in
   return lo;
 }
 
-constexpr int kFlatRun = 4;  // consecutive virtual positions per thread
+constexpr int kListThreads = 512;
+
+// The offsets of a list's applied columns, off[0..m].  SCAN (m <=
+// kListScanMax): every CTA sums the list itself, in shared memory, where the
+// searches of its threads then run: 4 KB of L2 reads for 1,024 entries.  On 512
+// accepted columns (20,000 non-zeros) the passes over z and u take 4.0 and 4.3
+// us; with a launch of its own for the offsets (4.8 us) and searches of nine
+// dependent loads in memory they took 4.4 and 6.6.  counters (not null): CTA 0 adds the updates and
+// the non-zeros to them.  Not SCAN: the offsets are in memory already.
+template <bool SCAN>
+__device__ __forceinline__ const uint32_t* list_offsets(const uint32_t* __restrict__ list, int64_t m,
+                                                        uint32_t* s_off, unsigned long long* counters) {
+  if (!SCAN) return list;
+  __shared__ uint32_t s_warp[kListThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, mi = (int)m;
+  uint32_t upd = 0;
+  for (int e = tid; e < mi; e += kListThreads) {
+    const uint32_t v = list[e];
+    upd += v >> 31;
+    s_off[e] = v & ~kApplied;
+  }
+  __syncthreads();
+  const int per = (mi + kListThreads - 1) / kListThreads;
+  const int e0 = min(tid * per, mi), e1 = min(e0 + per, mi);
+  uint32_t mine = 0;
+  for (int e = e0; e < e1; ++e) mine += s_off[e];
+  uint32_t incl = mine;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, d);
+    if (lane >= d) incl += y;
+  }
+  if (lane == 31) s_warp[wid] = incl;
+  __syncthreads();
+  uint32_t run = incl - mine, total = 0;
+#pragma unroll
+  for (int v = 0; v < kListThreads / 32; ++v) {
+    if (v < wid) run += s_warp[v];
+    total += s_warp[v];
+  }
+  for (int e = e0; e < e1; ++e) {
+    const uint32_t x = s_off[e];
+    s_off[e] = run;
+    run += x;
+  }
+  if (tid == 0) s_off[mi] = total;
+  if (counters && blockIdx.x == 0) {
+    upd = warp_sum(upd);
+    if (lane == 0 && upd) atomicAdd(counters + 0, (unsigned long long)upd);
+    if (tid == 0 && total) atomicAdd(counters + 1, (unsigned long long)total);
+  }
+  __syncthreads();
+  return s_off;
+}
 
 // z_i += delta_j X_ij over the applied columns (atomic: columns may share rows)
-template <typename V>
-__global__ void __launch_bounds__(kThreads)
+template <typename V, bool SCAN>
+__global__ void __launch_bounds__(kListThreads)
     k_update_flat(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
                   const V* __restrict__ val, const int32_t* __restrict__ J, const double* __restrict__ D,
-                  const uint32_t* __restrict__ off, int64_t m, double* __restrict__ z) {
-  const uint32_t total = off[m];
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x * kFlatRun;
-  for (int64_t q0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kFlatRun; q0 < total; q0 += stride) {
-    int64_t e = entry_of(off, m, (uint32_t)q0);
-    for (int r = 0; r < kFlatRun; ++r) {
-      const uint32_t q = (uint32_t)(q0 + r);
-      if (q >= total) break;
-      while (q >= off[e + 1]) ++e;
-      const int32_t j = J[e];
-      const int64_t p = col_ptr[j] + (q - off[e]);
-      atomicAdd(z + row_idx[p], D[e] * (double)val[p]);
-    }
+                  const uint32_t* __restrict__ list, int64_t m, double* __restrict__ z,
+                  unsigned long long* __restrict__ counters) {
+  __shared__ uint32_t s_off[SCAN ? kListScanMax + 1 : 1];
+  const uint32_t* off = list_offsets<SCAN>(list, m, s_off, counters);
+  const int64_t total = off[m], stride = (int64_t)gridDim.x * kListThreads;
+  for (int64_t q = (int64_t)blockIdx.x * kListThreads + threadIdx.x; q < total; q += stride) {
+    const int64_t e = entry_of(off, m, (uint32_t)q);
+    const int64_t p = col_ptr[J[e]] + ((uint32_t)q - off[e]);
+    atomicAdd(z + row_idx[p], D[e] * (double)val[p]);
   }
 }
 
 // u_i = l'(y_i, z_i) on the rows of the applied columns, or on all rows when
-// the iteration touched at least n entries (one dense pass is cheaper then)
-template <typename U>
-__global__ void __launch_bounds__(kThreads)
+// the iteration touched at least n entries (one dense pass is cheaper then).
+// Neighbouring warps of the range lie on different SMs: the logistic
+// derivative takes some 50 FP64 operations, which an SM starts about two a
+// cycle, so few rows have to be spread over all of them (FP64, 100,000 rows:
+// 7.7 us, 12.1 with neighbouring warps in one CTA).
+template <typename U, bool SCAN>
+__global__ void __launch_bounds__(kListThreads)
     k_refresh_flat(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
-                   const int32_t* __restrict__ J, const uint32_t* __restrict__ off, int64_t m,
+                   const int32_t* __restrict__ J, const uint32_t* __restrict__ list, int64_t m,
                    const double* __restrict__ y, const double* __restrict__ z, int64_t n, int loss,
-                   U* __restrict__ u) {
-  const uint32_t total = off[m];
-  if ((int64_t)total >= n) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-      u[i] = u_value<U>(loss, y[i], z[i]);
+                   U* __restrict__ u, unsigned long long* __restrict__ counters) {
+  __shared__ uint32_t s_off[SCAN ? kListScanMax + 1 : 1];
+  const uint32_t* off = list_offsets<SCAN>(list, m, s_off, counters);
+  const int64_t total = off[m], stride = (int64_t)gridDim.x * kListThreads;
+  const int64_t q0 = ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
+  if (total >= n) {
+    for (int64_t i = q0; i < n; i += stride) u[i] = u_value<U>(loss, y[i], z[i]);
     return;
   }
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x * kFlatRun;
-  for (int64_t q0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kFlatRun; q0 < total; q0 += stride) {
-    int64_t e = entry_of(off, m, (uint32_t)q0);
-    for (int r = 0; r < kFlatRun; ++r) {
-      const uint32_t q = (uint32_t)(q0 + r);
-      if (q >= total) break;
-      while (q >= off[e + 1]) ++e;
-      const int64_t p = col_ptr[J[e]] + (q - off[e]);
-      const int32_t i = row_idx[p];
-      u[i] = u_value<U>(loss, y[i], z[i]);
+  for (int64_t q = q0; q < total; q += stride) {
+    const int64_t e = entry_of(off, m, (uint32_t)q);
+    const int32_t i = row_idx[col_ptr[J[e]] + ((uint32_t)q - off[e])];
+    u[i] = u_value<U>(loss, y[i], z[i]);
+  }
+}
+
+// Shotgun's Propose, Accept (all of J) and the Update of w and z in one pass:
+// a proposal reads u and its own w_j only, so its column's step goes into z at
+// once (u follows when all have landed: k_refresh_flat).  A CTA takes `per`
+// <= 8 columns, one a warp; a column of more than kWarpColumn entries is left
+// to the whole CTA.
+//
+// Bound: latency (dependent loads, then the FP64 step), so every column has
+// its own warp at once and long ones 256 threads: this takes 13 us on 800
+// columns of 1 to 5,000 non-zeros (FP32); one warp a column took 32, with a
+// launch each for the list's plan (4.4) and z (5.2) after it.  The step is evaluated by one thread: a warp's
+// FP64 instruction holds the pipe for some 16 cycles an SM.
+constexpr int kWarpColumn = 256;
+constexpr int kShotgunCols = kThreads / 32;
+
+template <typename V, typename U>
+__global__ void __launch_bounds__(kThreads)
+    k_shotgun_step(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
+                   const V* __restrict__ val, const U* __restrict__ u, const double* __restrict__ bjs,
+                   const double* __restrict__ ib, const int32_t* __restrict__ J, int64_t m, int per, double n,
+                   double lam, double* __restrict__ w, float* __restrict__ w32, double* __restrict__ z,
+                   uint32_t* __restrict__ list, unsigned long long* __restrict__ counters) {
+  __shared__ int64_t s_long[kShotgunCols];
+  __shared__ int s_nlong;
+  __shared__ uint32_t s_len[kShotgunCols];
+  __shared__ double s_sum[kThreads / 32], s_d;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (tid == 0) s_nlong = 0;
+  if (lane == 0) s_len[wid] = 0u;
+  __syncthreads();
+  const int64_t first = (int64_t)blockIdx.x * per;
+  auto step = [&](int64_t e, int32_t j, double sum) {  // one thread: the column's step, applied to w
+    double d, f;
+    eq7_step(sum / n, w[j], lam, bjs[j], ib[j], d, f);
+    list[e] = d != 0.0 ? apply_column(j, d, col_ptr, w, w32) : 0u;
+    return d;
+  };
+  if (wid < per && first + wid < m) {
+    const int64_t e = first + wid;
+    const int32_t j = J[e];
+    const int64_t s = col_ptr[j];
+    const uint32_t len = (uint32_t)(col_ptr[j + 1] - s);
+    if (lane == 0) s_len[wid] = len;
+    if (len > (uint32_t)kWarpColumn) {
+      if (lane == 0) s_long[atomicAdd(&s_nlong, 1)] = e;
+    } else {
+      V acc = V(0);
+#pragma unroll 4
+      for (uint32_t t = lane; t < len; t += 32) acc = fma(val[s + t], (V)u[row_idx[s + t]], acc);
+      const double sum = warp_sum((double)acc);
+      double d = 0.0;
+      if (lane == 0) d = step(e, j, sum);
+      d = __shfl_sync(0xffffffffu, d, 0);
+      if (d != 0.0) {
+#pragma unroll 4
+        for (uint32_t t = lane; t < len; t += 32) atomicAdd(z + row_idx[s + t], d * (double)val[s + t]);
+      }
     }
+  }
+  __syncthreads();
+  const int nlong = s_nlong;
+  for (int q = 0; q < nlong; ++q) {  // uniform across the CTA
+    const int64_t e = s_long[q];
+    const int32_t j = J[e];
+    const int64_t s = col_ptr[j];
+    const uint32_t len = (uint32_t)(col_ptr[j + 1] - s);
+    V acc = V(0);
+#pragma unroll 4
+    for (uint32_t t = tid; t < len; t += kThreads) acc = fma(val[s + t], (V)u[row_idx[s + t]], acc);
+    const double part = warp_sum((double)acc);
+    if (lane == 0) s_sum[wid] = part;
+    __syncthreads();
+    if (tid == 0) {
+      double sum = 0.0;
+      for (int v = 0; v < kThreads / 32; ++v) sum += s_sum[v];
+      s_d = step(e, j, sum);
+    }
+    __syncthreads();
+    const double d = s_d;
+    if (d != 0.0) {
+#pragma unroll 4
+      for (uint32_t t = tid; t < len; t += kThreads) atomicAdd(z + row_idx[s + t], d * (double)val[s + t]);
+    }
+  }
+  if (tid == 0) {  // the non-zeros proposed on
+    unsigned long long work = 0;
+    for (int v = 0; v < kShotgunCols; ++v) work += s_len[v];
+    if (work) atomicAdd(counters + 1, work);
   }
 }
 
@@ -431,44 +506,89 @@ int launch_fill_u(gencd_problem* p, unsigned long long* counts, unsigned long lo
   return GENCD_OK;
 }
 
-// Update (Algorithm 3) for the list (J, d): w, then z (atomic), then u.
-int launch_update_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m, bool) {
+// w and list_off for the accepted entries of the list (J, d)
+int launch_apply_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m) {
+  if (m <= 0) return GENCD_OK;
+  k_apply_list<<<grid_for(m, kThreads, p->num_sms * 8), kThreads, 0, p->stream>>>(p->col_ptr, J, d, m, p->w, p->w32,
+                                                                                  p->list_off);
+  p->prof.launches[K_UPDATE] += 1;
+  GENCD_CUDA_TRY(cudaGetLastError());
+  return GENCD_OK;
+}
+
+// a long list's offsets, in list_off, and its counts
+static int prefix_long_list(gencd_problem* p, int64_t m) {
+  unsigned long long* ctr = reinterpret_cast<unsigned long long*>(p->dscal + 4);
+  k_list_lengths<<<grid_for(m + 1, kThreads, p->num_sms * 8), kThreads, 0, p->stream>>>(p->list_off, m, ctr);
+  p->prof.launches[K_UPDATE] += 1;
+  GENCD_CUDA_TRY(cudaGetLastError());
+  return exclusive_scan(p, p->list_off, p->list_off, m + 1, p->scan_tmp);
+}
+
+// CTAs of the passes over a list: two per SM, all resident
+static int list_grid(const gencd_problem* p) { return p->num_sms * 2; }
+
+// Update (Algorithm 3) of z for the list (J, d) whose w has been applied
+// (list_off), and the counters
+int launch_update_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m) {
   if (m <= 0) return GENCD_OK;
   unsigned long long* ctr = reinterpret_cast<unsigned long long*>(p->dscal + 4);
-  const int g = p->num_sms * 8;
+  const bool scan = m <= kListScanMax;
+  if (!scan) GENCD_TRY(prefix_long_list(p, m));
   cudaEvent_t ev = nullptr;
-  const bool one_cta = m <= kListPlanMax;
-  prof_begin(p, K_UPDATE, &ev, one_cta ? 2 : 3);  // plan kernel(s) and the scatter (+ the scan)
-  if (one_cta) {
-    k_list_plan<<<1, kListPlanThreads, 0, p->stream>>>(p->col_ptr, J, d, m, p->w, p->w32, p->list_off, ctr);
-  } else {
-    k_list_len<<<grid_for(m + 1, kThreads, g), kThreads, 0, p->stream>>>(p->col_ptr, J, d, m, p->list_off);
-    GENCD_TRY(exclusive_scan(p, p->list_off, p->list_off, m + 1, p->scan_tmp));
-    k_apply_w<<<grid_for(m, kThreads, g), kThreads, 0, p->stream>>>(p->col_ptr, J, d, m, p->w, p->w32, ctr);
-  }
+  prof_begin(p, K_UPDATE, &ev);
+  auto go = [&](auto kernel, auto* val) {
+    kernel<<<list_grid(p), kListThreads, 0, p->stream>>>(p->col_ptr, p->row_idx, val, J, d, p->list_off, m, p->z, ctr);
+  };
   if (p->precision == GENCD_F64)
-    k_update_flat<double><<<g, kThreads, 0, p->stream>>>(p->col_ptr, p->row_idx, (const double*)p->val, J, d,
-                                                         p->list_off, m, p->z);
+    go(scan ? k_update_flat<double, true> : k_update_flat<double, false>, (const double*)p->val);
   else
-    k_update_flat<float><<<g, kThreads, 0, p->stream>>>(p->col_ptr, p->row_idx, (const float*)p->val, J, d,
-                                                        p->list_off, m, p->z);
+    go(scan ? k_update_flat<float, true> : k_update_flat<float, false>, (const float*)p->val);
   prof_end(p, ev);
   GENCD_CUDA_TRY(cudaGetLastError());
   return GENCD_OK;
 }
 
-// needs the prefix list_off left by launch_update_list for the same list
-int launch_refresh_list(gencd_problem* p, const int32_t* J, const double*, int64_t m, bool) {
+// u on the rows of the list's applied columns, after z.  counted: the list's
+// counts are in the counters already (launch_update_list); else (Shotgun's
+// fused step) they are added here.
+int launch_refresh_list(gencd_problem* p, const int32_t* J, int64_t m, bool counted) {
   if (m <= 0) return GENCD_OK;
-  const int g = p->num_sms * 8;
+  unsigned long long* ctr = counted ? nullptr : reinterpret_cast<unsigned long long*>(p->dscal + 4);
+  const bool scan = m <= kListScanMax;
+  if (!scan && !counted) GENCD_TRY(prefix_long_list(p, m));
   cudaEvent_t ev = nullptr;
   prof_begin(p, K_REFRESH, &ev);
+  auto go = [&](auto kernel, auto* u) {
+    kernel<<<list_grid(p), kListThreads, 0, p->stream>>>(p->col_ptr, p->row_idx, J, p->list_off, m, p->y, p->z, p->n,
+                                                         p->loss, u, ctr);
+  };
   if (p->precision == GENCD_F64)
-    k_refresh_flat<double><<<g, kThreads, 0, p->stream>>>(p->col_ptr, p->row_idx, J, p->list_off, m, p->y, p->z,
-                                                           p->n, p->loss, (double*)p->u);
+    go(scan ? k_refresh_flat<double, true> : k_refresh_flat<double, false>, (double*)p->u);
   else
-    k_refresh_flat<float><<<g, kThreads, 0, p->stream>>>(p->col_ptr, p->row_idx, J, p->list_off, m, p->y, p->z,
-                                                          p->n, p->loss, (float*)p->u);
+    go(scan ? k_refresh_flat<float, true> : k_refresh_flat<float, false>, (float*)p->u);
+  prof_end(p, ev);
+  GENCD_CUDA_TRY(cudaGetLastError());
+  return GENCD_OK;
+}
+
+// Shotgun's iteration on the list J up to z: propose, accept all, w and z
+int launch_shotgun_step(gencd_problem* p, const int32_t* J, int64_t m) {
+  if (m <= 0) return GENCD_OK;
+  unsigned long long* ctr = reinterpret_cast<unsigned long long*>(p->dscal + 4);
+  // two CTAs per SM before a CTA takes a second column
+  const int per = (int)std::min<int64_t>(kShotgunCols, (m + 2 * p->num_sms - 1) / (2 * p->num_sms));
+  const unsigned grid = (unsigned)((m + per - 1) / per);
+  cudaEvent_t ev = nullptr;
+  prof_begin(p, K_PROPOSE_LIST, &ev);
+  if (p->precision == GENCD_F64)
+    k_shotgun_step<double, double><<<grid, kThreads, 0, p->stream>>>(
+        p->col_ptr, p->row_idx, (const double*)p->val, (const double*)p->u, p->bj, p->ib, J, m, per, (double)p->n,
+        p->lambda, p->w, p->w32, p->z, p->list_off, ctr);
+  else
+    k_shotgun_step<float, float><<<grid, kThreads, 0, p->stream>>>(
+        p->col_ptr, p->row_idx, (const float*)p->val, (const float*)p->u, p->bj, p->ib, J, m, per, (double)p->n,
+        p->lambda, p->w, p->w32, p->z, p->list_off, ctr);
   prof_end(p, ev);
   GENCD_CUDA_TRY(cudaGetLastError());
   return GENCD_OK;

@@ -837,3 +837,31 @@ def test_set_w_fits_sparse_and_dense_coefficients(gb, precision, frac, large):
             # sums of at most a few hundred terms of size 10 in FP64 (stored values rounded to FP32)
             np.testing.assert_allclose(p.z(), orc.fitted(w), rtol=0, atol=1e-11 if precision == "f64" else 2e-5)
             np.testing.assert_array_equal(p.w(), w)
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+@pytest.mark.parametrize("name,P", [("ragged-logistic", 1), ("ragged-logistic", 326), ("cfg1-logistic", 305),
+                                    ("cfg1-logistic", 4500)])
+def test_shotgun_steps_match(gb, name, P, precision):
+    # one and several columns a CTA, columns at the edges of one warp's share
+    # (255, 256, 257) and far beyond it, empty ones, lists on both sides of
+    # the 4,096 entries summed in shared memory; two steps from the same start
+    prob = PROBLEMS[name]()
+    orc = oracle.Oracle(prob)
+    lam = 0.05 * orc.lambda_max()
+    orc.set_lambda(lam)
+    w0 = _state(prob, 5)
+    w_cpu, z_cpu, _, st = orc.run("shotgun", 2, w=w0, P=P, seed=7)
+    with gb.Problem(prob, precision=precision) as p:
+        p.set_lambda(lam)
+        p.set_params(variant="shotgun", P=P, seed=7)
+        p.set_w(w0)
+        p.stats_reset()
+        p.iterate(2)
+        assert 0 < p.stats().updates <= st[0]  # the oracle counts steps of 0 too
+        w, z = p.w(), p.z()
+    # FP64 sums in another order; FP32: u and the stored values carry 2^-24,
+    # and a column's step divides its sum's error by beta_j
+    tol = 1e-10 if precision == "f64" else 2e-4
+    np.testing.assert_allclose(w, w_cpu, rtol=0, atol=tol * max(1.0, np.abs(w_cpu).max()))
+    np.testing.assert_allclose(z, z_cpu, rtol=0, atol=tol * max(1.0, np.abs(z_cpu).max()))
