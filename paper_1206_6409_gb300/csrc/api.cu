@@ -322,10 +322,10 @@ static int launch_top_accept(gencd_problem* p, int64_t B) {
 }
 
 // Shotgun's iteration on the selected list J (Jacobi: every proposal from the
-// start state's u)
-static int shotgun_on_list(gencd_problem* p, const int32_t* J, int64_t m) {
+// start state's u); early: J was written before the iteration
+static int shotgun_on_list(gencd_problem* p, const int32_t* J, int64_t m, bool early) {
   if (p->params.improve_steps <= 0) {
-    GENCD_TRY(launch_shotgun_step(p, J, m));
+    GENCD_TRY(launch_shotgun_step(p, J, m, early));
     return launch_refresh_list(p, J, m, false);
   }
   GENCD_TRY(launch_propose_list(p, J, m, p->list_d, p->phi));
@@ -376,7 +376,7 @@ static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt)
     GENCD_TRY(ensure_selection(p, e, p->k));                             // Select, random subset
     const int64_t lo = q * P, m = (lo + P <= p->k ? P : p->k - lo);
     const int32_t* J = p->perm + lo;
-    GENCD_TRY(shotgun_on_list(p, J, m));                                 // Propose, Accept all, Update
+    GENCD_TRY(shotgun_on_list(p, J, m, true));                           // Propose, Accept all, Update
   } else if (v == GENCD_SHOTGUN_BLOCKS) {
     const int32_t B = (int32_t)std::min<int64_t>(p->params.blocks > 0 ? p->params.blocks : 16, p->k);
     GENCD_TRY(compute_block_pstar(p, B));
@@ -396,7 +396,7 @@ static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt)
     k_block_select<<<1, kThreads, 0, p->stream>>>(p->t, B, p->block_lo, p->block_P, p->perm, p->list_j);
     p->prof.launches[K_SETUP] += 1;
     GENCD_CUDA_TRY(cudaGetLastError());
-    GENCD_TRY(shotgun_on_list(p, p->list_j, m));                        // Propose, Accept all, Update
+    GENCD_TRY(shotgun_on_list(p, p->list_j, m, false));                 // Propose, Accept all, Update
   } else if (v == GENCD_COLORING) {
     if (!p->color) GENCD_TRY(run_coloring(p));
     const int64_t C = p->ncolors;

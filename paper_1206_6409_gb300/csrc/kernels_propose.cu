@@ -383,6 +383,8 @@ __global__ void __launch_bounds__(kThreads)
   __shared__ G s_g[kRoundCols];
   __shared__ double s_w[F32 ? 1 : kRoundCols];
   __shared__ bool s_last;
+  pdl_trigger();
+  pdl_wait();
   uint64_t vmax64 = 0;
   uint32_t vmax32 = 0;
   const int64_t items = B * per;
@@ -711,18 +713,15 @@ int launch_finalize_accept(gencd_problem* p, int64_t B, bool want_kkt, bool appl
   const int grid = (int)std::min<int64_t>(B * per, 2 * resident);
   cudaEvent_t ev = nullptr;
   prof_begin(p, K_FINALIZE, &ev);
-  if (f64)
-    k_accept_partitions<double><<<grid, kThreads, 0, p->stream>>>(
-        (double*)p->gnat, c, B, (int)per, chunk, p->part_lo, want_kkt ? 1 : 0, p->slot_m, p->slot_j, p->slot_d,
-        p->slot_cnt, p->list_j, p->list_d, p->list_m, p->dscal + 0, p->col_ptr, p->w, p->w32,
-        apply ? p->list_off : nullptr);
-  else
-    k_accept_partitions<float><<<grid, kThreads, 0, p->stream>>>(
-        (float*)p->gnat, c, B, (int)per, chunk, p->part_lo, want_kkt ? 1 : 0, p->slot_m, p->slot_j, p->slot_d,
-        p->slot_cnt, p->list_j, p->list_d, p->list_m, p->dscal + 0, p->col_ptr, p->w, p->w32,
-        apply ? p->list_off : nullptr);
+  auto go = [&](auto kernel, auto* gacc) {
+    return launch_overlapped(kernel, grid, kThreads, 0, p->stream, gacc, c, B, (int)per, chunk, p->part_lo,
+                             want_kkt ? 1 : 0, p->slot_m, p->slot_j, p->slot_d, p->slot_cnt, p->list_j, p->list_d,
+                             p->list_m, p->dscal + 0, p->col_ptr, p->w, p->w32, apply ? p->list_off : nullptr);
+  };
+  const cudaError_t err = f64 ? go(k_accept_partitions<double>, (double*)p->gnat)
+                              : go(k_accept_partitions<float>, (float*)p->gnat);
   prof_end(p, ev);
-  GENCD_CUDA_TRY(cudaGetLastError());
+  GENCD_CUDA_TRY(err);
   return GENCD_OK;
 }
 

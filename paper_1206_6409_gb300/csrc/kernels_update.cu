@@ -150,6 +150,8 @@ __global__ void __launch_bounds__(kListThreads)
                   const uint32_t* __restrict__ list, int64_t m, double* __restrict__ z,
                   unsigned long long* __restrict__ counters) {
   __shared__ uint32_t s_off[SCAN ? kListScanMax + 1 : 1];
+  pdl_trigger();
+  pdl_wait();
   const uint32_t* off = list_offsets<SCAN>(list, m, s_off, counters);
   const int64_t total = off[m], stride = (int64_t)gridDim.x * kListThreads;
   for (int64_t q = (int64_t)blockIdx.x * kListThreads + threadIdx.x; q < total; q += stride) {
@@ -172,6 +174,8 @@ __global__ void __launch_bounds__(kListThreads)
                    const double* __restrict__ y, const double* __restrict__ z, int64_t n, int loss,
                    U* __restrict__ u, unsigned long long* __restrict__ counters) {
   __shared__ uint32_t s_off[SCAN ? kListScanMax + 1 : 1];
+  pdl_trigger();
+  pdl_wait();
   const uint32_t* off = list_offsets<SCAN>(list, m, s_off, counters);
   const int64_t total = off[m], stride = (int64_t)gridDim.x * kListThreads;
   const int64_t q0 = ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
@@ -204,43 +208,60 @@ template <typename V, typename U>
 __global__ void __launch_bounds__(kThreads)
     k_shotgun_step(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
                    const V* __restrict__ val, const U* __restrict__ u, const double* __restrict__ bjs,
-                   const double* __restrict__ ib, const int32_t* __restrict__ J, int64_t m, int per, double n,
-                   double lam, double* __restrict__ w, float* __restrict__ w32, double* __restrict__ z,
+                   const double* __restrict__ ib, const int32_t* __restrict__ J, int64_t m, int per, int early,
+                   double n, double lam, double* __restrict__ w, float* __restrict__ w32, double* __restrict__ z,
                    uint32_t* __restrict__ list, unsigned long long* __restrict__ counters) {
   __shared__ int64_t s_long[kShotgunCols];
   __shared__ int s_nlong;
   __shared__ uint32_t s_len[kShotgunCols];
   __shared__ double s_sum[kThreads / 32], s_d;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  pdl_trigger();
   if (tid == 0) s_nlong = 0;
   if (lane == 0) s_len[wid] = 0u;
   __syncthreads();
   const int64_t first = (int64_t)blockIdx.x * per;
+  const bool mine = wid < per && first + wid < m;  // this warp's column
+  if (!early) pdl_wait();  // J is an earlier kernel's output
+  int32_t wj = 0, r0 = 0;
+  int64_t ws = 0;
+  uint32_t wlen = 0;
+  V v0 = V(0);
+  if (mine) {  // its extent and first entries, which no iteration writes
+    wj = J[first + wid];
+    ws = col_ptr[wj];
+    wlen = (uint32_t)(col_ptr[wj + 1] - ws);
+    if ((uint32_t)lane < wlen) {
+      r0 = row_idx[ws + lane];
+      v0 = val[ws + lane];
+    }
+  }
+  if (early) pdl_wait();
   auto step = [&](int64_t e, int32_t j, double sum) {  // one thread: the column's step, applied to w
     double d, f;
     eq7_step(sum / n, w[j], lam, bjs[j], ib[j], d, f);
     list[e] = d != 0.0 ? apply_column(j, d, col_ptr, w, w32) : 0u;
     return d;
   };
-  if (wid < per && first + wid < m) {
-    const int64_t e = first + wid;
-    const int32_t j = J[e];
-    const int64_t s = col_ptr[j];
-    const uint32_t len = (uint32_t)(col_ptr[j + 1] - s);
+  if (mine) {
+    const int64_t e = first + wid, s = ws;
+    const int32_t j = wj;
+    const uint32_t len = wlen;
     if (lane == 0) s_len[wid] = len;
     if (len > (uint32_t)kWarpColumn) {
       if (lane == 0) s_long[atomicAdd(&s_nlong, 1)] = e;
     } else {
-      V acc = V(0);
+      V acc = (uint32_t)lane < len ? v0 * (V)u[r0] : V(0);
 #pragma unroll 4
-      for (uint32_t t = lane; t < len; t += 32) acc = fma(val[s + t], (V)u[row_idx[s + t]], acc);
+      for (uint32_t t = lane + 32; t < len; t += 32) acc = fma(val[s + t], (V)u[row_idx[s + t]], acc);
       const double sum = warp_sum((double)acc);
       double d = 0.0;
       if (lane == 0) d = step(e, j, sum);
       d = __shfl_sync(0xffffffffu, d, 0);
       if (d != 0.0) {
+        if ((uint32_t)lane < len) atomicAdd(z + r0, d * (double)v0);
 #pragma unroll 4
-        for (uint32_t t = lane; t < len; t += 32) atomicAdd(z + row_idx[s + t], d * (double)val[s + t]);
+        for (uint32_t t = lane + 32; t < len; t += 32) atomicAdd(z + row_idx[s + t], d * (double)val[s + t]);
       }
     }
   }
@@ -276,6 +297,14 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// One warp per column of the colour class.
+//
+// Bound: latency, a chain of ten dependent loads and FP64 operations, at one
+// launch per iteration.  So the class is spread thinly (a warp's FP64
+// instruction holds the pipe for some 16 cycles an SM), and what no iteration
+// writes (the class, the columns' extents, first entries and their y) is read
+// while the previous iteration still runs: 3.6 us an iteration on classes of
+// about 70 columns (FP64), 6.9 with eight warps a CTA and a plain launch.
 template <typename V, typename U>
 __global__ void __launch_bounds__(kThreads)
     k_coloring_iter(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
@@ -289,14 +318,25 @@ __global__ void __launch_bounds__(kThreads)
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  pdl_trigger();
   const int32_t colour = perm[q];
   const int32_t lo = color_ptr[colour], hi = color_ptr[colour + 1];
   unsigned long long upd = 0, work = 0;
+  bool waited = false;
   for (int64_t e = lo + warp; e < hi; e += nwarps) {
     const int32_t j = cols_by_color[e];
     const int64_t s = col_ptr[j], t = col_ptr[j + 1];
-    V acc = V(0);
-    for (int64_t p = s + lane; p < t; p += 32) acc = fma(val[p], (V)u[row_idx[p]], acc);
+    const bool have = s + lane < t;
+    const int32_t i0 = have ? row_idx[s + lane] : 0;
+    const V v0 = have ? val[s + lane] : V(0);
+    const double y0 = have ? y[i0] : 0.0;
+    if (!waited) {
+      pdl_wait();
+      waited = true;
+    }
+    const double z0 = have ? z[i0] : 0.0;  // no other column of the class has row i0
+    V acc = have ? v0 * (V)u[i0] : V(0);
+    for (int64_t p = s + lane + 32; p < t; p += 32) acc = fma(val[p], (V)u[row_idx[p]], acc);
     const double g = warp_sum((double)acc) / n;
     const double wj = w[j];
     double d, f;
@@ -304,7 +344,12 @@ __global__ void __launch_bounds__(kThreads)
     work += (unsigned long long)(t - s);
     if (d != 0.0) {
       // every lane has read its u values above (warp_sum synchronised them)
-      for (int64_t p = s + lane; p < t; p += 32) {
+      if (have) {
+        const double zi = z0 + d * (double)v0;
+        z[i0] = zi;
+        u[i0] = u_value<U>(loss, y0, zi);
+      }
+      for (int64_t p = s + lane + 32; p < t; p += 32) {
         const int32_t i = row_idx[p];
         const double zi = z[i] + d * (double)val[p];
         z[i] = zi;
@@ -318,6 +363,7 @@ __global__ void __launch_bounds__(kThreads)
       work += (unsigned long long)(t - s);
     }
   }
+  if (!waited) pdl_wait();
   if (lane == 0 && (upd | work)) {
     atomicAdd(counters + 0, upd);
     atomicAdd(counters + 1, work);
@@ -538,14 +584,16 @@ int launch_update_list(gencd_problem* p, const int32_t* J, const double* d, int6
   cudaEvent_t ev = nullptr;
   prof_begin(p, K_UPDATE, &ev);
   auto go = [&](auto kernel, auto* val) {
-    kernel<<<list_grid(p), kListThreads, 0, p->stream>>>(p->col_ptr, p->row_idx, val, J, d, p->list_off, m, p->z, ctr);
+    return launch_overlapped(kernel, list_grid(p), kListThreads, 0, p->stream, p->col_ptr, p->row_idx, val, J, d,
+                             p->list_off, m, p->z, ctr);
   };
+  cudaError_t err;
   if (p->precision == GENCD_F64)
-    go(scan ? k_update_flat<double, true> : k_update_flat<double, false>, (const double*)p->val);
+    err = go(scan ? k_update_flat<double, true> : k_update_flat<double, false>, (const double*)p->val);
   else
-    go(scan ? k_update_flat<float, true> : k_update_flat<float, false>, (const float*)p->val);
+    err = go(scan ? k_update_flat<float, true> : k_update_flat<float, false>, (const float*)p->val);
   prof_end(p, ev);
-  GENCD_CUDA_TRY(cudaGetLastError());
+  GENCD_CUDA_TRY(err);
   return GENCD_OK;
 }
 
@@ -560,20 +608,22 @@ int launch_refresh_list(gencd_problem* p, const int32_t* J, int64_t m, bool coun
   cudaEvent_t ev = nullptr;
   prof_begin(p, K_REFRESH, &ev);
   auto go = [&](auto kernel, auto* u) {
-    kernel<<<list_grid(p), kListThreads, 0, p->stream>>>(p->col_ptr, p->row_idx, J, p->list_off, m, p->y, p->z, p->n,
-                                                         p->loss, u, ctr);
+    return launch_overlapped(kernel, list_grid(p), kListThreads, 0, p->stream, p->col_ptr, p->row_idx, J, p->list_off,
+                             m, p->y, p->z, p->n, p->loss, u, ctr);
   };
+  cudaError_t err;
   if (p->precision == GENCD_F64)
-    go(scan ? k_refresh_flat<double, true> : k_refresh_flat<double, false>, (double*)p->u);
+    err = go(scan ? k_refresh_flat<double, true> : k_refresh_flat<double, false>, (double*)p->u);
   else
-    go(scan ? k_refresh_flat<float, true> : k_refresh_flat<float, false>, (float*)p->u);
+    err = go(scan ? k_refresh_flat<float, true> : k_refresh_flat<float, false>, (float*)p->u);
   prof_end(p, ev);
-  GENCD_CUDA_TRY(cudaGetLastError());
+  GENCD_CUDA_TRY(err);
   return GENCD_OK;
 }
 
-// Shotgun's iteration on the list J up to z: propose, accept all, w and z
-int launch_shotgun_step(gencd_problem* p, const int32_t* J, int64_t m) {
+// Shotgun's iteration on the list J up to z: propose, accept all, w and z.
+// early: no kernel still running may be writing J.
+int launch_shotgun_step(gencd_problem* p, const int32_t* J, int64_t m, bool early) {
   if (m <= 0) return GENCD_OK;
   unsigned long long* ctr = reinterpret_cast<unsigned long long*>(p->dscal + 4);
   // two CTAs per SM before a CTA takes a second column
@@ -581,35 +631,39 @@ int launch_shotgun_step(gencd_problem* p, const int32_t* J, int64_t m) {
   const unsigned grid = (unsigned)((m + per - 1) / per);
   cudaEvent_t ev = nullptr;
   prof_begin(p, K_PROPOSE_LIST, &ev);
+  cudaError_t err;
   if (p->precision == GENCD_F64)
-    k_shotgun_step<double, double><<<grid, kThreads, 0, p->stream>>>(
-        p->col_ptr, p->row_idx, (const double*)p->val, (const double*)p->u, p->bj, p->ib, J, m, per, (double)p->n,
-        p->lambda, p->w, p->w32, p->z, p->list_off, ctr);
+    err = launch_overlapped(k_shotgun_step<double, double>, grid, kThreads, 0, p->stream, p->col_ptr, p->row_idx,
+                            (const double*)p->val, (const double*)p->u, p->bj, p->ib, J, m, per, early ? 1 : 0,
+                            (double)p->n, p->lambda, p->w, p->w32, p->z, p->list_off, ctr);
   else
-    k_shotgun_step<float, float><<<grid, kThreads, 0, p->stream>>>(
-        p->col_ptr, p->row_idx, (const float*)p->val, (const float*)p->u, p->bj, p->ib, J, m, per, (double)p->n,
-        p->lambda, p->w, p->w32, p->z, p->list_off, ctr);
+    err = launch_overlapped(k_shotgun_step<float, float>, grid, kThreads, 0, p->stream, p->col_ptr, p->row_idx,
+                            (const float*)p->val, (const float*)p->u, p->bj, p->ib, J, m, per, early ? 1 : 0,
+                            (double)p->n, p->lambda, p->w, p->w32, p->z, p->list_off, ctr);
   prof_end(p, ev);
-  GENCD_CUDA_TRY(cudaGetLastError());
+  GENCD_CUDA_TRY(err);
   return GENCD_OK;
 }
 
 int launch_coloring_iter(gencd_problem* p, int64_t q) {
   const int64_t warps = p->max_class > 0 ? p->max_class : 1;
-  const int grid = grid_for(warps * 32, kThreads, p->num_sms * 8);
+  // two warps per SM before a CTA takes a second one
+  const int per = (int)std::min<int64_t>(kThreads / 32, (warps + 2 * p->num_sms - 1) / (2 * p->num_sms));
+  const int grid = grid_for(warps, per, p->num_sms * 8);
   unsigned long long* ctr = reinterpret_cast<unsigned long long*>(p->dscal + 4);
   cudaEvent_t ev = nullptr;
   prof_begin(p, K_COLOR_ITER, &ev);
+  cudaError_t err;
   if (p->precision == GENCD_F64)
-    k_coloring_iter<double, double><<<grid, kThreads, 0, p->stream>>>(
-        p->col_ptr, p->row_idx, (const double*)p->val, (double*)p->u, p->w, p->w32, p->bj, p->ib, p->z, p->y, p->perm, q,
-        p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, ctr);
+    err = launch_overlapped(k_coloring_iter<double, double>, grid, 32 * per, 0, p->stream, p->col_ptr, p->row_idx,
+                            (const double*)p->val, (double*)p->u, p->w, p->w32, p->bj, p->ib, p->z, p->y, p->perm, q,
+                            p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, ctr);
   else
-    k_coloring_iter<float, float><<<grid, kThreads, 0, p->stream>>>(
-        p->col_ptr, p->row_idx, (const float*)p->val, (float*)p->u, p->w, p->w32, p->bj, p->ib, p->z, p->y, p->perm, q,
-        p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, ctr);
+    err = launch_overlapped(k_coloring_iter<float, float>, grid, 32 * per, 0, p->stream, p->col_ptr, p->row_idx,
+                            (const float*)p->val, (float*)p->u, p->w, p->w32, p->bj, p->ib, p->z, p->y, p->perm, q,
+                            p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, ctr);
   prof_end(p, ev);
-  GENCD_CUDA_TRY(cudaGetLastError());
+  GENCD_CUDA_TRY(err);
   return GENCD_OK;
 }
 

@@ -360,6 +360,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                     int32_t slab_rows, G* __restrict__ gacc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   U* s_u = reinterpret_cast<U*>(smem_raw);
+  pdl_trigger();
+  pdl_wait();
   slab_pass<V, U, G, DEPTH, ITEMS, SV, 0>(s_row, s_val, pmask, pair_col, tile_start, tile_end, tile_pair, tile_slab,
                                           slab_tile_begin, cta_tile_begin[blockIdx.x],
                                           cta_tile_begin[blockIdx.x + 1], u, n, slab_rows, gacc, s_u,
@@ -506,6 +508,8 @@ __global__ void __launch_bounds__(kThreads, 3)
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  pdl_trigger();
+  pdl_wait();
   constexpr bool kPrefetch = sizeof(V) == 4;  // FP64 stages are too large to double in registers
   LightStage<SV> nxt;
   if (kPrefetch) load_light_stage<SV>(row, val, lmask, tile_lc, warp, ntiles, nnz, lane, nxt);
@@ -576,6 +580,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                     G* __restrict__ gacc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   U* s_u = reinterpret_cast<U*>(smem_raw);
+  pdl_trigger();
+  pdl_wait();
   const int warp = threadIdx.x >> 5;
   if (warp < SLAB_WARPS)
     slab_pass<V, U, G, DEPTH, ITEMS, SV, 32 * SLAB_WARPS>(
@@ -630,9 +636,10 @@ constexpr int kFusedSplits[] = {20, 24, 28, 31};
 constexpr int kNumFusedSplits = 4;
 
 template <typename V, typename U, typename G, typename SV, int DEPTH, int ITEMS, int SW>
-static void launch_fused(gencd_problem* p, const void* u_vec, size_t smem) {
+static cudaError_t launch_fused(gencd_problem* p, const void* u_vec, size_t smem) {
   ProposePlan& P = p->plan;
-  k_propose_fused<V, U, G, kFusedThreads, SW, DEPTH, ITEMS, SV><<<P.grid, kFusedThreads, smem, p->stream>>>(
+  return launch_overlapped(k_propose_fused<V, U, G, kFusedThreads, SW, DEPTH, ITEMS, SV>, P.grid, kFusedThreads, smem,
+                           p->stream,
       P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, P.tile_start, P.tile_end, P.tile_pair, P.tile_slab,
       P.slab_tile_begin, P.cta_tile_begin, P.light_row, (const SV*)P.light_val, P.lmask, P.light_tile_lc,
       P.light_cols, P.light_scale, P.light_nnz, P.light_ntiles, P.light_counter, (const U*)u_vec, p->n,
@@ -646,35 +653,36 @@ static int launch_plan_passes(gencd_problem* p, const void* u_vec) {
     const size_t smem = (size_t)(P.slab_rows + kSlabZeroSlot) * sizeof(U);
     cudaEvent_t e1 = nullptr;
     prof_begin(p, K_PROPOSE_FUSED, &e1);
+    cudaError_t err;
     switch (P.fused_split) {
-      case 20: launch_fused<V, U, G, SV, DEPTH, ITEMS, 20>(p, u_vec, smem); break;
-      case 24: launch_fused<V, U, G, SV, DEPTH, ITEMS, 24>(p, u_vec, smem); break;
-      case 28: launch_fused<V, U, G, SV, DEPTH, ITEMS, 28>(p, u_vec, smem); break;
-      default: launch_fused<V, U, G, SV, DEPTH, ITEMS, 31>(p, u_vec, smem); break;
+      case 20: err = launch_fused<V, U, G, SV, DEPTH, ITEMS, 20>(p, u_vec, smem); break;
+      case 24: err = launch_fused<V, U, G, SV, DEPTH, ITEMS, 24>(p, u_vec, smem); break;
+      case 28: err = launch_fused<V, U, G, SV, DEPTH, ITEMS, 28>(p, u_vec, smem); break;
+      default: err = launch_fused<V, U, G, SV, DEPTH, ITEMS, 31>(p, u_vec, smem); break;
     }
     prof_end(p, e1);
-    GENCD_CUDA_TRY(cudaGetLastError());
+    GENCD_CUDA_TRY(err);
     return scale_heavy<G, SV>(p);
   }
   if (P.nlight > 0) {
     cudaEvent_t e = nullptr;
     prof_begin(p, K_PROPOSE_LIGHT, &e);
     const int grid = grid_for(P.light_ntiles * 32, kThreads, p->num_sms * 3);  // resident CTAs: persistent warps
-    k_propose_light_runs<V, U, G, SV><<<grid, kThreads, 0, p->stream>>>(
-        P.light_row, (const SV*)P.light_val, P.lmask, P.light_tile_lc, P.light_cols, P.light_scale,
-        (const U*)u_vec, P.light_nnz, P.light_ntiles, (G*)p->gnat);
+    const cudaError_t err = launch_overlapped(
+        k_propose_light_runs<V, U, G, SV>, grid, kThreads, 0, p->stream, P.light_row, (const SV*)P.light_val, P.lmask,
+        P.light_tile_lc, P.light_cols, P.light_scale, (const U*)u_vec, P.light_nnz, P.light_ntiles, (G*)p->gnat);
     prof_end(p, e);
-    GENCD_CUDA_TRY(cudaGetLastError());
+    GENCD_CUDA_TRY(err);
   }
   if (P.nheavy > 0) {
     const size_t smem = (size_t)(P.slab_rows + kSlabZeroSlot) * sizeof(U);
     cudaEvent_t e1 = nullptr;
     prof_begin(p, K_PROPOSE_SLABS, &e1);
-    k_propose_slabs<V, U, G, THREADS, DEPTH, ITEMS, SV><<<P.grid, THREADS, smem, p->stream>>>(
-        P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, P.tile_start, P.tile_end, P.tile_pair, P.tile_slab,
+    const cudaError_t err = launch_overlapped(
+        k_propose_slabs<V, U, G, THREADS, DEPTH, ITEMS, SV>, P.grid, THREADS, smem, p->stream, P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, P.tile_start, P.tile_end, P.tile_pair, P.tile_slab,
         P.slab_tile_begin, P.cta_tile_begin, (const U*)u_vec, p->n, P.slab_rows, (G*)p->gnat);
     prof_end(p, e1);
-    GENCD_CUDA_TRY(cudaGetLastError());
+    GENCD_CUDA_TRY(err);
   }
   return scale_heavy<G, SV>(p);
 }
