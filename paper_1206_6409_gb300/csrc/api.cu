@@ -253,8 +253,10 @@ static int compute_block_pstar(gencd_problem* p, int32_t B);
 __global__ void k_block_select(int64_t t, int32_t B, const int64_t* __restrict__ blo, const int64_t* __restrict__ bP,
                                const int32_t* __restrict__ perm, int32_t* __restrict__ J);
 
-static int ensure_selection(gencd_problem* p, int64_t epoch, int64_t m) {
-  if (p->perm_epoch == epoch && p->perm_m == m) return GENCD_OK;
+// *fresh: the permutation was enqueued by this call
+static int ensure_selection(gencd_problem* p, int64_t epoch, int64_t m, bool* fresh) {
+  *fresh = !(p->perm_epoch == epoch && p->perm_m == m);
+  if (!*fresh) return GENCD_OK;
   GENCD_TRY(make_permutation(p, p->params.seed, epoch, m, p->perm));
   p->perm_epoch = epoch;
   p->perm_m = m;
@@ -373,10 +375,11 @@ static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt)
     if (P > p->k) P = p->k;
     const int64_t per_epoch = (p->k + P - 1) / P;
     const int64_t e = p->t / per_epoch, q = p->t % per_epoch;
-    GENCD_TRY(ensure_selection(p, e, p->k));                             // Select, random subset
+    bool fresh = false;
+    GENCD_TRY(ensure_selection(p, e, p->k, &fresh));                     // Select, random subset
     const int64_t lo = q * P, m = (lo + P <= p->k ? P : p->k - lo);
     const int32_t* J = p->perm + lo;
-    GENCD_TRY(shotgun_on_list(p, J, m, true));                           // Propose, Accept all, Update
+    GENCD_TRY(shotgun_on_list(p, J, m, !fresh));                         // Propose, Accept all, Update
   } else if (v == GENCD_SHOTGUN_BLOCKS) {
     const int32_t B = (int32_t)std::min<int64_t>(p->params.blocks > 0 ? p->params.blocks : 16, p->k);
     GENCD_TRY(compute_block_pstar(p, B));
@@ -401,8 +404,9 @@ static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt)
     if (!p->color) GENCD_TRY(run_coloring(p));
     const int64_t C = p->ncolors;
     const int64_t e = p->t / C, q = p->t % C;
-    GENCD_TRY(ensure_selection(p, e, C));                                // Select, random colour
-    GENCD_TRY(launch_coloring_iter(p, q));                               // Propose + Update fused
+    bool fresh = false;
+    GENCD_TRY(ensure_selection(p, e, C, &fresh));                        // Select, random colour
+    GENCD_TRY(launch_coloring_iter(p, q, !fresh));                       // Propose + Update fused
   } else {
     return fail(GENCD_EINVAL, "unknown variant");
   }

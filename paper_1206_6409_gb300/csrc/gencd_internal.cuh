@@ -315,7 +315,7 @@ int launch_apply_list(gencd_problem* p, const int32_t* J, const double* d, int64
 int launch_update_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m);  // z (after w)
 int launch_refresh_list(gencd_problem* p, const int32_t* J, int64_t m, bool counted);    // u (after z)
 int launch_shotgun_step(gencd_problem* p, const int32_t* J, int64_t m, bool early);      // propose, w and z
-int launch_coloring_iter(gencd_problem* p, int64_t q);
+int launch_coloring_iter(gencd_problem* p, int64_t q, bool early);
 int launch_csr_spmv(gencd_problem* p, const double* x, double* out);  // out = X x (FP64)
 int launch_state_from_w(gencd_problem* p);  // z, u and w32 from p->w (synchronises the stream)
 
@@ -369,7 +369,9 @@ void prof_end(gencd_problem* p, cudaEvent_t stop);
 //    permutation or colour classes may be read before it), so that completion
 //    stays transitive along the stream;
 //  - calls pdl_trigger() at its start: the next kernel's launch latency and its
-//    reads before its own pdl_wait() then overlap this kernel.
+//    reads before its own pdl_wait() then overlap this kernel.  The first kernel
+//    after a new permutation waits before that, so that no later one starts
+//    before the permutation is visible.
 // The gap between two dependent kernels of an iteration, 1.6 us launched
 // plainly, goes with it: Greedy on 800 x 100,000 took 687 us for 20 iterations
 // of five launches and takes 537.

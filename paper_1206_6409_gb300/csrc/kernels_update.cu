@@ -216,13 +216,13 @@ __global__ void __launch_bounds__(kThreads)
   __shared__ uint32_t s_len[kShotgunCols];
   __shared__ double s_sum[kThreads / 32], s_d;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (!early) pdl_wait();  // J is the output of an earlier kernel, which may still run
   pdl_trigger();
   if (tid == 0) s_nlong = 0;
   if (lane == 0) s_len[wid] = 0u;
   __syncthreads();
   const int64_t first = (int64_t)blockIdx.x * per;
   const bool mine = wid < per && first + wid < m;  // this warp's column
-  if (!early) pdl_wait();  // J is an earlier kernel's output
   int32_t wj = 0, r0 = 0;
   int64_t ws = 0;
   uint32_t wlen = 0;
@@ -313,16 +313,17 @@ __global__ void __launch_bounds__(kThreads)
                     double* __restrict__ z,
                     const double* __restrict__ y, const int32_t* __restrict__ perm, int64_t q,
                     const int32_t* __restrict__ color_ptr, const int32_t* __restrict__ cols_by_color,
-                    double n, double lam, int loss,
+                    double n, double lam, int loss, int early,
                     unsigned long long* __restrict__ counters) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  bool waited = !early;
+  if (!early) pdl_wait();  // perm is the output of an earlier kernel, which may still run
   pdl_trigger();
   const int32_t colour = perm[q];
   const int32_t lo = color_ptr[colour], hi = color_ptr[colour + 1];
   unsigned long long upd = 0, work = 0;
-  bool waited = false;
   for (int64_t e = lo + warp; e < hi; e += nwarps) {
     const int32_t j = cols_by_color[e];
     const int64_t s = col_ptr[j], t = col_ptr[j + 1];
@@ -645,7 +646,8 @@ int launch_shotgun_step(gencd_problem* p, const int32_t* J, int64_t m, bool earl
   return GENCD_OK;
 }
 
-int launch_coloring_iter(gencd_problem* p, int64_t q) {
+// early: no kernel still running may be writing the permutation
+int launch_coloring_iter(gencd_problem* p, int64_t q, bool early) {
   const int64_t warps = p->max_class > 0 ? p->max_class : 1;
   // two warps per SM before a CTA takes a second one
   const int per = (int)std::min<int64_t>(kThreads / 32, (warps + 2 * p->num_sms - 1) / (2 * p->num_sms));
@@ -657,11 +659,11 @@ int launch_coloring_iter(gencd_problem* p, int64_t q) {
   if (p->precision == GENCD_F64)
     err = launch_overlapped(k_coloring_iter<double, double>, grid, 32 * per, 0, p->stream, p->col_ptr, p->row_idx,
                             (const double*)p->val, (double*)p->u, p->w, p->w32, p->bj, p->ib, p->z, p->y, p->perm, q,
-                            p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, ctr);
+                            p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, early ? 1 : 0, ctr);
   else
     err = launch_overlapped(k_coloring_iter<float, float>, grid, 32 * per, 0, p->stream, p->col_ptr, p->row_idx,
                             (const float*)p->val, (float*)p->u, p->w, p->w32, p->bj, p->ib, p->z, p->y, p->perm, q,
-                            p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, ctr);
+                            p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, early ? 1 : 0, ctr);
   prof_end(p, ev);
   GENCD_CUDA_TRY(err);
   return GENCD_OK;

@@ -108,6 +108,13 @@ def test_lambda_max_and_objective(gb, precision):
                                        atol=1e-12 if precision == "f64" else 1e-5)
 
 
+@pytest.mark.parametrize("m", [2, 3, 31, 375, 4999, 16_383, 16_384, 16_385])
+def test_permutation_of_small_ranges_is_bit_exact(gb, m):
+    # by rank up to 16,384 entries, by the radix sort beyond
+    with gb.Problem(workloads.config1("logistic")) as p:
+        np.testing.assert_array_equal(p.permutation(5, 2, m), oracle.permutation(5, 2, m))
+
+
 def test_permutation_is_bit_exact(gb):
     prob = workloads.config1("logistic")
     with gb.Problem(prob) as p:
