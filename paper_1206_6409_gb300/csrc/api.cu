@@ -548,15 +548,11 @@ __global__ void __launch_bounds__(kThreads)
 
 static void free_problem(gencd_problem* p) {
   if (!p) return;
-  void* bufs[] = {p->col_ptr, p->row_idx, p->val, p->y, p->z, p->u, p->w, p->c, p->ib, p->tile_col, p->gacc,
-                  p->delta, p->phi, p->list_j, p->list_d, p->list_m, p->w_start, p->top_buf, p->dscal, p->red, p->perm,
-                  p->sort_tmp,
-                  p->row_ptr, p->col_idx, p->csr_val, p->color, p->color_ptr, p->cols_by_color,
-                  p->slot_m, p->slot_d, p->slot_j, p->slot_cnt, p->list_off, p->scan_tmp, p->bj, p->w32, p->bj32, p->ib32,
-                  p->part_lo, p->col_val, p->block_lo, p->block_P};
+  void* bufs[] = {p->mem, p->w_start, p->top_buf, p->sort_tmp, p->row_ptr, p->col_idx, p->csr_val, p->color,
+                  p->color_ptr, p->cols_by_color, p->slot_m, p->slot_d, p->slot_j, p->slot_cnt, p->part_lo, p->col_val,
+                  p->block_lo, p->block_P};
   if (p->stream) cudaStreamSynchronize(p->stream);
   free_propose_plan(p);
-  if (p->gnat && p->gnat != p->gacc) dev_free(p, p->gnat);
   for (void* b : bufs)
     if (b) dev_free(p, b);
   if (p->hpin && p->own_hpin) cudaFreeHost(p->hpin);
@@ -634,40 +630,40 @@ static int create_impl(gencd_problem* p, const int64_t* col_ptr, const int32_t* 
   p->ntiles = (nnz + tile - 1) / tile;
   const size_t vsz = p->precision == GENCD_F64 ? 8 : 4;
 
-  GENCD_TRY(dev_alloc(p, &p->col_ptr, k + 1));
-  GENCD_TRY(dev_alloc(p, &p->row_idx, p->nnz_pad));
-  GENCD_TRY(dev_alloc(p, (char**)&p->val, vsz * p->nnz_pad));
-  GENCD_TRY(dev_alloc(p, &p->y, n));
-  GENCD_TRY(dev_alloc(p, &p->z, n));
-  GENCD_TRY(dev_alloc(p, (char**)&p->u, vsz * (n + 1)));  // u[n] = 0: the row that padding entries may gather
-  GENCD_TRY(dev_alloc(p, &p->w, k));
-  GENCD_TRY(dev_alloc(p, &p->c, k));
-  GENCD_TRY(dev_alloc(p, &p->ib, k));
-  GENCD_TRY(dev_alloc(p, &p->bj, k));
+  // one allocation for the arrays every problem has
+  Arena a;
+  a.add(&p->col_ptr, k + 1);
+  a.add(&p->row_idx, p->nnz_pad);
+  a.add((char**)&p->val, (int64_t)vsz * p->nnz_pad);
+  a.add(&p->y, n);
+  a.add(&p->z, n);
+  a.add((char**)&p->u, (int64_t)vsz * (n + 1));  // u[n] = 0: the row that padding entries may gather
+  a.add(&p->w, k);
+  a.add(&p->c, k);
+  a.add(&p->ib, k);
+  a.add(&p->bj, k);
   if (p->precision == GENCD_F32) {
-    GENCD_TRY(dev_alloc(p, &p->w32, k));
-    GENCD_TRY(dev_alloc(p, &p->bj32, k));
-    GENCD_TRY(dev_alloc(p, &p->ib32, k));
+    a.add(&p->w32, k);
+    a.add(&p->bj32, k);
+    a.add(&p->ib32, k);
   }
-  GENCD_TRY(dev_alloc(p, &p->tile_col, p->ntiles + 1));
-  GENCD_TRY(dev_alloc(p, &p->gacc, k));
-  if (p->precision == GENCD_F64) {
-    p->gnat = p->gacc;
-  } else {
-    float* gf = nullptr;
-    GENCD_TRY(dev_alloc(p, &gf, k));
-    p->gnat = gf;
-  }
-  GENCD_TRY(dev_alloc(p, &p->delta, k));
-  GENCD_TRY(dev_alloc(p, &p->phi, k));
-  GENCD_TRY(dev_alloc(p, &p->list_j, k));
-  GENCD_TRY(dev_alloc(p, &p->list_d, k));
-  GENCD_TRY(dev_alloc(p, &p->list_m, k));
-  GENCD_TRY(dev_alloc(p, &p->perm, k));
-  GENCD_TRY(dev_alloc(p, &p->list_off, k + 2));
-  GENCD_TRY(dev_alloc(p, &p->scan_tmp, scan_tmp_words(k + 2)));
-  GENCD_TRY(dev_alloc(p, &p->dscal, kScalars));
-  GENCD_TRY(dev_alloc(p, &p->red, 3 * kRedBlocks));
+  a.add(&p->tile_col, p->ntiles + 1);
+  a.add(&p->gacc, k);
+  float* gf = nullptr;
+  if (p->precision != GENCD_F64) a.add(&gf, k);
+  a.add(&p->delta, k);
+  a.add(&p->phi, k);
+  a.add(&p->list_j, k);
+  a.add(&p->list_d, k);
+  a.add(&p->list_m, k);
+  a.add(&p->perm, k);
+  a.add(&p->list_off, k + 2);
+  a.add(&p->scan_tmp, scan_tmp_words(k + 2));
+  a.add(&p->dscal, kScalars);
+  a.add(&p->red, 3 * kRedBlocks);
+  GENCD_TRY(dev_alloc_bytes(p, &p->mem, a.bytes()));
+  a.place(p->mem);
+  p->gnat = p->precision == GENCD_F64 ? (void*)p->gacc : gf;
   GENCD_CUDA_TRY(cudaEventCreateWithFlags(&p->ev_scalars, cudaEventDisableTiming));
   if (!p->hpin && cudaMallocHost((void**)&p->hpin, kScalars * sizeof(double)) != cudaSuccess) {
     cudaGetLastError();

@@ -144,6 +144,7 @@ struct ProposePlan {
   int fused_split = 0;
   double tuned_ms[8] = {-1.0};
   unsigned int* light_counter = nullptr;
+  void* mem[2] = {nullptr, nullptr};  // the allocations that hold the arrays above
 };
 
 // ---------------------------------------------------------------------------
@@ -170,6 +171,8 @@ struct gencd_problem {
   int64_t t = 0;  // GenCD iteration counter (drives Select)
   int64_t stat_iters = 0;     // iterations since the last counter reset
   int64_t stat_host_nnz = 0;  // non-zeros streamed by full passes since the reset
+
+  void* mem = nullptr;  // the allocation that holds the arrays every problem has
 
   // CSC + rows + cols
   int64_t* col_ptr = nullptr;
@@ -297,8 +300,6 @@ size_t radix_tmp_words(int64_t m);
 int radix_sort_with_tmp(gencd_problem* p, uint32_t* keys, uint32_t* vals, int64_t m, int bits,
                         uint32_t* keys_alt, uint32_t* vals_alt, uint32_t* tmp, bool* result_in_alt);
 int bits_for_max(int64_t maxval);
-int lower_bounds_u32_to_i64(gencd_problem* p, const uint32_t* sorted, int64_t m, int64_t count, int64_t* out);
-int iota_u32(gencd_problem* p, uint32_t* a, int64_t m);
 int fail_plan(const char* msg);
 // tile_col[t] = column holding entry t * tile (columns without entries hold none)
 int launch_tile_map_of(gencd_problem* p, const int64_t* col_ptr, int64_t k, int64_t ntiles, int32_t* tile_col,
@@ -406,6 +407,31 @@ template <typename T>
 inline int dev_alloc(gencd_problem* p, T** ptr, size_t count) {
   return dev_alloc_bytes(p, reinterpret_cast<void**>(ptr), sizeof(T) * (count > 0 ? count : 1));
 }
+
+// Arrays that share one allocation: add() them, allocate bytes(), place() sets
+// their pointers (each 256-byte aligned).  An array of no elements gets a valid
+// address too.
+class Arena {
+ public:
+  template <typename T>
+  void add(T** ptr, int64_t count) {
+    *ptr = nullptr;
+    items_.push_back({reinterpret_cast<void**>(ptr), used_});
+    used_ += (sizeof(T) * (size_t)(count > 0 ? count : 1) + 255) / 256 * 256;
+  }
+  size_t bytes() const { return used_; }
+  void place(void* base) {
+    for (const Item& i : items_) *i.ptr = static_cast<char*>(base) + i.at;
+  }
+
+ private:
+  struct Item {
+    void** ptr;
+    size_t at;
+  };
+  std::vector<Item> items_;
+  size_t used_ = 0;
+};
 
 inline int grid_for(int64_t work, int threads, int max_blocks) {
   int64_t b = (work + threads - 1) / threads;

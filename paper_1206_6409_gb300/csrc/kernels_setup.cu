@@ -436,26 +436,6 @@ int bits_for_max(int64_t maxval) {
   return b;
 }
 
-int lower_bounds_u32_to_i64(gencd_problem* p, const uint32_t* sorted, int64_t m, int64_t count, int64_t* out) {
-  k_lower_bounds<<<grid_for(count + 1, kThreads, p->num_sms * 8), kThreads, 0, p->stream>>>(sorted, m, count, out,
-                                                                                            nullptr);
-  p->prof.launches[K_SETUP] += 1;
-  GENCD_CUDA_TRY(cudaGetLastError());
-  return GENCD_OK;
-}
-
-__global__ void k_iota_u32(uint32_t* __restrict__ a, int64_t m) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) a[i] = (uint32_t)i;
-}
-
-int iota_u32(gencd_problem* p, uint32_t* a, int64_t m) {
-  k_iota_u32<<<grid_for(m, kThreads, p->num_sms * 8), kThreads, 0, p->stream>>>(a, m);
-  p->prof.launches[K_SETUP] += 1;
-  GENCD_CUDA_TRY(cudaGetLastError());
-  return GENCD_OK;
-}
-
 int fail_plan(const char* msg) {
   set_error(msg);
   return GENCD_EINVAL;

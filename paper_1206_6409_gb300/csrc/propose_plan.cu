@@ -718,27 +718,34 @@ int launch_propose_plan(gencd_problem* p, const void* u_vec) {
 // ---------------------------------------------------------------------------
 // building the plan (once per problem)
 
+// Columns by kind, for the exclusive scans: hid and lid number the heavy and
+// the light ones, loff offsets the light ones' entries.
 __global__ void k_plan_classify(const int64_t* __restrict__ col_ptr, int64_t k, int64_t hmin,
                                 uint32_t* __restrict__ hid, uint32_t* __restrict__ lid,
-                                uint32_t* __restrict__ hoff, uint32_t* __restrict__ loff) {
+                                uint32_t* __restrict__ loff) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= k; j += stride) {
-    uint32_t len = j < k ? (uint32_t)(col_ptr[j + 1] - col_ptr[j]) : 0u;
+    const uint32_t len = j < k ? (uint32_t)(col_ptr[j + 1] - col_ptr[j]) : 0u;
     const bool heavy = len > 0 && (int64_t)len >= hmin;
     const bool light = len > 0 && !heavy;
     hid[j] = heavy;
     lid[j] = light;
-    hoff[j] = heavy ? len : 0u;
     loff[j] = light ? len : 0u;
   }
 }
 
+// light_scale (index-only storage): the value of every light column
 __global__ void k_plan_columns(const int64_t* __restrict__ col_ptr, int64_t k, int64_t hmin,
                                const uint32_t* __restrict__ hid, const uint32_t* __restrict__ lid,
                                const uint32_t* __restrict__ loff, int32_t* __restrict__ heavy_cols,
-                               int32_t* __restrict__ light_cols, int64_t* __restrict__ light_col_ptr) {
+                               int32_t* __restrict__ light_cols, int64_t* __restrict__ light_col_ptr,
+                               const float* __restrict__ col_val, float* __restrict__ light_scale) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < k; j += stride) {
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= k; j += stride) {
+    if (j == k) {
+      light_col_ptr[lid[k]] = loff[k];
+      continue;
+    }
     const int64_t len = col_ptr[j + 1] - col_ptr[j];
     if (len <= 0) continue;
     if (len >= hmin) {
@@ -746,33 +753,9 @@ __global__ void k_plan_columns(const int64_t* __restrict__ col_ptr, int64_t k, i
     } else {
       light_cols[lid[j]] = (int32_t)j;
       light_col_ptr[lid[j]] = loff[j];
+      if (light_scale) light_scale[lid[j]] = col_val[j];
     }
   }
-}
-
-template <typename V>
-__global__ void k_plan_copy_light(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
-                                  const V* __restrict__ val, int64_t k, int64_t hmin,
-                                  const uint32_t* __restrict__ loff, int32_t* __restrict__ lrow,
-                                  V* __restrict__ lval) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t j = warp; j < k; j += nwarps) {
-    const int64_t s = col_ptr[j], len = col_ptr[j + 1] - s;
-    if (len <= 0 || len >= hmin) continue;
-    for (int64_t t = lane; t < len; t += 32) {
-      lrow[loff[j] + t] = row_idx[s + t];
-      lval[loff[j] + t] = val[s + t];
-    }
-  }
-}
-
-// value storage of the plan: bfloat16 copies (the values are bfloat16-exact)
-__global__ void k_plan_to_bf16(const float* __restrict__ src, int64_t m, __nv_bfloat16* __restrict__ dst) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride)
-    dst[i] = __float2bfloat16_rn(src[i]);
 }
 
 template <typename T>
@@ -781,89 +764,139 @@ __global__ void k_plan_fill(T* __restrict__ a, int64_t m, T v) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += stride) a[i] = v;
 }
 
-// index-only storage: scale[c] = col_val[cols[c]]
-__global__ void k_plan_gather_scales(const int32_t* __restrict__ cols, int64_t m, const float* __restrict__ col_val,
-                                     float* __restrict__ scale) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < m; c += stride) scale[c] = col_val[cols[c]];
+// first entry of a column (rows r[0..len), ascending) at or beyond a row
+__device__ __forceinline__ uint32_t rows_below(const int32_t* __restrict__ r, uint32_t len, int64_t row) {
+  uint32_t lo = 0, hi = len;
+  while (lo < hi) {
+    const uint32_t mid = (lo + hi) >> 1;
+    if ((int64_t)r[mid] < row)
+      lo = mid + 1;
+    else
+      hi = mid;
+  }
+  return lo;
 }
 
-// bit p % 32 of word p / 32 (= bit p % 8 of byte p / 8) for the first entry p of
-// every light column
-__global__ void k_plan_light_starts(const int64_t* __restrict__ light_col_ptr, int64_t nlight,
-                                    uint32_t* __restrict__ words) {
+// The entries of heavy column h in slab r are one run of the column (its rows
+// ascend).  Slab-major, i = r nheavy + h: seg[i] the run's first entry within
+// the column, cnt[i] its length, pair[i] whether it is not empty (both for the
+// exclusive scans; index count holds 0).
+__global__ void k_plan_segments(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
+                                const int32_t* __restrict__ heavy_cols, int64_t nheavy, int64_t count, int32_t R,
+                                int32_t slab_rows, uint32_t* __restrict__ seg, uint32_t* __restrict__ cnt,
+                                uint32_t* __restrict__ pair) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; c < nlight; c += stride) {
-    const int64_t p = light_col_ptr[c];
-    atomicOr(words + (p >> 5), 1u << (p & 31));
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i <= count; i += stride) {
+    uint32_t n_i = 0;
+    if (i < count) {
+      const int64_t r = i / nheavy;
+      const int32_t j = heavy_cols[i - r * nheavy];
+      const int64_t s = col_ptr[j];
+      const uint32_t len = (uint32_t)(col_ptr[j + 1] - s);
+      const uint32_t a = r == 0 ? 0u : rows_below(row_idx + s, len, r * slab_rows);
+      const uint32_t b = r == R - 1 ? len : rows_below(row_idx + s, len, (r + 1) * slab_rows);
+      seg[i] = a;
+      n_i = b - a;
+    }
+    cnt[i] = n_i;
+    pair[i] = n_i > 0 ? 1u : 0u;
   }
 }
 
-// heavy entry e (column-major order): key = slab, plus its row, value, heavy id
+// entries before slab r (r = R: all of them), and the number of pairs
+__global__ void k_plan_slab_begins(const uint32_t* __restrict__ pos, const uint32_t* __restrict__ pair, int64_t nheavy,
+                                   int32_t R, int64_t* __restrict__ slab_begin) {
+  for (int32_t r = threadIdx.x; r <= R; r += blockDim.x) slab_begin[r] = pos[(int64_t)r * nheavy];
+  if (threadIdx.x == 0) slab_begin[R + 1] = pair[(int64_t)R * nheavy];
+}
+
 template <typename V>
-__global__ void k_plan_heavy_entries(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
-                                     const V* __restrict__ val, int64_t k, int64_t hmin,
-                                     const uint32_t* __restrict__ hid, const uint32_t* __restrict__ hoff,
-                                     int32_t slab_rows, uint32_t* __restrict__ keys, uint32_t* __restrict__ order,
-                                     uint32_t* __restrict__ hrow, uint32_t* __restrict__ hh, V* __restrict__ hval) {
-  const int lane = threadIdx.x & 31;
-  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t j = warp; j < k; j += nwarps) {
-    const int64_t s = col_ptr[j], len = col_ptr[j + 1] - s;
-    if (len <= 0 || len < hmin) continue;
-    for (int64_t t = lane; t < len; t += 32) {
-      const uint32_t e = hoff[j] + (uint32_t)t;
-      const int32_t r = row_idx[s + t];
-      keys[e] = (uint32_t)(r / slab_rows);
-      order[e] = e;
-      hrow[e] = (uint32_t)r;
-      hh[e] = hid[j];
-      hval[e] = val[s + t];
+__device__ __forceinline__ void plan_store(V* a, int64_t i, V v) {
+  a[i] = v;
+}
+__device__ __forceinline__ void plan_store(__nv_bfloat16* a, int64_t i, float v) {
+  a[i] = __float2bfloat16_rn(v);  // the values are bfloat16-exact
+}
+__device__ __forceinline__ void plan_store(NoVal*, int64_t, float) {}
+
+// Every entry to its place: a heavy one into its slab's run (pad_off[r] is
+// where the padded slab starts), a light one into the compact copy, in the
+// plan's value storage; the start bits of pairs and light columns (bit p % 32
+// of word p / 32 = bit p % 8 of byte p / 8), and each pair's first entry and
+// column.
+//
+// Bound: memory.  Consecutive lanes take consecutive entries, so reads and, run
+// by run, writes are coalesced; every entry finds its column within its tile
+// (the tile map): 142 us on 2.0e7 FP32 non-zeros, 41 at the copy rate.  The
+// entries' keys, order, rows, columns and values expanded (480 us: a warp walked
+// a whole column), sorted by slab (117) and gathered (163), and the pairs (62),
+// took 0.8 ms and 28 bytes of scratch a non-zero.
+template <typename V, typename SV>
+__global__ void __launch_bounds__(kThreads)
+    k_plan_place(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx, const V* __restrict__ val,
+                 const int32_t* __restrict__ tile_col, int64_t nnz, int64_t tile, int64_t hmin,
+                 const uint32_t* __restrict__ hid, const uint32_t* __restrict__ loff, int64_t nheavy,
+                 int32_t slab_rows, const uint32_t* __restrict__ seg, const uint32_t* __restrict__ pos,
+                 const uint32_t* __restrict__ pair, const int64_t* __restrict__ slab_begin,
+                 const int64_t* __restrict__ pad_off, uint16_t* __restrict__ s_row, SV* __restrict__ s_val,
+                 uint32_t* __restrict__ pmask, uint32_t* __restrict__ pair_start, uint32_t* __restrict__ pair_col,
+                 int32_t* __restrict__ lrow, SV* __restrict__ lval, uint32_t* __restrict__ lmask) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nnz; p += stride) {
+    const int64_t t = p / tile;
+    int32_t lo = __ldg(tile_col + t), hi = __ldg(tile_col + t + 1);  // last c with col_ptr[c] <= p
+    while (lo < hi) {
+      const int32_t mid = (lo + hi + 1) >> 1;
+      if (__ldg(col_ptr + mid) <= p)
+        lo = mid;
+      else
+        hi = mid - 1;
+    }
+    const int64_t s = __ldg(col_ptr + lo), len = __ldg(col_ptr + lo + 1) - s;
+    const int32_t row = row_idx[p];
+    const uint32_t at = (uint32_t)(p - s);
+    if (len >= hmin) {
+      const int32_t r = row / slab_rows;
+      const int64_t i = (int64_t)r * nheavy + __ldg(hid + lo);
+      const uint32_t first = __ldg(seg + i);
+      const int64_t d = __ldg(pad_off + r) - __ldg(slab_begin + r) + __ldg(pos + i) + (at - first);
+      s_row[d] = (uint16_t)(row - r * slab_rows);
+      plan_store(s_val, d, val[p]);
+      if (at == first) {
+        const uint32_t q = __ldg(pair + i);
+        atomicOr(pmask + (d >> 5), 1u << (d & 31));
+        pair_start[q] = (uint32_t)d;
+        pair_col[q] = (uint32_t)lo;
+      }
+    } else {
+      const int64_t d = (int64_t)__ldg(loff + lo) + at;
+      lrow[d] = row;
+      plan_store(lval, d, val[p]);
+      if (at == 0) atomicOr(lmask + (d >> 5), 1u << (d & 31));
     }
   }
 }
 
-// entries in slab order -> padded slab arrays, and the flag "a pair starts here"
-template <typename V>
-__global__ void k_plan_fill_slabs(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ se, int64_t E,
-                                  const int64_t* __restrict__ slab_begin, const int64_t* __restrict__ pad_off,
-                                  int32_t slab_rows, const uint32_t* __restrict__ hrow,
-                                  const uint32_t* __restrict__ hh, const V* __restrict__ hval,
-                                  uint16_t* __restrict__ s_row, V* __restrict__ s_val,
-                                  uint32_t* __restrict__ newpair, uint32_t* __restrict__ pmask_words) {
+// the padding of every slab's entries (and 8 entries past the last slab): row
+// pad_row, value 0
+__global__ void k_plan_pad(const int64_t* __restrict__ slab_begin, const int64_t* __restrict__ pad_off, int32_t R,
+                           int64_t entries, uint16_t pad_row, uint16_t* __restrict__ s_row, char* __restrict__ s_val,
+                           int vsz) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < E; i += stride) {
-    const uint32_t r = sk[i], e = se[i];
-    const int64_t ip = pad_off[r] + (i - slab_begin[r]);
-    s_row[ip] = (uint16_t)(hrow[e] - r * (uint32_t)slab_rows);
-    s_val[ip] = hval[e];
-    const bool starts = i == slab_begin[r] || hh[e] != hh[se[i - 1]];
-    newpair[i] = starts ? 1u : 0u;
-    // bit ip % 32 of word ip / 32 = bit ip % 8 of byte ip / 8 (little-endian)
-    if (starts) atomicOr(pmask_words + (ip >> 5), 1u << (ip & 31));
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < (int64_t)(R + 1) * kSlabPad; q += stride) {
+    const int64_t r = q / kSlabPad, x = q - r * kSlabPad;
+    int64_t d, end;
+    if (r < R) {
+      d = pad_off[r] + (slab_begin[r + 1] - slab_begin[r]) + x;
+      end = pad_off[r + 1];
+    } else {
+      d = entries + x;
+      end = entries + 8;
+    }
+    if (d >= end) continue;
+    s_row[d] = pad_row;
+    for (int b = 0; b < vsz; ++b) s_val[d * vsz + b] = 0;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) newpair[E] = 0u;
-}
-
-__global__ void k_plan_fill_pairs(const uint32_t* __restrict__ sk, const uint32_t* __restrict__ se, int64_t E,
-                                  const int64_t* __restrict__ slab_begin, const int64_t* __restrict__ pad_off,
-                                  const uint32_t* __restrict__ hh, const uint32_t* __restrict__ pidx,
-                                  uint32_t* __restrict__ pair_start, uint32_t* __restrict__ pair_h) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < E; i += stride) {
-    if (pidx[i + 1] == pidx[i]) continue;
-    const uint32_t q = pidx[i], r = sk[i];
-    pair_start[q] = (uint32_t)(pad_off[r] + (i - slab_begin[r]));
-    pair_h[q] = hh[se[i]];
-  }
-}
-
-__global__ void k_plan_pair_cols(const uint32_t* __restrict__ pair_h, int64_t npairs,
-                                 const int32_t* __restrict__ heavy_cols, uint32_t* __restrict__ pair_col) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < npairs; q += stride)
-    pair_col[q] = (uint32_t)heavy_cols[pair_h[q]];
 }
 
 __global__ void k_plan_tiles(const int32_t* __restrict__ slab_tile_begin, const int64_t* __restrict__ pad_off,
@@ -900,19 +933,9 @@ __global__ void k_plan_tiles(const int32_t* __restrict__ slab_tile_begin, const 
 }
 
 void free_propose_plan(gencd_problem* p) {
-  ProposePlan& P = p->plan;
-  void* bufs[] = {P.light_cols, P.light_col_ptr, P.light_row, P.light_val, P.light_tile_lc, P.lmask, P.light_scale,
-                  P.heavy_cols,
-                  P.s_row, P.s_val, P.pmask, P.pair_col, P.tile_start,
-                  P.tile_end, P.tile_pair, P.tile_slab, P.slab_tile_begin, P.cta_tile_begin, P.light_counter};
-  for (void* b : bufs)
+  for (void* b : p->plan.mem)
     if (b) dev_free(p, b);
-  P = ProposePlan();
-}
-
-template <typename T>
-static int palloc(gencd_problem* p, T** ptr, int64_t count) {
-  return dev_alloc(p, ptr, (size_t)(count > 0 ? count : 1));
+  p->plan = ProposePlan();
 }
 
 // scratch that is freed when the build returns
@@ -920,22 +943,37 @@ struct Scratch {
   gencd_problem* p;
   std::vector<void*> bufs;
   explicit Scratch(gencd_problem* q) : p(q) {}
-  template <typename T>
-  int get(T** ptr, int64_t count) {
-    int rc = palloc(p, ptr, count);
-    if (rc == GENCD_OK) bufs.push_back(*ptr);
-    return rc;
+  int get(Arena& a) {
+    void* base = nullptr;
+    GENCD_TRY(dev_alloc_bytes(p, &base, a.bytes()));
+    bufs.push_back(base);
+    a.place(base);
+    return GENCD_OK;
   }
   ~Scratch() {
     for (void* b : bufs) dev_free(p, b);
   }
 };
 
+template <typename V, typename SV>
+static void launch_place(gencd_problem* p, const uint32_t* hid, const uint32_t* loff, const uint32_t* seg,
+                         const uint32_t* pos, const uint32_t* pair, const int64_t* slab_begin, const int64_t* pad_off,
+                         uint32_t* pair_start) {
+  ProposePlan& P = p->plan;
+  k_plan_place<V, SV><<<grid_for(p->nnz, kThreads, p->num_sms * 32), kThreads, 0, p->stream>>>(
+      p->col_ptr, p->row_idx, (const V*)p->val, p->tile_col, p->nnz, 32LL * p->items, P.heavy_min, hid, loff, P.nheavy,
+      P.slab_rows, seg, pos, pair, slab_begin, pad_off, P.s_row, (SV*)P.s_val, (uint32_t*)P.pmask, pair_start,
+      P.pair_col, P.light_row, (SV*)P.light_val, (uint32_t*)P.lmask);
+}
+
+// Two allocations hold the plan and two the scratch: a cudaMalloc or cudaFree
+// of this size takes longer than most of the kernels here (some forty of them
+// took half of the 7 ms of a cold start on 2.0e7 non-zeros).
 static int build_plan_impl(gencd_problem* p, Scratch& S) {
   ProposePlan& P = p->plan;
   const int64_t k = p->k, n = p->n;
   const bool f64 = p->precision == GENCD_F64;
-  const size_t vsz = f64 ? 8 : 4;
+  const size_t vsz = f64 ? 8 : p->vmode == kValBf16 ? 2 : p->vmode == kValNone ? 0 : 4;  // as the plan stores them
   const int g = p->num_sms * 8;
   cudaStream_t st = p->stream;
   P.slab_rows = (int32_t)(kSlabBytes / (f64 ? 8 : 4));
@@ -948,226 +986,155 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   P.heavy_min = P.nslabs == 1 ? 1 : (f64 ? 8LL : 2LL) * P.nslabs;
 
   // classify, number and offset the columns
-  uint32_t *hid, *lid, *hoff, *loff, *tmp;
-  GENCD_TRY(S.get(&hid, k + 1));
-  GENCD_TRY(S.get(&lid, k + 1));
-  GENCD_TRY(S.get(&hoff, k + 1));
-  GENCD_TRY(S.get(&loff, k + 1));
-  GENCD_TRY(S.get(&tmp, scan_tmp_words(k + 1)));
-  k_plan_classify<<<grid_for(k + 1, kThreads, g), kThreads, 0, st>>>(p->col_ptr, k, P.heavy_min, hid, lid, hoff,
-                                                                      loff);
+  uint32_t *hid, *lid, *loff, *tmp;
+  Arena cols;
+  cols.add(&hid, k + 1);
+  cols.add(&lid, k + 1);
+  cols.add(&loff, k + 1);
+  cols.add(&tmp, scan_tmp_words(k + 1));
+  GENCD_TRY(S.get(cols));
+  k_plan_classify<<<grid_for(k + 1, kThreads, g), kThreads, 0, st>>>(p->col_ptr, k, P.heavy_min, hid, lid, loff);
   GENCD_TRY(exclusive_scan(p, hid, hid, k + 1, tmp));
   GENCD_TRY(exclusive_scan(p, lid, lid, k + 1, tmp));
-  GENCD_TRY(exclusive_scan(p, hoff, hoff, k + 1, tmp));
   GENCD_TRY(exclusive_scan(p, loff, loff, k + 1, tmp));
-  uint32_t tot[4];
+  uint32_t tot[3];
   GENCD_CUDA_TRY(cudaMemcpyAsync(&tot[0], hid + k, 4, cudaMemcpyDeviceToHost, st));
   GENCD_CUDA_TRY(cudaMemcpyAsync(&tot[1], lid + k, 4, cudaMemcpyDeviceToHost, st));
-  GENCD_CUDA_TRY(cudaMemcpyAsync(&tot[2], hoff + k, 4, cudaMemcpyDeviceToHost, st));
-  GENCD_CUDA_TRY(cudaMemcpyAsync(&tot[3], loff + k, 4, cudaMemcpyDeviceToHost, st));
+  GENCD_CUDA_TRY(cudaMemcpyAsync(&tot[2], loff + k, 4, cudaMemcpyDeviceToHost, st));
   GENCD_CUDA_TRY(cudaStreamSynchronize(st));
   P.nheavy = tot[0];
   P.nlight = tot[1];
-  const int64_t E = tot[2];
-  P.light_nnz = tot[3];
-
-  GENCD_TRY(palloc(p, &P.heavy_cols, P.nheavy));
-  GENCD_TRY(palloc(p, &P.light_cols, P.nlight));
-  GENCD_TRY(palloc(p, &P.light_col_ptr, P.nlight + 1));
-  k_plan_columns<<<grid_for(k, kThreads, g), kThreads, 0, st>>>(p->col_ptr, k, P.heavy_min, hid, lid, loff,
-                                                                 P.heavy_cols, P.light_cols, P.light_col_ptr);
-  GENCD_CUDA_TRY(cudaGetLastError());
-
-  // light columns: compact CSC copy and its tile map
-  if (P.nlight > 0) {
-    const int64_t lpad = ((P.light_nnz + kPadNnz - 1) / kPadNnz) * kPadNnz + kPadNnz;
-    GENCD_TRY(palloc(p, &P.light_row, lpad));
-    GENCD_TRY(palloc(p, (char**)&P.light_val, lpad * (int64_t)vsz));
-    GENCD_CUDA_TRY(cudaMemsetAsync(P.light_row, 0, sizeof(int32_t) * lpad, st));
-    GENCD_CUDA_TRY(cudaMemsetAsync(P.light_val, 0, vsz * lpad, st));
-    if (p->vmode == kValNone) {  // padding has no value to zero it: it gathers u[n] = 0 instead
-      k_plan_fill<int32_t><<<grid_for(lpad, kThreads, g), kThreads, 0, st>>>(P.light_row, lpad, (int32_t)n);
-      GENCD_CUDA_TRY(cudaGetLastError());
-    }
-    const int64_t ln = P.light_nnz;
-    GENCD_CUDA_TRY(cudaMemcpyAsync(P.light_col_ptr + P.nlight, &ln, 8, cudaMemcpyHostToDevice, st));
-    if (f64)
-      k_plan_copy_light<double><<<grid_for(k * 32, kThreads, g), kThreads, 0, st>>>(
-          p->col_ptr, p->row_idx, (const double*)p->val, k, P.heavy_min, loff, P.light_row, (double*)P.light_val);
-    else
-      k_plan_copy_light<float><<<grid_for(k * 32, kThreads, g), kThreads, 0, st>>>(
-          p->col_ptr, p->row_idx, (const float*)p->val, k, P.heavy_min, loff, P.light_row, (float*)P.light_val);
-    GENCD_CUDA_TRY(cudaGetLastError());
-    if (!f64 && p->vmode != kValPlain) {  // bfloat16 copy, or no values and a scale per column
-      if (p->vmode == kValBf16) {
-        __nv_bfloat16* b16 = nullptr;
-        GENCD_TRY(palloc(p, &b16, lpad));
-        k_plan_to_bf16<<<grid_for(lpad, kThreads, g), kThreads, 0, st>>>((const float*)P.light_val, lpad, b16);
-        GENCD_CUDA_TRY(cudaStreamSynchronize(st));
-        dev_free(p, P.light_val);
-        P.light_val = b16;
-      } else {
-        GENCD_CUDA_TRY(cudaStreamSynchronize(st));
-        dev_free(p, P.light_val);
-        P.light_val = nullptr;
-        GENCD_TRY(palloc(p, &P.light_scale, P.nlight));
-        k_plan_gather_scales<<<grid_for(P.nlight, kThreads, g), kThreads, 0, st>>>(P.light_cols, P.nlight, p->col_val,
-                                                                                    P.light_scale);
-      }
-      GENCD_CUDA_TRY(cudaGetLastError());
-    }
-    P.light_ntiles = (P.light_nnz + kLightTile - 1) / kLightTile;
-    GENCD_TRY(palloc(p, &P.light_tile_lc, P.light_ntiles + 1));
-    GENCD_TRY(launch_tile_map_of(p, P.light_col_ptr, P.nlight, P.light_ntiles, P.light_tile_lc, kLightTile));
-    const int64_t lwords = (lpad + 31) / 32;  // start bits, one byte per 8 entries
-    GENCD_TRY(palloc(p, (uint32_t**)&P.lmask, lwords));
-    GENCD_CUDA_TRY(cudaMemsetAsync(P.lmask, 0, 4 * (size_t)lwords, st));
-    k_plan_light_starts<<<grid_for(P.nlight, kThreads, g), kThreads, 0, st>>>(P.light_col_ptr, P.nlight,
-                                                                              (uint32_t*)P.lmask);
-    GENCD_CUDA_TRY(cudaGetLastError());
-  }
-  if (P.nheavy == 0) return GENCD_OK;
-
-  // heavy entries grouped by slab (stable: column-major order kept inside a slab)
-  uint32_t *keys, *order, *ka, *va, *hrow, *hh, *stmp;
-  char* hval;
-  GENCD_TRY(S.get(&keys, E));
-  GENCD_TRY(S.get(&order, E));
-  GENCD_TRY(S.get(&ka, E));
-  GENCD_TRY(S.get(&va, E));
-  GENCD_TRY(S.get(&hrow, E));
-  GENCD_TRY(S.get(&hh, E));
-  GENCD_TRY(S.get(&hval, E * (int64_t)vsz));
-  GENCD_TRY(S.get(&stmp, (int64_t)radix_tmp_words(E)));
-  if (f64)
-    k_plan_heavy_entries<double><<<grid_for(k * 32, kThreads, g), kThreads, 0, st>>>(
-        p->col_ptr, p->row_idx, (const double*)p->val, k, P.heavy_min, hid, hoff, P.slab_rows, keys, order, hrow,
-        hh, (double*)hval);
-  else
-    k_plan_heavy_entries<float><<<grid_for(k * 32, kThreads, g), kThreads, 0, st>>>(
-        p->col_ptr, p->row_idx, (const float*)p->val, k, P.heavy_min, hid, hoff, P.slab_rows, keys, order, hrow,
-        hh, (float*)hval);
-  GENCD_CUDA_TRY(cudaGetLastError());
-  bool in_alt = false;
-  GENCD_TRY(radix_sort_with_tmp(p, keys, order, E, bits_for_max(P.nslabs - 1), ka, va, stmp, &in_alt));
-  const uint32_t* sk = in_alt ? ka : keys;
-  const uint32_t* se = in_alt ? va : order;
-
-  // slab offsets (unpadded from the sorted keys; padded to 8 entries on the host)
+  P.light_nnz = tot[2];
+  const int64_t E = p->nnz - P.light_nnz;  // heavy entries
   const int R = P.nslabs;
+  const int64_t runs = (int64_t)R * P.nheavy;  // at most E / 2 with several slabs (heavy_min), E with one
+
+  // the plan's per-column arrays and the light columns' copy
+  const int64_t lpad = P.nlight > 0 ? ((P.light_nnz + kPadNnz - 1) / kPadNnz) * kPadNnz + kPadNnz : 0;
+  const int64_t lwords = (lpad + 31) / 32;  // start bits, one byte per 8 entries
+  P.light_ntiles = (P.light_nnz + kLightTile - 1) / kLightTile;
+  const bool fusable = !f64 && P.nlight > 0 && P.nheavy > 0;
+  Arena light;
+  light.add(&P.heavy_cols, P.nheavy);
+  light.add(&P.light_cols, P.nlight);
+  light.add(&P.light_col_ptr, P.nlight + 1);
+  light.add(&P.light_row, lpad);
+  light.add((char**)&P.light_val, lpad * (int64_t)vsz);
+  light.add(&P.light_tile_lc, P.light_ntiles + 1);
+  light.add((uint32_t**)&P.lmask, lwords);
+  if (p->vmode == kValNone && P.nlight > 0) light.add(&P.light_scale, P.nlight);
+  if (fusable) light.add(&P.light_counter, 2);  // tiles taken, warps finished
+  light.add(&P.slab_tile_begin, R + 1);
+  P.grid = p->num_sms;
+  light.add(&P.cta_tile_begin, P.grid + 1);
+  GENCD_TRY(dev_alloc_bytes(p, &P.mem[0], light.bytes()));
+  light.place(P.mem[0]);
+  k_plan_columns<<<grid_for(k + 1, kThreads, g), kThreads, 0, st>>>(p->col_ptr, k, P.heavy_min, hid, lid, loff,
+                                                                     P.heavy_cols, P.light_cols, P.light_col_ptr,
+                                                                     p->col_val, P.light_scale);
+  GENCD_CUDA_TRY(cudaGetLastError());
+  if (P.nlight > 0) {
+    if (p->vmode == kValNone) {  // padding has no value to zero it: it gathers u[n] = 0 instead
+      k_plan_fill<int32_t><<<grid_for(lpad - P.light_nnz, kThreads, g), kThreads, 0, st>>>(
+          P.light_row + P.light_nnz, lpad - P.light_nnz, (int32_t)n);
+      GENCD_CUDA_TRY(cudaGetLastError());
+    } else {
+      GENCD_CUDA_TRY(cudaMemsetAsync(P.light_row + P.light_nnz, 0, sizeof(int32_t) * (lpad - P.light_nnz), st));
+      GENCD_CUDA_TRY(cudaMemsetAsync((char*)P.light_val + vsz * P.light_nnz, 0, vsz * (lpad - P.light_nnz), st));
+    }
+    GENCD_CUDA_TRY(cudaMemsetAsync(P.lmask, 0, 4 * (size_t)lwords, st));
+    GENCD_TRY(launch_tile_map_of(p, P.light_col_ptr, P.nlight, P.light_ntiles, P.light_tile_lc, kLightTile));
+  }
+  if (fusable) GENCD_CUDA_TRY(cudaMemsetAsync(P.light_counter, 0, 2 * sizeof(unsigned int), st));
+
+  // the heavy columns' runs per slab, in slab order
+  uint32_t *seg, *pos, *pair, *pair_start, *rtmp;
   int64_t *slab_begin, *pad_off;
-  GENCD_TRY(S.get(&slab_begin, R + 1));
-  GENCD_TRY(S.get(&pad_off, R + 1));
-  GENCD_TRY(lower_bounds_u32_to_i64(p, sk, E, R, slab_begin));
-  std::vector<int64_t> hb(R + 1), hp(R + 1);
-  GENCD_CUDA_TRY(cudaMemcpyAsync(hb.data(), slab_begin, 8 * (R + 1), cudaMemcpyDeviceToHost, st));
-  GENCD_CUDA_TRY(cudaStreamSynchronize(st));
-  hp[0] = 0;
+  Arena heavy;
+  heavy.add(&seg, runs);
+  heavy.add(&pos, runs + 1);
+  heavy.add(&pair, runs + 1);
+  heavy.add(&pair_start, std::min(runs, E) + 1);  // a run that is not empty is a pair
+  heavy.add(&rtmp, scan_tmp_words(runs + 1));
+  heavy.add(&slab_begin, R + 2);
+  heavy.add(&pad_off, R + 1);
+  GENCD_TRY(S.get(heavy));
+  std::vector<int64_t> hb(R + 2, 0), hp(R + 1, 0);
+  if (P.nheavy > 0) {
+    k_plan_segments<<<grid_for(runs + 1, kThreads, p->num_sms * 32), kThreads, 0, st>>>(
+        p->col_ptr, p->row_idx, P.heavy_cols, P.nheavy, runs, R, P.slab_rows, seg, pos, pair);
+    GENCD_TRY(exclusive_scan(p, pos, pos, runs + 1, rtmp));
+    GENCD_TRY(exclusive_scan(p, pair, pair, runs + 1, rtmp));
+    k_plan_slab_begins<<<1, kThreads, 0, st>>>(pos, pair, P.nheavy, R, slab_begin);
+    GENCD_CUDA_TRY(cudaGetLastError());
+    GENCD_CUDA_TRY(cudaMemcpyAsync(hb.data(), slab_begin, 8 * (R + 2), cudaMemcpyDeviceToHost, st));
+    GENCD_CUDA_TRY(cudaStreamSynchronize(st));
+  }
+  P.npairs = hb[R + 1];
   for (int r = 0; r < R; ++r) hp[r + 1] = hp[r] + ((hb[r + 1] - hb[r] + kSlabPad - 1) / kSlabPad) * kSlabPad;
   P.entries = hp[R];
   if (P.entries >= (int64_t(1) << 32)) return fail_plan("heavy entries exceed 2^32");
-  GENCD_CUDA_TRY(cudaMemcpyAsync(pad_off, hp.data(), 8 * (R + 1), cudaMemcpyHostToDevice, st));
-
-  GENCD_TRY(palloc(p, &P.s_row, P.entries + 8));
-  GENCD_TRY(palloc(p, (char**)&P.s_val, (P.entries + 8) * (int64_t)vsz));
-  GENCD_CUDA_TRY(cudaMemsetAsync(P.s_row, 0, 2 * (P.entries + 8), st));
-  GENCD_CUDA_TRY(cudaMemsetAsync(P.s_val, 0, vsz * (P.entries + 8), st));
-  if (p->vmode == kValNone) {  // padding reads the zero slot past the slab
-    k_plan_fill<uint16_t><<<grid_for(P.entries + 8, kThreads, g), kThreads, 0, st>>>(P.s_row, P.entries + 8,
-                                                                                     (uint16_t)P.slab_rows);
-    GENCD_CUDA_TRY(cudaGetLastError());
-  }
-  // start bits: one byte per 8 entries, written as 32-bit words (entries + 8 bits, rounded up to words)
-  const int64_t mask_words = (P.entries + 8 + 31) / 32;
-  GENCD_TRY(palloc(p, (uint32_t**)&P.pmask, mask_words));
-  GENCD_CUDA_TRY(cudaMemsetAsync(P.pmask, 0, 4 * (size_t)mask_words, st));
-  uint32_t* pidx;
-  GENCD_TRY(S.get(&pidx, E + 1));
-  if (f64)
-    k_plan_fill_slabs<double><<<grid_for(E, kThreads, g), kThreads, 0, st>>>(
-        sk, se, E, slab_begin, pad_off, P.slab_rows, hrow, hh, (const double*)hval, P.s_row, (double*)P.s_val,
-        pidx, (uint32_t*)P.pmask);
-  else
-    k_plan_fill_slabs<float><<<grid_for(E, kThreads, g), kThreads, 0, st>>>(
-        sk, se, E, slab_begin, pad_off, P.slab_rows, hrow, hh, (const float*)hval, P.s_row, (float*)P.s_val, pidx,
-        (uint32_t*)P.pmask);
-  GENCD_CUDA_TRY(cudaGetLastError());
-  if (!f64 && p->vmode != kValPlain) {  // bfloat16 copy, or no values and a scale per column
-    if (p->vmode == kValBf16) {
-      __nv_bfloat16* b16 = nullptr;
-      GENCD_TRY(palloc(p, &b16, P.entries + 8));
-      k_plan_to_bf16<<<grid_for(P.entries + 8, kThreads, g), kThreads, 0, st>>>((const float*)P.s_val, P.entries + 8,
-                                                                                b16);
-      GENCD_CUDA_TRY(cudaStreamSynchronize(st));
-      dev_free(p, P.s_val);
-      P.s_val = b16;
-    } else {
-      GENCD_CUDA_TRY(cudaStreamSynchronize(st));
-      dev_free(p, P.s_val);
-      P.s_val = nullptr;  // k_scale_heavy applies col_val[j] after the pass
-    }
-    GENCD_CUDA_TRY(cudaGetLastError());
-  }
-  uint32_t* ptmp;
-  GENCD_TRY(S.get(&ptmp, scan_tmp_words(E + 1)));
-  GENCD_TRY(exclusive_scan(p, pidx, pidx, E + 1, ptmp));
-  uint32_t np32 = 0;
-  GENCD_CUDA_TRY(cudaMemcpyAsync(&np32, pidx + E, 4, cudaMemcpyDeviceToHost, st));
-  GENCD_CUDA_TRY(cudaStreamSynchronize(st));
-  P.npairs = np32;
-
-  // pairs: first entry and column
-  uint32_t *pair_start, *pair_h;
-  GENCD_TRY(S.get(&pair_start, P.npairs + 1));
-  GENCD_TRY(S.get(&pair_h, P.npairs));
-  k_plan_fill_pairs<<<grid_for(E, kThreads, g), kThreads, 0, st>>>(sk, se, E, slab_begin, pad_off, hh, pidx,
-                                                                    pair_start, pair_h);
-  const uint32_t ent32 = (uint32_t)P.entries;
-  GENCD_CUDA_TRY(cudaMemcpyAsync(pair_start + P.npairs, &ent32, 4, cudaMemcpyHostToDevice, st));
-  GENCD_TRY(palloc(p, &P.pair_col, P.npairs));
-  k_plan_pair_cols<<<grid_for(P.npairs, kThreads, g), kThreads, 0, st>>>(pair_h, P.npairs, P.heavy_cols,
-                                                                          P.pair_col);
-  GENCD_CUDA_TRY(cudaGetLastError());
 
   // tiles inside each slab, and contiguous runs of tiles per CTA
-  std::vector<int32_t> tb(R + 1);
+  std::vector<int32_t> tb(R + 1), ctb(P.grid + 1);
   tb[0] = 0;
   const int64_t tile = 32LL * (f64 ? kSlabItemsF64 : kSlabItemsF32);  // the kernel's tile
   for (int r = 0; r < R; ++r) tb[r + 1] = tb[r] + (int32_t)((hp[r + 1] - hp[r] + tile - 1) / tile);
   P.ntiles = tb[R];
-  GENCD_TRY(palloc(p, &P.slab_tile_begin, R + 1));
-  GENCD_TRY(palloc(p, &P.tile_start, P.ntiles));
-  GENCD_TRY(palloc(p, &P.tile_end, P.ntiles));
-  GENCD_TRY(palloc(p, &P.tile_pair, P.ntiles));
-  GENCD_TRY(palloc(p, &P.tile_slab, P.ntiles));
-  GENCD_CUDA_TRY(cudaMemcpyAsync(P.slab_tile_begin, tb.data(), 4 * (R + 1), cudaMemcpyHostToDevice, st));
-  k_plan_tiles<<<grid_for(P.ntiles, kThreads, g), kThreads, 0, st>>>(P.slab_tile_begin, pad_off, R, P.ntiles, tile,
-                                                                      pair_start, P.npairs, P.tile_start,
-                                                                      P.tile_end, P.tile_pair, P.tile_slab);
-  GENCD_CUDA_TRY(cudaGetLastError());
-  P.grid = p->num_sms;
-  // both passes may run in one kernel when there are light and heavy columns
-  // (FP32 arithmetic: FP64 stages do not fit the fused kernel's registers);
-  // the autotuner below decides
-  P.fused_split = 0;
-  if (!f64 && P.nlight > 0 && P.nheavy > 0) {
-    GENCD_TRY(palloc(p, &P.light_counter, 2));  // tiles taken, warps finished
-    GENCD_CUDA_TRY(cudaMemsetAsync(P.light_counter, 0, 2 * sizeof(unsigned int), st));
-  }
-  std::vector<int32_t> ctb(P.grid + 1);
   for (int b = 0; b <= P.grid; ++b) ctb[b] = (int32_t)((int64_t)b * P.ntiles / P.grid);
-  GENCD_TRY(palloc(p, &P.cta_tile_begin, P.grid + 1));
-  GENCD_CUDA_TRY(cudaMemcpyAsync(P.cta_tile_begin, ctb.data(), 4 * (P.grid + 1), cudaMemcpyHostToDevice, st));
-  if (f64)
-    GENCD_TRY(set_slab_smem<GENCD_PLAN_F64>(P));
-  else if (p->vmode == kValBf16)
-    GENCD_TRY(set_slab_smem<GENCD_PLAN_F32(__nv_bfloat16)>(P));
-  else if (p->vmode == kValNone)
-    GENCD_TRY(set_slab_smem<GENCD_PLAN_F32(NoVal)>(P));
-  else
-    GENCD_TRY(set_slab_smem<GENCD_PLAN_F32(float)>(P));
-  GENCD_CUDA_TRY(cudaStreamSynchronize(st));  // scratch is freed on return
-  p->prof.launches[K_SETUP] += 10;
+  if (P.nheavy > 0) {
+    const int64_t mask_words = (P.entries + 8 + 31) / 32;  // start bits: one byte per 8 entries
+    Arena slabs;
+    slabs.add(&P.s_row, P.entries + 8);
+    slabs.add((char**)&P.s_val, (P.entries + 8) * (int64_t)vsz);
+    slabs.add((uint32_t**)&P.pmask, mask_words);
+    slabs.add(&P.pair_col, P.npairs);
+    slabs.add(&P.tile_start, P.ntiles);
+    slabs.add(&P.tile_end, P.ntiles);
+    slabs.add(&P.tile_pair, P.ntiles);
+    slabs.add(&P.tile_slab, P.ntiles);
+    GENCD_TRY(dev_alloc_bytes(p, &P.mem[1], slabs.bytes()));
+    slabs.place(P.mem[1]);
+    GENCD_CUDA_TRY(cudaMemcpyAsync(pad_off, hp.data(), 8 * (R + 1), cudaMemcpyHostToDevice, st));
+    GENCD_CUDA_TRY(cudaMemcpyAsync(P.slab_tile_begin, tb.data(), 4 * (R + 1), cudaMemcpyHostToDevice, st));
+    GENCD_CUDA_TRY(cudaMemcpyAsync(P.cta_tile_begin, ctb.data(), 4 * (P.grid + 1), cudaMemcpyHostToDevice, st));
+    GENCD_CUDA_TRY(cudaMemsetAsync(P.pmask, 0, 4 * (size_t)mask_words, st));
+    k_plan_pad<<<grid_for((int64_t)(R + 1) * kSlabPad, kThreads, g), kThreads, 0, st>>>(
+        slab_begin, pad_off, R, P.entries, p->vmode == kValNone ? (uint16_t)P.slab_rows : (uint16_t)0, P.s_row,
+        (char*)P.s_val, (int)vsz);
+    GENCD_CUDA_TRY(cudaGetLastError());
+  }
+  if (p->nnz > 0) {
+    if (f64)
+      launch_place<double, double>(p, hid, loff, seg, pos, pair, slab_begin, pad_off, pair_start);
+    else if (p->vmode == kValBf16)
+      launch_place<float, __nv_bfloat16>(p, hid, loff, seg, pos, pair, slab_begin, pad_off, pair_start);
+    else if (p->vmode == kValNone)
+      launch_place<float, NoVal>(p, hid, loff, seg, pos, pair, slab_begin, pad_off, pair_start);
+    else
+      launch_place<float, float>(p, hid, loff, seg, pos, pair, slab_begin, pad_off, pair_start);
+    GENCD_CUDA_TRY(cudaGetLastError());
+  }
+  P.fused_split = 0;
+  if (P.nheavy > 0) {
+    k_plan_tiles<<<grid_for(P.ntiles, kThreads, g), kThreads, 0, st>>>(P.slab_tile_begin, pad_off, R, P.ntiles, tile,
+                                                                        pair_start, P.npairs, P.tile_start,
+                                                                        P.tile_end, P.tile_pair, P.tile_slab);
+    GENCD_CUDA_TRY(cudaGetLastError());
+    // both passes may run in one kernel when there are light and heavy columns
+    // (FP32 arithmetic: FP64 stages do not fit the fused kernel's registers);
+    // the autotuner below decides
+    if (f64)
+      GENCD_TRY(set_slab_smem<GENCD_PLAN_F64>(P));
+    else if (p->vmode == kValBf16)
+      GENCD_TRY(set_slab_smem<GENCD_PLAN_F32(__nv_bfloat16)>(P));
+    else if (p->vmode == kValNone)
+      GENCD_TRY(set_slab_smem<GENCD_PLAN_F32(NoVal)>(P));
+    else
+      GENCD_TRY(set_slab_smem<GENCD_PLAN_F32(float)>(P));
+  }
+  GENCD_CUDA_TRY(cudaStreamSynchronize(st));  // scratch and the host arrays go when this returns
+  p->prof.launches[K_SETUP] += 7;
   return GENCD_OK;
 }
 
@@ -1188,43 +1155,63 @@ int build_propose_plan(gencd_problem* p) {
 }
 
 // Autotuner of the streaming propose: times the separate light and slab
-// kernels and every split of the fused kernel on this problem (three
-// launches each, CUDA events, u as it stands) and keeps the fastest.  All
-// candidates compute the same sums; the scratch they leave is cleared.
+// kernels and every split of the fused kernel on this problem (CUDA events, u
+// as it stands: one launch each, then two more of those within kTuneClose of
+// the fastest) and keeps the fastest.  All candidates compute the same sums;
+// the scratch they leave is cleared.
+constexpr float kTuneClose = 1.15f;
+
 int tune_propose_plan(gencd_problem* p) {
+  constexpr int C = kNumFusedSplits + 1;
   ProposePlan& P = p->plan;
   P.tuned_ms[0] = -1.0;
   if (!P.built || !P.light_counter) return GENCD_OK;
-  cudaEvent_t ev[2] = {nullptr, nullptr};
-  GENCD_CUDA_TRY(cudaEventCreate(&ev[0]));
-  if (cudaEventCreate(&ev[1]) != cudaSuccess) {
-    cudaEventDestroy(ev[0]);
-    return fail_plan("cudaEventCreate failed");
-  }
+  cudaEvent_t ev[2 * C] = {};
+  int rc = GENCD_OK;
+  for (cudaEvent_t& e : ev)
+    if (rc == GENCD_OK && cudaEventCreate(&e) != cudaSuccess) rc = fail_plan("cudaEventCreate failed");
   const bool prof = p->prof.enabled;
   p->prof.enabled = false;
-  int rc = GENCD_OK;
-  float best_ms = 0.f;
-  int best = 0;
-  for (int c = 0; c <= kNumFusedSplits && rc == GENCD_OK; ++c) {
-    P.fused_split = c == 0 ? 0 : kFusedSplits[c - 1];
-    if ((rc = launch_propose_plan(p, p->u)) != GENCD_OK) break;  // warm-up
-    cudaEventRecord(ev[0], p->stream);
-    for (int r = 0; r < 3 && rc == GENCD_OK; ++r) rc = launch_propose_plan(p, p->u);
-    cudaEventRecord(ev[1], p->stream);
-    if (rc != GENCD_OK || cudaEventSynchronize(ev[1]) != cudaSuccess) {
-      rc = rc != GENCD_OK ? rc : fail_plan("autotuning the streaming propose failed");
+  const int kept = P.fused_split;
+  auto form = [](int c) { return c == 0 ? 0 : kFusedSplits[c - 1]; };
+  bool runs[C];
+  int reps[C] = {};
+  float total[C] = {};
+  for (bool& r : runs) r = true;
+  // each form once untimed (the first launch loads it), then the timed launches
+  for (int pass = 0; pass < 3 && rc == GENCD_OK; ++pass) {
+    const int n_launch = pass == 2 ? 2 : 1;
+    for (int c = 0; c < C && rc == GENCD_OK; ++c) {
+      if (!runs[c]) continue;
+      P.fused_split = form(c);
+      if (pass > 0) cudaEventRecord(ev[2 * c], p->stream);
+      for (int r = 0; r < n_launch && rc == GENCD_OK; ++r) rc = launch_propose_plan(p, p->u);
+      if (pass > 0) cudaEventRecord(ev[2 * c + 1], p->stream);
+    }
+    if (rc != GENCD_OK || pass == 0) continue;
+    if (cudaStreamSynchronize(p->stream) != cudaSuccess) {
+      rc = fail_plan("autotuning the streaming propose failed");
       break;
     }
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, ev[0], ev[1]);
-    P.tuned_ms[c] = ms / 3.0;
-    if (c == 0 || ms < best_ms) best_ms = ms, best = P.fused_split;
+    float best = 0.f;
+    for (int c = 0; c < C; ++c) {
+      if (!runs[c]) continue;
+      float ms = 0.f;
+      cudaEventElapsedTime(&ms, ev[2 * c], ev[2 * c + 1]);
+      total[c] += ms;
+      reps[c] += n_launch;
+      P.tuned_ms[c] = total[c] / reps[c];
+      if (c == 0 || (float)P.tuned_ms[c] < best) best = (float)P.tuned_ms[c];
+    }
+    for (int c = 0; c < C; ++c) runs[c] = (float)P.tuned_ms[c] <= kTuneClose * best;
   }
+  int best = 0;
+  for (int c = 1; c < C; ++c)
+    if (P.tuned_ms[c] < P.tuned_ms[best]) best = c;
   p->prof.enabled = prof;
-  P.fused_split = best;
-  cudaEventDestroy(ev[0]);
-  cudaEventDestroy(ev[1]);
+  P.fused_split = rc == GENCD_OK ? form(best) : kept;
+  for (cudaEvent_t e : ev)
+    if (e) cudaEventDestroy(e);
   if (rc != GENCD_OK) return rc;
   // the candidates' sums are scratch: the hot path expects them zero
   const size_t gsz = p->precision == GENCD_F64 ? sizeof(double) : sizeof(float);
