@@ -229,6 +229,7 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   if (gtid == 0) s_u[slab_rows] = U(0);  // the row of padding entries (index-only storage)
+  bool waited = false;
   while (t0 < t_end) {
     const int r = tile_slab[t0];
     const int tb = slab_tile_begin[r], tnext = slab_tile_begin[r + 1];
@@ -236,7 +237,16 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
     const uint32_t base = tile_start[tb], slab_end = tile_end[tnext - 1];  // the slab's entries
     const int64_t row0 = (int64_t)r * slab_rows;
     const int rows = (int)min((int64_t)slab_rows, n - row0);
+    TileStage<SV, ITEMS> stg[DEPTH > 0 ? DEPTH : 1];
+    int t = t0 + warp;
+#pragma unroll
+    for (int d = 0; d < DEPTH; ++d)
+      load_stage<SV, ITEMS>(s_row, s_val, pmask, tile_pair, t + d * nw, t1, base, tb, slab_end, lane, stg[d]);
     slab_barrier<BAR_THREADS>();  // the previous slab is no longer read
+    if (!waited) {  // the plan is read while the kernel that writes u still runs
+      pdl_wait();
+      waited = true;
+    }
     {  // 16-byte loads, four in flight per thread, when u + row0 is 16-byte aligned
       const bool al = (reinterpret_cast<uintptr_t>(u + row0) & 15u) == 0;
       const int nvec = al ? (int)(((int64_t)rows * (int64_t)sizeof(U)) / 16) : 0;
@@ -247,11 +257,6 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
       for (int i = (int)((int64_t)nvec * 16 / (int64_t)sizeof(U)) + gtid; i < rows; i += gthreads) s_u[i] = u[row0 + i];
     }
     slab_barrier<BAR_THREADS>();
-    TileStage<SV, ITEMS> stg[DEPTH > 0 ? DEPTH : 1];
-    int t = t0 + warp;
-#pragma unroll
-    for (int d = 0; d < DEPTH; ++d)
-      load_stage<SV, ITEMS>(s_row, s_val, pmask, tile_pair, t + d * nw, t1, base, tb, slab_end, lane, stg[d]);
     for (; t < t1; t += nw) {  // warp-uniform loop
       TileStage<SV, ITEMS> cur;
       if (DEPTH > 0) {
@@ -346,6 +351,7 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
     }
     t0 = t1;
   }
+  if (!waited) pdl_wait();
 }
 
 // THREADS per CTA (one CTA per SM); see slab_pass
@@ -361,7 +367,6 @@ __global__ void __launch_bounds__(THREADS, 1)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   U* s_u = reinterpret_cast<U*>(smem_raw);
   pdl_trigger();
-  pdl_wait();
   slab_pass<V, U, G, DEPTH, ITEMS, SV, 0>(s_row, s_val, pmask, pair_col, tile_start, tile_end, tile_pair, tile_slab,
                                           slab_tile_begin, cta_tile_begin[blockIdx.x],
                                           cta_tile_begin[blockIdx.x + 1], u, n, slab_rows, gacc, s_u,
@@ -509,10 +514,10 @@ __global__ void __launch_bounds__(kThreads, 3)
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   pdl_trigger();
-  pdl_wait();
   constexpr bool kPrefetch = sizeof(V) == 4;  // FP64 stages are too large to double in registers
   LightStage<SV> nxt;
   if (kPrefetch) load_light_stage<SV>(row, val, lmask, tile_lc, warp, ntiles, nnz, lane, nxt);
+  pdl_wait();
   for (int64_t t = warp; t < ntiles; t += nwarps) {  // warp-uniform
     LightStage<SV> cur;
     if (kPrefetch) {
@@ -581,13 +586,14 @@ __global__ void __launch_bounds__(THREADS, 1)
   extern __shared__ __align__(16) unsigned char smem_raw[];
   U* s_u = reinterpret_cast<U*>(smem_raw);
   pdl_trigger();
-  pdl_wait();
   const int warp = threadIdx.x >> 5;
   if (warp < SLAB_WARPS)
     slab_pass<V, U, G, DEPTH, ITEMS, SV, 32 * SLAB_WARPS>(
         s_row, s_val, pmask, pair_col, tile_start, tile_end, tile_pair, tile_slab, slab_tile_begin,
         cta_tile_begin[blockIdx.x], cta_tile_begin[blockIdx.x + 1], u, n, slab_rows, gacc, s_u, warp, SLAB_WARPS,
         threadIdx.x, 32 * SLAB_WARPS);
+  else
+    pdl_wait();
   light_pool<V, U, G, SV>(lrow, lval, lmask, tile_lc, light_cols, lscale, u, lnnz, lntiles, gacc, counter);
   // the last warp out resets the pool for the next launch: every warp has
   // taken its last tiles when it gets here (counter[1] counts the exits)
