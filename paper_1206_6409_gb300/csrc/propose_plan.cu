@@ -148,13 +148,16 @@ __device__ __forceinline__ uint32_t lane_mask(const uint8_t* __restrict__ pmask,
 
 // Segmented suffix sum over the lanes: T_L = x_L + x_{L+1} + ... + x_M where M
 // is the first lane >= L with stop set (all lanes to 31 when there is none);
-// ended_L reports whether such an M exists.  Five shuffle steps.
+// ended_L reports whether such an M exists.  Five shuffle steps; in FP64, whose
+// additions are what the passes wait for, only as many as the longest run of
+// the warp takes.
 template <typename V>
 __device__ __forceinline__ V lane_suffix_sum(V x, bool stop, int lane, bool& ended) {
   V t = x;
   bool e = stop;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
+    if (sizeof(V) == 8 && !__any_sync(0xffffffffu, !e && lane + d < 32)) break;
     const V tn = __shfl_down_sync(0xffffffffu, t, d);
     const bool en = __shfl_down_sync(0xffffffffu, (int)e, d) != 0;
     if (!e && lane + d < 32) {
