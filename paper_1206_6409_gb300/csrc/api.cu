@@ -661,6 +661,7 @@ static int create_impl(gencd_problem* p, const int64_t* col_ptr, const int32_t* 
   a.add(&p->scan_tmp, scan_tmp_words(k + 2));
   a.add(&p->dscal, kScalars);
   a.add(&p->red, 3 * kRedBlocks);
+  a.add(&p->ltab, kLogisticWords);
   GENCD_TRY(dev_alloc_bytes(p, &p->mem, a.bytes()));
   a.place(p->mem);
   p->gnat = p->precision == GENCD_F64 ? (void*)p->gacc : gf;
@@ -692,6 +693,8 @@ static int create_impl(gencd_problem* p, const int64_t* col_ptr, const int32_t* 
     }
   }
   GENCD_CUDA_TRY(cudaMemcpyAsync(p->y, y, sizeof(double) * n, kind_in(memory), st));
+  GENCD_CUDA_TRY(cudaMemcpyAsync(p->ltab, logistic_table().data(), sizeof(double) * kLogisticWords,
+                                 cudaMemcpyHostToDevice, st));
 
   int64_t bad_col = -1, bad_row = -1;
   int stage = 0;

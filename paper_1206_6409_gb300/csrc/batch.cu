@@ -755,7 +755,7 @@ __global__ void k_b_objective(const double* __restrict__ y, const double* __rest
                               const uint8_t* __restrict__ fold, int nfolds, int loss, int64_t n,
                               const double* __restrict__ w, int64_t k, int Sp, const int32_t* __restrict__ list,
                               const int32_t* __restrict__ list_set, int m, const double* __restrict__ dual_scale,
-                              double* __restrict__ acc) {
+                              const double* __restrict__ tab, double* __restrict__ acc) {
   __shared__ double red[3][8][33];
   const int q = threadIdx.x;
   double sl = 0.0, s1 = 0.0, sc = 0.0;
@@ -766,8 +766,8 @@ __global__ void k_b_objective(const double* __restrict__ y, const double* __rest
     for (int64_t i = (int64_t)blockIdx.x * 8 + threadIdx.y; i < n; i += stride)
       if (b_train(fold, i, set, nfolds)) {
         const double zi = z[i * Sp + s];
-        sl += loss_value(loss, y[i], zi);
-        if (dual_scale) sc += loss_conjugate(loss, y[i], sc_s * loss_deriv(loss, y[i], zi));
+        sl += loss_value(loss, y[i], zi, tab);
+        if (dual_scale) sc += loss_conjugate(loss, y[i], sc_s * loss_deriv(loss, y[i], zi, tab));
       }
     for (int64_t j = (int64_t)blockIdx.x * 8 + threadIdx.y; j < k; j += stride) s1 += fabs(w[j * Sp + s]);
   }
@@ -1201,7 +1201,7 @@ static int slot_objectives(gencd_batch* b, const std::vector<int32_t>& slots, st
     const int grid = (int)std::min<int64_t>((work + 7) / 8, (int64_t)b->X->num_sms * 8);
     k_b_objective<<<grid, dim3(32, 8), 0, b->st>>>(b->X->y, b->z, b->fold, b->nfolds, b->loss, b->n, b->w, b->k, b->S,
                                                   b->obj_list, b->obj_list + 32, m, gap ? b->obj_acc + 96 : nullptr,
-                                                  b->obj_acc);
+                                                  b->X->ltab, b->obj_acc);
     GENCD_CUDA_TRY(cudaGetLastError());
     double h[96];
     GENCD_CUDA_TRY(cudaMemcpyAsync(h, b->obj_acc, sizeof(double) * 3 * m, cudaMemcpyDeviceToHost, b->st));

@@ -6,14 +6,43 @@
 
 namespace gencd {
 
+// Taylor polynomials of f(a) = log(1 + e^-a) (table 0) and s(a) = 1 / (1 + e^a)
+// (table 1) for 0 <= a < kLogisticEnd, eight coefficients about each multiple
+// of 1/32 (logistic_table() in kernels_setup.cu).  Both functions' nearest
+// singularities are at +-i pi, so the first term left out is below 1e-18 of
+// the value, and the constant terms are rounded from extended precision: the
+// result is within about one unit in the last place.  Some 12 FP64 operations
+// and one 64-byte row of the table, where the exponential, the logarithm and the
+// division of the direct formula take 50 (s) and 150 (f): an SM starts about two
+// FP64 operations a cycle, and these evaluations were what the passes over rows
+// waited for.
+constexpr double kLogisticEnd = 20.0;
+constexpr int kLogisticRows = 20 * 32 + 1;
+constexpr int kLogisticWords = 2 * 8 * kLogisticRows;  // doubles
+
+__device__ __forceinline__ double logistic_poly(const double* __restrict__ tab, int which, double a) {
+  const double shift = 211106232532992.0;  // 1.5 * 2^47: adding it rounds a to a multiple of 1/32
+  const double t = a + shift;
+  const int row = (int)(uint32_t)(uint64_t)__double_as_longlong(t);  // a * 32, rounded
+  const double r = a - (t - shift);
+  const double2* c = reinterpret_cast<const double2*>(tab + 8 * (which * kLogisticRows + row));
+  const double2 c01 = __ldg(c), c23 = __ldg(c + 1), c45 = __ldg(c + 2), c67 = __ldg(c + 3);
+  const double r2 = r * r;
+  const double hi = fma(fma(c67.y, r, c67.x), r, c45.y);
+  const double q = fma(fma(hi, r2, fma(c45.x, r, c23.y)), r2, fma(c23.x, r, c01.y));
+  return fma(q, r, c01.x);
+}
+
 // Section 1 losses.  t is the fitted value (Xw)_i.
-__device__ __forceinline__ double loss_value(int loss, double y, double t) {
+__device__ __forceinline__ double loss_value(int loss, double y, double t, const double* __restrict__ tab) {
   if (loss == 0) {  // squared: (y - t)^2 / 2
     double r = y - t;
     return 0.5 * r * r;
   }
-  double m = -y * t;  // logistic: log(1 + e^m), overflow-free on both sides of 0
-  return m > 0.0 ? m + log1p(exp(-m)) : log1p(exp(m));
+  const double m = -y * t;  // logistic: log(1 + e^m), overflow-free on both sides of 0
+  const double a = fabs(m);
+  const double f = a < kLogisticEnd ? logistic_poly(tab, 0, a) : log1p(exp(-a));
+  return m > 0.0 ? m + f : f;
 }
 
 // Derivative of the loss in t, u_i = l'(y_i, z_i): t - y (squared),
@@ -26,6 +55,15 @@ __device__ __forceinline__ double loss_deriv(int loss, double y, double t) {
     return -y * e / (1.0 + e);
   }
   return -y / (1.0 + exp(m));
+}
+
+// the same from the table
+__device__ __forceinline__ double loss_deriv(int loss, double y, double t, const double* __restrict__ tab) {
+  if (loss == 0) return t - y;
+  const double m = y * t;
+  if (!(fabs(m) < kLogisticEnd)) return loss_deriv(loss, y, t);
+  const double s = logistic_poly(tab, 1, fabs(m));
+  return -y * (m > 0.0 ? s : 1.0 - s);
 }
 
 // Convex conjugate of the loss in t, l*(y, v) = sup_t (v t - l(y, t)) (the
@@ -45,15 +83,15 @@ __device__ __forceinline__ double loss_conjugate(int loss, double y, double v) {
 // evaluates the logistic derivative in FP32 arithmetic (its result is stored
 // in FP32 anyway), from the FP64 fitted value.
 template <typename U>
-__device__ __forceinline__ U u_value(int loss, double y, double t);
+__device__ __forceinline__ U u_value(int loss, double y, double t, const double* __restrict__ tab = nullptr);
 
 template <>
-__device__ __forceinline__ double u_value<double>(int loss, double y, double t) {
-  return loss_deriv(loss, y, t);
+__device__ __forceinline__ double u_value<double>(int loss, double y, double t, const double* __restrict__ tab) {
+  return loss_deriv(loss, y, t, tab);
 }
 
 template <>
-__device__ __forceinline__ float u_value<float>(int loss, double y, double t) {
+__device__ __forceinline__ float u_value<float>(int loss, double y, double t, const double* __restrict__) {
   if (loss == 0) return (float)(t - y);
   const float yf = (float)y;
   const float m = (float)(y * t);

@@ -233,6 +233,7 @@ struct gencd_problem {
   double* dscal = nullptr;
   double* red = nullptr;  // per-block partial sums (2 * kRedBlocks)
   double* hpin = nullptr; // pinned host mirror of dscal
+  double* ltab = nullptr; // logistic_table() on the device
 
   // selection
   int32_t* perm = nullptr;  // current epoch permutation (k, or C for Coloring)
@@ -321,6 +322,7 @@ int launch_csr_spmv(gencd_problem* p, const double* x, double* out);  // out = X
 int launch_state_from_w(gencd_problem* p);  // z, u and w32 from p->w (synchronises the stream)
 
 // kernels_setup.cu
+const std::vector<double>& logistic_table();
 int launch_col_scale(gencd_problem* p);
 int launch_tile_map(gencd_problem* p);
 int make_permutation(gencd_problem* p, uint64_t seed, int64_t epoch, int64_t m, int32_t* out);

@@ -527,7 +527,7 @@ __device__ __forceinline__ double block_sum(double v, double* sm) {
 __global__ void __launch_bounds__(kThreads)
     k_objective_partial(const double* __restrict__ y, const double* __restrict__ z, int64_t n,
                         const double* __restrict__ w, int64_t k, int loss, double lam, int gap,
-                        const double* __restrict__ dscal, double* __restrict__ red) {
+                        const double* __restrict__ dscal, const double* __restrict__ tab, double* __restrict__ red) {
   __shared__ double sm[kThreads / 32];
   double sl = 0.0, sw = 0.0, sc = 0.0;
   double scale = 1.0;
@@ -536,10 +536,11 @@ __global__ void __launch_bounds__(kThreads)
     scale = gm > lam ? lam / gm : 1.0;
   }
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  // neighbouring warps on different SMs: few rows keep all FP64 pipes busy
+  const int64_t i0 = ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
   for (int64_t i = i0; i < n; i += stride) {
-    sl += loss_value(loss, y[i], z[i]);
-    if (gap) sc += loss_conjugate(loss, y[i], scale * loss_deriv(loss, y[i], z[i]));
+    sl += loss_value(loss, y[i], z[i], tab);
+    if (gap) sc += loss_conjugate(loss, y[i], scale * loss_deriv(loss, y[i], z[i], tab));
   }
   for (int64_t j = i0; j < k; j += stride) sw += fabs(w[j]);
   sl = block_sum<kThreads>(sl, sm);
@@ -779,7 +780,7 @@ int launch_objective(gencd_problem* p, bool gap) {
   cudaEvent_t ev = nullptr;
   prof_begin(p, K_OBJECTIVE, &ev);
   k_objective_partial<<<grid, kThreads, 0, p->stream>>>(p->y, p->z, p->n, p->w, p->k, p->loss, p->lambda,
-                                                        gap ? 1 : 0, p->dscal, p->red);
+                                                        gap ? 1 : 0, p->dscal, p->ltab, p->red);
   k_objective_final<<<1, 32, 0, p->stream>>>(p->red, grid, (double)p->n, p->lambda, gap ? 1 : 0, p->dscal);
   prof_end(p, ev);
   p->prof.launches[K_OBJECTIVE] += 1;  // two launches per objective

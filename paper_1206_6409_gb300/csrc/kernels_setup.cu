@@ -16,12 +16,41 @@
 //    them uses;
 //  * the pieces of the power iteration for rho (Section 4.1).
 #include <algorithm>
+#include <cmath>
 #include <vector>
 
 #include "device_math.cuh"
 #include "gencd_internal.cuh"
 
 namespace gencd {
+
+// The Taylor coefficients read by logistic_poly, formed once in extended
+// precision: with y(r) = 1 / (1 + e^(c + r)), y' = y^2 - y gives the coefficients of
+// y one after another, and those of log(1 + e^-(c + r)) are -y_k / (k + 1).
+const std::vector<double>& logistic_table() {
+  static const std::vector<double> table = [] {
+    std::vector<double> t((size_t)kLogisticWords);
+    double *f = t.data(), *s = f + 8 * kLogisticRows;
+    for (int i = 0; i < kLogisticRows; ++i) {
+      const long double e = std::exp(-(long double)i / 32.0L);
+      long double y[8];
+      y[0] = e / (1.0L + e);
+      for (int k = 0; k < 7; ++k) {
+        long double sq = 0.0L;
+        for (int a = 0; a <= k; ++a) sq += y[a] * y[k - a];
+        y[k + 1] = (sq - y[k]) / (long double)(k + 1);
+      }
+      f[8 * i] = (double)std::log1p(e);
+      s[8 * i] = (double)y[0];
+      for (int k = 1; k < 8; ++k) {
+        f[8 * i + k] = (double)(-y[k - 1] / (long double)k);
+        s[8 * i + k] = (double)y[k];
+      }
+    }
+    return t;
+  }();
+  return table;
+}
 
 // ---------------------------------------------------------------------------
 // validation: err[0] <- smallest bad column, err[1] <- smallest bad row (y)

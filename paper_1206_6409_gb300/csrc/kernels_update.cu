@@ -25,10 +25,11 @@ namespace gencd {
 template <typename U>
 __global__ void __launch_bounds__(kThreads)
     k_fill_u(const double* __restrict__ y, const double* __restrict__ z, int64_t n, int loss,
-             U* __restrict__ u, unsigned long long* counts, unsigned long long* report) {
+             const double* __restrict__ tab, U* __restrict__ u, unsigned long long* counts,
+             unsigned long long* report) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (int64_t i = i0; i < n; i += stride) u[i] = u_value<U>(loss, y[i], z[i]);
+  for (int64_t i = i0; i < n; i += stride) u[i] = u_value<U>(loss, y[i], z[i], tab);
   if (report && i0 < 2) {  // z = Xw's counts to the host's copy, and reset for the next call
     report[i0] = counts[i0];
     counts[i0] = 0ull;
@@ -172,7 +173,7 @@ __global__ void __launch_bounds__(kListThreads)
     k_refresh_flat(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
                    const int32_t* __restrict__ J, const uint32_t* __restrict__ list, int64_t m,
                    const double* __restrict__ y, const double* __restrict__ z, int64_t n, int loss,
-                   U* __restrict__ u, unsigned long long* __restrict__ counters) {
+                   const double* __restrict__ tab, U* __restrict__ u, unsigned long long* __restrict__ counters) {
   __shared__ uint32_t s_off[SCAN ? kListScanMax + 1 : 1];
   pdl_trigger();
   pdl_wait();
@@ -180,13 +181,13 @@ __global__ void __launch_bounds__(kListThreads)
   const int64_t total = off[m], stride = (int64_t)gridDim.x * kListThreads;
   const int64_t q0 = ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
   if (total >= n) {
-    for (int64_t i = q0; i < n; i += stride) u[i] = u_value<U>(loss, y[i], z[i]);
+    for (int64_t i = q0; i < n; i += stride) u[i] = u_value<U>(loss, y[i], z[i], tab);
     return;
   }
   for (int64_t q = q0; q < total; q += stride) {
     const int64_t e = entry_of(off, m, (uint32_t)q);
     const int32_t i = row_idx[col_ptr[J[e]] + ((uint32_t)q - off[e])];
-    u[i] = u_value<U>(loss, y[i], z[i]);
+    u[i] = u_value<U>(loss, y[i], z[i], tab);
   }
 }
 
@@ -313,7 +314,7 @@ __global__ void __launch_bounds__(kThreads)
                     double* __restrict__ z,
                     const double* __restrict__ y, const int32_t* __restrict__ perm, int64_t q,
                     const int32_t* __restrict__ color_ptr, const int32_t* __restrict__ cols_by_color,
-                    double n, double lam, int loss, int early,
+                    double n, double lam, int loss, const double* __restrict__ tab, int early,
                     unsigned long long* __restrict__ counters) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -348,13 +349,13 @@ __global__ void __launch_bounds__(kThreads)
       if (have) {
         const double zi = z0 + d * (double)v0;
         z[i0] = zi;
-        u[i0] = u_value<U>(loss, y0, zi);
+        u[i0] = u_value<U>(loss, y0, zi, tab);
       }
       for (int64_t p = s + lane + 32; p < t; p += 32) {
         const int32_t i = row_idx[p];
         const double zi = z[i] + d * (double)val[p];
         z[i] = zi;
-        u[i] = u_value<U>(loss, y[i], zi);
+        u[i] = u_value<U>(loss, y[i], zi, tab);
       }
       if (lane == 0) {
         w[j] = wj + d;
@@ -545,9 +546,9 @@ int launch_fill_u(gencd_problem* p, unsigned long long* counts, unsigned long lo
   if (p->n == 0) return GENCD_OK;
   const int grid = grid_for(p->n, kThreads, p->num_sms * 8);
   if (p->precision == GENCD_F64)
-    k_fill_u<double><<<grid, kThreads, 0, p->stream>>>(p->y, p->z, p->n, p->loss, (double*)p->u, counts, report);
+    k_fill_u<double><<<grid, kThreads, 0, p->stream>>>(p->y, p->z, p->n, p->loss, p->ltab, (double*)p->u, counts, report);
   else
-    k_fill_u<float><<<grid, kThreads, 0, p->stream>>>(p->y, p->z, p->n, p->loss, (float*)p->u, counts, report);
+    k_fill_u<float><<<grid, kThreads, 0, p->stream>>>(p->y, p->z, p->n, p->loss, p->ltab, (float*)p->u, counts, report);
   p->prof.launches[K_SETUP] += 1;
   GENCD_CUDA_TRY(cudaGetLastError());
   return GENCD_OK;
@@ -610,7 +611,7 @@ int launch_refresh_list(gencd_problem* p, const int32_t* J, int64_t m, bool coun
   prof_begin(p, K_REFRESH, &ev);
   auto go = [&](auto kernel, auto* u) {
     return launch_overlapped(kernel, list_grid(p), kListThreads, 0, p->stream, p->col_ptr, p->row_idx, J, p->list_off,
-                             m, p->y, p->z, p->n, p->loss, u, ctr);
+                             m, p->y, p->z, p->n, p->loss, p->ltab, u, ctr);
   };
   cudaError_t err;
   if (p->precision == GENCD_F64)
@@ -659,11 +660,11 @@ int launch_coloring_iter(gencd_problem* p, int64_t q, bool early) {
   if (p->precision == GENCD_F64)
     err = launch_overlapped(k_coloring_iter<double, double>, grid, 32 * per, 0, p->stream, p->col_ptr, p->row_idx,
                             (const double*)p->val, (double*)p->u, p->w, p->w32, p->bj, p->ib, p->z, p->y, p->perm, q,
-                            p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, early ? 1 : 0, ctr);
+                            p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, p->ltab, early ? 1 : 0, ctr);
   else
     err = launch_overlapped(k_coloring_iter<float, float>, grid, 32 * per, 0, p->stream, p->col_ptr, p->row_idx,
                             (const float*)p->val, (float*)p->u, p->w, p->w32, p->bj, p->ib, p->z, p->y, p->perm, q,
-                            p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, early ? 1 : 0, ctr);
+                            p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, p->ltab, early ? 1 : 0, ctr);
   prof_end(p, ev);
   GENCD_CUDA_TRY(err);
   return GENCD_OK;

@@ -872,3 +872,29 @@ def test_shotgun_steps_match(gb, name, P, precision):
     tol = 1e-10 if precision == "f64" else 2e-4
     np.testing.assert_allclose(w, w_cpu, rtol=0, atol=tol * max(1.0, np.abs(w_cpu).max()))
     np.testing.assert_allclose(z, z_cpu, rtol=0, atol=tol * max(1.0, np.abs(z_cpu).max()))
+
+
+def test_logistic_values_over_the_whole_range(gb):
+    # X = I: z = w, and with lambda = 0 a step is -4 u_i; margins at and next to
+    # the table's centres (multiples of 1/32), half way between them, at the
+    # end of its range (20), beyond it, and at 0
+    k = np.arange(0, 20 * 32 + 1) / 32.0
+    a = np.unique(np.concatenate([k, k[:-1] + 1 / 64, np.nextafter(k[:-1] + 1 / 64, 99), np.nextafter(k[1:], 0),
+                                  np.linspace(1e-9, 45.0, 3001), [1e-300, 1e-17, 700.0, 745.0, 800.0]]))
+    w = np.concatenate([a, -a])
+    n = w.size
+    y = np.where(np.arange(n) % 2 == 0, 1.0, -1.0)
+    prob = workloads.Problem(n, n, np.arange(n + 1, dtype=np.int64), np.arange(n, dtype=np.int32), np.ones(n), y,
+                             "logistic", np.zeros(n), "identity")
+    with gb.Problem(prob) as p:
+        p.set_lambda(0.0)
+        p.set_w(w)
+        d, _ = p.propose_at(np.arange(n, dtype=np.int32))
+        obj, _ = p.objective()
+    m = y.astype(np.longdouble) * w.astype(np.longdouble)
+    u = -y / (1 + np.exp(m))
+    # u to about two units in the last place, then divided by n, multiplied by
+    # 1/beta and n; results below the normal range carry fewer bits
+    np.testing.assert_allclose(d, (-4 * u).astype(np.float64), rtol=2e-15, atol=1e-305)
+    loss = np.sum(np.maximum(-m, 0) + np.log1p(np.exp(-np.abs(m)))) / n
+    assert obj == pytest.approx(float(loss), rel=1e-14)
