@@ -13,8 +13,8 @@
 // the lane-segmented pass with gathers from L2.
 //
 // Within a slab the kernel works like the CSC pass: a warp owns a tile of
-// 256 consecutive entries, a lane 8 of them (128-bit loads of rows and
-// values), a lane sums its entries pair by pair in registers and adds each
+// consecutive entries, a lane 8 (FP32) or 16 (FP64) of them (128-bit loads of
+// rows and values), a lane sums its entries pair by pair in registers and adds each
 // run's sum into g_j (an atomic add that returns nothing: other slabs and
 // tiles add to the same column); a run cut by lane boundaries is combined by
 // a segmented warp suffix sum first, and a full tile inside one pair is
@@ -33,34 +33,46 @@
 namespace gencd {
 
 constexpr int kSlabBytes = 192 * 1024;
-constexpr int kSlabThreadsF32 = 1024;  // 32 warps, the next tile's loads in flight
-constexpr int kSlabThreadsF64 = 1024;  // 32 warps, loads issued tile by tile
-constexpr int kSlabItemsF32 = 8;   // entries per lane and tile step
-constexpr int kSlabItemsF64 = 8;
-constexpr int kSlabPad = 16;       // slab entry ranges are padded to this
+// Entries of a slab are stored in tiles of kSlabTile, in the order in which a
+// warp's lanes load them: a lane owns 16 consecutive entries (or 8, taking half
+// a tile at a time), and its v-th 16-byte vector lies next to the other lanes'
+// v-th ones, so every load of a warp is one contiguous 512 bytes whatever the
+// lane's share (slab_at, load_lane).
+constexpr int kSlabTile = 512;
+// Shape of the row-slab kernel: threads, tiles of loads in flight beyond the
+// current one, entries per lane.  FP32 is bound by instructions and loads in
+// flight: 1024 / 1 / 8 takes 83 us with the light columns on 4e7 non-zeros,
+// 768 / 1 / 16 92 and 512 / 1 / 16 112.  FP64 is bound by its pipe, and a lane's
+// 16 entries halve the additions that combine the lanes: 10 Thread-Greedy
+// iterations on 2e7 non-zeros take 1259 us with 768 / 0 / 16, 1284 with 512 / 1 /
+// 16, 1322 with 1024 / 0 / 8.
+constexpr int kSlabThreadsF32 = 1024;
+constexpr int kSlabThreadsF64 = 768;
+constexpr int kSlabDepthF32 = 1;
+constexpr int kSlabDepthF64 = 0;
+constexpr int kSlabItemsF32 = 8;
+constexpr int kSlabItemsF64 = 16;
+constexpr int kFusedItems = 8;  // the kernel that runs both passes (FP32): entries per lane
+constexpr int kSlabPad = kSlabTile;  // slabs are padded to whole tiles
 constexpr int kSlabZeroSlot = 4;   // shared u slots past the slab (16 B); the first holds 0
 
 // ---------------------------------------------------------------------------
 // the kernel
 
+// N values as 16-byte vectors, `step` values from one vector to the next
 template <typename V, int N>
-__device__ __forceinline__ void load_vals(const V* __restrict__ p, V (&v)[N]) {
+__device__ __forceinline__ void load_vals(const V* __restrict__ p, V (&v)[N], int step) {
   constexpr int PER = 16 / (int)sizeof(V);  // values per 128-bit load
 #pragma unroll
   for (int q = 0; q < N / PER; ++q) {
     if (sizeof(V) == 4) {
-      const float4 x = __ldcs(reinterpret_cast<const float4*>(p) + q);
+      const float4 x = __ldcs(reinterpret_cast<const float4*>(p + q * step));
       v[4 * q] = (V)x.x, v[4 * q + 1] = (V)x.y, v[4 * q + 2] = (V)x.z, v[4 * q + 3] = (V)x.w;
     } else {
-      const double2 x = __ldcs(reinterpret_cast<const double2*>(p) + q);
+      const double2 x = __ldcs(reinterpret_cast<const double2*>(p + q * step));
       v[2 * q] = (V)x.x, v[2 * q + 1] = (V)x.y;
     }
   }
-}
-
-template <typename V>
-__device__ __forceinline__ void load8(const V* __restrict__ p, V (&v)[8]) {
-  load_vals<V, 8>(p, v);
 }
 
 template <typename G>
@@ -91,24 +103,24 @@ struct ValRegs;
 template <int N>
 struct ValRegs<float, N> {
   float v[N];
-  __device__ __forceinline__ void load(const float* __restrict__ p) { load_vals<float, N>(p, v); }
+  __device__ __forceinline__ void load(const float* __restrict__ p, int step = 4) { load_vals<float, N>(p, v, step); }
   __device__ __forceinline__ float get(int i) const { return v[i]; }
 };
 
 template <int N>
 struct ValRegs<double, N> {
   double v[N];
-  __device__ __forceinline__ void load(const double* __restrict__ p) { load_vals<double, N>(p, v); }
+  __device__ __forceinline__ void load(const double* __restrict__ p, int step = 2) { load_vals<double, N>(p, v, step); }
   __device__ __forceinline__ double get(int i) const { return v[i]; }
 };
 
 template <int N>
 struct ValRegs<__nv_bfloat16, N> {
   uint32_t w[N / 2];  // value 2q in the low half of w[q], 2q + 1 in the high half
-  __device__ __forceinline__ void load(const __nv_bfloat16* __restrict__ p) {
+  __device__ __forceinline__ void load(const __nv_bfloat16* __restrict__ p, int step = 8) {
 #pragma unroll
     for (int q = 0; q < N / 8; ++q) {
-      const uint4 x = __ldcs(reinterpret_cast<const uint4*>(p) + q);
+      const uint4 x = __ldcs(reinterpret_cast<const uint4*>(p + q * step));
       w[4 * q] = x.x, w[4 * q + 1] = x.y, w[4 * q + 2] = x.z, w[4 * q + 3] = x.w;
     }
   }
@@ -120,9 +132,23 @@ struct ValRegs<__nv_bfloat16, N> {
 
 template <int N>
 struct ValRegs<NoVal, N> {
-  __device__ __forceinline__ void load(const NoVal*) {}
+  __device__ __forceinline__ void load(const NoVal*, int = 0) {}
   __device__ __forceinline__ float get(int) const { return 1.0f; }
 };
+
+// values per 16-byte vector of a stored value (index-only storage has none)
+template <typename SV>
+__host__ __device__ constexpr int vector_of() {
+  return std::is_same<SV, NoVal>::value ? 8 : 16 / (int)sizeof(SV);
+}
+
+// where entry x of a tile (x < kSlabTile, in pair order) is stored, in vectors of
+// VW elements
+template <int VW>
+__device__ __forceinline__ uint32_t slab_at(uint32_t x) {
+  const uint32_t owner = x >> 4, i = x & 15u;
+  return (i / VW) * (32 * VW) + owner * VW + i % VW;
+}
 
 // the entries of one lane: ITEMS in-slab rows (128-bit loads of 8) and values
 template <typename SV, int ITEMS>
@@ -131,12 +157,18 @@ struct LaneLoad {
   ValRegs<SV, ITEMS> val;
 };
 
+// a0: the first entry, in pair order, of the warp's 32 * ITEMS ones
 template <typename SV, int ITEMS>
 __device__ __forceinline__ void load_lane(const uint16_t* __restrict__ s_row, const SV* __restrict__ s_val,
-                                          uint32_t a, LaneLoad<SV, ITEMS>& L) {
+                                          uint32_t a0, int lane, LaneLoad<SV, ITEMS>& L) {
+  constexpr int VW = vector_of<SV>();
+  const uint32_t tile = a0 & ~(uint32_t)(kSlabTile - 1);
+  const uint32_t owner = ITEMS == 16 ? (uint32_t)lane : ((a0 >> 8) & 1u) * 16u + ((uint32_t)lane >> 1);
+  const uint32_t half = ITEMS == 16 ? 0u : (uint32_t)lane & 1u;  // which 8 of the owner's 16 entries
 #pragma unroll
-  for (int h = 0; h < ITEMS / 8; ++h) L.rr[h] = __ldcs(reinterpret_cast<const uint4*>(s_row + a) + h);
-  L.val.load(s_val + a);
+  for (int h = 0; h < ITEMS / 8; ++h)
+    L.rr[h] = __ldcs(reinterpret_cast<const uint4*>(s_row + tile + (half + h) * 256u + owner * 8u));
+  L.val.load(s_val + tile + half * (8 / VW) * (32 * VW) + owner * VW, 32 * VW);
 }
 
 // start bits of a lane's ITEMS entries (one byte per 8 entries, little-endian)
@@ -189,15 +221,12 @@ template <typename SV, int ITEMS>
 __device__ __forceinline__ void load_stage(const uint16_t* __restrict__ s_row, const SV* __restrict__ s_val,
                                            const uint8_t* __restrict__ pmask,
                                            const uint32_t* __restrict__ tile_pair, int t, int t1, uint32_t base,
-                                           int tb, uint32_t slab_end, int lane, TileStage<SV, ITEMS>& S) {
-  S.m = 0;
+                                           int tb, int lane, TileStage<SV, ITEMS>& S) {
   if (t < t1) {
     S.q0 = __ldg(tile_pair + t);
-    const uint32_t a = base + (uint32_t)(t - tb) * (32 * ITEMS) + lane * ITEMS;
-    if (a < slab_end) {
-      load_lane<SV, ITEMS>(s_row, s_val, a, S.L);
-      S.m = lane_mask<ITEMS>(pmask, a);
-    }
+    const uint32_t a0 = base + (uint32_t)(t - tb) * (32 * ITEMS);
+    load_lane<SV, ITEMS>(s_row, s_val, a0, lane, S.L);
+    S.m = lane_mask<ITEMS>(pmask, a0 + lane * ITEMS);
   }
 }
 
@@ -212,6 +241,15 @@ __device__ __forceinline__ void slab_barrier() {
     asm volatile("bar.sync 1, %0;" ::"n"(BAR_THREADS) : "memory");
 }
 
+// tiles of one size (32 lanes of 16 or of 8 entries) over the slabs' entries
+struct SlabTiles {
+  const uint32_t* tile_pair;        // pair holding a tile's first entry
+  const int32_t* tile_slab;         // slab of each tile
+  const int32_t* slab_tile_begin;   // nslabs + 1
+  const int32_t* cta_tile_begin;    // grid + 1
+  const uint32_t* slab_off;         // first entry of each slab
+};
+
 // The row-slab pass of one CTA's contiguous run of tiles [t0, t_end), by the
 // warps warp = 0 .. nw - 1 of the slab group (ITEMS entries per lane, a tile
 // is 32 * ITEMS entries; DEPTH tiles of loads in flight per warp beyond the
@@ -219,32 +257,26 @@ __device__ __forceinline__ void slab_barrier() {
 template <typename V, typename U, typename G, int DEPTH, int ITEMS, typename SV, int BAR_THREADS>
 __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, const SV* __restrict__ s_val,
                                           const uint8_t* __restrict__ pmask, const uint32_t* __restrict__ pair_col,
-                                          const uint32_t* __restrict__ tile_start,
-                                          const uint32_t* __restrict__ tile_end,
-                                          const uint32_t* __restrict__ tile_pair,
-                                          const int32_t* __restrict__ tile_slab,
-                                          const int32_t* __restrict__ slab_tile_begin, int t0, const int t_end,
+                                          const SlabTiles& T, int t0, const int t_end,
                                           const U* __restrict__ u, int64_t n, int32_t slab_rows,
                                           G* __restrict__ gacc, U* s_u, const int warp, const int nw,
                                           const int gtid, const int gthreads) {
-  constexpr int TILE = 32 * ITEMS;
   constexpr uint32_t NOT_FIRST = ((1u << ITEMS) - 1u) & ~1u;  // start bits after a lane's first entry
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   if (gtid == 0) s_u[slab_rows] = U(0);  // the row of padding entries (index-only storage)
   bool waited = false;
   while (t0 < t_end) {
-    const int r = tile_slab[t0];
-    const int tb = slab_tile_begin[r], tnext = slab_tile_begin[r + 1];
-    const int t1 = min(t_end, tnext);
-    const uint32_t base = tile_start[tb], slab_end = tile_end[tnext - 1];  // the slab's entries
+    const int r = T.tile_slab[t0];
+    const int tb = T.slab_tile_begin[r], t1 = min(t_end, T.slab_tile_begin[r + 1]);
+    const uint32_t base = T.slab_off[r];  // the slab's entries
     const int64_t row0 = (int64_t)r * slab_rows;
     const int rows = (int)min((int64_t)slab_rows, n - row0);
     TileStage<SV, ITEMS> stg[DEPTH > 0 ? DEPTH : 1];
     int t = t0 + warp;
 #pragma unroll
     for (int d = 0; d < DEPTH; ++d)
-      load_stage<SV, ITEMS>(s_row, s_val, pmask, tile_pair, t + d * nw, t1, base, tb, slab_end, lane, stg[d]);
+      load_stage<SV, ITEMS>(s_row, s_val, pmask, T.tile_pair, t + d * nw, t1, base, tb, lane, stg[d]);
     slab_barrier<BAR_THREADS>();  // the previous slab is no longer read
     if (!waited) {  // the plan is read while the kernel that writes u still runs
       pdl_wait();
@@ -266,19 +298,13 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
         cur = stg[0];
 #pragma unroll
         for (int d = 0; d + 1 < DEPTH; ++d) stg[d] = stg[d + 1];
-        load_stage<SV, ITEMS>(s_row, s_val, pmask, tile_pair, t + DEPTH * nw, t1, base, tb, slab_end, lane,
-                              stg[DEPTH - 1]);
+        load_stage<SV, ITEMS>(s_row, s_val, pmask, T.tile_pair, t + DEPTH * nw, t1, base, tb, lane, stg[DEPTH - 1]);
       } else {
-        load_stage<SV, ITEMS>(s_row, s_val, pmask, tile_pair, t, t1, base, tb, slab_end, lane, cur);
+        load_stage<SV, ITEMS>(s_row, s_val, pmask, T.tile_pair, t, t1, base, tb, lane, cur);
       }
-      const uint32_t ts = base + (uint32_t)(t - tb) * TILE;
-      const uint32_t te = slab_end - ts < (uint32_t)TILE ? slab_end : ts + TILE;
-      const uint32_t q0 = cur.q0;
-      uint32_t m = cur.m;
-      const uint32_t a = ts + lane * ITEMS;
-      const bool active = a < te;  // slab ends are multiples of ITEMS
-      if (!active) m = 0;
-      // pair of the lane's first entry: q0 + start bits in (ts, a] of the tile
+      const uint32_t q0 = cur.q0, m = cur.m;
+      // pair of the lane's first entry: q0 + the tile's start bits after its
+      // first entry and up to the lane's
       const uint32_t cnt = __popc(lane == 0 ? (m & NOT_FIRST) : m);
       uint32_t incl = cnt;
 #pragma unroll
@@ -289,12 +315,12 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
       uint32_t q = q0 + (incl - cnt) + (lane > 0 ? (m & 1u) : 0u);
       // columns of the pairs this lane may emit, loaded early: the tile's
       // first pair (lane 0) and the pair of the lane's last run
-      const bool lead = lane == 0 && active && !(m & 1u);
+      const bool lead = lane == 0 && !(m & 1u);
       const uint32_t col0 = lead ? __ldg(pair_col + q0) : 0u;
-      const uint32_t col_last = (active && m != 0u) ? __ldg(pair_col + q + __popc(m & NOT_FIRST)) : 0u;
+      const uint32_t col_last = m != 0u ? __ldg(pair_col + q + __popc(m & NOT_FIRST)) : 0u;
       V cont = V(0), tail = V(0);
       bool has_tail = false;
-      if (active) {
+      {
         U uu[ITEMS];
 #pragma unroll
         for (int h = 0; h < ITEMS / 8; ++h) {
@@ -339,7 +365,7 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
           cont = acc;
         }
       }
-      const bool stop = !active || m != 0u;
+      const bool stop = m != 0u;
       if (__ballot_sync(FULL, stop) == 0u) {
         // the whole tile lies inside pair q0
         const V sum = warp_sum(cont);
@@ -361,18 +387,13 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
 template <typename V, typename U, typename G, int THREADS, int DEPTH, int ITEMS, typename SV>
 __global__ void __launch_bounds__(THREADS, 1)
     k_propose_slabs(const uint16_t* __restrict__ s_row, const SV* __restrict__ s_val,
-                    const uint8_t* __restrict__ pmask, const uint32_t* __restrict__ pair_col,
-                    const uint32_t* __restrict__ tile_start,
-                    const uint32_t* __restrict__ tile_end, const uint32_t* __restrict__ tile_pair,
-                    const int32_t* __restrict__ tile_slab, const int32_t* __restrict__ slab_tile_begin,
-                    const int32_t* __restrict__ cta_tile_begin, const U* __restrict__ u, int64_t n,
-                    int32_t slab_rows, G* __restrict__ gacc) {
+                    const uint8_t* __restrict__ pmask, const uint32_t* __restrict__ pair_col, SlabTiles T,
+                    const U* __restrict__ u, int64_t n, int32_t slab_rows, G* __restrict__ gacc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   U* s_u = reinterpret_cast<U*>(smem_raw);
   pdl_trigger();
-  slab_pass<V, U, G, DEPTH, ITEMS, SV, 0>(s_row, s_val, pmask, pair_col, tile_start, tile_end, tile_pair, tile_slab,
-                                          slab_tile_begin, cta_tile_begin[blockIdx.x],
-                                          cta_tile_begin[blockIdx.x + 1], u, n, slab_rows, gacc, s_u,
+  slab_pass<V, U, G, DEPTH, ITEMS, SV, 0>(s_row, s_val, pmask, pair_col, T, T.cta_tile_begin[blockIdx.x],
+                                          T.cta_tile_begin[blockIdx.x + 1], u, n, slab_rows, gacc, s_u,
                                           threadIdx.x >> 5, blockDim.x >> 5, threadIdx.x, blockDim.x);
 }
 
@@ -577,10 +598,7 @@ __device__ __forceinline__ void light_pool(const int32_t* __restrict__ row, cons
 template <typename V, typename U, typename G, int THREADS, int SLAB_WARPS, int DEPTH, int ITEMS, typename SV>
 __global__ void __launch_bounds__(THREADS, 1)
     k_propose_fused(const uint16_t* __restrict__ s_row, const SV* __restrict__ s_val,
-                    const uint8_t* __restrict__ pmask, const uint32_t* __restrict__ pair_col,
-                    const uint32_t* __restrict__ tile_start, const uint32_t* __restrict__ tile_end,
-                    const uint32_t* __restrict__ tile_pair, const int32_t* __restrict__ tile_slab,
-                    const int32_t* __restrict__ slab_tile_begin, const int32_t* __restrict__ cta_tile_begin,
+                    const uint8_t* __restrict__ pmask, const uint32_t* __restrict__ pair_col, SlabTiles T,
                     const int32_t* __restrict__ lrow, const SV* __restrict__ lval,
                     const uint8_t* __restrict__ lmask, const int32_t* __restrict__ tile_lc,
                     const int32_t* __restrict__ light_cols, const float* __restrict__ lscale, int64_t lnnz,
@@ -592,9 +610,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   const int warp = threadIdx.x >> 5;
   if (warp < SLAB_WARPS)
     slab_pass<V, U, G, DEPTH, ITEMS, SV, 32 * SLAB_WARPS>(
-        s_row, s_val, pmask, pair_col, tile_start, tile_end, tile_pair, tile_slab, slab_tile_begin,
-        cta_tile_begin[blockIdx.x], cta_tile_begin[blockIdx.x + 1], u, n, slab_rows, gacc, s_u, warp, SLAB_WARPS,
-        threadIdx.x, 32 * SLAB_WARPS);
+        s_row, s_val, pmask, pair_col, T, T.cta_tile_begin[blockIdx.x], T.cta_tile_begin[blockIdx.x + 1], u, n,
+        slab_rows, gacc, s_u, warp, SLAB_WARPS, threadIdx.x, 32 * SLAB_WARPS);
   else
     pdl_wait();
   light_pool<V, U, G, SV>(lrow, lval, lmask, tile_lc, light_cols, lscale, u, lnnz, lntiles, gacc, counter);
@@ -635,6 +652,10 @@ static int scale_heavy(gencd_problem* p) {
   return GENCD_OK;
 }
 
+static SlabTiles tiles_of(const ProposePlan& P, const ProposePlan::Tiles& t) {
+  return SlabTiles{t.pair, t.slab, t.slab_begin, t.cta_begin, P.slab_off};
+}
+
 // the two streaming passes for one value storage SV (V compute type, U type
 // of u, G accumulator)
 constexpr int kFusedThreads = 1024;
@@ -644,34 +665,39 @@ constexpr int kFusedThreads = 1024;
 constexpr int kFusedSplits[] = {20, 24, 28, 31};
 constexpr int kNumFusedSplits = 4;
 
-template <typename V, typename U, typename G, typename SV, int DEPTH, int ITEMS, int SW>
+template <typename V, typename U, typename G, typename SV, int SW>
 static cudaError_t launch_fused(gencd_problem* p, const void* u_vec, size_t smem) {
   ProposePlan& P = p->plan;
-  return launch_overlapped(k_propose_fused<V, U, G, kFusedThreads, SW, DEPTH, ITEMS, SV>, P.grid, kFusedThreads, smem,
-                           p->stream,
-      P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, P.tile_start, P.tile_end, P.tile_pair, P.tile_slab,
-      P.slab_tile_begin, P.cta_tile_begin, P.light_row, (const SV*)P.light_val, P.lmask, P.light_tile_lc,
-      P.light_cols, P.light_scale, P.light_nnz, P.light_ntiles, P.light_counter, (const U*)u_vec, p->n,
-      P.slab_rows, (G*)p->gnat);
+  return launch_overlapped(k_propose_fused<V, U, G, kFusedThreads, SW, 1, kFusedItems, SV>, P.grid, kFusedThreads, smem,
+                           p->stream, P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P, P.fused),
+                           P.light_row, (const SV*)P.light_val, P.lmask, P.light_tile_lc, P.light_cols, P.light_scale,
+                           P.light_nnz, P.light_ntiles, P.light_counter, (const U*)u_vec, p->n, P.slab_rows,
+                           (G*)p->gnat);
+}
+
+// both passes in one kernel
+template <typename V, typename U, typename G, typename SV>
+static int launch_fused_passes(gencd_problem* p, const void* u_vec) {
+  const size_t smem = (size_t)(p->plan.slab_rows + kSlabZeroSlot) * sizeof(U);
+  cudaEvent_t e1 = nullptr;
+  prof_begin(p, K_PROPOSE_FUSED, &e1);
+  cudaError_t err;
+  switch (p->plan.fused_split) {
+    case 20: err = launch_fused<V, U, G, SV, 20>(p, u_vec, smem); break;
+    case 24: err = launch_fused<V, U, G, SV, 24>(p, u_vec, smem); break;
+    case 28: err = launch_fused<V, U, G, SV, 28>(p, u_vec, smem); break;
+    default: err = launch_fused<V, U, G, SV, 31>(p, u_vec, smem); break;
+  }
+  prof_end(p, e1);
+  GENCD_CUDA_TRY(err);
+  return scale_heavy<G, SV>(p);
 }
 
 template <typename V, typename U, typename G, typename SV, int THREADS, int DEPTH, int ITEMS>
 static int launch_plan_passes(gencd_problem* p, const void* u_vec) {
   ProposePlan& P = p->plan;
-  if (P.fused_split > 0) {  // both passes in one kernel
-    const size_t smem = (size_t)(P.slab_rows + kSlabZeroSlot) * sizeof(U);
-    cudaEvent_t e1 = nullptr;
-    prof_begin(p, K_PROPOSE_FUSED, &e1);
-    cudaError_t err;
-    switch (P.fused_split) {
-      case 20: err = launch_fused<V, U, G, SV, DEPTH, ITEMS, 20>(p, u_vec, smem); break;
-      case 24: err = launch_fused<V, U, G, SV, DEPTH, ITEMS, 24>(p, u_vec, smem); break;
-      case 28: err = launch_fused<V, U, G, SV, DEPTH, ITEMS, 28>(p, u_vec, smem); break;
-      default: err = launch_fused<V, U, G, SV, DEPTH, ITEMS, 31>(p, u_vec, smem); break;
-    }
-    prof_end(p, e1);
-    GENCD_CUDA_TRY(err);
-    return scale_heavy<G, SV>(p);
+  if constexpr (sizeof(V) == 4) {
+    if (P.fused_split > 0) return launch_fused_passes<V, U, G, SV>(p, u_vec);
   }
   if (P.nlight > 0) {
     cudaEvent_t e = nullptr;
@@ -688,8 +714,9 @@ static int launch_plan_passes(gencd_problem* p, const void* u_vec) {
     cudaEvent_t e1 = nullptr;
     prof_begin(p, K_PROPOSE_SLABS, &e1);
     const cudaError_t err = launch_overlapped(
-        k_propose_slabs<V, U, G, THREADS, DEPTH, ITEMS, SV>, P.grid, THREADS, smem, p->stream, P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, P.tile_start, P.tile_end, P.tile_pair, P.tile_slab,
-        P.slab_tile_begin, P.cta_tile_begin, (const U*)u_vec, p->n, P.slab_rows, (G*)p->gnat);
+        k_propose_slabs<V, U, G, THREADS, DEPTH, ITEMS, SV>, P.grid, THREADS, smem, p->stream, P.s_row,
+        (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P, P.tiles), (const U*)u_vec, p->n, P.slab_rows,
+        (G*)p->gnat);
     prof_end(p, e1);
     GENCD_CUDA_TRY(err);
   }
@@ -701,21 +728,23 @@ static int set_slab_smem(const ProposePlan& P) {
   const int smem = (int)((size_t)(P.slab_rows + kSlabZeroSlot) * sizeof(U));
   GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_slabs<V, U, G, THREADS, DEPTH, ITEMS, SV>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  if (P.light_counter) {
-    GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 31, DEPTH, ITEMS, SV>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 20, DEPTH, ITEMS, SV>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 24, DEPTH, ITEMS, SV>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 28, DEPTH, ITEMS, SV>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  if constexpr (sizeof(V) == 4) {
+    if (P.light_counter) {
+      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 20, 1, kFusedItems, SV>,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 24, 1, kFusedItems, SV>,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 28, 1, kFusedItems, SV>,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 31, 1, kFusedItems, SV>,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    }
   }
   return GENCD_OK;
 }
 
-#define GENCD_PLAN_F64 double, double, double, double, kSlabThreadsF64, 0, kSlabItemsF64
-#define GENCD_PLAN_F32(SV) float, float, float, SV, kSlabThreadsF32, 1, kSlabItemsF32
+#define GENCD_PLAN_F64 double, double, double, double, kSlabThreadsF64, kSlabDepthF64, kSlabItemsF64
+#define GENCD_PLAN_F32(SV) float, float, float, SV, kSlabThreadsF32, kSlabDepthF32, kSlabItemsF32
 
 int launch_propose_plan(gencd_problem* p, const void* u_vec) {
   if (p->precision == GENCD_F64) return launch_plan_passes<GENCD_PLAN_F64>(p, u_vec);
@@ -827,6 +856,11 @@ __device__ __forceinline__ void plan_store(__nv_bfloat16* a, int64_t i, float v)
   a[i] = __float2bfloat16_rn(v);  // the values are bfloat16-exact
 }
 __device__ __forceinline__ void plan_store(NoVal*, int64_t, float) {}
+template <typename SV>
+__device__ __forceinline__ void plan_zero(SV* a, int64_t i) {
+  a[i] = SV(0.0f);
+}
+__device__ __forceinline__ void plan_zero(NoVal*, int64_t) {}
 
 // Every entry to its place: a heavy one into its slab's run (pad_off[r] is
 // where the padded slab starts), a light one into the compact copy, in the
@@ -869,8 +903,10 @@ __global__ void __launch_bounds__(kThreads)
       const int64_t i = (int64_t)r * nheavy + __ldg(hid + lo);
       const uint32_t first = __ldg(seg + i);
       const int64_t d = __ldg(pad_off + r) - __ldg(slab_begin + r) + __ldg(pos + i) + (at - first);
-      s_row[d] = (uint16_t)(row - r * slab_rows);
-      plan_store(s_val, d, val[p]);
+      const int64_t d0 = d & ~(int64_t)(kSlabTile - 1);
+      const uint32_t x = (uint32_t)(d - d0);
+      s_row[d0 + slab_at<8>(x)] = (uint16_t)(row - r * slab_rows);
+      plan_store(s_val, d0 + slab_at<vector_of<SV>()>(x), val[p]);
       if (at == first) {
         const uint32_t q = __ldg(pair + i);
         atomicOr(pmask + (d >> 5), 1u << (d & 31));
@@ -886,33 +922,24 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// the padding of every slab's entries (and 8 entries past the last slab): row
-// pad_row, value 0
+// the padding of every slab's last tile: the row past the slab, which reads a
+// zero from shared memory, and value 0
+template <typename SV>
 __global__ void k_plan_pad(const int64_t* __restrict__ slab_begin, const int64_t* __restrict__ pad_off, int32_t R,
-                           int64_t entries, uint16_t pad_row, uint16_t* __restrict__ s_row, char* __restrict__ s_val,
-                           int vsz) {
+                           uint16_t pad_row, uint16_t* __restrict__ s_row, SV* __restrict__ s_val) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < (int64_t)(R + 1) * kSlabPad; q += stride) {
-    const int64_t r = q / kSlabPad, x = q - r * kSlabPad;
-    int64_t d, end;
-    if (r < R) {
-      d = pad_off[r] + (slab_begin[r + 1] - slab_begin[r]) + x;
-      end = pad_off[r + 1];
-    } else {
-      d = entries + x;
-      end = entries + 8;
-    }
-    if (d >= end) continue;
-    s_row[d] = pad_row;
-    for (int b = 0; b < vsz; ++b) s_val[d * vsz + b] = 0;
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < (int64_t)R * kSlabTile; q += stride) {
+    const int64_t r = q / kSlabTile, end = pad_off[r + 1];
+    const uint32_t x = (uint32_t)(q - r * kSlabTile);  // place in the slab's last tile
+    if (end == pad_off[r] || end - kSlabTile + x < pad_off[r] + (slab_begin[r + 1] - slab_begin[r])) continue;
+    s_row[end - kSlabTile + slab_at<8>(x)] = pad_row;
+    plan_zero(s_val, end - kSlabTile + slab_at<vector_of<SV>()>(x));
   }
 }
 
 __global__ void k_plan_tiles(const int32_t* __restrict__ slab_tile_begin, const int64_t* __restrict__ pad_off,
                              int32_t R, int64_t T, int64_t tile, const uint32_t* __restrict__ pair_start,
-                             int64_t npairs,
-                             uint32_t* __restrict__ tile_start, uint32_t* __restrict__ tile_end,
-                             uint32_t* __restrict__ tile_pair, int32_t* __restrict__ tile_slab) {
+                             int64_t npairs, uint32_t* __restrict__ tile_pair, int32_t* __restrict__ tile_slab) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < T; t += stride) {
     int32_t lo = 0, hi = R - 1;  // slab: last r with slab_tile_begin[r] <= t
@@ -925,9 +952,6 @@ __global__ void k_plan_tiles(const int32_t* __restrict__ slab_tile_begin, const 
     }
     const int32_t r = lo;
     const int64_t s = pad_off[r] + (t - slab_tile_begin[r]) * tile;
-    const int64_t e = s + tile < pad_off[r + 1] ? s + tile : pad_off[r + 1];
-    tile_start[t] = (uint32_t)s;
-    tile_end[t] = (uint32_t)e;
     tile_slab[t] = r;
     int64_t a = 0, b = npairs - 1;  // pair of the tile's first entry: last q with pair_start[q] <= s
     while (a < b) {
@@ -973,6 +997,9 @@ static void launch_place(gencd_problem* p, const uint32_t* hid, const uint32_t* 
       p->col_ptr, p->row_idx, (const V*)p->val, p->tile_col, p->nnz, 32LL * p->items, P.heavy_min, hid, loff, P.nheavy,
       P.slab_rows, seg, pos, pair, slab_begin, pad_off, P.s_row, (SV*)P.s_val, (uint32_t*)P.pmask, pair_start,
       P.pair_col, P.light_row, (SV*)P.light_val, (uint32_t*)P.lmask);
+  if (P.nheavy > 0)
+    k_plan_pad<SV><<<grid_for((int64_t)P.nslabs * kSlabTile, kThreads, p->num_sms * 8), kThreads, 0, p->stream>>>(
+        slab_begin, pad_off, P.nslabs, (uint16_t)P.slab_rows, P.s_row, (SV*)P.s_val);
 }
 
 // Two allocations hold the plan and two the scratch: a cudaMalloc or cudaFree
@@ -1033,9 +1060,7 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   light.add((uint32_t**)&P.lmask, lwords);
   if (p->vmode == kValNone && P.nlight > 0) light.add(&P.light_scale, P.nlight);
   if (fusable) light.add(&P.light_counter, 2);  // tiles taken, warps finished
-  light.add(&P.slab_tile_begin, R + 1);
   P.grid = p->num_sms;
-  light.add(&P.cta_tile_begin, P.grid + 1);
   GENCD_TRY(dev_alloc_bytes(p, &P.mem[0], light.bytes()));
   light.place(P.mem[0]);
   k_plan_columns<<<grid_for(k + 1, kThreads, g), kThreads, 0, st>>>(p->col_ptr, k, P.heavy_min, hid, lid, loff,
@@ -1084,34 +1109,42 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   P.entries = hp[R];
   if (P.entries >= (int64_t(1) << 32)) return fail_plan("heavy entries exceed 2^32");
 
-  // tiles inside each slab, and contiguous runs of tiles per CTA
-  std::vector<int32_t> tb(R + 1), ctb(P.grid + 1);
-  tb[0] = 0;
-  const int64_t tile = 32LL * (f64 ? kSlabItemsF64 : kSlabItemsF32);  // the kernel's tile
-  for (int r = 0; r < R; ++r) tb[r + 1] = tb[r] + (int32_t)((hp[r + 1] - hp[r] + tile - 1) / tile);
-  P.ntiles = tb[R];
-  for (int b = 0; b <= P.grid; ++b) ctb[b] = (int32_t)((int64_t)b * P.ntiles / P.grid);
   if (P.nheavy > 0) {
-    const int64_t mask_words = (P.entries + 8 + 31) / 32;  // start bits: one byte per 8 entries
+    // tiles of both sizes in use inside each slab, and contiguous runs of
+    // tiles per CTA
+    ProposePlan::Tiles* sets[2] = {&P.tiles, fusable ? &P.fused : nullptr};
+    const int64_t tile[2] = {32LL * (f64 ? kSlabItemsF64 : kSlabItemsF32), 32LL * kFusedItems};
+    const int64_t mask_words = (P.entries + 31) / 32;  // start bits: one byte per 8 entries
+    std::vector<uint32_t> off(R + 1);
+    for (int r = 0; r <= R; ++r) off[r] = (uint32_t)hp[r];
     Arena slabs;
-    slabs.add(&P.s_row, P.entries + 8);
-    slabs.add((char**)&P.s_val, (P.entries + 8) * (int64_t)vsz);
+    slabs.add(&P.s_row, P.entries);
+    slabs.add((char**)&P.s_val, P.entries * (int64_t)vsz);
     slabs.add((uint32_t**)&P.pmask, mask_words);
     slabs.add(&P.pair_col, P.npairs);
-    slabs.add(&P.tile_start, P.ntiles);
-    slabs.add(&P.tile_end, P.ntiles);
-    slabs.add(&P.tile_pair, P.ntiles);
-    slabs.add(&P.tile_slab, P.ntiles);
+    slabs.add(&P.slab_off, R + 1);
+    for (int i = 0; i < 2; ++i)
+      if (sets[i]) {
+        sets[i]->count = P.entries / tile[i];
+        slabs.add(&sets[i]->pair, sets[i]->count);
+        slabs.add(&sets[i]->slab, sets[i]->count);
+        slabs.add(&sets[i]->slab_begin, R + 1);
+        slabs.add(&sets[i]->cta_begin, P.grid + 1);
+      }
     GENCD_TRY(dev_alloc_bytes(p, &P.mem[1], slabs.bytes()));
     slabs.place(P.mem[1]);
     GENCD_CUDA_TRY(cudaMemcpyAsync(pad_off, hp.data(), 8 * (R + 1), cudaMemcpyHostToDevice, st));
-    GENCD_CUDA_TRY(cudaMemcpyAsync(P.slab_tile_begin, tb.data(), 4 * (R + 1), cudaMemcpyHostToDevice, st));
-    GENCD_CUDA_TRY(cudaMemcpyAsync(P.cta_tile_begin, ctb.data(), 4 * (P.grid + 1), cudaMemcpyHostToDevice, st));
+    GENCD_CUDA_TRY(cudaMemcpyAsync(P.slab_off, off.data(), 4 * (R + 1), cudaMemcpyHostToDevice, st));
     GENCD_CUDA_TRY(cudaMemsetAsync(P.pmask, 0, 4 * (size_t)mask_words, st));
-    k_plan_pad<<<grid_for((int64_t)(R + 1) * kSlabPad, kThreads, g), kThreads, 0, st>>>(
-        slab_begin, pad_off, R, P.entries, p->vmode == kValNone ? (uint16_t)P.slab_rows : (uint16_t)0, P.s_row,
-        (char*)P.s_val, (int)vsz);
-    GENCD_CUDA_TRY(cudaGetLastError());
+    std::vector<int32_t> tb(R + 1), ctb(P.grid + 1);  // pageable sources: read when the copy returns
+    for (int i = 0; i < 2; ++i)
+      if (sets[i]) {
+        for (int r = 0; r <= R; ++r) tb[r] = (int32_t)(hp[r] / tile[i]);
+        for (int b = 0; b <= P.grid; ++b) ctb[b] = (int32_t)((int64_t)b * sets[i]->count / P.grid);
+        GENCD_CUDA_TRY(cudaMemcpyAsync(sets[i]->slab_begin, tb.data(), 4 * (R + 1), cudaMemcpyHostToDevice, st));
+        GENCD_CUDA_TRY(cudaMemcpyAsync(sets[i]->cta_begin, ctb.data(), 4 * (P.grid + 1), cudaMemcpyHostToDevice, st));
+        GENCD_CUDA_TRY(cudaStreamSynchronize(st));
+      }
   }
   if (p->nnz > 0) {
     if (f64)
@@ -1126,9 +1159,11 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   }
   P.fused_split = 0;
   if (P.nheavy > 0) {
-    k_plan_tiles<<<grid_for(P.ntiles, kThreads, g), kThreads, 0, st>>>(P.slab_tile_begin, pad_off, R, P.ntiles, tile,
-                                                                        pair_start, P.npairs, P.tile_start,
-                                                                        P.tile_end, P.tile_pair, P.tile_slab);
+    for (ProposePlan::Tiles* t : {&P.tiles, &P.fused})
+      if (t->count > 0)
+        k_plan_tiles<<<grid_for(t->count, kThreads, g), kThreads, 0, st>>>(t->slab_begin, pad_off, R, t->count,
+                                                                            P.entries / t->count, pair_start, P.npairs,
+                                                                            t->pair, t->slab);
     GENCD_CUDA_TRY(cudaGetLastError());
     // both passes may run in one kernel when there are light and heavy columns
     // (FP32 arithmetic: FP64 stages do not fit the fused kernel's registers);
