@@ -303,11 +303,11 @@ int gencd_permutation(gencd_problem* p, uint64_t seed, int64_t epoch, int64_t m,
 
 /* Kernel launch counts and, when profiling is enabled, summed device time
  * (ms, CUDA events on the problem's stream) and number of timed invocations
- * per kernel family: 0 streaming propose (the whole family: 9 + 10, or 12,
- * and 11 with index-only storage), 1 finalize, 2 accept, 3 update,
+ * per kernel family: 0 streaming propose (the whole family: 9 + 10, or 12),
+ * 1 finalize, 2 accept, 3 update,
  * 4 refresh, 5 list propose, 6 Coloring iteration, 7 objective,
- * 8 setup/selection, 9 light-column pass, 10 row-slab pass, 11 the heavy
- * columns' g_j times their value (index-only storage), 12 row-slab and
+ * 8 setup/selection, 9 light-column pass, 10 row-slab pass, 11 (none;
+ * index-only storage's values are applied with the steps), 12 row-slab and
  * light-column passes in one kernel.  ms / calls is the mean duration of one
  * invocation; ms, launches, calls may be NULL. */
 int gencd_profile_enable(gencd_problem* p, int32_t enable);

@@ -75,7 +75,7 @@ enum KernelId {
   K_SETUP,            // one-time and selection kernels
   K_PROPOSE_LIGHT,    // streaming propose: lane-segmented pass over the light columns
   K_PROPOSE_SLABS,    // streaming propose: row-slab pass over the heavy columns
-  K_SCALE_HEAVY,      // streaming propose, index-only storage: heavy columns' g_j times their value
+  K_SCALE_HEAVY,      // (no kernel: the Accept and the finalize apply the index-only storage's values)
   K_PROPOSE_FUSED,    // streaming propose: row-slab and light passes in one kernel
   K_NUM
 };
@@ -119,7 +119,6 @@ struct ProposePlan {
   int32_t* light_row = nullptr;
   void* light_val = nullptr;
   int32_t* light_tile_lc = nullptr;  // light column of each 256-entry tile's first entry
-  float* light_scale = nullptr;      // index-only storage: the value of light column lc
   uint8_t* lmask = nullptr;          // per 8 light entries: bit i = entry 8g + i starts a column
   // heavy columns
   int64_t nheavy = 0, entries = 0, npairs = 0;
@@ -196,7 +195,8 @@ struct gencd_problem {
   int64_t ntiles = 0;
   int32_t* tile_col = nullptr;
   double* gacc = nullptr;   // FP64 sums (setup passes, power iteration)
-  void* gnat = nullptr;     // sums of the hot path in the storage precision (== gacc in FP64 mode)
+  void* gnat = nullptr;     // sums of the hot path in the storage precision (== gacc in FP64 mode); index-only
+                            // storage: sums of u over the columns' rows, col_val[j] still to be applied
   double* delta = nullptr;
   double* phi = nullptr;
 

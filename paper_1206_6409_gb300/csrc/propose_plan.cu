@@ -91,7 +91,7 @@ struct NoVal {};
 
 // a heavy column's run sum into g_j: other slabs and tiles add to the same
 // column, so always atomically (index-only storage: the sum of u over the
-// column's rows; k_scale_heavy applies the column's value afterwards)
+// column's rows; who reads g_j applies the column's value)
 template <typename G>
 __device__ __forceinline__ void add_col(G* __restrict__ gacc, uint32_t j, G v) {
   atomicAdd(gacc + j, v);
@@ -438,15 +438,13 @@ __device__ __forceinline__ void load_light_stage(const int32_t* __restrict__ row
   }
 }
 
-// One light tile's sums from its loads `cur` (lscale: index-only columns,
-// each column's sum scaled by its value); results go to out[light_cols[lc]].
+// One light tile's sums from its loads `cur` (index-only columns: the sums of u
+// over their rows); results go to out[light_cols[lc]].
 template <typename V, typename U, typename G, typename SV>
 __device__ __forceinline__ void light_tile(const LightStage<SV>& cur, int64_t t, int64_t nnz,
                                            const int32_t* __restrict__ light_cols,
-                                           const float* __restrict__ lscale, const U* __restrict__ u,
-                                           G* __restrict__ out, int lane) {
+                                           const U* __restrict__ u, G* __restrict__ out, int lane) {
   const unsigned FULL = 0xffffffffu;
-  constexpr bool kScaled = std::is_same<SV, NoVal>::value;
   const int64_t a = t * kLightTile + (int64_t)lane * kLightItems;
   const bool active = a < nnz;
   const uint32_t m = cur.m, lc0 = cur.lc0;
@@ -464,11 +462,6 @@ __device__ __forceinline__ void light_tile(const LightStage<SV>& cur, int64_t t,
   const uint32_t ql = q + __popc(m & 0xfeu);
   const int32_t j0 = lead ? __ldg(light_cols + lc0) : 0;
   const int32_t jl = (active && m != 0u) ? __ldg(light_cols + ql) : 0;
-  V s0 = V(1), sl = V(1);
-  if (kScaled) {
-    s0 = lead ? (V)__ldg(lscale + lc0) : V(1);
-    sl = (active && m != 0u) ? (V)__ldg(lscale + ql) : V(1);
-  }
   V cont = V(0), tail = V(0);
   bool has_tail = false;
   if (active) {
@@ -487,8 +480,7 @@ __device__ __forceinline__ void light_tile(const LightStage<SV>& cur, int64_t t,
         if (i == bf) {
           first = acc;
         } else {  // a whole column inside the lane
-          const V sc = kScaled ? (V)__ldg(lscale + qi) : V(1);
-          out[__ldg(light_cols + qi)] = (G)(acc * sc);
+          out[__ldg(light_cols + qi)] = (G)acc;
         }
         acc = V(0);
         ++qi;
@@ -497,8 +489,7 @@ __device__ __forceinline__ void light_tile(const LightStage<SV>& cur, int64_t t,
     }
     if (inner) {
       if (m & 1u) {  // started at entry 0, ended inside
-        const V sc = kScaled ? (V)__ldg(lscale + q) : V(1);
-        out[__ldg(light_cols + q)] = (G)(first * sc);
+        out[__ldg(light_cols + q)] = (G)first;
       } else {
         cont = first;
       }
@@ -514,16 +505,16 @@ __device__ __forceinline__ void light_tile(const LightStage<SV>& cur, int64_t t,
   const bool stop = !active || m != 0u;
   if (__ballot_sync(FULL, stop) == 0u) {
     const V sum = warp_sum(cont);  // the whole tile is inside column lc0
-    if (lane == 0) atomicAdd(out + j0, (G)(sum * s0));
+    if (lane == 0) atomicAdd(out + j0, (G)sum);
   } else {
     bool ended;
     const V tsum = lane_suffix_sum(cont, stop, lane, ended);
     const V t1s = __shfl_down_sync(FULL, tsum, 1);
     const bool e1 = __shfl_down_sync(FULL, (int)ended, 1) != 0;
-    if (lead) atomicAdd(out + j0, (G)(tsum * s0));  // column from the previous tile
+    if (lead) atomicAdd(out + j0, (G)tsum);  // column from the previous tile
     if (has_tail) {
       const V sum = tail + (lane < 31 ? t1s : V(0));
-      emit_pair<G>(out, (uint32_t)jl, (G)(sum * sl), lane < 31 && e1);
+      emit_pair<G>(out, (uint32_t)jl, (G)sum, lane < 31 && e1);
     }
   }
 }
@@ -532,8 +523,7 @@ template <typename V, typename U, typename G, typename SV>
 __global__ void __launch_bounds__(kThreads, 3)
     k_propose_light_runs(const int32_t* __restrict__ row, const SV* __restrict__ val,
                          const uint8_t* __restrict__ lmask, const int32_t* __restrict__ tile_lc,
-                         const int32_t* __restrict__ light_cols, const float* __restrict__ lscale,
-                         const U* __restrict__ u, int64_t nnz, int64_t ntiles, G* __restrict__ out) {
+                         const int32_t* __restrict__ light_cols, const U* __restrict__ u, int64_t nnz, int64_t ntiles, G* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -550,7 +540,7 @@ __global__ void __launch_bounds__(kThreads, 3)
     } else {
       load_light_stage<SV>(row, val, lmask, tile_lc, t, ntiles, nnz, lane, cur);
     }
-    light_tile<V, U, G, SV>(cur, t, nnz, light_cols, lscale, u, out, lane);
+    light_tile<V, U, G, SV>(cur, t, nnz, light_cols, u, out, lane);
   }
 }
 
@@ -563,7 +553,7 @@ template <typename V, typename U, typename G, typename SV>
 __device__ __forceinline__ void light_pool(const int32_t* __restrict__ row, const SV* __restrict__ val,
                                            const uint8_t* __restrict__ lmask, const int32_t* __restrict__ tile_lc,
                                            const int32_t* __restrict__ light_cols,
-                                           const float* __restrict__ lscale, const U* __restrict__ u, int64_t nnz,
+                                           const U* __restrict__ u, int64_t nnz,
                                            int64_t ntiles, G* __restrict__ out, unsigned int* counter) {
   const int lane = threadIdx.x & 31;
   auto grab = [&](int64_t& t, int64_t& t_end) {
@@ -584,7 +574,7 @@ __device__ __forceinline__ void light_pool(const int32_t* __restrict__ row, cons
     if (++t >= t_end) grab(t, t_end);
     const bool more = t < ntiles;
     if (more) load_light_stage<SV>(row, val, lmask, tile_lc, t, ntiles, nnz, lane, nxt);  // next tile in flight
-    light_tile<V, U, G, SV>(cur, tc, nnz, light_cols, lscale, u, out, lane);
+    light_tile<V, U, G, SV>(cur, tc, nnz, light_cols, u, out, lane);
     if (!more) break;
   }
 }
@@ -601,7 +591,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     const uint8_t* __restrict__ pmask, const uint32_t* __restrict__ pair_col, SlabTiles T,
                     const int32_t* __restrict__ lrow, const SV* __restrict__ lval,
                     const uint8_t* __restrict__ lmask, const int32_t* __restrict__ tile_lc,
-                    const int32_t* __restrict__ light_cols, const float* __restrict__ lscale, int64_t lnnz,
+                    const int32_t* __restrict__ light_cols, int64_t lnnz,
                     int64_t lntiles, unsigned int* counter, const U* __restrict__ u, int64_t n, int32_t slab_rows,
                     G* __restrict__ gacc) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -614,7 +604,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         slab_rows, gacc, s_u, warp, SLAB_WARPS, threadIdx.x, 32 * SLAB_WARPS);
   else
     pdl_wait();
-  light_pool<V, U, G, SV>(lrow, lval, lmask, tile_lc, light_cols, lscale, u, lnnz, lntiles, gacc, counter);
+  light_pool<V, U, G, SV>(lrow, lval, lmask, tile_lc, light_cols, u, lnnz, lntiles, gacc, counter);
   // the last warp out resets the pool for the next launch: every warp has
   // taken its last tiles when it gets here (counter[1] counts the exits)
   if ((threadIdx.x & 31) == 0) {
@@ -625,31 +615,6 @@ __global__ void __launch_bounds__(THREADS, 1)
       counter[1] = 0u;
     }
   }
-}
-
-// index-only storage: g_j of every heavy column times the column's value
-// (the row-slab pass adds the sums of u over the column's rows)
-template <typename G>
-__global__ void k_scale_heavy(const int32_t* __restrict__ heavy_cols, int64_t nheavy,
-                              const float* __restrict__ col_val, G* __restrict__ gacc) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t h = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; h < nheavy; h += stride) {
-    const int32_t j = heavy_cols[h];
-    gacc[j] *= (G)col_val[j];
-  }
-}
-
-template <typename G, typename SV>
-static int scale_heavy(gencd_problem* p) {
-  ProposePlan& P = p->plan;
-  if (!std::is_same<SV, NoVal>::value || P.nheavy == 0) return GENCD_OK;
-  cudaEvent_t e = nullptr;
-  prof_begin(p, K_SCALE_HEAVY, &e);
-  k_scale_heavy<G><<<grid_for(P.nheavy, kThreads, p->num_sms * 8), kThreads, 0, p->stream>>>(
-      P.heavy_cols, P.nheavy, p->col_val, (G*)p->gnat);
-  prof_end(p, e);
-  GENCD_CUDA_TRY(cudaGetLastError());
-  return GENCD_OK;
 }
 
 static SlabTiles tiles_of(const ProposePlan& P, const ProposePlan::Tiles& t) {
@@ -670,7 +635,7 @@ static cudaError_t launch_fused(gencd_problem* p, const void* u_vec, size_t smem
   ProposePlan& P = p->plan;
   return launch_overlapped(k_propose_fused<V, U, G, kFusedThreads, SW, 1, kFusedItems, SV>, P.grid, kFusedThreads, smem,
                            p->stream, P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P, P.fused),
-                           P.light_row, (const SV*)P.light_val, P.lmask, P.light_tile_lc, P.light_cols, P.light_scale,
+                           P.light_row, (const SV*)P.light_val, P.lmask, P.light_tile_lc, P.light_cols,
                            P.light_nnz, P.light_ntiles, P.light_counter, (const U*)u_vec, p->n, P.slab_rows,
                            (G*)p->gnat);
 }
@@ -690,7 +655,7 @@ static int launch_fused_passes(gencd_problem* p, const void* u_vec) {
   }
   prof_end(p, e1);
   GENCD_CUDA_TRY(err);
-  return scale_heavy<G, SV>(p);
+  return GENCD_OK;
 }
 
 template <typename V, typename U, typename G, typename SV, int THREADS, int DEPTH, int ITEMS>
@@ -705,7 +670,7 @@ static int launch_plan_passes(gencd_problem* p, const void* u_vec) {
     const int grid = grid_for(P.light_ntiles * 32, kThreads, p->num_sms * 3);  // resident CTAs: persistent warps
     const cudaError_t err = launch_overlapped(
         k_propose_light_runs<V, U, G, SV>, grid, kThreads, 0, p->stream, P.light_row, (const SV*)P.light_val, P.lmask,
-        P.light_tile_lc, P.light_cols, P.light_scale, (const U*)u_vec, P.light_nnz, P.light_ntiles, (G*)p->gnat);
+        P.light_tile_lc, P.light_cols, (const U*)u_vec, P.light_nnz, P.light_ntiles, (G*)p->gnat);
     prof_end(p, e);
     GENCD_CUDA_TRY(err);
   }
@@ -720,7 +685,7 @@ static int launch_plan_passes(gencd_problem* p, const void* u_vec) {
     prof_end(p, e1);
     GENCD_CUDA_TRY(err);
   }
-  return scale_heavy<G, SV>(p);
+  return GENCD_OK;
 }
 
 template <typename V, typename U, typename G, typename SV, int THREADS, int DEPTH, int ITEMS>
@@ -772,12 +737,10 @@ __global__ void k_plan_classify(const int64_t* __restrict__ col_ptr, int64_t k, 
   }
 }
 
-// light_scale (index-only storage): the value of every light column
 __global__ void k_plan_columns(const int64_t* __restrict__ col_ptr, int64_t k, int64_t hmin,
                                const uint32_t* __restrict__ hid, const uint32_t* __restrict__ lid,
                                const uint32_t* __restrict__ loff, int32_t* __restrict__ heavy_cols,
-                               int32_t* __restrict__ light_cols, int64_t* __restrict__ light_col_ptr,
-                               const float* __restrict__ col_val, float* __restrict__ light_scale) {
+                               int32_t* __restrict__ light_cols, int64_t* __restrict__ light_col_ptr) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j <= k; j += stride) {
     if (j == k) {
@@ -791,7 +754,6 @@ __global__ void k_plan_columns(const int64_t* __restrict__ col_ptr, int64_t k, i
     } else {
       light_cols[lid[j]] = (int32_t)j;
       light_col_ptr[lid[j]] = loff[j];
-      if (light_scale) light_scale[lid[j]] = col_val[j];
     }
   }
 }
@@ -1058,14 +1020,12 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   light.add((char**)&P.light_val, lpad * (int64_t)vsz);
   light.add(&P.light_tile_lc, P.light_ntiles + 1);
   light.add((uint32_t**)&P.lmask, lwords);
-  if (p->vmode == kValNone && P.nlight > 0) light.add(&P.light_scale, P.nlight);
   if (fusable) light.add(&P.light_counter, 2);  // tiles taken, warps finished
   P.grid = p->num_sms;
   GENCD_TRY(dev_alloc_bytes(p, &P.mem[0], light.bytes()));
   light.place(P.mem[0]);
   k_plan_columns<<<grid_for(k + 1, kThreads, g), kThreads, 0, st>>>(p->col_ptr, k, P.heavy_min, hid, lid, loff,
-                                                                     P.heavy_cols, P.light_cols, P.light_col_ptr,
-                                                                     p->col_val, P.light_scale);
+                                                                     P.heavy_cols, P.light_cols, P.light_col_ptr);
   GENCD_CUDA_TRY(cudaGetLastError());
   if (P.nlight > 0) {
     if (p->vmode == kValNone) {  // padding has no value to zero it: it gathers u[n] = 0 instead
