@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(kAcceptThreads)
     const float lam = sa.lam32[s], invn = sa.invn32[s];
     const float* bjv = bj32 + (int64_t)set * k;
     const float* ibv = ib32 + (int64_t)set * k;
+#pragma unroll 4
     for (int64_t j = lo + r; j < hi; j += R) {
       const float g = __ldg(G + j * Sp + s) * invn;
       const float wj = __ldg(w32 + j * Sp + s);
@@ -430,6 +431,7 @@ __global__ void k_b_update(const int32_t* __restrict__ acc_j, const double* __re
       atomicAdd(ctr, (unsigned long long)(e - a));
       atomicAdd(ctr + 1, 1ull);
     }
+#pragma unroll 4
     for (int64_t t = a + lane; t < e; t += 32) atomicAdd(z + (int64_t)row[t] * Sp + s, d * (double)val[t]);
   }
 }
@@ -745,6 +747,90 @@ __global__ void k_b_fill_col(const double* __restrict__ y, const uint8_t* __rest
   }
 }
 
+// Slots that a path starts, finishes or clears together, passed by value: one
+// launch for all of them, lanes over slots, whose values of a row or column
+// are contiguous.  A path of 32 chains of two solves on 4e6 non-zeros, 60 steps
+// of 32 slots, takes 9.3 ms; slot by slot, with five launches and six copies a
+// start and a copy and a wait for every w, it took 13.9.
+struct SlotWave {
+  int32_t m = 0;
+  int16_t slot[kBatchMaxSlots];
+  int16_t set[kBatchMaxSlots];     // -1: no training rows (a cleared slot)
+  int32_t chain[kBatchMaxSlots];   // row of w_last the slot starts from or finishes to; -1: starts from w = 0
+  void add(int s, int st, int c) {
+    slot[m] = (int16_t)s;
+    set[m] = (int16_t)st;
+    chain[m] = c;
+    ++m;
+  }
+};
+
+// w, its float copy and w_start[s] from the chains' w_last (or 0), and z = 0;
+// block 32 x 8, threadIdx.x = place in the wave
+__global__ void k_b_wave_start(SlotWave v, const double* __restrict__ w_last, int64_t k, int64_t n, int Sp,
+                               double* __restrict__ w, float* __restrict__ w32, double* __restrict__ w_start,
+                               double* __restrict__ z) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.y, r0 = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
+  for (int q = threadIdx.x; q < v.m; q += 32) {
+    const int s = v.slot[q], c = v.chain[q];
+    for (int64_t j = r0; j < k; j += stride) {
+      const double x = c >= 0 ? w_last[(int64_t)c * k + j] : 0.0;
+      w[j * Sp + s] = x;
+      w32[j * Sp + s] = w_mirror(x);
+      w_start[(int64_t)s * k + j] = x;
+    }
+    for (int64_t i = r0; i < n; i += stride) z[i * Sp + s] = 0.0;
+  }
+}
+
+// z_s += w_js X_j for every column with w_js != 0 and listed slot (one warp
+// per column)
+__global__ void k_b_wave_scatter(SlotWave v, const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row,
+                                 const float* __restrict__ val, const double* __restrict__ w, int64_t k, int Sp,
+                                 double* __restrict__ z) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int q0 = 0; q0 < v.m; q0 += 32) {
+    const int q = q0 + lane;
+    const int s = q < v.m && v.chain[q] >= 0 ? v.slot[q] : -1;
+    for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < k; j += nw) {  // warp-uniform
+      const double wj = s >= 0 ? w[j * Sp + s] : 0.0;
+      unsigned todo = __ballot_sync(FULL, wj != 0.0);
+      if (!todo) continue;
+      const int64_t a = col_ptr[j], e = col_ptr[j + 1];
+      for (; todo; todo &= todo - 1) {
+        const int l = __ffs(todo) - 1;
+        const double wl = __shfl_sync(FULL, wj, l);
+        const int sl = __shfl_sync(FULL, s, l);
+        for (int64_t t = a + lane; t < e; t += 32) atomicAdd(z + (int64_t)row[t] * Sp + sl, wl * (double)val[t]);
+      }
+    }
+  }
+}
+
+// u_s on every row of the listed slots (block 32 x 8)
+__global__ void k_b_wave_fill(SlotWave v, const double* __restrict__ y, const uint8_t* __restrict__ fold, int nfolds,
+                              int loss, const double* __restrict__ z, int64_t n, int Sp, float* __restrict__ U) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.y, r0 = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
+  for (int q = threadIdx.x; q < v.m; q += 32) {
+    const int s = v.slot[q], set = v.set[q];
+    for (int64_t i = r0; i < n; i += stride) {
+      const int64_t o = i * Sp + s;
+      U[o] = (set >= 0 && b_train(fold, i, set, nfolds)) ? u_value<float>(loss, y[i], z[o]) : 0.0f;
+    }
+  }
+}
+
+// w_last[chain] = w_s of the listed slots (block 32 x 8)
+__global__ void k_b_wave_get(SlotWave v, const double* __restrict__ w, int64_t k, int Sp, double* __restrict__ w_last) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.y, r0 = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
+  for (int q = threadIdx.x; q < v.m; q += 32) {
+    const int s = v.slot[q], c = v.chain[q];
+    for (int64_t j = r0; j < k; j += stride) w_last[(int64_t)c * k + j] = w[j * Sp + s];
+  }
+}
+
 // acc[q] += loss sum over slot list[q]'s training rows; acc[m + q] += ||w_s||_1
 // (block: 32 x 8 threads, threadIdx.x = list position)
 // dual_scale (nullable): per listed slot, s = lambda_s / max(lambda_s,
@@ -852,7 +938,7 @@ struct gencd_batch {
   int32_t* obj_list = nullptr;
   double* tmp_k = nullptr;  // k doubles (w in/out)
 
-  // per-slot parameters (device) and their host copy
+  // per-slot parameters (device, one allocation from d_lam on) and their host copy
   int32_t* d_set = nullptr;
   int32_t* d_group = nullptr;
   double *d_lam = nullptr, *d_invn = nullptr;
@@ -883,23 +969,23 @@ static SlotArgs slot_args(const gencd_batch* b) {
   return SlotArgs{b->d_set, b->d_group, b->d_lam, b->d_lam32, b->d_invn, b->d_invn32};
 }
 
+// The slots' parameters to the device, in one copy (the arrays share one
+// allocation; a pageable source has been read when the call returns)
 static int upload_slots(gencd_batch* b) {
   const int S = b->S;
-  std::vector<float> l32(S), i32(S);
-  std::vector<double> inv(S);
+  std::vector<double> img((size_t)4 * S);  // 32 bytes a slot
+  double *lam = img.data(), *inv = lam + S;
+  int32_t *set = reinterpret_cast<int32_t*>(inv + S), *group = set + S;
+  float *l32 = reinterpret_cast<float*>(group + S), *i32 = l32 + S;
   for (int s = 0; s < S; ++s) {
-    const int set = b->h_set[s];
-    inv[s] = set >= 0 && b->set_rows[set] > 0 ? 1.0 / (double)b->set_rows[set] : 0.0;
-    l32[s] = (float)b->h_lam[s];
+    set[s] = b->h_set[s];
+    group[s] = b->h_group[s];
+    lam[s] = b->h_lam[s];
+    inv[s] = set[s] >= 0 && b->set_rows[set[s]] > 0 ? 1.0 / (double)b->set_rows[set[s]] : 0.0;
+    l32[s] = (float)lam[s];
     i32[s] = (float)inv[s];
   }
-  // pageable sources: each copy has read its source when the call returns
-  GENCD_CUDA_TRY(cudaMemcpyAsync(b->d_set, b->h_set.data(), 4 * S, cudaMemcpyHostToDevice, b->st));
-  GENCD_CUDA_TRY(cudaMemcpyAsync(b->d_group, b->h_group.data(), 4 * S, cudaMemcpyHostToDevice, b->st));
-  GENCD_CUDA_TRY(cudaMemcpyAsync(b->d_lam, b->h_lam.data(), 8 * S, cudaMemcpyHostToDevice, b->st));
-  GENCD_CUDA_TRY(cudaMemcpyAsync(b->d_invn, inv.data(), 8 * S, cudaMemcpyHostToDevice, b->st));
-  GENCD_CUDA_TRY(cudaMemcpyAsync(b->d_lam32, l32.data(), 4 * S, cudaMemcpyHostToDevice, b->st));
-  GENCD_CUDA_TRY(cudaMemcpyAsync(b->d_invn32, i32.data(), 4 * S, cudaMemcpyHostToDevice, b->st));
+  GENCD_CUDA_TRY(cudaMemcpyAsync(b->d_lam, img.data(), 32 * (size_t)S, cudaMemcpyHostToDevice, b->st));
   return GENCD_OK;
 }
 
@@ -1163,6 +1249,43 @@ static int slot_clear(gencd_batch* b, int s) {
   return GENCD_OK;
 }
 
+static int wave_grid(const gencd_batch* b, int64_t rows) { return grid_for(rows, 8, b->X->num_sms * 8); }
+
+static int wave_fill(gencd_batch* b, const SlotWave& v) {
+  k_b_wave_fill<<<wave_grid(b, b->n), dim3(32, 8), 0, b->st>>>(v, b->X->y, b->fold, b->nfolds, b->loss, b->z, b->n,
+                                                              b->S, b->U);
+  GENCD_CUDA_TRY(cudaGetLastError());
+  return GENCD_OK;
+}
+
+// starts the listed slots (h_set, h_lam and h_group are set) from their chains'
+// w_last, or from w = 0
+static int wave_start(gencd_batch* b, const SlotWave& v, const double* w_last, double* w_start) {
+  if (v.m == 0) return GENCD_OK;
+  k_b_wave_start<<<wave_grid(b, std::max(b->k, b->n)), dim3(32, 8), 0, b->st>>>(v, w_last, b->k, b->n, b->S, b->w,
+                                                                               b->w32, w_start, b->z);
+  bool warm = false;
+  for (int q = 0; q < v.m; ++q) warm = warm || v.chain[q] >= 0;
+  if (warm)
+    k_b_wave_scatter<<<grid_for(b->k * 32, kThreads, b->X->num_sms * 8), kThreads, 0, b->st>>>(
+        v, b->X->col_ptr, b->X->row_idx, (const float*)b->X->val, b->w, b->k, b->S, b->z);
+  GENCD_CUDA_TRY(cudaGetLastError());
+  return wave_fill(b, v);
+}
+
+// clears the listed slots (host state and u = 0)
+static int wave_clear(gencd_batch* b, SlotWave v) {
+  if (v.m == 0) return GENCD_OK;
+  for (int q = 0; q < v.m; ++q) {
+    v.set[q] = -1;
+    b->h_set[v.slot[q]] = -1;
+    b->h_lam[v.slot[q]] = 0.0;
+    b->h_group[v.slot[q]] = 1;
+  }
+  GENCD_TRY(upload_slots(b));
+  return wave_fill(b, v);
+}
+
 // objectives of the listed slots (FP64), synchronising; gap (nullable): their
 // duality gaps, which need the max |g_js| of the slots' current state (a
 // propose pass over the current state must have run since the last step)
@@ -1273,8 +1396,7 @@ static void free_batch(gencd_batch* b) {
   drop_graph(b);
   void* bufs[] = {b->fold, b->inv_n, b->sq, b->bj, b->ib, b->bj32, b->ib32, b->tstart, b->tile_cc, b->nzcols,
                   b->bnd, b->w, b->z, b->w32, b->U, b->G, b->acc_j, b->acc_d, b->acc_phi, b->part_lo, b->kkt_bits,
-                  b->ctr, b->obj_acc, b->obj_list, b->tmp_k, b->d_set, b->d_group, b->d_lam, b->d_invn,
-                  b->d_lam32, b->d_invn32};
+                  b->ctr, b->obj_acc, b->obj_list, b->tmp_k, b->d_lam};
   for (void* q : bufs) cudaFree(q);
   cudaGetLastError();
   if (b->X) gencd_destroy(b->X);
@@ -1425,12 +1547,12 @@ static int create_batch(gencd_batch* b, const uint8_t* fold, int32_t memory) {
   GENCD_TRY(balloc(&b->obj_acc, 128));
   GENCD_TRY(balloc(&b->obj_list, 64));
   GENCD_TRY(balloc(&b->tmp_k, k));
-  GENCD_TRY(balloc(&b->d_set, S));
-  GENCD_TRY(balloc(&b->d_group, S));
-  GENCD_TRY(balloc(&b->d_lam, S));
-  GENCD_TRY(balloc(&b->d_invn, S));
-  GENCD_TRY(balloc(&b->d_lam32, S));
-  GENCD_TRY(balloc(&b->d_invn32, S));
+  GENCD_TRY(balloc(&b->d_lam, 4 * (size_t)S));  // all six arrays (upload_slots)
+  b->d_invn = b->d_lam + S;
+  b->d_set = reinterpret_cast<int32_t*>(b->d_invn + S);
+  b->d_group = b->d_set + S;
+  b->d_lam32 = reinterpret_cast<float*>(b->d_group + S);
+  b->d_invn32 = b->d_lam32 + S;
   b->h_set.assign(S, -1);
   b->h_group.assign(S, 1);
   b->h_lam.assign(S, 0.0);
@@ -1750,29 +1872,37 @@ static int batch_path(gencd_batch* b, const gencd_path* path, gencd_path_solve* 
     solves[q].slot = -1;
   }
   int rc = GENCD_OK;
-  for (int s = 0; s < S && rc == GENCD_OK; ++s) rc = slot_clear(b, s);
+  {
+    SlotWave all;
+    for (int s = 0; s < S; ++s) all.add(s, -1, -1);
+    rc = wave_clear(b, all);
+  }
   GENCD_CUDA_TRY(cudaMemsetAsync(b->ctr, 0, 16, b->st));
   const int64_t steps0 = b->steps;
   int done = 0, all_ok = 1;
   std::vector<double> kv;
   std::vector<int32_t> started;
   while (rc == GENCD_OK && done < C * L) {
-    // start ready solves in free slots, chains in turn
+    // start ready solves in free slots, chains in turn: from a live slot's
+    // iterate at once, the others together
+    SlotWave fresh;
     for (int c = 0, free_s = 0; c < C && rc == GENCD_OK; ++c) {
       if (!ready[c] || next[c] >= L) continue;
       while (free_s < S && slot_solve[free_s] >= 0) ++free_s;
       if (free_s >= S) break;
       const int t = next[c], q = c * L + t, s = free_s;
       const double lam = path->lambda[q];
-      if (t == 0 || !path->warm)
-        rc = slot_set(b, s, cset[c], lam, nullptr, chain_group[c]);
-      else if (pred_slot[c] >= 0)
+      if (t > 0 && path->warm && pred_slot[c] >= 0) {
         rc = slot_copy(b, s, pred_slot[c], cset[c], lam, chain_group[c]);
-      else
-        rc = slot_set(b, s, cset[c], lam, w_last + (size_t)c * b->k, chain_group[c]);
-      if (rc == GENCD_OK)
-        k_b_get_w<<<grid_for(b->k, kThreads, g_sm), kThreads, 0, b->st>>>(b->w, b->k, S, s,
-                                                                           w_start + (size_t)s * b->k);
+        if (rc == GENCD_OK)
+          k_b_get_w<<<grid_for(b->k, kThreads, g_sm), kThreads, 0, b->st>>>(b->w, b->k, S, s,
+                                                                             w_start + (size_t)s * b->k);
+      } else {
+        b->h_set[s] = cset[c];
+        b->h_lam[s] = lam;
+        b->h_group[s] = chain_group[c];
+        fresh.add(s, cset[c], t > 0 && path->warm ? c : -1);
+      }
       slot_solve[s] = q;
       slot_epoch[s] = fails[c];
       slot_iters[s] = 0;
@@ -1785,6 +1915,10 @@ static int batch_path(gencd_batch* b, const gencd_path* path, gencd_path_solve* 
       next[c] += 1;
       ready[c] = 0;
       started.push_back(s);
+    }
+    if (rc == GENCD_OK && fresh.m > 0) {
+      rc = upload_slots(b);
+      if (rc == GENCD_OK) rc = wave_start(b, fresh, w_last, w_start);
     }
     if (rc != GENCD_OK) break;
     if (!started.empty()) {  // the objective each new solve starts from (the backoff's reference)
@@ -1903,6 +2037,21 @@ static int batch_path(gencd_batch* b, const gencd_path* path, gencd_path_solve* 
     if (rc != GENCD_OK || retire.empty()) continue;
     std::vector<double> ob;
     rc = slot_objectives(b, retire, &ob);
+    // the finished solves' w to their chains' w_last, all in one launch, and out
+    SlotWave finished, cleared;
+    std::vector<int> finished_q;
+    std::vector<char> taken(C, 0);
+    auto take = [&](SlotWave& v, std::vector<int>& qs) -> int {
+      if (v.m == 0) return GENCD_OK;
+      k_b_wave_get<<<wave_grid(b, b->k), dim3(32, 8), 0, b->st>>>(v, b->w, b->k, S, w_last);
+      GENCD_CUDA_TRY(cudaGetLastError());
+      for (int i = 0; w_out && i < v.m; ++i)
+        GENCD_CUDA_TRY(cudaMemcpyAsync(w_out + (size_t)qs[i] * b->k, w_last + (size_t)v.chain[i] * b->k, 8 * b->k,
+                                       cudaMemcpyDeviceToHost, b->st));
+      v.m = 0;
+      qs.clear();
+      return GENCD_OK;
+    };
     for (size_t r = 0; r < retire.size() && rc == GENCD_OK; ++r) {
       const int s = retire[r], q = slot_solve[s], c = q / L;
       solves[q].objective = ob[r];
@@ -1914,19 +2063,31 @@ static int batch_path(gencd_batch* b, const gencd_path* path, gencd_path_solve* 
         chain_group[c] = 1;
       }
       // the chain's latest finished lambda is the warm start of the solves still to come
-      double* dst = q > last_q[c] ? w_last + (size_t)c * b->k : b->tmp_k;
-      if (q > last_q[c]) last_q[c] = q;
-      k_b_get_w<<<grid_for(b->k, kThreads, b->X->num_sms * 8), kThreads, 0, b->st>>>(b->w, b->k, S, s, dst);
-      if (w_out && (cudaMemcpyAsync(w_out + (size_t)q * b->k, dst, 8 * b->k, cudaMemcpyDeviceToHost, b->st) !=
-                        cudaSuccess ||
-                    cudaStreamSynchronize(b->st) != cudaSuccess))
-        rc = bfail(GENCD_ECUDA, "copy of w failed");
-      if (rc == GENCD_OK) rc = slot_clear(b, s);
+      if (q > last_q[c] && !taken[c]) {
+        last_q[c] = q;
+        taken[c] = 1;
+        finished.add(s, -1, c);
+        finished_q.push_back(q);
+      } else {  // an earlier lambda of its chain, or the chain's second solve to finish here
+        double* dst = q > last_q[c] ? w_last + (size_t)c * b->k : b->tmp_k;
+        if (dst != b->tmp_k) rc = take(finished, finished_q);  // the first one's w leaves w_last
+        if (q > last_q[c]) last_q[c] = q;
+        if (rc == GENCD_OK) {
+          k_b_get_w<<<grid_for(b->k, kThreads, g_sm), kThreads, 0, b->st>>>(b->w, b->k, S, s, dst);
+          if (w_out && (cudaMemcpyAsync(w_out + (size_t)q * b->k, dst, 8 * b->k, cudaMemcpyDeviceToHost, b->st) !=
+                            cudaSuccess ||
+                        cudaStreamSynchronize(b->st) != cudaSuccess))
+            rc = bfail(GENCD_ECUDA, "copy of w failed");
+        }
+      }
+      cleared.add(s, -1, -1);
       slot_solve[s] = -1;
       if (pred_slot[c] == s) pred_slot[c] = -1;
       if (next[c] == (q % L) + 1) ready[c] = 1;  // the successor starts from the final w
       done += 1;
     }
+    if (rc == GENCD_OK) rc = take(finished, finished_q);
+    if (rc == GENCD_OK) rc = wave_clear(b, cleared);
     if (rc == GENCD_OK && cudaStreamSynchronize(b->st) != cudaSuccess)
       rc = bfail(GENCD_ECUDA, std::string("path: ") + cudaGetErrorString(cudaGetLastError()));
   }
