@@ -690,7 +690,8 @@ static int launch_plan_passes(gencd_problem* p, const void* u_vec) {
 
 template <typename V, typename U, typename G, typename SV, int THREADS, int DEPTH, int ITEMS>
 static int set_slab_smem(const ProposePlan& P) {
-  const int smem = (int)((size_t)(P.slab_rows + kSlabZeroSlot) * sizeof(U));
+  // the limit belongs to the kernel, not to the problem: the largest slab's
+  const int smem = (int)(kSlabBytes + kSlabZeroSlot * sizeof(U));
   GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_slabs<V, U, G, THREADS, DEPTH, ITEMS, SV>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   if constexpr (sizeof(V) == 4) {
@@ -933,6 +934,40 @@ void free_propose_plan(gencd_problem* p) {
   p->plan = ProposePlan();
 }
 
+// First tile of each of `grid` CTAs, from the slabs' first tiles tb[0..R].
+// Equal runs of all tiles make some CTAs load two slabs of u, which takes as
+// long as about kSlabSwitch entries; CTAs that keep to one slab have unequal
+// runs.  The split whose longest CTA is shorter.
+constexpr int64_t kSlabSwitch = 16384;
+
+static std::vector<int32_t> split_tiles(const std::vector<int32_t>& tb, int grid, int64_t tile) {
+  const int R = (int)tb.size() - 1;
+  const int64_t T = tb[R];
+  std::vector<int32_t> first(grid + 1);
+  for (int b = 0; b <= grid; ++b) first[b] = (int32_t)(b * T / grid);
+  if (R < 2 || R > grid || T == 0) return first;
+  std::vector<int> ctas(R);  // proportional to the slabs' tiles, at least one each
+  int left = grid;
+  for (int r = 0; r < R; ++r) {
+    ctas[r] = std::max<int>(1, (int)((int64_t)grid * (tb[r + 1] - tb[r]) / T));
+    left -= ctas[r];
+  }
+  int64_t longest = 0;
+  for (; left > 0; --left) {  // the rest to the slab with the longest runs
+    int most = 0;
+    for (int r = 1; r < R; ++r)
+      if ((int64_t)(tb[r + 1] - tb[r]) * ctas[most] > (int64_t)(tb[most + 1] - tb[most]) * ctas[r]) most = r;
+    ctas[most] += 1;
+  }
+  for (int r = 0; r < R; ++r) longest = std::max<int64_t>(longest, (tb[r + 1] - tb[r] + ctas[r] - 1) / ctas[r]);
+  if (left < 0 || longest > (T + grid - 1) / grid + kSlabSwitch / tile) return first;
+  int b = 0;
+  for (int r = 0; r < R; ++r)
+    for (int q = 0; q < ctas[r]; ++q)
+      first[b++] = (int32_t)(tb[r] + (int64_t)q * (tb[r + 1] - tb[r]) / ctas[r]);
+  return first;
+}
+
 // scratch that is freed when the build returns
 struct Scratch {
   gencd_problem* p;
@@ -974,8 +1009,13 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   const size_t vsz = f64 ? 8 : p->vmode == kValBf16 ? 2 : p->vmode == kValNone ? 0 : 4;  // as the plan stores them
   const int g = p->num_sms * 8;
   cudaStream_t st = p->stream;
-  P.slab_rows = (int32_t)(kSlabBytes / (f64 ? 8 : 4));
-  P.nslabs = (int32_t)((n + P.slab_rows - 1) / P.slab_rows);
+  // as few slabs as hold n rows, and all alike: a last slab with the few rows
+  // left over has runs of one or two entries, whose sums and atomic adds made
+  // its CTAs take 72 us where the others took 51 (4e7 non-zeros, n = 200,000:
+  // 3,392 rows left).  Multiples of 8 rows keep the slabs' u 16-byte aligned.
+  const int64_t most_rows = kSlabBytes / (f64 ? 8 : 4);
+  P.nslabs = (int32_t)((n + most_rows - 1) / most_rows);
+  P.slab_rows = (int32_t)(((n + P.nslabs - 1) / P.nslabs + 7) / 8 * 8);
   // one slab: every non-empty column reads u from shared memory; otherwise a
   // column takes this layout once it averages >= 2 entries per slab in FP32
   // arithmetic (the fused pass and the warp reduction of the partials make
@@ -1096,11 +1136,11 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
     GENCD_CUDA_TRY(cudaMemcpyAsync(pad_off, hp.data(), 8 * (R + 1), cudaMemcpyHostToDevice, st));
     GENCD_CUDA_TRY(cudaMemcpyAsync(P.slab_off, off.data(), 4 * (R + 1), cudaMemcpyHostToDevice, st));
     GENCD_CUDA_TRY(cudaMemsetAsync(P.pmask, 0, 4 * (size_t)mask_words, st));
-    std::vector<int32_t> tb(R + 1), ctb(P.grid + 1);  // pageable sources: read when the copy returns
+    std::vector<int32_t> tb(R + 1), ctb;  // pageable sources: read when the copy returns
     for (int i = 0; i < 2; ++i)
       if (sets[i]) {
         for (int r = 0; r <= R; ++r) tb[r] = (int32_t)(hp[r] / tile[i]);
-        for (int b = 0; b <= P.grid; ++b) ctb[b] = (int32_t)((int64_t)b * sets[i]->count / P.grid);
+        ctb = split_tiles(tb, P.grid, tile[i]);
         GENCD_CUDA_TRY(cudaMemcpyAsync(sets[i]->slab_begin, tb.data(), 4 * (R + 1), cudaMemcpyHostToDevice, st));
         GENCD_CUDA_TRY(cudaMemcpyAsync(sets[i]->cta_begin, ctb.data(), 4 * (P.grid + 1), cudaMemcpyHostToDevice, st));
         GENCD_CUDA_TRY(cudaStreamSynchronize(st));

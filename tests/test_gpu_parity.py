@@ -898,3 +898,26 @@ def test_logistic_values_over_the_whole_range(gb):
     np.testing.assert_allclose(d, (-4 * u).astype(np.float64), rtol=2e-15, atol=1e-305)
     loss = np.sum(np.maximum(-m, 0) + np.log1p(np.exp(-np.abs(m)))) / n
     assert obj == pytest.approx(float(loss), rel=1e-14)
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("n", [24_576, 24_577, 49_152, 49_153, 147_457, 640_000])
+def test_propose_at_the_slabs_edges(gb, n, precision):
+    # rows that fill 1, 2, 3 slabs exactly or by one more (24,576 rows in FP64,
+    # 49,152 in FP32), and many slabs for few CTAs each
+    prob = workloads.zipf_problem(n, 1_500, 150_000, cap=n // 2, n_planted=10, loss="squared", seed=n % 89)
+    if precision == "bf16":
+        prob = oracle.stored_problem(prob, "bf16")
+    orc = oracle.Oracle(prob)
+    lam = 0.05 * orc.lambda_max()
+    orc.set_lambda(lam)
+    w = _state(prob, 17)
+    z = orc.fitted(w)
+    J = np.arange(prob.k, dtype=np.int32)
+    d_cpu, f_cpu = orc.propose(w, z, J)
+    with gb.Problem(prob, precision=precision) as p:
+        p.set_lambda(lam)
+        p.set_w(w)
+        for _ in range(2):
+            d, f, _ = p.propose_all()
+            assert_steps_close(prob, z, w, lam, J, d, f, d_cpu, f_cpu, TOL[precision if precision == "f64" else "f32"])
