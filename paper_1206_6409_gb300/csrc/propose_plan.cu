@@ -179,25 +179,21 @@ __device__ __forceinline__ uint32_t lane_mask(const uint8_t* __restrict__ pmask,
 }
 
 // Segmented suffix sum over the lanes: T_L = x_L + x_{L+1} + ... + x_M where M
-// is the first lane >= L with stop set (all lanes to 31 when there is none);
-// ended_L reports whether such an M exists.  Five shuffle steps; in FP64, whose
-// additions are what the passes wait for, only as many as the longest run of
-// the warp takes.
+// is the first lane >= L whose bit is set in `stops` (all lanes to 31 when there
+// is none).  M is known from the ballot, so a step is one shuffle and one
+// addition; in FP64, whose additions are what the passes wait for, only as many
+// steps as the longest run of the warp takes.
 template <typename V>
-__device__ __forceinline__ V lane_suffix_sum(V x, bool stop, int lane, bool& ended) {
+__device__ __forceinline__ V lane_suffix_sum(V x, uint32_t stops, int lane) {
+  const uint32_t from = stops >> lane;
+  const int last = from ? lane + __ffs(from) - 1 : 31;
   V t = x;
-  bool e = stop;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
-    if (sizeof(V) == 8 && !__any_sync(0xffffffffu, !e && lane + d < 32)) break;
+    if (sizeof(V) == 8 && !__any_sync(0xffffffffu, lane + d <= last)) break;
     const V tn = __shfl_down_sync(0xffffffffu, t, d);
-    const bool en = __shfl_down_sync(0xffffffffu, (int)e, d) != 0;
-    if (!e && lane + d < 32) {
-      t += tn;
-      e = en;
-    }
+    if (lane + d <= last) t += tn;
   }
-  ended = e;
   return t;
 }
 
@@ -365,14 +361,13 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
           cont = acc;
         }
       }
-      const bool stop = m != 0u;
-      if (__ballot_sync(FULL, stop) == 0u) {
+      const uint32_t stops = __ballot_sync(FULL, m != 0u);
+      if (stops == 0u) {
         // the whole tile lies inside pair q0
         const V sum = warp_sum(cont);
         if (lane == 0) add_col<G>(gacc, col0, (G)sum);
       } else {
-        bool ended;
-        const V tsum = lane_suffix_sum(cont, stop, lane, ended);
+        const V tsum = lane_suffix_sum(cont, stops, lane);
         const V t1s = __shfl_down_sync(FULL, tsum, 1);
         if (lead) add_col<G>(gacc, col0, (G)tsum);  // pair from the previous tile
         if (has_tail) add_col<G>(gacc, col_last, (G)(tail + (lane < 31 ? t1s : V(0))));
@@ -502,19 +497,17 @@ __device__ __forceinline__ void light_tile(const LightStage<SV>& cur, int64_t t,
       cont = acc;
     }
   }
-  const bool stop = !active || m != 0u;
-  if (__ballot_sync(FULL, stop) == 0u) {
+  const uint32_t stops = __ballot_sync(FULL, !active || m != 0u);
+  if (stops == 0u) {
     const V sum = warp_sum(cont);  // the whole tile is inside column lc0
     if (lane == 0) atomicAdd(out + j0, (G)sum);
   } else {
-    bool ended;
-    const V tsum = lane_suffix_sum(cont, stop, lane, ended);
+    const V tsum = lane_suffix_sum(cont, stops, lane);
     const V t1s = __shfl_down_sync(FULL, tsum, 1);
-    const bool e1 = __shfl_down_sync(FULL, (int)ended, 1) != 0;
     if (lead) atomicAdd(out + j0, (G)tsum);  // column from the previous tile
     if (has_tail) {
       const V sum = tail + (lane < 31 ? t1s : V(0));
-      emit_pair<G>(out, (uint32_t)jl, (G)sum, lane < 31 && e1);
+      emit_pair<G>(out, (uint32_t)jl, (G)sum, lane < 31 && (stops >> (lane + 1)) != 0u);
     }
   }
 }
