@@ -330,21 +330,18 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
         // one FMA chain over the lane's entries; at each start bit after
         // entry 0 the running sum closes a run: the first run (continuing
         // from the left, or a whole run when it began at entry 0) or a run
-        // between two start bits (whole: stored); the last run stays in acc
+        // between two start bits (whole: stored); the last run stays in acc.
+        // Only the latter are a branch: some lane of the warp has a start at
+        // almost every i, and a branch there cost all lanes its instructions.
         const uint32_t inner = m & NOT_FIRST;
-        const int bf = inner ? __ffs(inner) - 1 : ITEMS;  // first start bit after entry 0
+        const uint32_t earliest = inner & (0u - inner), later = inner ^ earliest;  // the first start bit, the others
         V acc = V(0), first = V(0);
-        uint32_t qi = q;
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
-          if ((inner >> i) & 1u) {
-            if (i == bf)
-              first = acc;
-            else
-              add_col<G>(gacc, __ldg(pair_col + qi), (G)acc);  // started and ended inside the lane
-            acc = V(0);
-            ++qi;
-          }
+          if ((later >> i) & 1u)  // a run that started and ended inside the lane
+            add_col<G>(gacc, __ldg(pair_col + q + __popc(inner & ((1u << i) - 1u))), (G)acc);
+          first = (earliest >> i) & 1u ? acc : first;
+          acc = (inner >> i) & 1u ? V(0) : acc;
           acc = fma((V)cur.L.val.get(i), (V)uu[i], acc);
         }
         if (inner) {
