@@ -7,7 +7,8 @@
  * is free and the HBM it needs fits the budget, solves it to its KKT
  * tolerance (gencd_solve's loop: Algorithm 1 with the configured variant and
  * its accept backoff) and returns its memory for the next.  Device memory
- * comes from one memory pool reserved at the start of the call, so no
+ * comes from one memory pool (the most that the requests can hold at once is
+ * reserved at the start of the call), so no
  * request allocates or frees device memory itself (cudaMalloc / cudaFree
  * would stall the device for the others).  Every slot owns a CUDA stream; one
  * host thread creates the admitted requests' problems and another advances
@@ -48,7 +49,7 @@ typedef struct {
   int32_t workers;      /* slots: requests in flight at most (one stream each), 1..64  */
   int32_t precision;    /* gencd_precision of every request                             */
   double hbm_fraction;  /* share of the device's free memory at the start that the
-                           memory pool reserves and the requests in flight may hold
+                           requests in flight may hold by their estimates
                            (0 < f <= 1); a request whose estimate exceeds the whole
                            budget runs alone                                          */
   gencd_params params;  /* iteration parameters of every solve                         */

@@ -5,12 +5,12 @@
 // value, which makes a plain CSC pass L2-bound long before HBM is saturated.
 // Here the rows are cut into slabs of at most 192 KB of u.  A persistent CTA
 // (one per SM, 1024 threads) copies the u slab of its work into shared memory
-// once and gathers from there.  Only columns with at least heavy_min
-// non-zeros use this layout (their entries are regrouped slab by slab, with
-// 16-bit in-slab rows); every (slab, column) "pair" produces one partial sum,
-// added atomically into the column's g_j.  Columns with fewer non-zeros would
-// produce about one partial per non-zero, so they keep a compact CSC copy and
-// the lane-segmented pass with gathers from L2.
+// once and gathers from there.  Every (slab, column) "pair" (entries regrouped
+// slab by slab, with 16-bit in-slab rows) produces one partial sum, added
+// atomically into the column's g_j.  Columns that would produce about two
+// partials per non-zero or more ("light", when there are many: the rule is in
+// build_plan_impl) keep a compact CSC copy and the lane-segmented pass with
+// gathers from L2.
 //
 // Within a slab the kernel works like the CSC pass: a warp owns a tile of
 // consecutive entries, a lane 8 (FP32) or 16 (FP64) of them (128-bit loads of
@@ -712,6 +712,28 @@ int launch_propose_plan(gencd_problem* p, const void* u_vec) {
 // ---------------------------------------------------------------------------
 // building the plan (once per problem)
 
+// What the choice of the heavy columns needs: out[0] columns that are not
+// empty, out[1] entries of those shorter than hmin, out[2] and out[3] columns
+// below and from `forms` entries
+__global__ void __launch_bounds__(kThreads)
+    k_plan_count(const int64_t* __restrict__ col_ptr, int64_t k, int64_t hmin, int64_t forms,
+                 unsigned long long* __restrict__ out) {
+  unsigned long long c[4] = {0, 0, 0, 0};
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < k; j += stride) {
+    const int64_t len = col_ptr[j + 1] - col_ptr[j];
+    if (len <= 0) continue;
+    c[0] += 1;
+    if (len < hmin) c[1] += (unsigned long long)len;
+    c[len < forms ? 2 : 3] += 1;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    c[q] = warp_sum(c[q]);
+    if ((threadIdx.x & 31) == 0 && c[q]) atomicAdd(out + q, c[q]);
+  }
+}
+
 // Columns by kind, for the exclusive scans: hid and lid number the heavy and
 // the light ones, loff offsets the light ones' entries.
 __global__ void k_plan_classify(const int64_t* __restrict__ col_ptr, int64_t k, int64_t hmin,
@@ -1006,12 +1028,36 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   const int64_t most_rows = kSlabBytes / (f64 ? 8 : 4);
   P.nslabs = (int32_t)((n + most_rows - 1) / most_rows);
   P.slab_rows = (int32_t)(((n + P.nslabs - 1) / P.nslabs + 7) / 8 * 8);
-  // one slab: every non-empty column reads u from shared memory; otherwise a
-  // column takes this layout once it averages >= 2 entries per slab in FP32
-  // arithmetic (the fused pass and the warp reduction of the partials make
-  // that pay: fewer entries left to the light pass's gathers of u from L2,
-  // one L1 wavefront each) and >= 8 in FP64 (two separate passes)
-  P.heavy_min = P.nslabs == 1 ? 1 : (f64 ? 8LL : 2LL) * P.nslabs;
+  // Heavy columns.  One slab: every column.  Otherwise a column's run in a slab
+  // costs about as much as gathering its entries from L2 (one L1 wavefront
+  // each) once it averages half an entry per slab in FP32 arithmetic (uniform
+  // columns, a pass over 9.0e7 and 1.8e7 entries as slabs / as light columns:
+  // 1.4 a slab 255 / 343 us, 0.3 a slab 118 / 88) and two in FP64 (0.7 a slab 465
+  // / 400).  The light pass is a kernel of its own, though: what few entries
+  // would be left to it join the slabs (2e8 Zipf non-zeros: 4341 us for ten
+  // iterations from two a slab, 4106 from a half, 3772 with none left; FP64 2e7
+  // 1137 / 1044), while the runs (R per column) are no more than the non-zeros,
+  // which bounds the scratch of the build.
+  constexpr int64_t kFewLight = int64_t(1) << 22;
+  P.heavy_min = 1;
+  P.forms = false;
+  if (P.nslabs > 1) {
+    P.heavy_min = f64 ? 2LL * P.nslabs : std::max<int64_t>(2, (P.nslabs + 1) / 2);
+    unsigned long long* stats = nullptr;
+    Arena count;
+    count.add(&stats, 4);
+    GENCD_TRY(S.get(count));
+    GENCD_CUDA_TRY(cudaMemsetAsync(stats, 0, 4 * sizeof(*stats), st));
+    k_plan_count<<<grid_for(k, kThreads, g), kThreads, 0, st>>>(p->col_ptr, k, P.heavy_min, 2LL * P.nslabs, stats);
+    unsigned long long c[4];
+    GENCD_CUDA_TRY(cudaMemcpyAsync(c, stats, sizeof(c), cudaMemcpyDeviceToHost, st));
+    GENCD_CUDA_TRY(cudaStreamSynchronize(st));
+    if ((int64_t)c[1] <= std::max(kFewLight, p->nnz / 10) && (int64_t)c[0] * P.nslabs <= std::max(kFewLight, p->nnz))
+      P.heavy_min = 1;
+    // the schedules of both passes stay selectable wherever columns lie on both
+    // sides of two entries a slab, whether or not the rule leaves light ones
+    P.forms = !f64 && c[2] > 0 && c[3] > 0;
+  }
 
   // classify, number and offset the columns
   uint32_t *hid, *lid, *loff, *tmp;
@@ -1035,13 +1081,13 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   P.light_nnz = tot[2];
   const int64_t E = p->nnz - P.light_nnz;  // heavy entries
   const int R = P.nslabs;
-  const int64_t runs = (int64_t)R * P.nheavy;  // at most E / 2 with several slabs (heavy_min), E with one
+  const int64_t runs = (int64_t)R * P.nheavy;  // at most two per heavy entry (heavy_min), or p->nnz (or 2^22)
 
   // the plan's per-column arrays and the light columns' copy
   const int64_t lpad = P.nlight > 0 ? ((P.light_nnz + kPadNnz - 1) / kPadNnz) * kPadNnz + kPadNnz : 0;
   const int64_t lwords = (lpad + 31) / 32;  // start bits, one byte per 8 entries
   P.light_ntiles = (P.light_nnz + kLightTile - 1) / kLightTile;
-  const bool fusable = !f64 && P.nlight > 0 && P.nheavy > 0;
+  const bool fusable = P.forms;
   Arena light;
   light.add(&P.heavy_cols, P.nheavy);
   light.add(&P.light_cols, P.nlight);
@@ -1198,8 +1244,9 @@ constexpr float kTuneClose = 1.15f;
 int tune_propose_plan(gencd_problem* p) {
   constexpr int C = kNumFusedSplits + 1;
   ProposePlan& P = p->plan;
-  P.tuned_ms[0] = -1.0;
-  if (!P.built || !P.light_counter) return GENCD_OK;
+  for (double& ms : P.tuned_ms) ms = -1.0;
+  P.fused_split = 0;
+  if (!P.built || !P.light_counter || P.nlight == 0) return GENCD_OK;
   cudaEvent_t ev[2 * C] = {};
   int rc = GENCD_OK;
   for (cudaEvent_t& e : ev)

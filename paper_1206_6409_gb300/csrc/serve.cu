@@ -88,7 +88,7 @@ double footprint(const gencd_request& r, int precision, const gencd_params& para
   const double vsz = precision == GENCD_F64 ? 8.0 : 4.0;
   const double nnz = (double)r.nnz, n = (double)r.n, k = (double)r.k;
   double b = nnz * (4.0 + vsz)               // CSC
-             + nnz * (4.0 + vsz + 0.25)      // streaming plan
+             + nnz * (6.0 + vsz + 0.25)      // streaming plan (2-byte rows; at most a 4-byte pair an entry)
              + nnz * (4.0 + vsz) + 8.0 * n   // row-major copy
              + nnz * 24.0                    // its sort scratch
              + n * (16.0 + vsz)              // y, z, u

@@ -921,3 +921,40 @@ def test_propose_at_the_slabs_edges(gb, n, precision):
         for _ in range(2):
             d, f, _ = p.propose_all()
             assert_steps_close(prob, z, w, lam, J, d, f, d_cpu, f_cpu, TOL[precision if precision == "f64" else "f32"])
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32", "bf16", "binary"])
+def test_propose_with_light_and_heavy_columns(gb, precision):
+    # columns that average less than half an entry per slab of rows keep the
+    # light pass when they hold more than 2^22 non-zeros: 1.2e6 of 4 entries
+    # beside 2,000 of 300 and a long one, 10 slabs in FP32 and 20 in FP64; every
+    # schedule of the two passes
+    rng = np.random.default_rng(12)
+    n = 480_000
+    counts = np.full(1_200_000, 4, np.int64)
+    counts[rng.permutation(counts.size)[:2000]] = 300
+    counts[77] = 100_000
+    counts[[0, 5, counts.size - 1]] = 0
+    col_ptr = np.zeros(counts.size + 1, np.int64)
+    np.cumsum(counts, out=col_ptr[1:])
+    rows = workloads.synthetic._distinct_rows(n, counts, rng)
+    val = np.repeat(rng.lognormal(0.0, 0.5, counts.size), counts)
+    if precision != "binary":
+        val = val * rng.lognormal(0.0, 0.5, rows.size)
+    prob = workloads.Problem(n, counts.size, col_ptr, rows, val, rng.normal(size=n), "squared",
+                             np.zeros(counts.size), "light-heavy")
+    sp = oracle.stored_problem(prob, precision) if precision in ("bf16", "binary") else prob
+    orc = oracle.Oracle(sp)
+    lam = 0.05 * orc.lambda_max()
+    orc.set_lambda(lam)
+    w = _state(prob, 17, frac=0.01)
+    z = orc.fitted(w)
+    J = np.arange(prob.k, dtype=np.int32)
+    d_cpu, f_cpu = orc.propose(w, z, J)
+    with gb.Problem(prob, precision=precision) as p:
+        p.set_lambda(lam)
+        p.set_w(w)
+        for split in [0] if precision == "f64" else [0, 20, 31]:
+            gb.gencd_set_propose_schedule(p.h, split)
+            d, f, _ = p.propose_all()
+            assert_steps_close(sp, z, w, lam, J, d, f, d_cpu, f_cpu, TOL["f64" if precision == "f64" else "f32"])
