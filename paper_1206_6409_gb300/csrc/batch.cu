@@ -42,7 +42,7 @@ namespace gencd {
 constexpr int kBatchMaxSlots = 256;
 constexpr int kBatchMaxFolds = 31;
 constexpr int kSpmmThreads = 256;
-constexpr int kAcceptThreads = 512;  // per partition: slots x column strides
+constexpr int kAcceptThreads = 1024;  // per partition: slots x column strides
 constexpr int kObjChecks = 8;        // convergence checks between objective evaluations of a path solve
 constexpr int kStallIters = 500;     // iterations without progress taken as a stall (as gencd_solve)
 constexpr double kStallGain = 1e-2;  // a new lowest KKT value is 1% below the previous one
@@ -198,6 +198,8 @@ __global__ void k_b_absmax(const float* __restrict__ G0, int64_t k, int nsets, u
 // zero the G rows added atomically by k_b_spmm, and the per-slot KKT maxima
 __global__ void k_b_prep(const int32_t* __restrict__ bnd, int64_t nb, int Sp, float* __restrict__ G,
                          unsigned int* __restrict__ kkt_bits) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t total = nb * Sp;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += stride) {
@@ -234,6 +236,8 @@ __global__ void __launch_bounds__(kSpmmThreads)
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  pdl_trigger();
+  pdl_wait();
   if (w >= W) return;
   const int64_t t0 = ntiles * w / W, t1 = ntiles * (w + 1) / W;
   if (t0 >= t1) return;
@@ -308,6 +312,8 @@ __global__ void __launch_bounds__(kAcceptThreads)
   __shared__ uint32_t s_mag[kAcceptThreads];
   __shared__ int32_t s_col[kAcceptThreads];
   __shared__ float s_v[kAcceptThreads];
+  pdl_trigger();
+  pdl_wait();
   const int b = blockIdx.x;
   const int s = threadIdx.x % Sp, r = threadIdx.x / Sp;
   const bool live = r < R;
@@ -391,6 +397,8 @@ __global__ void __launch_bounds__(kAcceptThreads)
 // the lower partition).  G = B is Greedy.
 __global__ void k_b_merge(int32_t* __restrict__ acc_j, const double* __restrict__ acc_phi, int B, int Sp,
                           const int32_t* __restrict__ group) {
+  pdl_trigger();
+  pdl_wait();
   const int q = blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= B * Sp) return;
   const int b = q / Sp, s = q % Sp;
@@ -415,6 +423,8 @@ __global__ void k_b_update(const int32_t* __restrict__ acc_j, const double* __re
                            const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row,
                            const float* __restrict__ val, double* __restrict__ w, float* __restrict__ w32,
                            double* __restrict__ z, unsigned long long* __restrict__ ctr) {
+  pdl_trigger();
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int nw = (gridDim.x * blockDim.x) >> 5;
   for (int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < npairs; q += nw) {
@@ -448,6 +458,8 @@ __global__ void k_b_update_grouped(const int32_t* __restrict__ acc_j, const doub
                                    int Sp, const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row,
                                    const float* __restrict__ val, double* __restrict__ w, float* __restrict__ w32,
                                    double* __restrict__ z, unsigned long long* __restrict__ ctr) {
+  pdl_trigger();
+  pdl_wait();
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int per = (Sp + 31) / 32;
@@ -511,6 +523,8 @@ __global__ void k_b_refresh(const int32_t* __restrict__ acc_j, int npairs, int S
                             const int32_t* __restrict__ row, const double* __restrict__ y,
                             const uint8_t* __restrict__ fold, int nfolds, int loss, const int32_t* __restrict__ sset,
                             const double* __restrict__ z, float* __restrict__ U) {
+  pdl_trigger();
+  pdl_wait();
   const int lane = threadIdx.x & 31;
   const int nw = (gridDim.x * blockDim.x) >> 5;
   for (int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < npairs; q += nw) {
@@ -532,6 +546,8 @@ __global__ void k_b_refresh(const int32_t* __restrict__ acc_j, int npairs, int S
 __global__ void k_b_refresh_all(const double* __restrict__ y, const uint8_t* __restrict__ fold, int nfolds, int loss,
                                 const int32_t* __restrict__ sset, const double* __restrict__ z, int64_t n, int Sp,
                                 float* __restrict__ U) {
+  pdl_trigger();
+  pdl_wait();
   const int s = threadIdx.x;
   const int set = sset[s];
   const int64_t stride = (int64_t)gridDim.x * blockDim.y;
@@ -571,6 +587,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     k_b_spmm_runs8(const int32_t* __restrict__ row, const float* __restrict__ val, const uint8_t* __restrict__ smask,
                    const int32_t* __restrict__ tile_cc, const int32_t* __restrict__ nzcols,
                    const float* __restrict__ U, int S, float* __restrict__ G, int64_t nnz, int64_t ntiles) {
+  pdl_trigger();
+  pdl_wait();
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const float* __restrict__ Uc = U + 8 * blockIdx.y;
@@ -992,8 +1010,8 @@ static int upload_slots(gencd_batch* b) {
 template <int NC>
 static int launch_spmm_nc(gencd_batch* b, const float* U, float* G) {
   constexpr int GRP = NC <= 2 ? 8 : 4;
-  k_b_spmm<NC, GRP><<<b->spmm_grid, kSpmmThreads, 0, b->st>>>(b->X->row_idx, (const float*)b->X->val, b->tstart,
-                                                              b->tile_cc, b->nzcols, U, G, b->ntiles, b->W);
+  GENCD_CUDA_TRY(launch_overlapped(k_b_spmm<NC, GRP>, dim3(b->spmm_grid), dim3(kSpmmThreads), 0, b->st, b->X->row_idx,
+                                   (const float*)b->X->val, b->tstart, b->tile_cc, b->nzcols, U, G, b->ntiles, b->W));
   return GENCD_OK;
 }
 
@@ -1007,9 +1025,9 @@ static int launch_spmm(gencd_batch* b, int kind, const float* U, float* G) {
     const int64_t t256 = (b->nnz + 255) / 256;
     if (t256 == 0) return GENCD_OK;
     const dim3 grid(grid_for(t256 * 32, kThreads, b->X->num_sms * 2), b->S / 8);
-    k_b_spmm_runs8<<<grid, kThreads, 0, b->st>>>(b->X->row_idx, (const float*)b->X->val,
-                                                  reinterpret_cast<const uint8_t*>(b->tstart), b->tile_cc, b->nzcols,
-                                                  U, b->S, G, b->nnz, t256);
+    GENCD_CUDA_TRY(launch_overlapped(k_b_spmm_runs8, grid, dim3(kThreads), 0, b->st, b->X->row_idx,
+                                     (const float*)b->X->val, reinterpret_cast<const uint8_t*>(b->tstart), b->tile_cc,
+                                     b->nzcols, U, b->S, G, b->nnz, t256));
     return GENCD_OK;
   }
   switch (NC) {
@@ -1057,27 +1075,21 @@ static int enqueue_propose(gencd_batch* b, bool accept) {
   const int g = b->X->num_sms * 8;
   // the lanes-over-entries pass zeroes all of G itself
   const int64_t nb = (b->NC == 0 || b->spmm_kind == 0) ? 0 : 2 * b->W;
-  k_b_prep<<<grid_for(std::max<int64_t>(1, nb * b->S), kThreads, g), kThreads, 0, b->st>>>(b->bnd, nb, b->S, b->G,
-                                                                                          b->kkt_bits);
+  GENCD_CUDA_TRY(launch_overlapped(k_b_prep, dim3(grid_for(std::max<int64_t>(1, nb * b->S), kThreads, g)),
+                                   dim3(kThreads), 0, b->st, b->bnd, nb, b->S, b->G, b->kkt_bits));
   GENCD_TRY(launch_spmm(b, b->spmm_kind, b->U, b->G));
   const int R = accept_R(b);
-  if (accept)
-    k_b_accept<1><<<b->B, b->S * R, 0, b->st>>>(b->G, b->w32, b->w, b->bj32, b->ib32, b->bj, b->ib, b->k,
-                                                 slot_args(b), b->part_lo, b->S, R, b->acc_j, b->acc_d,
-                                                 b->acc_phi, b->kkt_bits);
-  else
-    k_b_accept<0><<<b->B, b->S * R, 0, b->st>>>(b->G, b->w32, b->w, b->bj32, b->ib32, b->bj, b->ib, b->k,
-                                                 slot_args(b), b->part_lo, b->S, R, nullptr, nullptr, nullptr,
-                                                 b->kkt_bits);
-  GENCD_CUDA_TRY(cudaGetLastError());
+  GENCD_CUDA_TRY(launch_overlapped(accept ? k_b_accept<1> : k_b_accept<0>, dim3(b->B), dim3(b->S * R), 0, b->st, b->G,
+                                   b->w32, b->w, b->bj32, b->ib32, b->bj, b->ib, b->k, slot_args(b), b->part_lo, b->S,
+                                   R, b->acc_j, b->acc_d, b->acc_phi, b->kkt_bits));
   return GENCD_OK;
 }
 
 static int launch_refresh_all(gencd_batch* b) {
   const int rows = std::max(1, 256 / b->S);
   const int g = grid_for(b->n, rows, b->X->num_sms * 16);
-  k_b_refresh_all<<<g, dim3(b->S, rows), 0, b->st>>>(b->X->y, b->fold, b->nfolds, b->loss, b->d_set, b->z, b->n,
-                                                     b->S, b->U);
+  GENCD_CUDA_TRY(launch_overlapped(k_b_refresh_all, dim3(g), dim3(b->S, rows), 0, b->st, b->X->y, b->fold, b->nfolds,
+                                   b->loss, b->d_set, b->z, b->n, b->S, b->U));
   return GENCD_OK;
 }
 
@@ -1085,24 +1097,26 @@ static int enqueue_step(gencd_batch* b) {
   GENCD_TRY(enqueue_propose(b, true));
   const int npairs = b->B * b->S;
   if (b->B > 1)
-    k_b_merge<<<(npairs + kThreads - 1) / kThreads, kThreads, 0, b->st>>>(b->acc_j, b->acc_phi, b->B, b->S,
-                                                                         b->d_group);
+    GENCD_CUDA_TRY(launch_overlapped(k_b_merge, dim3((npairs + kThreads - 1) / kThreads), dim3(kThreads), 0, b->st,
+                                     b->acc_j, b->acc_phi, b->B, b->S, b->d_group));
   const int g = grid_for((int64_t)npairs * 32, kThreads, b->X->num_sms * 8);
   if (b->update_kind == 1) {
     const int per = (b->S + 31) / 32;
-    k_b_update_grouped<<<grid_for((int64_t)b->B * per * 32, kThreads, b->X->num_sms * 8), kThreads, 0, b->st>>>(
-        b->acc_j, b->acc_d, b->B, b->S, b->X->col_ptr, b->X->row_idx, (const float*)b->X->val, b->w, b->w32, b->z,
-        b->ctr);
+    const int gg = grid_for((int64_t)b->B * per * 32, kThreads, b->X->num_sms * 8);
+    GENCD_CUDA_TRY(launch_overlapped(k_b_update_grouped, dim3(gg), dim3(kThreads), 0, b->st, b->acc_j, b->acc_d, b->B,
+                                     b->S, b->X->col_ptr, b->X->row_idx, (const float*)b->X->val, b->w, b->w32, b->z,
+                                     b->ctr));
   } else {
-    k_b_update<<<g, kThreads, 0, b->st>>>(b->acc_j, b->acc_d, npairs, b->S, b->X->col_ptr, b->X->row_idx,
-                                          (const float*)b->X->val, b->w, b->w32, b->z, b->ctr);
+    GENCD_CUDA_TRY(launch_overlapped(k_b_update, dim3(g), dim3(kThreads), 0, b->st, b->acc_j, b->acc_d, npairs, b->S,
+                                     b->X->col_ptr, b->X->row_idx, (const float*)b->X->val, b->w, b->w32, b->z,
+                                     b->ctr));
   }
   if (b->dense_refresh)
     GENCD_TRY(launch_refresh_all(b));
   else
-    k_b_refresh<<<g, kThreads, 0, b->st>>>(b->acc_j, npairs, b->S, b->X->col_ptr, b->X->row_idx, b->X->y, b->fold,
-                                           b->nfolds, b->loss, b->d_set, b->z, b->U);
-  GENCD_CUDA_TRY(cudaGetLastError());
+    GENCD_CUDA_TRY(launch_overlapped(k_b_refresh, dim3(g), dim3(kThreads), 0, b->st, b->acc_j, npairs, b->S,
+                                     b->X->col_ptr, b->X->row_idx, b->X->y, b->fold, b->nfolds, b->loss, b->d_set,
+                                     b->z, b->U));
   b->steps += 1;
   return GENCD_OK;
 }
