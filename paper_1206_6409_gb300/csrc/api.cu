@@ -333,8 +333,7 @@ static int shotgun_on_list(gencd_problem* p, const int32_t* J, int64_t m, bool e
   GENCD_TRY(launch_propose_list(p, J, m, p->list_d, p->phi));
   GENCD_TRY(launch_improve_list(p, J, p->list_d, m));  // Improve delta_j: from the start state's z
   GENCD_TRY(launch_apply_list(p, J, p->list_d, m));
-  GENCD_TRY(launch_update_list(p, J, p->list_d, m));
-  return launch_refresh_list(p, J, m, true);
+  return launch_update_refresh(p, J, p->list_d, m);
 }
 
 // one GenCD iteration (Algorithm 1) of the configured variant, enqueued
@@ -352,8 +351,7 @@ static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt)
       GENCD_TRY(launch_improve_list(p, p->list_j, p->list_d, B));  // Improve delta_j (Algorithm 3), if asked
       GENCD_TRY(launch_apply_list(p, p->list_j, p->list_d, B));
     }
-    GENCD_TRY(launch_update_list(p, p->list_j, p->list_d, B));  // Update (atomic z)
-    GENCD_TRY(launch_refresh_list(p, p->list_j, B, true));
+    GENCD_TRY(launch_update_refresh(p, p->list_j, p->list_d, B));  // Update (atomic z; u)
     *host_nnz += p->nnz;
     p->stat_host_nnz += p->nnz;
   } else if (v == GENCD_TOP_GREEDY) {
@@ -365,8 +363,7 @@ static int enqueue_iteration(gencd_problem* p, int64_t* host_nnz, bool want_kkt)
     GENCD_TRY(launch_top_accept(p, B));                 // Accept: the B lowest proxies
     GENCD_TRY(launch_improve_list(p, p->list_j, p->list_d, B));
     GENCD_TRY(launch_apply_list(p, p->list_j, p->list_d, B));
-    GENCD_TRY(launch_update_list(p, p->list_j, p->list_d, B));  // Update (atomic z)
-    GENCD_TRY(launch_refresh_list(p, p->list_j, B, true));
+    GENCD_TRY(launch_update_refresh(p, p->list_j, p->list_d, B));  // Update (atomic z; u)
     *host_nnz += p->nnz;
     p->stat_host_nnz += p->nnz;
   } else if (v == GENCD_SHOTGUN) {

@@ -177,6 +177,7 @@ struct gencd_problem {
   int64_t stat_host_nnz = 0;  // non-zeros streamed by full passes since the reset
 
   void* mem = nullptr;  // the allocation that holds the arrays every problem has
+  int64_t max_len = 0;  // non-zeros of the longest column
 
   // CSC + rows + cols
   int64_t* col_ptr = nullptr;
@@ -319,7 +320,7 @@ int launch_inv_beta(gencd_problem* p);   // ib_j = 1 / beta_j for the current be
 // u = l'(y, z); with report (pinned host memory), counts[0..1] are copied there and reset
 int launch_fill_u(gencd_problem* p, unsigned long long* counts = nullptr, unsigned long long* report = nullptr);
 int launch_apply_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m);   // w, list_off
-int launch_update_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m);  // z (after w)
+int launch_update_refresh(gencd_problem* p, const int32_t* J, const double* d, int64_t m);  // z and u (after w)
 int launch_refresh_list(gencd_problem* p, const int32_t* J, int64_t m, bool counted);    // u (after z)
 int launch_shotgun_step(gencd_problem* p, const int32_t* J, int64_t m, bool early);      // propose, w and z
 int launch_coloring_iter(gencd_problem* p, int64_t q, bool early);
@@ -386,20 +387,32 @@ void prof_end(gencd_problem* p, cudaEvent_t stop);
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+//
+// launch_cluster_overlapped: the same with the grid as one cluster of CTAs.
 template <typename... P, typename... A>
-inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
-                                     A... args) {
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
+inline cudaError_t launch_cluster_overlapped(void (*kernel)(P...), unsigned cluster, dim3 grid, dim3 block, size_t smem,
+                                             cudaStream_t stream, A... args) {
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+                                     A... args) {
+  return launch_cluster_overlapped(kernel, 1u, grid, block, smem, stream, args...);
 }
 
 // grow a device allocation

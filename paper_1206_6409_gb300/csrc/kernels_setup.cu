@@ -53,15 +53,20 @@ const std::vector<double>& logistic_table() {
 }
 
 // ---------------------------------------------------------------------------
-// validation: err[0] <- smallest bad column, err[1] <- smallest bad row (y)
+// validation: err[0] <- smallest bad column, err[1] <- smallest bad row (y);
+// err[2] <- the longest column
 __global__ void k_validate_colptr(const int64_t* __restrict__ col_ptr, int64_t k, int64_t nnz,
                                   unsigned long long* __restrict__ err) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  unsigned longest = 0;
   for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < k; j += stride) {
     const int64_t s = col_ptr[j], t = col_ptr[j + 1];
+    if (t > s) longest = t - s > (int64_t)longest ? (unsigned)(t - s) : longest;
     bool bad = s < 0 || t < s || t > nnz || (j == 0 && s != 0) || (j == k - 1 && t != nnz);
     if (bad) atomicMin(err, (unsigned long long)j);
   }
+  longest = __reduce_max_sync(0xffffffffu, longest);
+  if ((threadIdx.x & 31) == 0 && longest) atomicMax(err + 2, (unsigned long long)longest);
 }
 
 // bit p of starts is set when nnz position p begins a non-empty column
@@ -722,7 +727,8 @@ int launch_tile_map(gencd_problem* p) {
 int validate_input(gencd_problem* p, int64_t* bad_col, int64_t* bad_row, int* stage) {
   unsigned long long* err = nullptr;
   GENCD_TRY(dev_alloc_bytes(p, (void**)&err, 3 * sizeof(unsigned long long)));
-  GENCD_CUDA_TRY(cudaMemsetAsync(err, 0xff, 3 * sizeof(unsigned long long), p->stream));
+  GENCD_CUDA_TRY(cudaMemsetAsync(err, 0xff, 2 * sizeof(unsigned long long), p->stream));
+  GENCD_CUDA_TRY(cudaMemsetAsync(err + 2, 0, sizeof(unsigned long long), p->stream));
   const int g = p->num_sms * 8;
   k_validate_colptr<<<grid_for(p->k, kThreads, g), kThreads, 0, p->stream>>>(p->col_ptr, p->k, p->nnz, err);
   unsigned long long h[3] = {0, 0, 0};
@@ -735,6 +741,7 @@ int validate_input(gencd_problem* p, int64_t* bad_col, int64_t* bad_row, int* st
     return GENCD_OK;
   }
   *stage = 1;
+  p->max_len = (int64_t)h[2];
   uint32_t* starts = nullptr;
   const int64_t words = (p->nnz + 31) / 32 + 1;
   GENCD_TRY(dev_alloc_bytes(p, (void**)&starts, words * sizeof(uint32_t)));

@@ -201,6 +201,43 @@ __global__ void __launch_bounds__(kListThreads)
   }
 }
 
+// Both passes over a short list in one launch: the CTAs are one cluster, whose
+// barrier stands between the last addition into z and the first u.  Every launch
+// of an iteration of little work costs 2 us or more, on the device and on the
+// host; kClusterCtas SMs refresh up to short_list() non-zeros in about that time.
+constexpr int kClusterCtas = 8;
+
+template <typename V, typename U>
+__global__ void __launch_bounds__(kListThreads)
+    k_update_refresh(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
+                     const V* __restrict__ val, const int32_t* __restrict__ J, const double* __restrict__ D,
+                     const uint32_t* __restrict__ list, int64_t m, const double* __restrict__ y, double* z, int64_t n,
+                     int loss, const double* __restrict__ tab, U* __restrict__ u,
+                     unsigned long long* __restrict__ counters) {
+  __shared__ uint32_t s_off[kListScanMax + 1];
+  pdl_trigger();
+  pdl_wait();
+  const uint32_t* off = list_offsets<true>(list, m, s_off, counters);
+  const int64_t total = off[m], threads = (int64_t)kClusterCtas * kListThreads;
+  // neighbouring warps on different SMs, as in k_refresh_flat
+  const int64_t q0 = ((int64_t)(threadIdx.x >> 5) * kClusterCtas + blockIdx.x) * 32 + (threadIdx.x & 31);
+  for (int64_t q = q0; q < total; q += threads) {
+    const int64_t e = entry_of(off, m, (uint32_t)q);
+    const int64_t p = col_ptr[J[e]] + ((uint32_t)q - off[e]);
+    atomicAdd(z + row_idx[p], D[e] * (double)val[p]);
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (total >= n) {
+    for (int64_t i = q0; i < n; i += threads) u[i] = u_value<U>(loss, y[i], __ldcg(z + i), tab);
+    return;
+  }
+  for (int64_t q = q0; q < total; q += threads) {
+    const int64_t e = entry_of(off, m, (uint32_t)q);
+    const int32_t i = row_idx[col_ptr[J[e]] + ((uint32_t)q - off[e])];
+    u[i] = u_value<U>(loss, y[i], __ldcg(z + i), tab);
+  }
+}
+
 // Shotgun's Propose, Accept (all of J) and the Update of w and z in one pass:
 // a proposal reads u and its own w_j only, so its column's step goes into z at
 // once (u follows when all have landed: k_refresh_flat).  A CTA takes `per`
@@ -586,11 +623,33 @@ static int prefix_long_list(gencd_problem* p, int64_t m) {
 // CTAs of the passes over a list: as many threads as are resident
 static int list_grid(const gencd_problem* p) { return p->num_sms * 4; }
 
+// Non-zeros up to which a list's two passes go in one launch (k_update_refresh).
+// Twenty Thread-Greedy iterations on uniform columns, in one launch / in two:
+// FP64 2,000 non-zeros a list 638 / 669 us, 320 518 / 577; FP32 3,840 non-zeros
+// 522 / 557, 320 431 / 478; beyond, eight SMs are too few: 18,000 to 19,000 FP32
+// non-zeros 678 to 697 / 525 to 529.
+static int64_t short_list(const gencd_problem* p) { return p->precision == GENCD_F64 ? 4096 : 8192; }
+
 // Update (Algorithm 3) of z for the list (J, d) whose w has been applied
-// (list_off), and the counters
-int launch_update_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m) {
+// (list_off), the counters, and u
+int launch_update_refresh(gencd_problem* p, const int32_t* J, const double* d, int64_t m) {
   if (m <= 0) return GENCD_OK;
   unsigned long long* ctr = reinterpret_cast<unsigned long long*>(p->dscal + 4);
+  if (m <= kListScanMax && m * p->max_len <= short_list(p)) {
+    cudaEvent_t ev = nullptr;
+    prof_begin(p, K_UPDATE, &ev);
+    auto go = [&](auto kernel, auto* val, auto* u) {
+      return launch_cluster_overlapped(kernel, kClusterCtas, dim3(kClusterCtas), dim3(kListThreads), 0, p->stream,
+                                       p->col_ptr, p->row_idx, val, J, d, p->list_off, m, p->y, p->z, p->n, p->loss,
+                                       p->ltab, u, ctr);
+    };
+    const cudaError_t err = p->precision == GENCD_F64
+                                ? go(k_update_refresh<double, double>, (const double*)p->val, (double*)p->u)
+                                : go(k_update_refresh<float, float>, (const float*)p->val, (float*)p->u);
+    prof_end(p, ev);
+    GENCD_CUDA_TRY(err);
+    return GENCD_OK;
+  }
   const bool scan = m <= kListScanMax;
   if (!scan) GENCD_TRY(prefix_long_list(p, m));
   cudaEvent_t ev = nullptr;
@@ -606,7 +665,7 @@ int launch_update_list(gencd_problem* p, const int32_t* J, const double* d, int6
     err = go(scan ? k_update_flat<float, true> : k_update_flat<float, false>, (const float*)p->val);
   prof_end(p, ev);
   GENCD_CUDA_TRY(err);
-  return GENCD_OK;
+  return launch_refresh_list(p, J, m, true);
 }
 
 // u on the rows of the list's applied columns, after z.  counted: the list's

@@ -958,3 +958,32 @@ def test_propose_with_light_and_heavy_columns(gb, precision):
             gb.gencd_set_propose_schedule(p.h, split)
             d, f, _ = p.propose_all()
             assert_steps_close(sp, z, w, lam, J, d, f, d_cpu, f_cpu, TOL["f64" if precision == "f64" else "f32"])
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
+@pytest.mark.parametrize("n", [3_000, 30_000])
+@pytest.mark.parametrize("B", [1, 256, 257, 512, 513])
+def test_update_and_refresh_on_both_sides_of_one_launch(gb, n, B, precision):
+    # columns of 16: up to 256 (FP64) and 512 (FP32) partitions z and u take
+    # one launch, with fewer rows than touched (all refreshed) and more; z has
+    # to be X w, and u is what the proposals of the new state see
+    prob = workloads.uniform_problem(n, 8_000, 16, values="lognormal", loss="logistic", n_planted=30, seed=2)
+    assert prob.col_nnz().max() == 16
+    orc = oracle.Oracle(prob)
+    lam = 0.02 * orc.lambda_max()
+    orc.set_lambda(lam)
+    with gb.Problem(prob, precision=precision) as p:
+        p.set_lambda(lam)
+        p.set_params(variant="thread_greedy", blocks=B)
+        p.iterate(3)
+        w, z = p.w(), p.z()
+        d, f, _ = p.propose_all()
+    assert np.count_nonzero(w) > 0
+    tol = TOL[precision]
+    # sums of n_i terms of w_j x_ij: 2^-53 each and per partial sum (some tens of
+    # columns a row, three times over); stored values carry 2^-24 in FP32
+    terms = np.bincount(prob.row_idx, weights=np.abs(prob.val * np.repeat(w, prob.col_nnz())), minlength=n).max()
+    np.testing.assert_allclose(z, orc.fitted(w), rtol=0, atol=(3e-14 if precision == "f64" else 1.2e-7) * terms)
+    J = np.arange(prob.k, dtype=np.int32)
+    d_cpu, f_cpu = orc.propose(w, z, J)
+    assert_steps_close(prob, z, w, lam, J, d, f, d_cpu, f_cpu, tol)
