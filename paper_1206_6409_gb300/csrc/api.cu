@@ -647,7 +647,7 @@ static int create_impl(gencd_problem* p, const int64_t* col_ptr, const int32_t* 
   a.add(&p->tile_col, p->ntiles + 1);
   a.add(&p->gacc, k);
   float* gf = nullptr;
-  if (p->precision != GENCD_F64) a.add(&gf, k);
+  if (p->precision != GENCD_F64) a.add(&gf, 2 * k);  // two sums a column (ProposePlan::second)
   a.add(&p->delta, k);
   a.add(&p->phi, k);
   a.add(&p->list_j, k);
@@ -718,7 +718,7 @@ static int create_impl(gencd_problem* p, const int64_t* col_ptr, const int32_t* 
   GENCD_CUDA_TRY(cudaMemsetAsync(p->w, 0, sizeof(double) * k, st));
   if (p->w32) GENCD_CUDA_TRY(cudaMemsetAsync(p->w32, 0, sizeof(float) * k, st));
   GENCD_CUDA_TRY(cudaMemsetAsync(p->gacc, 0, sizeof(double) * k, st));
-  if (p->gnat != p->gacc) GENCD_CUDA_TRY(cudaMemsetAsync(p->gnat, 0, sizeof(float) * k, st));
+  if (p->gnat != p->gacc) GENCD_CUDA_TRY(cudaMemsetAsync(p->gnat, 0, 2 * sizeof(float) * k, st));
   GENCD_CUDA_TRY(cudaMemsetAsync(p->dscal, 0, kScalars * sizeof(double), st));
   GENCD_TRY(launch_tile_map(p));
   GENCD_TRY(launch_col_scale(p));

@@ -112,6 +112,7 @@ struct ProposePlan {
   bool built = false;
   int32_t slab_rows = 0, nslabs = 0;
   int64_t heavy_min = 0;
+  int64_t second = 0;  // offset of the second sum of a column in gnat (0: one sum)
   bool forms = false;  // the schedules with both passes in one kernel can be set
   // light columns
   int64_t nlight = 0, light_nnz = 0, light_ntiles = 0;

@@ -225,11 +225,12 @@ constexpr int kRoundCols = kColsPerThread * kThreads;  // columns a CTA scans pe
 // queues the active ones in shared memory; after a barrier the queue is
 // processed packed (one active column per thread), so FP64 work is
 // proportional to the number of active columns, not to the warps that hold
-// one.  scale (index-only storage): each column's value, applied to its sum.  Returns the queue length; the queue holds (j, raw sum, w_j).
+// one.  second: offset of a column's second sum (0: none).  scale (index-only
+// storage): each column's value, applied to its sum.  Returns the queue length; the queue holds (j, raw sum, w_j).
 template <typename G>
 __device__ __forceinline__ int scan_round(G* __restrict__ gacc, const double* __restrict__ w, int64_t base,
-                                          int64_t hi, uint64_t lnb64, uint32_t lnb32, const float* __restrict__ scale,
-                                          int* s_n, int64_t* s_j, double* s_g, double* s_w, double* delta,
+                                          int64_t hi, uint64_t lnb64, uint32_t lnb32, int64_t second,
+                                          const float* __restrict__ scale, int* s_n, int64_t* s_j, double* s_g, double* s_w, double* delta,
                                           double* phi) {
   G ga[kColsPerThread];
   double wv[kColsPerThread];
@@ -238,6 +239,7 @@ __device__ __forceinline__ int scan_round(G* __restrict__ gacc, const double* __
     const int64_t j = base + q * kThreads + threadIdx.x;
     ga[q] = j < hi ? gacc[j] : G(0);
     wv[q] = j < hi ? w[j] : 0.0;
+    if (second && j < hi) ga[q] += gacc[j + second];
     if (scale && j < hi) ga[q] *= (G)scale[j];
   }
 #pragma unroll
@@ -245,6 +247,7 @@ __device__ __forceinline__ int scan_round(G* __restrict__ gacc, const double* __
     const int64_t j = base + q * kThreads + threadIdx.x;
     if (j >= hi) continue;
     gacc[j] = G(0);
+    if (second) gacc[j + second] = G(0);
     if (!idle_raw(ga[q], wv[q], lnb64, lnb32)) {
       const int slot = atomicAdd(s_n, 1);
       s_j[slot] = j;
@@ -266,7 +269,7 @@ template <typename G>
 __global__ void __launch_bounds__(kThreads)
     k_finalize(G* __restrict__ gacc, const double* __restrict__ w, const double* __restrict__ bjs,
                const double* __restrict__ ib, int64_t k, double inv_n, double lam, uint64_t lnb64, uint32_t lnb32,
-               const float* __restrict__ scale, double* __restrict__ delta, double* __restrict__ phi,
+               int64_t second, const float* __restrict__ scale, double* __restrict__ delta, double* __restrict__ phi,
                double* __restrict__ kkt_out, int write_steps) {
   __shared__ int s_n;
   __shared__ int64_t s_j[kRoundCols];
@@ -275,7 +278,7 @@ __global__ void __launch_bounds__(kThreads)
   for (int64_t base = (int64_t)blockIdx.x * kRoundCols; base < k; base += (int64_t)gridDim.x * kRoundCols) {
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
-    const int na = scan_round(gacc, w, base, k, lnb64, lnb32, scale, &s_n, s_j, s_g, s_w,
+    const int na = scan_round(gacc, w, base, k, lnb64, lnb32, second, scale, &s_n, s_j, s_g, s_w,
                               write_steps ? delta : nullptr, phi);
     for (int e = threadIdx.x; e < na; e += kThreads) {
       const int64_t j = s_j[e];
@@ -320,6 +323,7 @@ struct AcceptCols {
   const double *w, *bj, *ib;
   const float *w32, *bj32, *ib32;
   const float* scale;  // index-only storage: the columns' values (else null)
+  int64_t second;      // offset of the columns' second sums (0: none)
   double inv_n, lam;
   float inv_nf, lamf;  // converted on the host: a conversion runs on the FP64 pipe (16 cycles a warp)
   uint64_t lnb64;
@@ -328,14 +332,15 @@ struct AcceptCols {
 
 // scan_round for FP32 sums and the float copy of w: the queue holds (j, raw sum)
 __device__ __forceinline__ int scan_round_f32(float* __restrict__ gacc, const float* __restrict__ w32,
-                                              const float* __restrict__ scale, int64_t base, int64_t hi,
-                                              uint32_t lnb32, int* s_n, int32_t* s_j, float* s_g) {
+                                              const float* __restrict__ scale, int64_t second, int64_t base,
+                                              int64_t hi, uint32_t lnb32, int* s_n, int32_t* s_j, float* s_g) {
   float ga[kColsPerThread], wv[kColsPerThread];
 #pragma unroll
   for (int q = 0; q < kColsPerThread; ++q) {
     const int64_t j = base + q * kThreads + threadIdx.x;
     ga[q] = j < hi ? gacc[j] : 0.0f;
     wv[q] = j < hi ? w32[j] : 0.0f;
+    if (second && j < hi) ga[q] += gacc[j + second];
     if (scale && j < hi) ga[q] *= scale[j];
   }
 #pragma unroll
@@ -343,6 +348,7 @@ __device__ __forceinline__ int scan_round_f32(float* __restrict__ gacc, const fl
     const int64_t j = base + q * kThreads + threadIdx.x;
     if (j >= hi) continue;
     gacc[j] = 0.0f;
+    if (second) gacc[j + second] = 0.0f;
     const bool idle = (__float_as_uint(wv[q]) << 1) == 0 && (__float_as_uint(ga[q]) & 0x7fffffffu) <= lnb32;
     if (!idle) {
       const int slot = atomicAdd(s_n, 1);
@@ -407,9 +413,9 @@ __global__ void __launch_bounds__(kThreads)
       __syncthreads();
       int na;
       if constexpr (F32)
-        na = scan_round_f32(gacc, c.w32, c.scale, base, hi, c.lnb32, &s_n, s_j, s_g);
+        na = scan_round_f32(gacc, c.w32, c.scale, c.second, base, hi, c.lnb32, &s_n, s_j, s_g);
       else
-        na = scan_round(gacc, c.w, base, hi, c.lnb64, c.lnb32, (const float*)nullptr, &s_n, s_j, s_g, s_w,
+        na = scan_round(gacc, c.w, base, hi, c.lnb64, c.lnb32, (int64_t)0, (const float*)nullptr, &s_n, s_j, s_g, s_w,
                         (double*)nullptr, (double*)nullptr);
       for (int e = threadIdx.x; e < na; e += kThreads) {
         const int64_t j = s_j[e];
@@ -668,10 +674,10 @@ int launch_finalize(gencd_problem* p, double lambda, bool write_steps) {
   prof_begin(p, K_FINALIZE, &ev);
   if (p->precision == GENCD_F64)
     k_finalize<double><<<grid, kThreads, 0, p->stream>>>((double*)p->gnat, p->w, p->bj, p->ib, p->k, inv_n, lambda,
-                                                         b64, b32, p->col_val, p->delta, p->phi, p->dscal + 0, write_steps ? 1 : 0);
+                                                         b64, b32, p->plan.second, p->col_val, p->delta, p->phi, p->dscal + 0, write_steps ? 1 : 0);
   else
     k_finalize<float><<<grid, kThreads, 0, p->stream>>>((float*)p->gnat, p->w, p->bj, p->ib, p->k, inv_n, lambda,
-                                                        b64, b32, p->col_val, p->delta, p->phi, p->dscal + 0, write_steps ? 1 : 0);
+                                                        b64, b32, p->plan.second, p->col_val, p->delta, p->phi, p->dscal + 0, write_steps ? 1 : 0);
   prof_end(p, ev);
   GENCD_CUDA_TRY(cudaGetLastError());
   return GENCD_OK;
@@ -709,7 +715,7 @@ int launch_finalize_accept(gencd_problem* p, int64_t B, bool want_kkt, bool appl
   lambda_bits(p, p->lambda, &b64, &b32);
   const bool f64 = p->precision == GENCD_F64;
   GENCD_TRY(ensure_part_bounds(p, B));
-  const AcceptCols c{p->w, p->bj, p->ib, p->w32, p->bj32, p->ib32, p->col_val, 1.0 / (double)p->n, p->lambda,
+  const AcceptCols c{p->w, p->bj, p->ib, p->w32, p->bj32, p->ib32, p->col_val, p->plan.second, 1.0 / (double)p->n, p->lambda,
                      (float)(1.0 / (double)p->n), (float)p->lambda, b64, b32};
   const int64_t resident = (int64_t)p->num_sms * 8;
   const int64_t most = (p->k + B - 1) / B;  // columns of the largest partition

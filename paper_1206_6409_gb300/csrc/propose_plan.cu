@@ -255,7 +255,7 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
                                           const uint8_t* __restrict__ pmask, const uint32_t* __restrict__ pair_col,
                                           const SlabTiles& T, int t0, const int t_end,
                                           const U* __restrict__ u, int64_t n, int32_t slab_rows,
-                                          G* __restrict__ gacc, U* s_u, const int warp, const int nw,
+                                          G* __restrict__ sums, int64_t second, U* s_u, const int warp, const int nw,
                                           const int gtid, const int gthreads) {
   constexpr uint32_t NOT_FIRST = ((1u << ITEMS) - 1u) & ~1u;  // start bits after a lane's first entry
   const unsigned FULL = 0xffffffffu;
@@ -266,6 +266,7 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
     const int r = T.tile_slab[t0];
     const int tb = T.slab_tile_begin[r], t1 = min(t_end, T.slab_tile_begin[r + 1]);
     const uint32_t base = T.slab_off[r];  // the slab's entries
+    G* __restrict__ gacc = sums + (r & 1 ? second : 0);
     const int64_t row0 = (int64_t)r * slab_rows;
     const int rows = (int)min((int64_t)slab_rows, n - row0);
     TileStage<SV, ITEMS> stg[DEPTH > 0 ? DEPTH : 1];
@@ -380,12 +381,12 @@ template <typename V, typename U, typename G, int THREADS, int DEPTH, int ITEMS,
 __global__ void __launch_bounds__(THREADS, 1)
     k_propose_slabs(const uint16_t* __restrict__ s_row, const SV* __restrict__ s_val,
                     const uint8_t* __restrict__ pmask, const uint32_t* __restrict__ pair_col, SlabTiles T,
-                    const U* __restrict__ u, int64_t n, int32_t slab_rows, G* __restrict__ gacc) {
+                    const U* __restrict__ u, int64_t n, int32_t slab_rows, G* __restrict__ gacc, int64_t second) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   U* s_u = reinterpret_cast<U*>(smem_raw);
   pdl_trigger();
   slab_pass<V, U, G, DEPTH, ITEMS, SV, 0>(s_row, s_val, pmask, pair_col, T, T.cta_tile_begin[blockIdx.x],
-                                          T.cta_tile_begin[blockIdx.x + 1], u, n, slab_rows, gacc, s_u,
+                                          T.cta_tile_begin[blockIdx.x + 1], u, n, slab_rows, gacc, second, s_u,
                                           threadIdx.x >> 5, blockDim.x >> 5, threadIdx.x, blockDim.x);
 }
 
@@ -583,7 +584,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                     const uint8_t* __restrict__ lmask, const int32_t* __restrict__ tile_lc,
                     const int32_t* __restrict__ light_cols, int64_t lnnz,
                     int64_t lntiles, unsigned int* counter, const U* __restrict__ u, int64_t n, int32_t slab_rows,
-                    G* __restrict__ gacc) {
+                    G* __restrict__ gacc, int64_t second) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   U* s_u = reinterpret_cast<U*>(smem_raw);
   pdl_trigger();
@@ -591,7 +592,7 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (warp < SLAB_WARPS)
     slab_pass<V, U, G, DEPTH, ITEMS, SV, 32 * SLAB_WARPS>(
         s_row, s_val, pmask, pair_col, T, T.cta_tile_begin[blockIdx.x], T.cta_tile_begin[blockIdx.x + 1], u, n,
-        slab_rows, gacc, s_u, warp, SLAB_WARPS, threadIdx.x, 32 * SLAB_WARPS);
+        slab_rows, gacc, second, s_u, warp, SLAB_WARPS, threadIdx.x, 32 * SLAB_WARPS);
   else
     pdl_wait();
   light_pool<V, U, G, SV>(lrow, lval, lmask, tile_lc, light_cols, u, lnnz, lntiles, gacc, counter);
@@ -627,7 +628,7 @@ static cudaError_t launch_fused(gencd_problem* p, const void* u_vec, size_t smem
                            p->stream, P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P, P.fused),
                            P.light_row, (const SV*)P.light_val, P.lmask, P.light_tile_lc, P.light_cols,
                            P.light_nnz, P.light_ntiles, P.light_counter, (const U*)u_vec, p->n, P.slab_rows,
-                           (G*)p->gnat);
+                           (G*)p->gnat, P.second);
 }
 
 // both passes in one kernel
@@ -671,7 +672,7 @@ static int launch_plan_passes(gencd_problem* p, const void* u_vec) {
     const cudaError_t err = launch_overlapped(
         k_propose_slabs<V, U, G, THREADS, DEPTH, ITEMS, SV>, P.grid, THREADS, smem, p->stream, P.s_row,
         (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P, P.tiles), (const U*)u_vec, p->n, P.slab_rows,
-        (G*)p->gnat);
+        (G*)p->gnat, P.second);
     prof_end(p, e1);
     GENCD_CUDA_TRY(err);
   }
@@ -1039,6 +1040,12 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   // 1137 / 1044), while the runs (R per column) are no more than the non-zeros,
   // which bounds the scratch of the build.
   constexpr int64_t kFewLight = int64_t(1) << 22;
+  // FP32 sums of many slabs go to two accumulators, odd slabs to the second: a
+  // column's sums are added one after another, and two chains half as long keep
+  // the error of short columns below that of the light pass, which adds in a
+  // tree (columns of 30 over 21 slabs: 7.56e-8 of the norm with two, 8.74e-8 with
+  // one, 7.52e-8 as light columns; Zipf columns in all 6.25e-8, 6.77e-8, 6.52e-8)
+  P.second = !f64 && P.nslabs >= 8 ? k : 0;
   P.heavy_min = 1;
   P.forms = false;
   if (P.nslabs > 1) {
@@ -1296,7 +1303,7 @@ int tune_propose_plan(gencd_problem* p) {
   if (rc != GENCD_OK) return rc;
   // the candidates' sums are scratch: the hot path expects them zero
   const size_t gsz = p->precision == GENCD_F64 ? sizeof(double) : sizeof(float);
-  GENCD_CUDA_TRY(cudaMemsetAsync(p->gnat, 0, gsz * (size_t)p->k, p->stream));
+  GENCD_CUDA_TRY(cudaMemsetAsync(p->gnat, 0, gsz * (size_t)(p->k + P.second), p->stream));
   return GENCD_OK;
 }
 
