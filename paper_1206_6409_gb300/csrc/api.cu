@@ -257,6 +257,8 @@ __global__ void k_block_select(int64_t t, int32_t B, const int64_t* __restrict__
 static int ensure_selection(gencd_problem* p, int64_t epoch, int64_t m, bool* fresh) {
   *fresh = !(p->perm_epoch == epoch && p->perm_m == m);
   if (!*fresh) return GENCD_OK;
+  // block Shotgun's permutations lie in perm too, and do not any more
+  std::fill(p->hblock_epoch.begin(), p->hblock_epoch.end(), int64_t(-1));
   GENCD_TRY(make_permutation(p, p->params.seed, epoch, m, p->perm));
   p->perm_epoch = epoch;
   p->perm_m = m;

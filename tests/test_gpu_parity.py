@@ -656,6 +656,34 @@ def test_block_shotgun_matches_the_oracle(gb, loss):
     np.testing.assert_allclose(w_gpu, w_cpu, rtol=0, atol=1e-10)
 
 
+@pytest.mark.parametrize("between", ["shotgun", "coloring"])
+def test_block_shotgun_redraws_after_another_selection(gb, between):
+    # Shotgun's and Coloring's permutations take the place of the blocks' ones:
+    # within the same epoch and with the same seed, block Shotgun draws its own
+    # again and continues as if the other variant had not run
+    prob = workloads.config1("squared")
+    lam = 0.05 * oracle.Oracle(prob).lambda_max()
+    with gb.Problem(prob) as p:
+        p.set_lambda(lam)
+
+        def blocks(w, t):
+            p.set_params(variant="shotgun_blocks", blocks=7, seed=4)
+            p.set_w(w)
+            p.set_iteration(t)
+            p.iterate(1)
+            return p.w()
+
+        w1 = blocks(np.zeros(prob.k), 0)
+        want = blocks(w1, 1)
+        blocks(np.zeros(prob.k), 0)
+        p.set_params(variant=between, P=100, seed=4)
+        p.iterate(1)
+        got = blocks(w1, 1)
+    assert np.count_nonzero(want != w1) > 0
+    np.testing.assert_array_equal(got != w1, want != w1)
+    np.testing.assert_allclose(got, want, rtol=0, atol=1e-10)  # FP64 sums in another order
+
+
 def test_block_shotgun_solve_reaches_the_optimum(gb):
     prob = workloads.uniform_problem(1000, 2000, 10, values="pm1", loss="logistic", n_planted=30, seed=21)
     orc = oracle.Oracle(prob)
