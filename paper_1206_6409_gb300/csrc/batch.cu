@@ -196,8 +196,7 @@ __global__ void k_b_absmax(const float* __restrict__ G0, int64_t k, int nsets, u
 // the step
 
 // zero the G rows added atomically by k_b_spmm, and the per-slot KKT maxima
-__global__ void k_b_prep(const int32_t* __restrict__ bnd, int64_t nb, int Sp, float* __restrict__ G,
-                         unsigned int* __restrict__ kkt_bits) {
+__global__ void k_b_prep(const int32_t* __restrict__ bnd, int64_t nb, int Sp, float* G, unsigned int* kkt_bits) {
   pdl_trigger();
   pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -211,7 +210,7 @@ __global__ void k_b_prep(const int32_t* __restrict__ bnd, int64_t nb, int Sp, fl
 }
 
 template <int NC>
-__device__ __forceinline__ void b_flush(float* __restrict__ G, const int32_t* __restrict__ nzcols, int32_t cc,
+__device__ __forceinline__ void b_flush(float* G, const int32_t* __restrict__ nzcols, int32_t cc,
                                         const float (&acc)[NC], bool atomic, int lane) {
   float* g = G + (int64_t)__ldg(nzcols + cc) * (32 * NC) + lane;
 #pragma unroll
@@ -230,8 +229,8 @@ __device__ __forceinline__ void b_flush(float* __restrict__ G, const int32_t* __
 template <int NC, int GRP>
 __global__ void __launch_bounds__(kSpmmThreads)
     k_b_spmm(const int32_t* __restrict__ row, const float* __restrict__ val, const uint32_t* __restrict__ tstart,
-             const int32_t* __restrict__ tile_cc, const int32_t* __restrict__ nzcols, const float* __restrict__ U,
-             float* __restrict__ G, int64_t ntiles, int64_t W) {
+             const int32_t* __restrict__ tile_cc, const int32_t* __restrict__ nzcols, const float* U, float* G,
+             int64_t ntiles, int64_t W) {
   constexpr int Sp = 32 * NC;
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
@@ -270,7 +269,7 @@ __global__ void __launch_bounds__(kSpmmThreads)
 #pragma unroll
       for (int q = 0; q < GRP; ++q)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) uu[q][c] = __ldg(U + (int64_t)r[q] * Sp + 32 * c + lane);
+        for (int c = 0; c < NC; ++c) uu[q][c] = U[(int64_t)r[q] * Sp + 32 * c + lane];
 #pragma unroll
       for (int q = 0; q < GRP; ++q) {
         if ((m >> (g + q)) & 1u) {  // warp-uniform: entry g + q starts the next column
@@ -304,11 +303,10 @@ struct SlotArgs {
 // KKT only.
 template <int MODE>
 __global__ void __launch_bounds__(kAcceptThreads)
-    k_b_accept(const float* __restrict__ G, const float* __restrict__ w32, const double* __restrict__ w,
+    k_b_accept(const float* G, const float* w32, const double* w,
                const float* __restrict__ bj32, const float* __restrict__ ib32, const double* __restrict__ bjs,
                const double* __restrict__ ibs, int64_t k, SlotArgs sa, const int64_t* __restrict__ part_lo, int Sp,
-               int R, int32_t* __restrict__ acc_j, double* __restrict__ acc_d, double* __restrict__ acc_phi,
-               unsigned int* __restrict__ kkt_bits) {
+               int R, int32_t* acc_j, double* acc_d, double* acc_phi, unsigned int* kkt_bits) {
   __shared__ uint32_t s_mag[kAcceptThreads];
   __shared__ int32_t s_col[kAcceptThreads];
   __shared__ float s_v[kAcceptThreads];
@@ -328,8 +326,8 @@ __global__ void __launch_bounds__(kAcceptThreads)
     const float* ibv = ib32 + (int64_t)set * k;
 #pragma unroll 4
     for (int64_t j = lo + r; j < hi; j += R) {
-      const float g = __ldg(G + j * Sp + s) * invn;
-      const float wj = __ldg(w32 + j * Sp + s);
+      const float g = G[j * Sp + s] * invn;
+      const float wj = w32[j * Sp + s];
       float d, phi;
       eq7_step_f32(g, wj, lam, __ldg(bjv + j), __ldg(ibv + j), d, phi);
       const uint32_t m = candidate_mag32(phi);
@@ -395,7 +393,7 @@ __global__ void __launch_bounds__(kAcceptThreads)
 // Accept backoff: a slot whose group size G > 1 keeps, of every G
 // consecutive partitions, only the one whose accepted proxy is lowest (ties:
 // the lower partition).  G = B is Greedy.
-__global__ void k_b_merge(int32_t* __restrict__ acc_j, const double* __restrict__ acc_phi, int B, int Sp,
+__global__ void k_b_merge(int32_t* acc_j, const double* acc_phi, int B, int Sp,
                           const int32_t* __restrict__ group) {
   pdl_trigger();
   pdl_wait();
@@ -419,10 +417,9 @@ __global__ void k_b_merge(int32_t* __restrict__ acc_j, const double* __restrict_
 }
 
 // w += delta and z_s += delta X_j for every accepted (partition, slot)
-__global__ void k_b_update(const int32_t* __restrict__ acc_j, const double* __restrict__ acc_d, int npairs, int Sp,
+__global__ void k_b_update(const int32_t* acc_j, const double* acc_d, int npairs, int Sp,
                            const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row,
-                           const float* __restrict__ val, double* __restrict__ w, float* __restrict__ w32,
-                           double* __restrict__ z, unsigned long long* __restrict__ ctr) {
+                           const float* __restrict__ val, double* w, float* w32, double* z, unsigned long long* ctr) {
   pdl_trigger();
   pdl_wait();
   const int lane = threadIdx.x & 31;
@@ -454,10 +451,10 @@ __global__ void k_b_update(const int32_t* __restrict__ acc_j, const double* __re
 // accepted by fewer slots is walked by the lanes, one slot after another.
 constexpr int kGroupMin = 4;
 
-__global__ void k_b_update_grouped(const int32_t* __restrict__ acc_j, const double* __restrict__ acc_d, int B,
-                                   int Sp, const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row,
-                                   const float* __restrict__ val, double* __restrict__ w, float* __restrict__ w32,
-                                   double* __restrict__ z, unsigned long long* __restrict__ ctr) {
+__global__ void k_b_update_grouped(const int32_t* acc_j, const double* acc_d, int B, int Sp,
+                                   const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row,
+                                   const float* __restrict__ val, double* w, float* w32, double* z,
+                                   unsigned long long* ctr) {
   pdl_trigger();
   pdl_wait();
   const unsigned FULL = 0xffffffffu;
@@ -519,10 +516,10 @@ __device__ __forceinline__ bool b_train(const uint8_t* __restrict__ fold, int64_
 }
 
 // u_s on the rows of every accepted (partition, slot)'s column
-__global__ void k_b_refresh(const int32_t* __restrict__ acc_j, int npairs, int Sp, const int64_t* __restrict__ col_ptr,
+__global__ void k_b_refresh(const int32_t* acc_j, int npairs, int Sp, const int64_t* __restrict__ col_ptr,
                             const int32_t* __restrict__ row, const double* __restrict__ y,
                             const uint8_t* __restrict__ fold, int nfolds, int loss, const int32_t* __restrict__ sset,
-                            const double* __restrict__ z, float* __restrict__ U) {
+                            const double* z, float* U) {
   pdl_trigger();
   pdl_wait();
   const int lane = threadIdx.x & 31;
@@ -544,8 +541,7 @@ __global__ void k_b_refresh(const int32_t* __restrict__ acc_j, int npairs, int S
 // dense form of k_b_refresh, cheaper when the accepted columns touch more
 // (row, slot) entries than there are rows times slots
 __global__ void k_b_refresh_all(const double* __restrict__ y, const uint8_t* __restrict__ fold, int nfolds, int loss,
-                                const int32_t* __restrict__ sset, const double* __restrict__ z, int64_t n, int Sp,
-                                float* __restrict__ U) {
+                                const int32_t* __restrict__ sset, const double* z, int64_t n, int Sp, float* U) {
   pdl_trigger();
   pdl_wait();
   const int s = threadIdx.x;
@@ -567,18 +563,18 @@ __global__ void k_b_refresh_all(const double* __restrict__ y, const uint8_t* __r
 // leaving to the right (tail) is combined across the warp by a segmented
 // suffix sum, so only a tile's first and last column are added atomically.
 // G must be zero before the launch.
-__device__ __forceinline__ void b_row8(const float* __restrict__ p, float (&u)[8]) {
-  const float4 a = __ldg(reinterpret_cast<const float4*>(p));
-  const float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+__device__ __forceinline__ void b_row8(const float* p, float (&u)[8]) {
+  const float4 a = reinterpret_cast<const float4*>(p)[0];
+  const float4 b = reinterpret_cast<const float4*>(p)[1];
   u[0] = a.x, u[1] = a.y, u[2] = a.z, u[3] = a.w, u[4] = b.x, u[5] = b.y, u[6] = b.z, u[7] = b.w;
 }
 
-__device__ __forceinline__ void b_store8(float* __restrict__ p, const float (&v)[8]) {
+__device__ __forceinline__ void b_store8(float* p, const float (&v)[8]) {
   reinterpret_cast<float4*>(p)[0] = make_float4(v[0], v[1], v[2], v[3]);
   reinterpret_cast<float4*>(p)[1] = make_float4(v[4], v[5], v[6], v[7]);
 }
 
-__device__ __forceinline__ void b_add8(float* __restrict__ p, const float (&v)[8]) {
+__device__ __forceinline__ void b_add8(float* p, const float (&v)[8]) {
 #pragma unroll
   for (int q = 0; q < 8; ++q) atomicAdd(p + q, v[q]);
 }
@@ -586,13 +582,13 @@ __device__ __forceinline__ void b_add8(float* __restrict__ p, const float (&v)[8
 __global__ void __launch_bounds__(kThreads, 2)
     k_b_spmm_runs8(const int32_t* __restrict__ row, const float* __restrict__ val, const uint8_t* __restrict__ smask,
                    const int32_t* __restrict__ tile_cc, const int32_t* __restrict__ nzcols,
-                   const float* __restrict__ U, int S, float* __restrict__ G, int64_t nnz, int64_t ntiles) {
+                   const float* U, int S, float* G, int64_t nnz, int64_t ntiles) {
   pdl_trigger();
   pdl_wait();
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  const float* __restrict__ Uc = U + 8 * blockIdx.y;
-  float* __restrict__ Gc = G + 8 * blockIdx.y;
+  const float* Uc = U + 8 * blockIdx.y;
+  float* Gc = G + 8 * blockIdx.y;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t t = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < ntiles; t += nwarps) {
     const int64_t a = t * 256 + (int64_t)lane * 8;

@@ -381,15 +381,53 @@ void prof_end(gencd_problem* p, cudaEvent_t stop);
 //  - calls pdl_trigger() at its start: the next kernel's launch latency and its
 //    reads before its own pdl_wait() then overlap this kernel.  The first kernel
 //    after a new permutation waits before that, so that no later one starts
-//    before the permutation is visible.
+//    before the permutation is visible;
+//  - takes what kernels launched this way write (z, u, w, w32, the sums, lists
+//    and slots; a batch's U, G, w, z and acc arrays) through pointers without
+//    __restrict__, and reads it after the wait by plain loads or load_l2().  Such
+//    memory changes while the kernel is resident: the read-only path (__ldg, or
+//    the loads the compiler makes of const __restrict__) is defined for memory
+//    that does not change, and neither its loads nor those of a restrict pointer
+//    are ordered by the wait's memory clobber.
 // The gap between two dependent kernels of an iteration, 1.6 us launched
 // plainly, goes with it: Greedy on 800 x 100,000 took 687 us for 20 iterations
 // of five launches and takes 537.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-//
-// launch_cluster_overlapped: the same with the grid as one cluster of CTAs.
+// A load from L2, where other SMs' writes are, in program order with the waits
+// and barriers around it (__ldcg is not: it may be taken for a function of its
+// address alone).
+__device__ __forceinline__ float load_l2(const float* p) {
+  float v;
+  asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ double load_l2(const double* p) {
+  double v;
+  asm volatile("ld.global.cg.f64 %0, [%1];" : "=d"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ int32_t load_l2(const int32_t* p) {
+  int32_t v;
+  asm volatile("ld.global.cg.s32 %0, [%1];" : "=r"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ uint64_t load_l2(const uint64_t* p) {
+  uint64_t v;
+  asm volatile("ld.global.cg.u64 %0, [%1];" : "=l"(v) : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+__device__ __forceinline__ uint4 load_l2(const uint4* p) {
+  uint4 v;
+  asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "l"(__cvta_generic_to_global(p)));
+  return v;
+}
+
+// launch_cluster_overlapped: such a launch with the whole grid, `cluster` CTAs,
+// as one cluster (cluster = 1: no cluster).
 template <typename... P, typename... A>
 inline cudaError_t launch_cluster_overlapped(void (*kernel)(P...), unsigned cluster, dim3 grid, dim3 block, size_t smem,
                                              cudaStream_t stream, A... args) {

@@ -228,7 +228,7 @@ constexpr int kRoundCols = kColsPerThread * kThreads;  // columns a CTA scans pe
 // one.  second: offset of a column's second sum (0: none).  scale (index-only
 // storage): each column's value, applied to its sum.  Returns the queue length; the queue holds (j, raw sum, w_j).
 template <typename G>
-__device__ __forceinline__ int scan_round(G* __restrict__ gacc, const double* __restrict__ w, int64_t base,
+__device__ __forceinline__ int scan_round(G* gacc, const double* w, int64_t base,
                                           int64_t hi, uint64_t lnb64, uint32_t lnb32, int64_t second,
                                           const float* __restrict__ scale, int* s_n, int64_t* s_j, double* s_g, double* s_w, double* delta,
                                           double* phi) {
@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(kThreads)
 // FP64 step and proxy of the ranked winner (raw sum ga): the accepted delta,
 // or no acceptance (false) when that proxy is not negative
 __device__ __forceinline__ bool accept_fp64(double ga, int32_t j, double inv_n, double lam,
-                                            const double* __restrict__ w, const double* __restrict__ bjs,
+                                            const double* w, const double* __restrict__ bjs,
                                             const double* __restrict__ ib, double& d) {
   double f;
   eq7_step(ga * inv_n, w[j], lam, bjs[j], ib[j], d, f);
@@ -331,7 +331,7 @@ struct AcceptCols {
 };
 
 // scan_round for FP32 sums and the float copy of w: the queue holds (j, raw sum)
-__device__ __forceinline__ int scan_round_f32(float* __restrict__ gacc, const float* __restrict__ w32,
+__device__ __forceinline__ int scan_round_f32(float* gacc, const float* w32,
                                               const float* __restrict__ scale, int64_t second, int64_t base,
                                               int64_t hi, uint32_t lnb32, int* s_n, int32_t* s_j, float* s_g) {
   float ga[kColsPerThread], wv[kColsPerThread];
@@ -382,12 +382,11 @@ __device__ __forceinline__ int scan_round_f32(float* __restrict__ gacc, const fl
 // beta_j (89 us on k = 4,000,000).
 template <typename G>
 __global__ void __launch_bounds__(kThreads)
-    k_accept_partitions(G* __restrict__ gacc, AcceptCols c, int64_t B, int per, int64_t chunk,
-                        const int64_t* __restrict__ part_lo, int want_kkt, uint64_t* __restrict__ slot_m,
-                        int32_t* __restrict__ slot_j, double* __restrict__ slot_x, unsigned int* __restrict__ slot_cnt,
-                        int32_t* __restrict__ list_j, double* __restrict__ list_d, uint64_t* __restrict__ list_m,
-                        double* __restrict__ kkt_out, const int64_t* __restrict__ col_ptr, double* w_out,
-                        float* w32_out, uint32_t* __restrict__ list_len) {
+    k_accept_partitions(G* gacc, AcceptCols c, int64_t B, int per, int64_t chunk,
+                        const int64_t* __restrict__ part_lo, int want_kkt, uint64_t* slot_m, int32_t* slot_j,
+                        double* slot_x, unsigned int* slot_cnt, int32_t* list_j, double* list_d, uint64_t* list_m,
+                        double* kkt_out, const int64_t* __restrict__ col_ptr, double* w_out, float* w32_out,
+                        uint32_t* list_len) {
   constexpr bool F32 = sizeof(G) == 4;
   using J = typename std::conditional<F32, int32_t, int64_t>::type;
   __shared__ int s_n;  // the active columns of a round, processed packed
@@ -466,12 +465,12 @@ __global__ void __launch_bounds__(kThreads)
         bj = INT32_MAX;
         bx = G(0);
         for (int64_t q = b * per + threadIdx.x; q < (b + 1) * per; q += kThreads) {
-          const uint64_t m = __ldcg(slot_m + q);
-          const int32_t j = __ldcg(slot_j + q);
+          const uint64_t m = load_l2(slot_m + q);
+          const int32_t j = load_l2(slot_j + q);
           if (cand_better(m, j, bm, bj)) {
             bm = m;
             bj = j;
-            bx = (G)__ldcg(slot_x + q);
+            bx = (G)load_l2(slot_x + q);
           }
         }
         block_best(bm, bj, bx);

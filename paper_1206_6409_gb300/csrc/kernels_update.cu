@@ -98,7 +98,7 @@ constexpr int kListThreads = 512;
 // dependent loads in memory they took 4.4 and 6.6.  counters (not null): CTA 0 adds the updates and
 // the non-zeros to them.  Not SCAN: the offsets are in memory already.
 template <bool SCAN>
-__device__ __forceinline__ const uint32_t* list_offsets(const uint32_t* __restrict__ list, int64_t m,
+__device__ __forceinline__ const uint32_t* list_offsets(const uint32_t* list, int64_t m,
                                                         uint32_t* s_off, unsigned long long* counters) {
   if (!SCAN) return list;
   __shared__ uint32_t s_warp[kListThreads / 32];
@@ -152,9 +152,8 @@ __device__ __forceinline__ const uint32_t* list_offsets(const uint32_t* __restri
 template <typename V, bool SCAN>
 __global__ void __launch_bounds__(kListThreads)
     k_update_flat(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
-                  const V* __restrict__ val, const int32_t* __restrict__ J, const double* __restrict__ D,
-                  const uint32_t* __restrict__ list, int64_t m, double* __restrict__ z,
-                  unsigned long long* __restrict__ counters) {
+                  const V* __restrict__ val, const int32_t* J, const double* D, const uint32_t* list, int64_t m,
+                  double* z, unsigned long long* counters) {
   __shared__ uint32_t s_off[SCAN ? kListScanMax + 1 : 1];
   pdl_trigger();
   pdl_wait();
@@ -162,12 +161,17 @@ __global__ void __launch_bounds__(kListThreads)
   const int64_t total = off[m], threads = (int64_t)gridDim.x * kListThreads;
   const int run = total > threads ? 4 : 1;
   for (int64_t q0 = ((int64_t)blockIdx.x * kListThreads + threadIdx.x) * run; q0 < total; q0 += threads * run) {
-    int64_t e = entry_of(off, m, (uint32_t)q0);
+    int64_t e = entry_of(off, m, (uint32_t)q0), end = off[e + 1], at = col_ptr[J[e]] - off[e];
+    double d = D[e];
 #pragma unroll 1
     for (int64_t q = q0; q < q0 + run && q < total; ++q) {
-      while (q >= off[e + 1]) ++e;
-      const int64_t p = col_ptr[J[e]] + ((uint32_t)q - off[e]);
-      atomicAdd(z + row_idx[p], D[e] * (double)val[p]);
+      if (q >= end) {  // the next applied column
+        do end = off[++e + 1];
+        while (q >= end);
+        at = col_ptr[J[e]] - off[e];
+        d = D[e];
+      }
+      atomicAdd(z + row_idx[at + q], d * (double)val[at + q]);
     }
   }
 }
@@ -181,9 +185,8 @@ __global__ void __launch_bounds__(kListThreads)
 template <typename U, bool SCAN>
 __global__ void __launch_bounds__(kListThreads)
     k_refresh_flat(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
-                   const int32_t* __restrict__ J, const uint32_t* __restrict__ list, int64_t m,
-                   const double* __restrict__ y, const double* __restrict__ z, int64_t n, int loss,
-                   const double* __restrict__ tab, U* __restrict__ u, unsigned long long* __restrict__ counters) {
+                   const int32_t* J, const uint32_t* list, int64_t m, const double* __restrict__ y, const double* z,
+                   int64_t n, int loss, const double* __restrict__ tab, U* u, unsigned long long* counters) {
   __shared__ uint32_t s_off[SCAN ? kListScanMax + 1 : 1];
   pdl_trigger();
   pdl_wait();
@@ -210,10 +213,9 @@ constexpr int kClusterCtas = 8;
 template <typename V, typename U>
 __global__ void __launch_bounds__(kListThreads)
     k_update_refresh(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
-                     const V* __restrict__ val, const int32_t* __restrict__ J, const double* __restrict__ D,
-                     const uint32_t* __restrict__ list, int64_t m, const double* __restrict__ y, double* z, int64_t n,
-                     int loss, const double* __restrict__ tab, U* __restrict__ u,
-                     unsigned long long* __restrict__ counters) {
+                     const V* __restrict__ val, const int32_t* J, const double* D, const uint32_t* list, int64_t m,
+                     const double* __restrict__ y, double* z, int64_t n, int loss, const double* __restrict__ tab,
+                     U* u, unsigned long long* counters) {
   __shared__ uint32_t s_off[kListScanMax + 1];
   pdl_trigger();
   pdl_wait();
@@ -228,13 +230,13 @@ __global__ void __launch_bounds__(kListThreads)
   }
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
   if (total >= n) {
-    for (int64_t i = q0; i < n; i += threads) u[i] = u_value<U>(loss, y[i], __ldcg(z + i), tab);
+    for (int64_t i = q0; i < n; i += threads) u[i] = u_value<U>(loss, y[i], load_l2(z + i), tab);
     return;
   }
   for (int64_t q = q0; q < total; q += threads) {
     const int64_t e = entry_of(off, m, (uint32_t)q);
     const int32_t i = row_idx[col_ptr[J[e]] + ((uint32_t)q - off[e])];
-    u[i] = u_value<U>(loss, y[i], __ldcg(z + i), tab);
+    u[i] = u_value<U>(loss, y[i], load_l2(z + i), tab);
   }
 }
 
@@ -255,10 +257,9 @@ constexpr int kShotgunCols = kThreads / 32;
 template <typename V, typename U>
 __global__ void __launch_bounds__(kThreads)
     k_shotgun_step(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
-                   const V* __restrict__ val, const U* __restrict__ u, const double* __restrict__ bjs,
-                   const double* __restrict__ ib, const int32_t* __restrict__ J, int64_t m, int per, int early,
-                   double n, double lam, double* __restrict__ w, float* __restrict__ w32, double* __restrict__ z,
-                   uint32_t* __restrict__ list, unsigned long long* __restrict__ counters) {
+                   const V* __restrict__ val, const U* u, const double* __restrict__ bjs,
+                   const double* __restrict__ ib, const int32_t* J, int64_t m, int per, int early, double n, double lam,
+                   double* w, float* w32, double* z, uint32_t* list, unsigned long long* counters) {
   __shared__ int64_t s_long[kShotgunCols];
   __shared__ int s_nlong;
   __shared__ uint32_t s_len[kShotgunCols];
@@ -356,13 +357,11 @@ __global__ void __launch_bounds__(kThreads)
 template <typename V, typename U>
 __global__ void __launch_bounds__(kThreads)
     k_coloring_iter(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
-                    const V* __restrict__ val, U* __restrict__ u, double* __restrict__ w,
-                    float* __restrict__ w32, const double* __restrict__ bjs, const double* __restrict__ ib,
-                    double* __restrict__ z,
-                    const double* __restrict__ y, const int32_t* __restrict__ perm, int64_t q,
-                    const int32_t* __restrict__ color_ptr, const int32_t* __restrict__ cols_by_color,
+                    const V* __restrict__ val, U* u, double* w, float* w32, const double* __restrict__ bjs,
+                    const double* __restrict__ ib, double* z, const double* __restrict__ y, const int32_t* perm,
+                    int64_t q, const int32_t* __restrict__ color_ptr, const int32_t* __restrict__ cols_by_color,
                     double n, double lam, int loss, const double* __restrict__ tab, int early,
-                    unsigned long long* __restrict__ counters) {
+                    unsigned long long* counters) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;

@@ -76,7 +76,7 @@ __device__ __forceinline__ void load_vals(const V* __restrict__ p, V (&v)[N], in
 }
 
 template <typename G>
-__device__ __forceinline__ void emit_pair(G* __restrict__ out, uint32_t slot, G s, bool whole) {
+__device__ __forceinline__ void emit_pair(G* out, uint32_t slot, G s, bool whole) {
   if (whole)
     out[slot] = s;
   else
@@ -93,7 +93,7 @@ struct NoVal {};
 // column, so always atomically (index-only storage: the sum of u over the
 // column's rows; who reads g_j applies the column's value)
 template <typename G>
-__device__ __forceinline__ void add_col(G* __restrict__ gacc, uint32_t j, G v) {
+__device__ __forceinline__ void add_col(G* gacc, uint32_t j, G v) {
   atomicAdd(gacc + j, v);
 }
 
@@ -254,8 +254,8 @@ template <typename V, typename U, typename G, int DEPTH, int ITEMS, typename SV,
 __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, const SV* __restrict__ s_val,
                                           const uint8_t* __restrict__ pmask, const uint32_t* __restrict__ pair_col,
                                           const SlabTiles& T, int t0, const int t_end,
-                                          const U* __restrict__ u, int64_t n, int32_t slab_rows,
-                                          G* __restrict__ sums, int64_t second, U* s_u, const int warp, const int nw,
+                                          const U* u, int64_t n, int32_t slab_rows,
+                                          G* sums, int64_t second, U* s_u, const int warp, const int nw,
                                           const int gtid, const int gthreads) {
   constexpr uint32_t NOT_FIRST = ((1u << ITEMS) - 1u) & ~1u;  // start bits after a lane's first entry
   const unsigned FULL = 0xffffffffu;
@@ -266,7 +266,7 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
     const int r = T.tile_slab[t0];
     const int tb = T.slab_tile_begin[r], t1 = min(t_end, T.slab_tile_begin[r + 1]);
     const uint32_t base = T.slab_off[r];  // the slab's entries
-    G* __restrict__ gacc = sums + (r & 1 ? second : 0);
+    G* gacc = sums + (r & 1 ? second : 0);
     const int64_t row0 = (int64_t)r * slab_rows;
     const int rows = (int)min((int64_t)slab_rows, n - row0);
     TileStage<SV, ITEMS> stg[DEPTH > 0 ? DEPTH : 1];
@@ -284,9 +284,16 @@ __device__ __forceinline__ void slab_pass(const uint16_t* __restrict__ s_row, co
       const int nvec = al ? (int)(((int64_t)rows * (int64_t)sizeof(U)) / 16) : 0;
       const uint4* src = reinterpret_cast<const uint4*>(u + row0);
       uint4* dst = reinterpret_cast<uint4*>(s_u);
-#pragma unroll 4
-      for (int i = gtid; i < nvec; i += gthreads) dst[i] = __ldcg(src + i);
-      for (int i = (int)((int64_t)nvec * 16 / (int64_t)sizeof(U)) + gtid; i < rows; i += gthreads) s_u[i] = u[row0 + i];
+      int i0 = gtid;
+      for (; i0 + 3 * gthreads < nvec; i0 += 4 * gthreads) {
+        uint4 x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) x[q] = load_l2(src + i0 + q * gthreads);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dst[i0 + q * gthreads] = x[q];
+      }
+      for (; i0 < nvec; i0 += gthreads) dst[i0] = load_l2(src + i0);
+      for (int i = (int)((int64_t)nvec * 16 / (int64_t)sizeof(U)) + gtid; i < rows; i += gthreads) s_u[i] = load_l2(u + row0 + i);
     }
     slab_barrier<BAR_THREADS>();
     for (; t < t1; t += nw) {  // warp-uniform loop
@@ -381,7 +388,7 @@ template <typename V, typename U, typename G, int THREADS, int DEPTH, int ITEMS,
 __global__ void __launch_bounds__(THREADS, 1)
     k_propose_slabs(const uint16_t* __restrict__ s_row, const SV* __restrict__ s_val,
                     const uint8_t* __restrict__ pmask, const uint32_t* __restrict__ pair_col, SlabTiles T,
-                    const U* __restrict__ u, int64_t n, int32_t slab_rows, G* __restrict__ gacc, int64_t second) {
+                    const U* u, int64_t n, int32_t slab_rows, G* gacc, int64_t second) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   U* s_u = reinterpret_cast<U*>(smem_raw);
   pdl_trigger();
@@ -436,7 +443,7 @@ __device__ __forceinline__ void load_light_stage(const int32_t* __restrict__ row
 template <typename V, typename U, typename G, typename SV>
 __device__ __forceinline__ void light_tile(const LightStage<SV>& cur, int64_t t, int64_t nnz,
                                            const int32_t* __restrict__ light_cols,
-                                           const U* __restrict__ u, G* __restrict__ out, int lane) {
+                                           const U* u, G* out, int lane) {
   const unsigned FULL = 0xffffffffu;
   const int64_t a = t * kLightTile + (int64_t)lane * kLightItems;
   const bool active = a < nnz;
@@ -461,7 +468,7 @@ __device__ __forceinline__ void light_tile(const LightStage<SV>& cur, int64_t t,
     U uu[8];
 #pragma unroll
     // gathers of u through L2 without allocating in L1 (no reuse to keep)
-    for (int i = 0; i < 8; ++i) uu[i] = __ldcg(u + r[i]);  // padding rows are 0, values 0
+    for (int i = 0; i < 8; ++i) uu[i] = load_l2(u + r[i]);  // padding rows are 0, values 0
     // first run, last run and the whole columns between (see k_propose_slabs)
     const uint32_t inner = m & 0xfeu;
     const int bf = inner ? __ffs(inner) - 1 : 8;
@@ -514,7 +521,7 @@ template <typename V, typename U, typename G, typename SV>
 __global__ void __launch_bounds__(kThreads, 3)
     k_propose_light_runs(const int32_t* __restrict__ row, const SV* __restrict__ val,
                          const uint8_t* __restrict__ lmask, const int32_t* __restrict__ tile_lc,
-                         const int32_t* __restrict__ light_cols, const U* __restrict__ u, int64_t nnz, int64_t ntiles, G* __restrict__ out) {
+                         const int32_t* __restrict__ light_cols, const U* u, int64_t nnz, int64_t ntiles, G* out) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -543,9 +550,8 @@ constexpr int kLightChunk = 4;
 template <typename V, typename U, typename G, typename SV>
 __device__ __forceinline__ void light_pool(const int32_t* __restrict__ row, const SV* __restrict__ val,
                                            const uint8_t* __restrict__ lmask, const int32_t* __restrict__ tile_lc,
-                                           const int32_t* __restrict__ light_cols,
-                                           const U* __restrict__ u, int64_t nnz,
-                                           int64_t ntiles, G* __restrict__ out, unsigned int* counter) {
+                                           const int32_t* __restrict__ light_cols, const U* u, int64_t nnz,
+                                           int64_t ntiles, G* out, unsigned int* counter) {
   const int lane = threadIdx.x & 31;
   auto grab = [&](int64_t& t, int64_t& t_end) {
     unsigned int b = 0;
@@ -583,8 +589,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                     const int32_t* __restrict__ lrow, const SV* __restrict__ lval,
                     const uint8_t* __restrict__ lmask, const int32_t* __restrict__ tile_lc,
                     const int32_t* __restrict__ light_cols, int64_t lnnz,
-                    int64_t lntiles, unsigned int* counter, const U* __restrict__ u, int64_t n, int32_t slab_rows,
-                    G* __restrict__ gacc, int64_t second) {
+                    int64_t lntiles, unsigned int* counter, const U* u, int64_t n, int32_t slab_rows, G* gacc,
+                    int64_t second) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   U* s_u = reinterpret_cast<U*>(smem_raw);
   pdl_trigger();
