@@ -216,7 +216,11 @@ int gencd_set_iteration(gencd_problem* p, int64_t t);
 int gencd_get_iteration(gencd_problem* p, int64_t* t);
 
 /* Copies w (double[k]) out to, or in from, a caller buffer.  gencd_set_w
- * recomputes z = Xw (from a row-major copy of X built on first use) and u. */
+ * recomputes z = Xw and u.  Up to 2^20 non-zeros, and for a w whose columns hold
+ * more than 2/5 of them, z is summed row by row in a fixed order (from a
+ * row-major copy of X built on first use).  Otherwise the columns with w_j != 0
+ * are added into z with FP64 atomics: two calls with the same w may then differ
+ * in the last bits of z, u and what follows from them. */
 int gencd_get_w(gencd_problem* p, double* w, int64_t k, int32_t memory);
 int gencd_set_w(gencd_problem* p, const double* w, int64_t k, int32_t memory);
 /* Copies z = Xw (double[n], maintained incrementally by Algorithm 3). */

@@ -652,11 +652,11 @@ static int create_impl(gencd_problem* p, const int64_t* col_ptr, const int32_t* 
   if (p->precision != GENCD_F64) a.add(&gf, 2 * k);  // two sums a column (ProposePlan::second)
   a.add(&p->delta, k);
   a.add(&p->phi, k);
-  a.add(&p->list_j, k);
+  a.add(&p->list_j, list_cap(k, nnz));
   a.add(&p->list_d, k);
   a.add(&p->list_m, k);
   a.add(&p->perm, k);
-  a.add(&p->list_off, k + 2);
+  a.add(&p->list_off, list_cap(k, nnz) + 2);
   a.add(&p->scan_tmp, scan_tmp_words(k + 2));
   a.add(&p->dscal, kScalars);
   a.add(&p->red, 3 * kRedBlocks);

@@ -61,6 +61,10 @@ constexpr uint32_t kApplied = 0x80000000u;  // list_off entry, before its prefix
 constexpr int32_t kMaxShotgunBlocks = 1024;  // column blocks of block Shotgun (one selection CTA)
 constexpr int kScalars = 16;  // device scalars of a problem (dscal / hpin)
 constexpr int kScalFit = 10;  // the first of the two that z = Xw uses
+// z = Xw from the columns of a sparse w: entries a segment, and the size of
+// problem from which the columns are taken at all (launch_state_from_w)
+constexpr int kSegEntries = 512;
+constexpr int64_t kFitRowsNnz = int64_t(1) << 20;
 
 // kernel ids for launch counting / profiling
 enum KernelId {
@@ -203,14 +207,15 @@ struct gencd_problem {
   double* delta = nullptr;
   double* phi = nullptr;
 
-  // accepted / selected lists (capacity k)
+  // accepted / selected lists (capacity k; list_j and list_off also hold the
+  // segments of z = Xw, list_cap() entries)
   int32_t* list_j = nullptr;
   uint64_t* list_m = nullptr;   // candidate magnitude of each partition's accepted column (accept backoff)
   uint32_t* top_buf = nullptr;  // global top-|J'| Accept: sort keys and indices (6 k words)
   double* w_start = nullptr;    // w at the start of a solve (restarts of the accept backoff)
   int64_t accept_group = 1;     // Thread-Greedy partitions merged per accept group (1: none)
   double* list_d = nullptr;
-  uint32_t* list_off = nullptr;  // the listed columns' nnz | kApplied, or their exclusive prefix (k + 2)
+  uint32_t* list_off = nullptr;  // the listed columns' nnz | kApplied, or their exclusive prefix (k + 1)
   uint32_t* scan_tmp = nullptr;  // scratch of the prefix sum
 
   // Thread-Greedy partition bounds floor(b k / B), b = 0..part_B
@@ -326,6 +331,8 @@ int launch_refresh_list(gencd_problem* p, const int32_t* J, int64_t m, bool coun
 int launch_shotgun_step(gencd_problem* p, const int32_t* J, int64_t m, bool early);      // propose, w and z
 int launch_coloring_iter(gencd_problem* p, int64_t q, bool early);
 int launch_csr_spmv(gencd_problem* p, const double* x, double* out);  // out = X x (FP64)
+// entries of list_j and list_off: a column of len non-zeros has ceil(len / kSegEntries) segments
+inline int64_t list_cap(int64_t k, int64_t nnz) { return k + (nnz > kFitRowsNnz ? nnz / kSegEntries : 0); }
 int launch_state_from_w(gencd_problem* p);  // z, u and w32 from p->w (synchronises the stream)
 
 // kernels_setup.cu

@@ -444,13 +444,11 @@ __global__ void k_mirror_w(const double* __restrict__ w, int64_t k, float* __res
 // non-zeros so that a long column is spread over many warps.  Pass 1 lists the
 // segments (writes the float copy of w and zeroes z): a CTA counts its columns'
 // segments, takes their place in the list with one atomic add, and also sums
-// the listed non-zeros into *total.  A list beyond `cap` is not written (the
-// count says so).
-constexpr int kSegEntries = 512;
-
+// the listed non-zeros into *total.  The list holds list_cap(k, nnz) segments,
+// those of all columns.
 __global__ void __launch_bounds__(kThreads)
     k_w_segments(const double* __restrict__ w, float* __restrict__ w32, const int64_t* __restrict__ col_ptr, int64_t k,
-                 int32_t* __restrict__ seg_j, uint32_t* __restrict__ seg_t, int64_t cap,
+                 int32_t* __restrict__ seg_j, uint32_t* __restrict__ seg_t,
                  unsigned long long* __restrict__ count, unsigned long long* __restrict__ total, int64_t n,
                  double* __restrict__ z) {
   constexpr int PER = 4;
@@ -496,26 +494,25 @@ __global__ void __launch_bounds__(kThreads)
     uint64_t pos = s_base + before + (incl - mine);
 #pragma unroll
     for (int q = 0; q < PER; ++q)
-      for (uint32_t t = 0; t < nseg[q]; ++t, ++pos)
-        if ((int64_t)pos < cap) {
-          seg_j[pos] = (int32_t)(base + q * kThreads + threadIdx.x);
-          seg_t[pos] = t;
-        }
+      for (uint32_t t = 0; t < nseg[q]; ++t, ++pos) {
+        seg_j[pos] = (int32_t)(base + q * kThreads + threadIdx.x);
+        seg_t[pos] = t;
+      }
     __syncthreads();  // s_warp and s_base are reused
   }
 }
 
 // pass 2: a warp per segment adds w_j X_ij into z (FP64 atomics); nothing when
-// the listed non-zeros exceed `limit` or the list overflowed
+// the listed non-zeros exceed `limit`
 template <typename V>
 __global__ void __launch_bounds__(kThreads)
-    k_scatter_segments(const int32_t* __restrict__ seg_j, const uint32_t* __restrict__ seg_t, int64_t cap,
+    k_scatter_segments(const int32_t* __restrict__ seg_j, const uint32_t* __restrict__ seg_t,
                        const unsigned long long* __restrict__ count, const unsigned long long* __restrict__ total,
                        unsigned long long limit, const int64_t* __restrict__ col_ptr,
                        const int32_t* __restrict__ row_idx, const V* __restrict__ val, const double* __restrict__ w,
                        double* __restrict__ z) {
   const int64_t m = (int64_t)*count;
-  if (*total > limit || m > cap) return;
+  if (*total > limit) return;
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < m; g += nwarps) {
@@ -753,8 +750,6 @@ int launch_coloring_iter(gencd_problem* p, int64_t q, bool early) {
 // longer there than listing w's segments, and the sums have a fixed order, so
 // that equal problems get equal z to the last bit (the scatter's atomic adds
 // do not).
-constexpr int64_t kFitRowsNnz = int64_t(1) << 20;
-
 static int state_by_rows(gencd_problem* p) {
   GENCD_TRY(build_csr(p));
   GENCD_TRY(launch_csr_spmv(p, p->w, p->z));
@@ -778,19 +773,18 @@ int launch_state_from_w(gencd_problem* p) {
   const unsigned long long limit = (unsigned long long)(p->nnz / 5 * 2);
   const int g = p->num_sms * 8;
   k_w_segments<<<grid_for(std::max((p->k + 3) / 4, p->n), kThreads, g), kThreads, 0, p->stream>>>(
-      p->w, p->w32, p->col_ptr, p->k, p->list_j, p->list_off, p->k, count, total, p->n, p->z);
+      p->w, p->w32, p->col_ptr, p->k, p->list_j, p->list_off, count, total, p->n, p->z);
   if (p->precision == GENCD_F64)
-    k_scatter_segments<double><<<g, kThreads, 0, p->stream>>>(p->list_j, p->list_off, p->k, count, total, limit,
-                                                              p->col_ptr, p->row_idx, (const double*)p->val, p->w,
-                                                              p->z);
+    k_scatter_segments<double><<<g, kThreads, 0, p->stream>>>(p->list_j, p->list_off, count, total, limit, p->col_ptr,
+                                                              p->row_idx, (const double*)p->val, p->w, p->z);
   else
-    k_scatter_segments<float><<<g, kThreads, 0, p->stream>>>(p->list_j, p->list_off, p->k, count, total, limit,
-                                                             p->col_ptr, p->row_idx, (const float*)p->val, p->w, p->z);
+    k_scatter_segments<float><<<g, kThreads, 0, p->stream>>>(p->list_j, p->list_off, count, total, limit, p->col_ptr,
+                                                             p->row_idx, (const float*)p->val, p->w, p->z);
   p->prof.launches[K_SETUP] += 2;
   GENCD_CUDA_TRY(cudaGetLastError());
   GENCD_TRY(launch_fill_u(p, total, host));
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
-  if (host[0] <= limit && host[1] <= (unsigned long long)p->k) return GENCD_OK;
+  if (host[0] <= limit) return GENCD_OK;
   return state_by_rows(p);
 }
 

@@ -875,6 +875,29 @@ def test_set_w_fits_sparse_and_dense_coefficients(gb, precision, frac, large):
 
 
 @pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_set_w_scatters_few_columns_of_many_segments(gb, precision):
+    # 100 columns of 15,000 non-zeros: 3,000 segments, 120 of them of the four
+    # columns set; their scatter is three launches, without the row-major copy
+    rng = np.random.default_rng(5)
+    n, k, m = 60_000, 100, 15_000
+    rows = np.concatenate([np.sort(rng.permutation(n)[:m]) for _ in range(k)]).astype(np.int32)
+    prob = workloads.Problem(n, k, np.arange(k + 1, dtype=np.int64) * m, rows, rng.normal(size=k * m),
+                             rng.normal(size=n), "squared", np.zeros(k), "long-columns")
+    orc = oracle.Oracle(prob)
+    w = np.zeros(k)
+    w[[3, 40, 41, 99]] = [0.5, -1.0, 0.25, 2.0]
+    with gb.Problem(prob, precision=precision) as p:
+        before = gb.gencd_profile_read(p.h, 8)[1]
+        p.set_w(w)
+        assert gb.gencd_profile_read(p.h, 8)[1] - before == 3
+        # sums of at most four terms of size 10 (stored values rounded to FP32)
+        np.testing.assert_allclose(p.z(), orc.fitted(w), rtol=0, atol=1e-13 if precision == "f64" else 2e-6)
+        w = rng.normal(size=k)  # dense: by rows
+        p.set_w(w)
+        np.testing.assert_allclose(p.z(), orc.fitted(w), rtol=0, atol=1e-11 if precision == "f64" else 2e-5)
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
 @pytest.mark.parametrize("name,P", [("ragged-logistic", 1), ("ragged-logistic", 326), ("cfg1-logistic", 305),
                                     ("cfg1-logistic", 4500)])
 def test_shotgun_steps_match(gb, name, P, precision):
