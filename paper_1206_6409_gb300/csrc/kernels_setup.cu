@@ -475,8 +475,7 @@ int fail_plan(const char* msg) {
   return GENCD_EINVAL;
 }
 
-int build_csr(gencd_problem* p) {
-  if (p->row_ptr) return GENCD_OK;
+static int build_csr_arrays(gencd_problem* p) {
   const int64_t nnz = p->nnz;
   const size_t vsz = p->precision == GENCD_F64 ? 8 : 4;
   GENCD_TRY(dev_alloc_bytes(p, (void**)&p->row_ptr, sizeof(int64_t) * (size_t)(p->n + 1)));
@@ -511,6 +510,21 @@ int build_csr(gencd_problem* p) {
   p->prof.launches[K_SETUP] += 2;
   GENCD_CUDA_TRY(cudaGetLastError());
   return GENCD_OK;
+}
+
+// row_ptr says that the copy is there, so a build that fails leaves none of it
+int build_csr(gencd_problem* p) {
+  if (p->row_ptr) return GENCD_OK;
+  const int rc = build_csr_arrays(p);
+  if (rc != GENCD_OK) {
+    dev_free(p, p->row_ptr);
+    dev_free(p, p->col_idx);
+    dev_free(p, p->csr_val);
+    p->row_ptr = nullptr;
+    p->col_idx = nullptr;
+    p->csr_val = nullptr;
+  }
+  return rc;
 }
 
 // ---------------------------------------------------------------------------

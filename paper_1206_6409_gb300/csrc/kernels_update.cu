@@ -422,7 +422,8 @@ template <typename V>
 __global__ void __launch_bounds__(kThreads)
     k_csr_spmv(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
                const V* __restrict__ csr_val, const double* __restrict__ x, int64_t n,
-               double* __restrict__ out) {
+               double* __restrict__ out, const unsigned long long* __restrict__ total, unsigned long long limit) {
+  if (total && *total <= limit) return;
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -740,11 +741,14 @@ int launch_coloring_iter(gencd_problem* p, int64_t q, bool early) {
 //
 // Sparse coefficients: their columns are scattered into z, which reads no more
 // of X than those columns and needs no row-major copy (whose build sorts every
-// non-zero).  Otherwise the rows are summed (the row-major copy is built on
-// first use).  The line is drawn at 2/5 of the non-zeros: a call took, by
-// columns with w_j != 0, scattered / by rows, on 4.0e7 FP32 non-zeros 48 / 276
-// us at 0.5%, 84 / 276 at 12.5%, 155 / 276 at 40%, 309 / 276 at 100%, and on
-// 2.0e7 FP64 non-zeros 52 / 123, 74 / 123, 116 / 123 and 164 / 123 us.
+// non-zero).  Otherwise the rows are summed: once the row-major copy is there,
+// the device decides from the listed non-zeros which of the two launches does
+// the work; before that the host does, after a wait, and builds it.  The line
+// is drawn at 2/5 of the non-zeros: a call took, by columns with w_j != 0,
+// scattered / by rows, on 4.0e7 FP32 non-zeros 48 / 276 us at 0.5%, 84 / 276 at
+// 12.5%, 155 / 276 at 40%, 309 / 276 at 100%, and on 2.0e7 FP64 non-zeros 52 /
+// 123, 74 / 123, 116 / 123 and 164 / 123 us.  Deciding costs a dense w some 10 us
+// (287 and 131 us in all; 298 and 145 with the host deciding on every call).
 //
 // At most kFitRowsNnz non-zeros: always by rows.  Reading all of X takes no
 // longer there than listing w's segments, and the sums have a fixed order, so
@@ -782,21 +786,24 @@ int launch_state_from_w(gencd_problem* p) {
                                                              p->row_idx, (const float*)p->val, p->w, p->z);
   p->prof.launches[K_SETUP] += 2;
   GENCD_CUDA_TRY(cudaGetLastError());
+  const bool rows_too = p->row_ptr != nullptr;
+  if (rows_too) GENCD_TRY(launch_csr_spmv(p, p->w, p->z, total, limit));
   GENCD_TRY(launch_fill_u(p, total, host));
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
-  if (host[0] <= limit) return GENCD_OK;
+  if (rows_too || host[0] <= limit) return GENCD_OK;
   return state_by_rows(p);
 }
 
-int launch_csr_spmv(gencd_problem* p, const double* x, double* out) {
+int launch_csr_spmv(gencd_problem* p, const double* x, double* out, const unsigned long long* total,
+                    unsigned long long limit) {
   if (p->n == 0) return GENCD_OK;
   const int grid = grid_for(p->n * 32, kThreads, p->num_sms * 8);
   if (p->precision == GENCD_F64)
     k_csr_spmv<double><<<grid, kThreads, 0, p->stream>>>(p->row_ptr, p->col_idx, (const double*)p->csr_val,
-                                                         x, p->n, out);
+                                                         x, p->n, out, total, limit);
   else
     k_csr_spmv<float><<<grid, kThreads, 0, p->stream>>>(p->row_ptr, p->col_idx, (const float*)p->csr_val,
-                                                        x, p->n, out);
+                                                        x, p->n, out, total, limit);
   p->prof.launches[K_SETUP] += 1;
   GENCD_CUDA_TRY(cudaGetLastError());
   return GENCD_OK;
