@@ -236,14 +236,14 @@ static int enqueue_evaluate(gencd_problem* p, bool gap = false) {
 }
 
 static int read_scalars(gencd_problem* p) {
-  GENCD_CUDA_TRY(cudaMemcpyAsync(p->hpin, p->dscal, kScalars * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
+  GENCD_CUDA_TRY(cudaMemcpyAsync(p->hpin, p->dscal, kScalFit * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
   return GENCD_OK;
 }
 
 // the device scalars to hpin without waiting; ev_scalars marks their arrival
 static int read_scalars_async(gencd_problem* p) {
-  GENCD_CUDA_TRY(cudaMemcpyAsync(p->hpin, p->dscal, kScalars * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
+  GENCD_CUDA_TRY(cudaMemcpyAsync(p->hpin, p->dscal, kScalFit * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
   GENCD_CUDA_TRY(cudaEventRecord(p->ev_scalars, p->stream));
   return GENCD_OK;
 }
@@ -813,6 +813,12 @@ static int solve_finish(gencd_problem* p, SolveRun* S) {
 
 int solve_advance(gencd_problem* p, SolveRun* S) {
   const gencd_params& a = p->params;
+  const int refit = finish_state_from_w(p);  // a restart from a w of many columns: z by rows
+  GENCD_TRY(refit);
+  if (refit == 1) {
+    GENCD_TRY(solve_evaluate(p, S));
+    return 1;
+  }
   if (!S->started) {
     S->obj_start = p->hpin[1];
     S->started = true;
@@ -1134,7 +1140,12 @@ int gencd_set_w(gencd_problem* p, const double* w, int64_t k, int32_t memory) {
       if (!std::isfinite(w[j])) return fail(GENCD_EINVAL, "w[" + std::to_string(j) + "] is not finite");
   }
   GENCD_CUDA_TRY(cudaMemcpyAsync(p->w, w, sizeof(double) * k, kind_in(memory), p->stream));
-  return launch_state_from_w(p);
+  GENCD_TRY(launch_state_from_w(p));
+  GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
+  const int refit = finish_state_from_w(p);
+  GENCD_TRY(refit);
+  if (refit == 1) GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
+  return GENCD_OK;
 }
 
 int gencd_duality_gap(gencd_problem* p, double* gap, double* primal, double* dual) {

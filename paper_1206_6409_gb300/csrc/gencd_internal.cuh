@@ -236,7 +236,7 @@ struct gencd_problem {
   float* bj32 = nullptr;
   float* ib32 = nullptr;
 
-  // device scalars (kScalars doubles, mirrored to hpin): [0] kkt bits,
+  // device scalars (kScalars doubles, [0..9] mirrored to hpin): [0] kkt bits,
   // [1] objective, [2] loss sum, [3] l1 sum, [4] updates (int64), [5] nnz
   // processed (int64), [6] scratch, [7] max_j |g_j| of the last full
   // evaluation (bits; idle columns count as lambda), [8] the duality gap's
@@ -244,7 +244,8 @@ struct gencd_problem {
   // segments of the columns that z = Xw scatters (int64)
   double* dscal = nullptr;
   double* red = nullptr;  // per-block partial sums (2 * kRedBlocks)
-  double* hpin = nullptr; // pinned host mirror of dscal
+  double* hpin = nullptr; // pinned host memory: dscal's first kScalFit, then what z = Xw reports
+  bool fit_open = false;  // whether the columns sufficed for z = Xw is in hpin once the stream gets there
   double* ltab = nullptr; // logistic_table() on the device
 
   // selection
@@ -335,7 +336,11 @@ int launch_csr_spmv(gencd_problem* p, const double* x, double* out, const unsign
                     unsigned long long limit = 0);
 // entries of list_j and list_off: a column of len non-zeros has ceil(len / kSegEntries) segments
 inline int64_t list_cap(int64_t k, int64_t nnz) { return k + (nnz > kFitRowsNnz ? nnz / kSegEntries : 0); }
-int launch_state_from_w(gencd_problem* p);  // z, u and w32 from p->w (synchronises the stream)
+// z, u and w32 from p->w, without waiting.  When p->fit_open is then set, the
+// state may still lack z: once the stream has been waited for,
+// finish_state_from_w enqueues the rest and returns 1, or 0 if nothing is missing.
+int launch_state_from_w(gencd_problem* p);
+int finish_state_from_w(gencd_problem* p);
 
 // kernels_setup.cu
 const std::vector<double>& logistic_table();

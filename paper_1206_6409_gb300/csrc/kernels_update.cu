@@ -737,13 +737,14 @@ int launch_coloring_iter(gencd_problem* p, int64_t q, bool early) {
 }
 
 // z = Xw, u = l'(y, z) and (FP32 mode) the float copy of w, from the
-// coefficients in p->w; synchronises the stream.
+// coefficients in p->w.
 //
 // Sparse coefficients: their columns are scattered into z, which reads no more
 // of X than those columns and needs no row-major copy (whose build sorts every
 // non-zero).  Otherwise the rows are summed: once the row-major copy is there,
 // the device decides from the listed non-zeros which of the two launches does
-// the work; before that the host does, after a wait, and builds it.  The line
+// the work; before that the host does, after a wait (finish_state_from_w), and
+// builds it.  The line
 // is drawn at 2/5 of the non-zeros: a call took, by columns with w_j != 0,
 // scattered / by rows, on 4.0e7 FP32 non-zeros 48 / 276 us at 0.5%, 84 / 276 at
 // 12.5%, 155 / 276 at 40%, 309 / 276 at 100%, and on 2.0e7 FP64 non-zeros 52 /
@@ -757,12 +758,14 @@ int launch_coloring_iter(gencd_problem* p, int64_t q, bool early) {
 static int state_by_rows(gencd_problem* p) {
   GENCD_TRY(build_csr(p));
   GENCD_TRY(launch_csr_spmv(p, p->w, p->z));
-  GENCD_TRY(launch_fill_u(p));
-  GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
-  return GENCD_OK;
+  return launch_fill_u(p);
 }
 
+// non-zeros of the listed columns up to which they are scattered
+static unsigned long long fit_limit(const gencd_problem* p) { return (unsigned long long)(p->nnz / 5 * 2); }
+
 int launch_state_from_w(gencd_problem* p) {
+  p->fit_open = false;
   if (p->nnz <= kFitRowsNnz) {
     if (p->w32) {
       k_mirror_w<<<grid_for(p->k, kThreads, p->num_sms * 8), kThreads, 0, p->stream>>>(p->w, p->k, p->w32);
@@ -774,7 +777,7 @@ int launch_state_from_w(gencd_problem* p) {
   unsigned long long* total = reinterpret_cast<unsigned long long*>(p->dscal + kScalFit);  // zero between calls
   unsigned long long* count = total + 1;
   unsigned long long* host = reinterpret_cast<unsigned long long*>(p->hpin + kScalFit);
-  const unsigned long long limit = (unsigned long long)(p->nnz / 5 * 2);
+  const unsigned long long limit = fit_limit(p);
   const int g = p->num_sms * 8;
   k_w_segments<<<grid_for(std::max((p->k + 3) / 4, p->n), kThreads, g), kThreads, 0, p->stream>>>(
       p->w, p->w32, p->col_ptr, p->k, p->list_j, p->list_off, count, total, p->n, p->z);
@@ -789,9 +792,16 @@ int launch_state_from_w(gencd_problem* p) {
   const bool rows_too = p->row_ptr != nullptr;
   if (rows_too) GENCD_TRY(launch_csr_spmv(p, p->w, p->z, total, limit));
   GENCD_TRY(launch_fill_u(p, total, host));
-  GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
-  if (rows_too || host[0] <= limit) return GENCD_OK;
-  return state_by_rows(p);
+  p->fit_open = !rows_too;
+  return GENCD_OK;
+}
+
+int finish_state_from_w(gencd_problem* p) {
+  if (!p->fit_open) return 0;
+  p->fit_open = false;
+  if (reinterpret_cast<const unsigned long long*>(p->hpin + kScalFit)[0] <= fit_limit(p)) return 0;
+  GENCD_TRY(state_by_rows(p));
+  return 1;
 }
 
 int launch_csr_spmv(gencd_problem* p, const double* x, double* out, const unsigned long long* total,

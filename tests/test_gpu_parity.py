@@ -903,6 +903,39 @@ def test_set_w_scatters_few_columns_of_many_segments(gb, precision):
             np.testing.assert_allclose(p.z(), orc.fitted(w), rtol=0, atol=1e-11 if precision == "f64" else 2e-5)
 
 
+@pytest.mark.parametrize("start", ["few", "dense", "grown"])
+def test_restarts_of_large_problems_start_from_their_w(gb, start):
+    # 1.2e6 non-zeros (z = Xw from the columns): Thread-Greedy's first steps
+    # overshoot, so the solve restarts, from a w of few columns, from one whose
+    # columns hold more than 2/5 of the non-zeros, and from such a one that
+    # iterations grew (no row-major copy yet: z by rows is decided at the next
+    # check).  The solve's z belongs to its w, and its objective falls
+    prob = workloads.uniform_problem(3_000, 40_000, 30, values="lognormal", loss="squared", n_planted=20, seed=6)
+    assert prob.nnz > 1 << 20
+    orc = oracle.Oracle(prob)
+    lam = (1e-4 if start == "grown" else 0.1) * orc.lambda_max()
+    orc.set_lambda(lam)
+    rng = np.random.default_rng(1)
+    w0 = np.where(rng.random(prob.k) < (0.7 if start == "dense" else 1e-3), rng.normal(0, 1e-4, prob.k), 0.0)
+    with gb.Problem(prob, precision="f64") as p:
+        p.set_lambda(lam)
+        p.set_w(w0)
+        if start == "grown":
+            p.set_params(variant="shotgun", P=40)
+            p.iterate(1000)
+            w0 = p.w()
+            assert prob.col_nnz()[w0 != 0].sum() > 0.4 * prob.nnz
+        p.set_params(variant="thread_greedy", blocks=1024, max_iter=200, check_every=10, tol_kkt=0.0)
+        before = gb.gencd_profile_read(p.h, 8)[1]
+        r = p.solve()
+        assert gb.gencd_profile_read(p.h, 8)[1] - before >= 3  # it restarted
+        w, z = p.w(), p.z()
+    assert r.iters == 200
+    np.testing.assert_allclose(z, orc.fitted(w), rtol=0, atol=1e-11 * max(1.0, np.abs(z).max()))
+    assert r.objective == pytest.approx(orc.objective(w), rel=1e-9)
+    assert r.objective < orc.objective(w0)
+
+
 @pytest.mark.parametrize("precision", ["f64", "f32"])
 @pytest.mark.parametrize("name,P", [("ragged-logistic", 1), ("ragged-logistic", 326), ("cfg1-logistic", 305),
                                     ("cfg1-logistic", 4500)])
