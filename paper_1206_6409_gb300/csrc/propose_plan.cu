@@ -1040,12 +1040,19 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   // each) once it averages half an entry per slab in FP32 arithmetic (uniform
   // columns, a pass over 9.0e7 and 1.8e7 entries as slabs / as light columns:
   // 1.4 a slab 255 / 343 us, 0.3 a slab 118 / 88) and two in FP64 (0.7 a slab 465
-  // / 400).  The light pass is a kernel of its own, though: what few entries
-  // would be left to it join the slabs (2e8 Zipf non-zeros: 4341 us for ten
-  // iterations from two a slab, 4106 from a half, 3772 with none left; FP64 2e7
-  // 1137 / 1044), while the runs (R per column) are no more than the non-zeros,
-  // which bounds the scratch of the build.
-  constexpr int64_t kFewLight = int64_t(1) << 22;
+  // / 400).  The light pass is a kernel of its own, though: beside heavy columns,
+  // what few entries would be left to it join the slabs (2e8 Zipf non-zeros: 4341
+  // us for ten iterations from two a slab, 4106 from a half, 3772 with none left;
+  // FP64 2e7 1137 / 1044), while the runs (R per column) are no more than the
+  // non-zeros, which bounds the scratch of the build.  An iteration with three
+  // columns of 20,000 beside uniform ones takes, in slabs / with the light pass,
+  // 21.8 / 26.2 us (FP32, 1e5 columns of 3 over 7 slabs), 27.9 / 29.0 (1.9e5 of 8
+  // over 21), 43.5 / 47.0 (FP64, 5e5 of 8 over 5); in FP64 it does not pay for
+  // many entries at less than one a slab (9e4 columns of 40 over 41 slabs 45.0 /
+  // 41.2; of 10 30.4 / 29.2, of 12 over 9 46.8 / 45.8).  Light columns alone
+  // keep their pass, which is then the only kernel (FP32 19.5 / 19.4, 26.9 / 23.7;
+  // FP64 44.1 / 41.7, 44.5 / 33.0 us).
+  constexpr int64_t kFewLight = int64_t(1) << 22, kFewSparse = int64_t(1) << 20;
   // FP32 sums of many slabs go to two accumulators, odd slabs to the second: a
   // column's sums are added one after another, and two chains half as long keep
   // the error of short columns below that of the light pass, which adds in a
@@ -1065,7 +1072,10 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
     unsigned long long c[4];
     GENCD_CUDA_TRY(cudaMemcpyAsync(c, stats, sizeof(c), cudaMemcpyDeviceToHost, st));
     GENCD_CUDA_TRY(cudaStreamSynchronize(st));
-    if ((int64_t)c[1] <= std::max(kFewLight, p->nnz / 10) && (int64_t)c[0] * P.nslabs <= std::max(kFewLight, p->nnz))
+    const int64_t columns = (int64_t)c[0], light = (int64_t)c[1], short_columns = (int64_t)c[2];  // FP64: the light ones
+    if (light < p->nnz && light <= std::max(kFewLight, p->nnz / 10) &&
+        columns * P.nslabs <= std::max(kFewLight, p->nnz) &&
+        (!f64 || light <= kFewSparse || light >= short_columns * P.nslabs))
       P.heavy_min = 1;
     // the schedules of both passes stay selectable wherever columns lie on both
     // sides of two entries a slab, whether or not the rule leaves light ones

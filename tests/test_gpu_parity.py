@@ -1051,6 +1051,41 @@ def test_propose_with_light_and_heavy_columns(gb, precision):
 
 
 @pytest.mark.parametrize("precision", ["f64", "f32"])
+@pytest.mark.parametrize("n,per_col,long,passes", [
+    (300_000, 3, 0, "light"), (300_000, 3, 20_000, "slabs"),  # 7 slabs in FP32, 13 in FP64
+    (300_000, 60, 0, "slabs"), (40_000, 3, 0, None)])
+def test_light_columns_alone_keep_their_pass(gb, n, per_col, long, passes, precision):
+    # few short columns join the slabs beside heavy ones only: alone, their own
+    # pass is the one kernel; either way the proposals are the oracle's
+    rng = np.random.default_rng(n + per_col)
+    counts = np.full(50_000, per_col, np.int64)
+    if long:
+        counts[777] = long
+    col_ptr = np.zeros(counts.size + 1, np.int64)
+    np.cumsum(counts, out=col_ptr[1:])
+    rows = workloads.synthetic._distinct_rows(n, counts, rng)
+    prob = workloads.Problem(n, counts.size, col_ptr, rows, rng.normal(size=rows.size), rng.normal(size=n), "squared",
+                             np.zeros(counts.size), "light")
+    orc = oracle.Oracle(prob)
+    lam = 0.05 * orc.lambda_max()
+    orc.set_lambda(lam)
+    w = _state(prob, 3, frac=0.01)
+    z = orc.fitted(w)
+    J = np.arange(prob.k, dtype=np.int32)
+    d_cpu, f_cpu = orc.propose(w, z, J)
+    with gb.Problem(prob, precision=precision) as p:
+        p.set_lambda(lam)
+        p.set_w(w)
+        gb.gencd_profile_reset(p.h)
+        d, f, _ = p.propose_all()
+        ran = [gb.gencd_profile_read(p.h, kernel)[1] for kernel in (9, 10, 12)]  # light, slabs, both in one
+    if passes is None:
+        passes = "slabs" if precision == "f32" else "light"  # one slab in FP32, two in FP64
+    assert ran == ([1, 0, 0] if passes == "light" else [0, 1, 0])
+    assert_steps_close(prob, z, w, lam, J, d, f, d_cpu, f_cpu, TOL[precision])
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
 @pytest.mark.parametrize("n", [3_000, 30_000])
 @pytest.mark.parametrize("B", [1, 256, 257, 512, 513])
 def test_update_and_refresh_on_both_sides_of_one_launch(gb, n, B, precision):
