@@ -167,6 +167,7 @@ struct gencd_problem {
   // serving loop, which must not synchronise the device), else cudaMalloc
   cudaMemPool_t pool = nullptr;
   bool own_hpin = true;               // hpin allocated by the problem (else lent by its owner)
+  bool overlap = true;                // launches overlap their predecessor (LaunchOn)
   cudaEvent_t ev_scalars = nullptr;   // recorded after each copy of dscal to hpin
   int64_t n = 0, k = 0, nnz = 0, nnz_pad = 0;
   int32_t loss = GENCD_LOSS_LOGISTIC;
@@ -440,32 +441,48 @@ __device__ __forceinline__ uint4 load_l2(const uint4* p) {
   return v;
 }
 
+// LaunchOn: the stream, and whether launches on it overlap.  Not for large
+// problems that share the device (a serving slot's, serve.cu): CTAs that wait
+// hold their SM's shared memory and threads, and other streams' ready kernels
+// cannot start there.
 // launch_cluster_overlapped: such a launch with the whole grid, `cluster` CTAs,
 // as one cluster (cluster = 1: no cluster).
+struct LaunchOn {
+  cudaStream_t stream;
+  bool overlap;
+  LaunchOn(cudaStream_t s, bool o = true) : stream(s), overlap(o) {}
+};
+inline LaunchOn launch_on(const gencd_problem* p) { return LaunchOn(p->stream, p->overlap); }
+
 template <typename... P, typename... A>
 inline cudaError_t launch_cluster_overlapped(void (*kernel)(P...), unsigned cluster, dim3 grid, dim3 block, size_t smem,
-                                             cudaStream_t stream, A... args) {
+                                             LaunchOn on, A... args) {
   cudaLaunchAttribute attr[2];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  attr[1].id = cudaLaunchAttributeClusterDimension;
-  attr[1].val.clusterDim.x = cluster;
-  attr[1].val.clusterDim.y = 1;
-  attr[1].val.clusterDim.z = 1;
+  unsigned attrs = 0;
+  if (on.overlap) {
+    attr[attrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[attrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[attrs].id = cudaLaunchAttributeClusterDimension;
+    attr[attrs].val.clusterDim.x = cluster;
+    attr[attrs].val.clusterDim.y = 1;
+    attr[attrs++].val.clusterDim.z = 1;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
+  cfg.stream = on.stream;
   cfg.attrs = attr;
-  cfg.numAttrs = cluster > 1 ? 2 : 1;
+  cfg.numAttrs = attrs;
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
 template <typename... P, typename... A>
-inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
+inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, LaunchOn on,
                                      A... args) {
-  return launch_cluster_overlapped(kernel, 1u, grid, block, smem, stream, args...);
+  return launch_cluster_overlapped(kernel, 1u, grid, block, smem, on, args...);
 }
 
 // grow a device allocation

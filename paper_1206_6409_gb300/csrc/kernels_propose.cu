@@ -726,7 +726,7 @@ int launch_finalize_accept(gencd_problem* p, int64_t B, bool want_kkt, bool appl
   cudaEvent_t ev = nullptr;
   prof_begin(p, K_FINALIZE, &ev);
   auto go = [&](auto kernel, auto* gacc) {
-    return launch_overlapped(kernel, grid, kThreads, 0, p->stream, gacc, c, B, (int)per, chunk, p->part_lo,
+    return launch_overlapped(kernel, grid, kThreads, 0, launch_on(p), gacc, c, B, (int)per, chunk, p->part_lo,
                              want_kkt ? 1 : 0, p->slot_m, p->slot_j, p->slot_d, p->slot_cnt, p->list_j, p->list_d,
                              p->list_m, p->dscal + 0, p->col_ptr, p->w, p->w32, apply ? p->list_off : nullptr);
   };

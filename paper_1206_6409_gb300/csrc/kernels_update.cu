@@ -636,7 +636,7 @@ int launch_update_refresh(gencd_problem* p, const int32_t* J, const double* d, i
     cudaEvent_t ev = nullptr;
     prof_begin(p, K_UPDATE, &ev);
     auto go = [&](auto kernel, auto* val, auto* u) {
-      return launch_cluster_overlapped(kernel, kClusterCtas, dim3(kClusterCtas), dim3(kListThreads), 0, p->stream,
+      return launch_cluster_overlapped(kernel, kClusterCtas, dim3(kClusterCtas), dim3(kListThreads), 0, launch_on(p),
                                        p->col_ptr, p->row_idx, val, J, d, p->list_off, m, p->y, p->z, p->n, p->loss,
                                        p->ltab, u, ctr);
     };
@@ -652,7 +652,7 @@ int launch_update_refresh(gencd_problem* p, const int32_t* J, const double* d, i
   cudaEvent_t ev = nullptr;
   prof_begin(p, K_UPDATE, &ev);
   auto go = [&](auto kernel, auto* val) {
-    return launch_overlapped(kernel, list_grid(p), kListThreads, 0, p->stream, p->col_ptr, p->row_idx, val, J, d,
+    return launch_overlapped(kernel, list_grid(p), kListThreads, 0, launch_on(p), p->col_ptr, p->row_idx, val, J, d,
                              p->list_off, m, p->z, ctr);
   };
   cudaError_t err;
@@ -676,7 +676,7 @@ int launch_refresh_list(gencd_problem* p, const int32_t* J, int64_t m, bool coun
   cudaEvent_t ev = nullptr;
   prof_begin(p, K_REFRESH, &ev);
   auto go = [&](auto kernel, auto* u) {
-    return launch_overlapped(kernel, list_grid(p), kListThreads, 0, p->stream, p->col_ptr, p->row_idx, J, p->list_off,
+    return launch_overlapped(kernel, list_grid(p), kListThreads, 0, launch_on(p), p->col_ptr, p->row_idx, J, p->list_off,
                              m, p->y, p->z, p->n, p->loss, p->ltab, u, ctr);
   };
   cudaError_t err;
@@ -701,11 +701,11 @@ int launch_shotgun_step(gencd_problem* p, const int32_t* J, int64_t m, bool earl
   prof_begin(p, K_PROPOSE_LIST, &ev);
   cudaError_t err;
   if (p->precision == GENCD_F64)
-    err = launch_overlapped(k_shotgun_step<double, double>, grid, kThreads, 0, p->stream, p->col_ptr, p->row_idx,
+    err = launch_overlapped(k_shotgun_step<double, double>, grid, kThreads, 0, launch_on(p), p->col_ptr, p->row_idx,
                             (const double*)p->val, (const double*)p->u, p->bj, p->ib, J, m, per, early ? 1 : 0,
                             (double)p->n, p->lambda, p->w, p->w32, p->z, p->list_off, ctr);
   else
-    err = launch_overlapped(k_shotgun_step<float, float>, grid, kThreads, 0, p->stream, p->col_ptr, p->row_idx,
+    err = launch_overlapped(k_shotgun_step<float, float>, grid, kThreads, 0, launch_on(p), p->col_ptr, p->row_idx,
                             (const float*)p->val, (const float*)p->u, p->bj, p->ib, J, m, per, early ? 1 : 0,
                             (double)p->n, p->lambda, p->w, p->w32, p->z, p->list_off, ctr);
   prof_end(p, ev);
@@ -724,11 +724,11 @@ int launch_coloring_iter(gencd_problem* p, int64_t q, bool early) {
   prof_begin(p, K_COLOR_ITER, &ev);
   cudaError_t err;
   if (p->precision == GENCD_F64)
-    err = launch_overlapped(k_coloring_iter<double, double>, grid, 32 * per, 0, p->stream, p->col_ptr, p->row_idx,
+    err = launch_overlapped(k_coloring_iter<double, double>, grid, 32 * per, 0, launch_on(p), p->col_ptr, p->row_idx,
                             (const double*)p->val, (double*)p->u, p->w, p->w32, p->bj, p->ib, p->z, p->y, p->perm, q,
                             p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, p->ltab, early ? 1 : 0, ctr);
   else
-    err = launch_overlapped(k_coloring_iter<float, float>, grid, 32 * per, 0, p->stream, p->col_ptr, p->row_idx,
+    err = launch_overlapped(k_coloring_iter<float, float>, grid, 32 * per, 0, launch_on(p), p->col_ptr, p->row_idx,
                             (const float*)p->val, (float*)p->u, p->w, p->w32, p->bj, p->ib, p->z, p->y, p->perm, q,
                             p->color_ptr, p->cols_by_color, (double)p->n, p->lambda, p->loss, p->ltab, early ? 1 : 0, ctr);
   prof_end(p, ev);

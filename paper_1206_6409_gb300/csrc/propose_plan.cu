@@ -631,7 +631,7 @@ template <typename V, typename U, typename G, typename SV, int SW>
 static cudaError_t launch_fused(gencd_problem* p, const void* u_vec, size_t smem) {
   ProposePlan& P = p->plan;
   return launch_overlapped(k_propose_fused<V, U, G, kFusedThreads, SW, 1, kFusedItems, SV>, P.grid, kFusedThreads, smem,
-                           p->stream, P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P, P.fused),
+                           launch_on(p), P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P, P.fused),
                            P.light_row, (const SV*)P.light_val, P.lmask, P.light_tile_lc, P.light_cols,
                            P.light_nnz, P.light_ntiles, P.light_counter, (const U*)u_vec, p->n, P.slab_rows,
                            (G*)p->gnat, P.second);
@@ -666,7 +666,7 @@ static int launch_plan_passes(gencd_problem* p, const void* u_vec) {
     prof_begin(p, K_PROPOSE_LIGHT, &e);
     const int grid = grid_for(P.light_ntiles * 32, kThreads, p->num_sms * 3);  // resident CTAs: persistent warps
     const cudaError_t err = launch_overlapped(
-        k_propose_light_runs<V, U, G, SV>, grid, kThreads, 0, p->stream, P.light_row, (const SV*)P.light_val, P.lmask,
+        k_propose_light_runs<V, U, G, SV>, grid, kThreads, 0, launch_on(p), P.light_row, (const SV*)P.light_val, P.lmask,
         P.light_tile_lc, P.light_cols, (const U*)u_vec, P.light_nnz, P.light_ntiles, (G*)p->gnat);
     prof_end(p, e);
     GENCD_CUDA_TRY(err);
@@ -676,7 +676,7 @@ static int launch_plan_passes(gencd_problem* p, const void* u_vec) {
     cudaEvent_t e1 = nullptr;
     prof_begin(p, K_PROPOSE_SLABS, &e1);
     const cudaError_t err = launch_overlapped(
-        k_propose_slabs<V, U, G, THREADS, DEPTH, ITEMS, SV>, P.grid, THREADS, smem, p->stream, P.s_row,
+        k_propose_slabs<V, U, G, THREADS, DEPTH, ITEMS, SV>, P.grid, THREADS, smem, launch_on(p), P.s_row,
         (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P, P.tiles), (const U*)u_vec, p->n, P.slab_rows,
         (G*)p->gnat, P.second);
     prof_end(p, e1);

@@ -63,6 +63,25 @@ def test_serve_results_are_the_same_alone_and_in_the_mix(gb, stream):
                                label=f"request {q}")
 
 
+def test_large_requests_in_the_mix_match_a_solve_alone(gb, stream):
+    # above 2^20 non-zeros a request's kernels launch plainly beside other slots
+    # (and early when it has the device to itself)
+    problems, fracs, arrivals = stream
+    big = [workloads.uniform_problem(4_000, 30_000, 40, values="lognormal", loss=loss, n_planted=30, seed=8)
+           for loss in ("squared", "logistic")]
+    assert all(p.nnz > 1 << 20 for p in big)
+    params = dict(variant="thread_greedy", blocks=64, tol_kkt=0.0, tol_gap=1e-6, max_iter=100_000, check_every=10)
+    mix, w_mix = gb.gencd_serve(big + problems[:4], [0.3, 0.3] + list(fracs[:4]), [0.0] * 6, workers=3, want_w=True,
+                                **params)
+    alone, _ = gb.gencd_serve(big, [0.3, 0.3], [0.0] * 2, workers=1, **params)
+    for q, p in enumerate(big):
+        assert mix[q]["status"] == 0 and alone[q]["status"] == 0
+        assert mix[q]["objective"] == pytest.approx(alone[q]["objective"], rel=2e-6)  # both within their gap
+        orc = oracle.Oracle(oracle.stored_problem(p, "f32"))
+        orc.set_lambda(mix[q]["lambda_"])
+        assert mix[q]["objective"] == pytest.approx(orc.objective(w_mix[q]), rel=1e-9)
+
+
 def test_serve_admits_by_the_hbm_budget(gb, stream):
     # a budget below every request's estimate: each runs alone, in order
     problems, fracs, arrivals = stream

@@ -111,3 +111,14 @@ def test_overlapped_kernels_read_changing_memory_coherently(kernel):
             ldg = set(re.findall(r"__ldg\(\s*(?:reinterpret_cast<[^>]*>\()?(\w+)", body))
             assert ldg <= LDG, (kernel, name, ldg - LDG)
         assert "__ldcg" not in body, (kernel, name)
+
+
+def test_a_problems_launches_follow_its_overlap():
+    # large problems of a serving slot launch plainly: every overlapped launch
+    # for a problem takes the stream together with the problem's choice
+    for f in ("kernels_propose.cu", "kernels_update.cu", "propose_plan.cu"):
+        with open(os.path.join(CSRC, f)) as fh:
+            text = fh.read()
+        calls = [text[m.start():_matching(text, m.end() - 1, "(", ")")]
+                 for m in re.finditer(r"\blaunch_(?:cluster_)?overlapped\(", text)]
+        assert calls and all("launch_on(p)" in c and "p->stream" not in c for c in calls), f
