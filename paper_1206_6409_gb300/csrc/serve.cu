@@ -83,9 +83,13 @@ struct Server {
 // its sort (built when a solve restarts from its start state or needs z =
 // Xw), per-row state (y, z, u), per-column state (w, c, beta_j, sums, steps,
 // proxies, lists, the Thread-Greedy backoff's start point, the top-|J'|
-// Accept's sort buffers) and a fixed allowance for small buffers.
+// Accept's sort buffers) and a fixed allowance for small buffers, which is all
+// that a request counts for whose sizes gencd_create refuses.
 double footprint(const gencd_request& r, int precision, const gencd_params& params) {
   const double vsz = precision == GENCD_F64 ? 8.0 : 4.0;
+  constexpr double kAllowance = 64.0 * (1 << 20);
+  constexpr int64_t kMost = int64_t(1) << 31;
+  if (r.n < 1 || r.k < 1 || r.nnz < 0 || r.n >= kMost || r.k >= kMost || r.nnz >= kMost) return kAllowance;
   const double nnz = (double)r.nnz, n = (double)r.n, k = (double)r.k;
   double b = nnz * (4.0 + vsz)               // CSC
              + nnz * (6.0 + vsz + 0.25)      // streaming plan (2-byte rows; at most a 4-byte pair an entry)
@@ -93,7 +97,7 @@ double footprint(const gencd_request& r, int precision, const gencd_params& para
              + nnz * 24.0                    // its sort scratch
              + n * (16.0 + vsz)              // y, z, u
              + k * 128.0                     // per-column state and lists
-             + 64.0 * (1 << 20);
+             + kAllowance;
   if (params.variant == GENCD_THREAD_GREEDY || params.variant == GENCD_TOP_GREEDY) b += 8.0 * k;  // backoff start
   if (params.variant == GENCD_TOP_GREEDY) b += 28.0 * k;  // sort keys, indices and scratch
   return b;

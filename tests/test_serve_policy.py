@@ -51,6 +51,20 @@ def test_the_budget_admits_by_estimate(gb):
     assert _overlap(big) == 1 and len(big) == 3
 
 
+def test_requests_with_refused_sizes_hold_the_allowance_only(gb):
+    # sizes that gencd_create refuses: their estimate is neither negative (it
+    # would admit others beyond the budget) nor the whole budget
+    bad = [(-(1 << 40), 10, 10), (10, -5, 10), (10, 10, -(1 << 40)), (10, 10, 1 << 62), (1 << 31, 10, 10)]
+    res = gb.gencd_serve_dry_run(bad + [(1000, 1000, 5000)], [0.0] * 6, [0.0] * 6, budget_bytes=1e12, workers=2)
+    assert [r["bytes"] for r in res[:5]] == [64 << 20] * 5
+    assert res[5]["bytes"] > 64 << 20
+    # two good requests that fill the budget: a refused one does not make room for a third
+    est = res[5]["bytes"]
+    sizes = [(1000, 1000, 5000), (-(1 << 40), 10, 10), (1000, 1000, 5000), (1000, 1000, 5000)]
+    res = gb.gencd_serve_dry_run(sizes, [0.0] * 4, [0.05] * 4, budget_bytes=2.2 * est, workers=4)
+    assert _overlap(res) == 2
+
+
 def test_requests_wait_for_their_arrival(gb):
     arrivals = [0.0, 0.05, 0.10, 0.15]
     res = gb.gencd_serve_dry_run([(1000, 1000, 5000)] * 4, arrivals, [0.01] * 4, budget_bytes=1e12, workers=4)
