@@ -19,6 +19,21 @@ static thread_local std::string g_err;
 void set_error(const std::string& m) { g_err = m; }
 const char* last_error() { return g_err.c_str(); }
 
+int caught() noexcept {
+  try {
+    throw;
+  } catch (const std::exception& e) {
+    try {
+      set_error(std::string("host allocation failed: ") + e.what());
+    } catch (...) {  // not even for the message
+      g_err.clear();
+    }
+  } catch (...) {
+    g_err.clear();
+  }
+  return GENCD_ENOMEM;
+}
+
 static int fail(int code, const std::string& m) {
   set_error(m);
   return code;
@@ -908,7 +923,7 @@ extern "C" {
 
 const char* gencd_last_error(void) { return last_error(); }
 
-int gencd_default_params(gencd_params* out) {
+int gencd_default_params(gencd_params* out) try {
   if (!out) return fail(GENCD_EINVAL, "params is NULL");
   std::memset(out, 0, sizeof(*out));
   out->variant = GENCD_THREAD_GREEDY;
@@ -922,13 +937,15 @@ int gencd_default_params(gencd_params* out) {
   out->timeout_s = 0.0;
   return GENCD_OK;
 }
+GENCD_CATCH
 
 int gencd_create(gencd_problem** out, int64_t n, int64_t k, int64_t nnz, const int64_t* col_ptr,
                  const int32_t* row_idx, const void* val, int32_t val_dtype, const double* y, int32_t loss,
-                 int32_t precision, int32_t memory, void* stream) {
+                 int32_t precision, int32_t memory, void* stream) try {
   return create_problem(out, n, k, nnz, col_ptr, row_idx, val, val_dtype, y, loss, precision, memory,
                         (cudaStream_t)stream, nullptr, nullptr);
 }
+GENCD_CATCH
 
 }  // extern "C"
 
@@ -965,11 +982,14 @@ int create_problem(gencd_problem** out, int64_t n, int64_t k, int64_t nnz, const
     p->hpin = hpin;
     p->own_hpin = false;
   }
-  int rc = create_impl(p, col_ptr, row_idx, val, val_dtype, y, memory);
-  if (rc != GENCD_OK) {
-    std::string keep = last_error();
+  int rc;
+  try {
+    rc = create_impl(p, col_ptr, row_idx, val, val_dtype, y, memory);
+  } catch (...) {
+    rc = caught();
+  }
+  if (rc != GENCD_OK) {  // freeing a problem leaves the message
     free_problem(p);
-    set_error(keep);
     return rc;
   }
   *out = p;
@@ -982,14 +1002,15 @@ extern "C" {
 
 void gencd_destroy(gencd_problem* p) { free_problem(p); }
 
-int gencd_set_lambda(gencd_problem* p, double lambda) {
+int gencd_set_lambda(gencd_problem* p, double lambda) try {
   GENCD_CHECK_HANDLE(p);
   if (!(lambda >= 0.0) || !std::isfinite(lambda)) return fail(GENCD_EINVAL, "lambda must be finite and >= 0");
   p->lambda = lambda;
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_set_loss(gencd_problem* p, int32_t loss) {
+int gencd_set_loss(gencd_problem* p, int32_t loss) try {
   GENCD_CHECK_HANDLE(p);
   if (loss != GENCD_LOSS_SQUARED && loss != GENCD_LOSS_LOGISTIC) return fail(GENCD_EINVAL, "unknown loss");
   if (loss == p->loss) return GENCD_OK;
@@ -1015,15 +1036,17 @@ int gencd_set_loss(gencd_problem* p, int32_t loss) {
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_lambda_max(gencd_problem* p, double* lambda_max) {
+int gencd_lambda_max(gencd_problem* p, double* lambda_max) try {
   GENCD_CHECK_HANDLE(p);
   if (!lambda_max) return fail(GENCD_EINVAL, "lambda_max is NULL");
   *lambda_max = p->lambda_max;
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_set_params(gencd_problem* p, const gencd_params* a) {
+int gencd_set_params(gencd_problem* p, const gencd_params* a) try {
   GENCD_CHECK_HANDLE(p);
   if (!a) return fail(GENCD_EINVAL, "params is NULL");
   if (a->variant < 0 || a->variant > 5) return fail(GENCD_EINVAL, "unknown variant");
@@ -1044,30 +1067,34 @@ int gencd_set_params(gencd_problem* p, const gencd_params* a) {
   GENCD_TRY(launch_inv_beta(p));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_get_params(gencd_problem* p, gencd_params* a) {
+int gencd_get_params(gencd_problem* p, gencd_params* a) try {
   GENCD_CHECK_HANDLE(p);
   if (!a) return fail(GENCD_EINVAL, "params is NULL");
   *a = p->params;
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_set_iteration(gencd_problem* p, int64_t t) {
+int gencd_set_iteration(gencd_problem* p, int64_t t) try {
   GENCD_CHECK_HANDLE(p);
   if (t < 0) return fail(GENCD_EINVAL, "iteration must be >= 0");
   p->t = t;
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_get_iteration(gencd_problem* p, int64_t* t) {
+int gencd_get_iteration(gencd_problem* p, int64_t* t) try {
   GENCD_CHECK_HANDLE(p);
   if (!t) return fail(GENCD_EINVAL, "t is NULL");
   *t = p->t;
   return GENCD_OK;
 }
+GENCD_CATCH
 
 
-int gencd_iterate(gencd_problem* p, int64_t iters, gencd_result* out) {
+int gencd_iterate(gencd_problem* p, int64_t iters, gencd_result* out) try {
   GENCD_CHECK_HANDLE(p);
   if (iters < 0) return fail(GENCD_EINVAL, "iters must be >= 0");
   auto t0 = std::chrono::steady_clock::now();
@@ -1087,8 +1114,9 @@ int gencd_iterate(gencd_problem* p, int64_t iters, gencd_result* out) {
   fill_result(p, out, GENCD_OK, iters, host_nnz, secs);
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_solve(gencd_problem* p, gencd_result* out) {
+int gencd_solve(gencd_problem* p, gencd_result* out) try {
   GENCD_CHECK_HANDLE(p);
   SolveRun S;
   GENCD_TRY(solve_begin(p, &S));
@@ -1101,38 +1129,43 @@ int gencd_solve(gencd_problem* p, gencd_result* out) {
   solve_result(p, &S, out);
   return S.status;
 }
+GENCD_CATCH
 
-int gencd_stats(gencd_problem* p, gencd_result* out) {
+int gencd_stats(gencd_problem* p, gencd_result* out) try {
   GENCD_CHECK_HANDLE(p);
   if (!out) return fail(GENCD_EINVAL, "out is NULL");
   GENCD_TRY(read_scalars(p));
   fill_result(p, out, GENCD_OK, p->stat_iters, p->stat_host_nnz, 0.0);
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_stats_reset(gencd_problem* p) {
+int gencd_stats_reset(gencd_problem* p) try {
   GENCD_CHECK_HANDLE(p);
   GENCD_TRY(reset_counters(p));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_get_w(gencd_problem* p, double* w, int64_t k, int32_t memory) {
+int gencd_get_w(gencd_problem* p, double* w, int64_t k, int32_t memory) try {
   GENCD_CHECK_HANDLE(p);
   if (!w || k != p->k) return fail(GENCD_EINVAL, "w must hold exactly k doubles");
   GENCD_CUDA_TRY(cudaMemcpyAsync(w, p->w, sizeof(double) * k, kind_out(memory), p->stream));
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_get_z(gencd_problem* p, double* z, int64_t n, int32_t memory) {
+int gencd_get_z(gencd_problem* p, double* z, int64_t n, int32_t memory) try {
   GENCD_CHECK_HANDLE(p);
   if (!z || n != p->n) return fail(GENCD_EINVAL, "z must hold exactly n doubles");
   GENCD_CUDA_TRY(cudaMemcpyAsync(z, p->z, sizeof(double) * n, kind_out(memory), p->stream));
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_set_w(gencd_problem* p, const double* w, int64_t k, int32_t memory) {
+int gencd_set_w(gencd_problem* p, const double* w, int64_t k, int32_t memory) try {
   GENCD_CHECK_HANDLE(p);
   if (!w || k != p->k) return fail(GENCD_EINVAL, "w must hold exactly k doubles");
   if (memory == GENCD_HOST) {
@@ -1147,8 +1180,9 @@ int gencd_set_w(gencd_problem* p, const double* w, int64_t k, int32_t memory) {
   if (refit == 1) GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_duality_gap(gencd_problem* p, double* gap, double* primal, double* dual) {
+int gencd_duality_gap(gencd_problem* p, double* gap, double* primal, double* dual) try {
   GENCD_CHECK_HANDLE(p);
   GENCD_TRY(enqueue_evaluate(p, true));
   GENCD_TRY(read_scalars(p));
@@ -1157,8 +1191,9 @@ int gencd_duality_gap(gencd_problem* p, double* gap, double* primal, double* dua
   if (dual) *dual = p->hpin[1] - p->hpin[9];
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_objective(gencd_problem* p, double* objective, double* kkt) {
+int gencd_objective(gencd_problem* p, double* objective, double* kkt) try {
   GENCD_CHECK_HANDLE(p);
   GENCD_TRY(enqueue_evaluate(p));
   GENCD_TRY(read_scalars(p));
@@ -1166,9 +1201,10 @@ int gencd_objective(gencd_problem* p, double* objective, double* kkt) {
   if (kkt) *kkt = p->hpin[0];
   return GENCD_OK;
 }
+GENCD_CATCH
 
 int gencd_propose_at(gencd_problem* p, const int32_t* J, int64_t m, double* delta, double* phi,
-                     int32_t memory) {
+                     int32_t memory) try {
   GENCD_CHECK_HANDLE(p);
   if (m < 0 || (m > 0 && (!J || !delta || !phi))) return fail(GENCD_EINVAL, "bad J / outputs");
   if (m == 0) return GENCD_OK;
@@ -1198,8 +1234,9 @@ int gencd_propose_at(gencd_problem* p, const int32_t* J, int64_t m, double* delt
   dev_free(p, df);
   return rc;
 }
+GENCD_CATCH
 
-int gencd_propose_all(gencd_problem* p, double* delta, double* phi, int32_t memory, double* kkt) {
+int gencd_propose_all(gencd_problem* p, double* delta, double* phi, int32_t memory, double* kkt) try {
   GENCD_CHECK_HANDLE(p);
   GENCD_CUDA_TRY(cudaMemsetAsync(p->dscal, 0, sizeof(double), p->stream));
   GENCD_TRY(launch_propose_all(p, p->u, p->precision == GENCD_F64));
@@ -1210,8 +1247,9 @@ int gencd_propose_all(gencd_problem* p, double* delta, double* phi, int32_t memo
   if (kkt) *kkt = p->hpin[0];
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_spectral_radius(gencd_problem* p, double* rho, int64_t* pstar, int32_t* iters) {
+int gencd_spectral_radius(gencd_problem* p, double* rho, int64_t* pstar, int32_t* iters) try {
   GENCD_CHECK_HANDLE(p);
   int32_t it = 0;
   GENCD_TRY(compute_pstar(p, &it));
@@ -1220,8 +1258,9 @@ int gencd_spectral_radius(gencd_problem* p, double* rho, int64_t* pstar, int32_t
   if (iters) *iters = it;
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_block_pstar(gencd_problem* p, int32_t B, int64_t* pstar, double* rho) {
+int gencd_block_pstar(gencd_problem* p, int32_t B, int64_t* pstar, double* rho) try {
   GENCD_CHECK_HANDLE(p);
   if (B < 1 || B > kMaxShotgunBlocks || B > p->k)
     return fail(GENCD_EINVAL, "B must be in [1, min(k, " + std::to_string(kMaxShotgunBlocks) + ")]");
@@ -1232,15 +1271,17 @@ int gencd_block_pstar(gencd_problem* p, int32_t B, int64_t* pstar, double* rho) 
   }
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_color(gencd_problem* p, int32_t* ncolors) {
+int gencd_color(gencd_problem* p, int32_t* ncolors) try {
   GENCD_CHECK_HANDLE(p);
   GENCD_TRY(run_coloring(p));
   if (ncolors) *ncolors = p->ncolors;
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_get_colors(gencd_problem* p, int32_t* colors, int64_t k, int32_t memory) {
+int gencd_get_colors(gencd_problem* p, int32_t* colors, int64_t k, int32_t memory) try {
   GENCD_CHECK_HANDLE(p);
   if (!colors || k != p->k) return fail(GENCD_EINVAL, "colors must hold exactly k ints");
   if (!p->color) return fail(GENCD_ESTATE, "no colouring yet: call gencd_color or gencd_set_colors");
@@ -1248,8 +1289,9 @@ int gencd_get_colors(gencd_problem* p, int32_t* colors, int64_t k, int32_t memor
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_set_colors(gencd_problem* p, const int32_t* colors, int64_t k, int32_t memory) {
+int gencd_set_colors(gencd_problem* p, const int32_t* colors, int64_t k, int32_t memory) try {
   GENCD_CHECK_HANDLE(p);
   if (!colors || k != p->k) return fail(GENCD_EINVAL, "colors must hold exactly k ints");
   GENCD_TRY(build_csr(p));
@@ -1286,8 +1328,9 @@ int gencd_set_colors(gencd_problem* p, const int32_t* colors, int64_t k, int32_t
   p->ncolors = (int32_t)h[1] + 1;
   return build_color_classes(p);
 }
+GENCD_CATCH
 
-int gencd_permutation(gencd_problem* p, uint64_t seed, int64_t epoch, int64_t m, int32_t* perm) {
+int gencd_permutation(gencd_problem* p, uint64_t seed, int64_t epoch, int64_t m, int32_t* perm) try {
   GENCD_CHECK_HANDLE(p);
   if (m < 0 || epoch < 0 || (m > 0 && !perm)) return fail(GENCD_EINVAL, "bad permutation arguments");
   if (m == 0) return GENCD_OK;
@@ -1301,8 +1344,9 @@ int gencd_permutation(gencd_problem* p, uint64_t seed, int64_t epoch, int64_t m,
   dev_free(p, d);
   return rc;
 }
+GENCD_CATCH
 
-int gencd_profile_enable(gencd_problem* p, int32_t enable) {
+int gencd_profile_enable(gencd_problem* p, int32_t enable) try {
   GENCD_CHECK_HANDLE(p);
   if (!enable) prof_flush(p);
   if (enable && p->prof.pool.empty()) {  // event pairs, created on first use
@@ -1316,8 +1360,9 @@ int gencd_profile_enable(gencd_problem* p, int32_t enable) {
   p->prof.enabled = enable != 0;
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_profile_read(gencd_problem* p, int32_t kernel, double* ms, int64_t* launches, int64_t* calls) {
+int gencd_profile_read(gencd_problem* p, int32_t kernel, double* ms, int64_t* launches, int64_t* calls) try {
   GENCD_CHECK_HANDLE(p);
   if (kernel < 0 || kernel >= K_NUM) return fail(GENCD_EINVAL, "unknown kernel family");
   prof_flush(p);
@@ -1326,8 +1371,9 @@ int gencd_profile_read(gencd_problem* p, int32_t kernel, double* ms, int64_t* la
   if (calls) *calls = p->prof.calls[kernel];
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_set_propose_schedule(gencd_problem* p, int32_t split) {
+int gencd_set_propose_schedule(gencd_problem* p, int32_t split) try {
   GENCD_CHECK_HANDLE(p);
   if (split == -1) return tune_propose_plan(p);
   const bool fusable = p->plan.built && p->plan.light_counter != nullptr;
@@ -1337,8 +1383,9 @@ int gencd_set_propose_schedule(gencd_problem* p, int32_t split) {
   p->plan.fused_split = split;
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_propose_schedule(gencd_problem* p, int32_t* split, double* ms, int32_t nms) {
+int gencd_propose_schedule(gencd_problem* p, int32_t* split, double* ms, int32_t nms) try {
   GENCD_CHECK_HANDLE(p);
   if (nms < 0 || (nms > 0 && !ms)) return fail(GENCD_EINVAL, "ms must hold nms >= 0 values");
   if (split) *split = p->plan.fused_split;
@@ -1346,8 +1393,9 @@ int gencd_propose_schedule(gencd_problem* p, int32_t* split, double* ms, int32_t
   for (int32_t i = 0; i < nms; ++i) ms[i] = (timed && i < 5) ? p->plan.tuned_ms[i] : -1.0;
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_profile_reset(gencd_problem* p) {
+int gencd_profile_reset(gencd_problem* p) try {
   GENCD_CHECK_HANDLE(p);
   prof_flush(p);
   for (int i = 0; i < K_NUM; ++i) {
@@ -1357,5 +1405,6 @@ int gencd_profile_reset(gencd_problem* p) {
   }
   return GENCD_OK;
 }
+GENCD_CATCH
 
 }  // extern "C"

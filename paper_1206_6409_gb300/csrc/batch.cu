@@ -1667,7 +1667,7 @@ static int batch_create(gencd_batch** out, int64_t n, int64_t k, int64_t nnz, co
 
 void gencd_batch_destroy(gencd_batch* b) { free_batch(b); }
 
-int gencd_batch_schedule(gencd_batch* b, int32_t* spmm_kind, int32_t* update_kind, double* ms, int32_t nms) {
+int gencd_batch_schedule(gencd_batch* b, int32_t* spmm_kind, int32_t* update_kind, double* ms, int32_t nms) try {
   if (!b) return bfail(GENCD_EINVAL, "batch handle is NULL");
   if (nms < 0 || (nms > 0 && !ms)) return bfail(GENCD_EINVAL, "ms must hold nms >= 0 values");
   if (spmm_kind) *spmm_kind = b->spmm_kind;
@@ -1675,8 +1675,9 @@ int gencd_batch_schedule(gencd_batch* b, int32_t* spmm_kind, int32_t* update_kin
   for (int32_t i = 0; i < nms; ++i) ms[i] = i < 4 ? b->tuned_ms[i] : -1.0;
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_batch_set_schedule(gencd_batch* b, int32_t spmm_kind, int32_t update_kind) {
+int gencd_batch_set_schedule(gencd_batch* b, int32_t spmm_kind, int32_t update_kind) try {
   if (!b) return bfail(GENCD_EINVAL, "batch handle is NULL");
   if (spmm_kind < -1 || spmm_kind > 1 || update_kind < -1 || update_kind > 1)
     return bfail(GENCD_EINVAL, "schedule kinds are -1 (autotune), 0 or 1");
@@ -1693,22 +1694,25 @@ int gencd_batch_set_schedule(gencd_batch* b, int32_t spmm_kind, int32_t update_k
   drop_graph(b);
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_batch_slots(gencd_batch* b, int32_t* slots) {
+int gencd_batch_slots(gencd_batch* b, int32_t* slots) try {
   if (!b || !slots) return bfail(GENCD_EINVAL, "NULL argument");
   *slots = b->S;
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_batch_lambda_max(gencd_batch* b, int32_t held_out, double* lambda_max) {
+int gencd_batch_lambda_max(gencd_batch* b, int32_t held_out, double* lambda_max) try {
   if (!b || !lambda_max) return bfail(GENCD_EINVAL, "NULL argument");
   int set;
   GENCD_TRY(set_of(b, held_out, &set));
   *lambda_max = b->lam_max[set];
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_batch_set_params(gencd_batch* b, const gencd_params* a) {
+int gencd_batch_set_params(gencd_batch* b, const gencd_params* a) try {
   if (!b || !a) return bfail(GENCD_EINVAL, "NULL argument");
   if (a->variant != GENCD_THREAD_GREEDY && a->variant != GENCD_GREEDY)
     return bfail(GENCD_EINVAL, "the batch runs Thread-Greedy or Greedy");
@@ -1721,9 +1725,10 @@ int gencd_batch_set_params(gencd_batch* b, const gencd_params* a) {
   if (betas) GENCD_TRY(set_betas(b));
   return GENCD_OK;
 }
+GENCD_CATCH
 
 int gencd_batch_set_slot(gencd_batch* b, int32_t slot, int32_t held_out, double lambda, const double* w,
-                         int32_t memory) {
+                         int32_t memory) try {
   GENCD_TRY(check_slot(b, slot));
   int set;
   GENCD_TRY(set_of(b, held_out, &set));
@@ -1743,8 +1748,9 @@ int gencd_batch_set_slot(gencd_batch* b, int32_t slot, int32_t held_out, double 
   GENCD_CUDA_TRY(cudaStreamSynchronize(b->st));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_batch_copy_slot(gencd_batch* b, int32_t dst, int32_t src, int32_t held_out, double lambda) {
+int gencd_batch_copy_slot(gencd_batch* b, int32_t dst, int32_t src, int32_t held_out, double lambda) try {
   GENCD_TRY(check_slot(b, dst));
   GENCD_TRY(check_slot(b, src));
   if (b->h_set[src] < 0) return bfail(GENCD_ESTATE, "source slot is not active");
@@ -1763,15 +1769,17 @@ int gencd_batch_copy_slot(gencd_batch* b, int32_t dst, int32_t src, int32_t held
   GENCD_CUDA_TRY(cudaStreamSynchronize(b->st));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_batch_clear_slot(gencd_batch* b, int32_t slot) {
+int gencd_batch_clear_slot(gencd_batch* b, int32_t slot) try {
   GENCD_TRY(check_slot(b, slot));
   GENCD_TRY(slot_clear(b, slot));
   GENCD_CUDA_TRY(cudaStreamSynchronize(b->st));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_batch_get_w(gencd_batch* b, int32_t slot, double* w, int64_t k, int32_t memory) {
+int gencd_batch_get_w(gencd_batch* b, int32_t slot, double* w, int64_t k, int32_t memory) try {
   GENCD_TRY(check_slot(b, slot));
   if (!w || k != b->k) return bfail(GENCD_EINVAL, "w must hold exactly k doubles");
   k_b_get_w<<<grid_for(b->k, kThreads, b->X->num_sms * 8), kThreads, 0, b->st>>>(b->w, b->k, b->S, slot, b->tmp_k);
@@ -1780,16 +1788,18 @@ int gencd_batch_get_w(gencd_batch* b, int32_t slot, double* w, int64_t k, int32_
   GENCD_CUDA_TRY(cudaStreamSynchronize(b->st));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_batch_iterate(gencd_batch* b, int64_t iters, int32_t sync) {
+int gencd_batch_iterate(gencd_batch* b, int64_t iters, int32_t sync) try {
   if (!b) return bfail(GENCD_EINVAL, "batch handle is NULL");
   if (iters < 0) return bfail(GENCD_EINVAL, "iters must be >= 0");
   for (int64_t i = 0; i < iters; ++i) GENCD_TRY(enqueue_step(b));
   if (sync) GENCD_CUDA_TRY(cudaStreamSynchronize(b->st));
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_batch_objective(gencd_batch* b, double* objective, double* kkt) {
+int gencd_batch_objective(gencd_batch* b, double* objective, double* kkt) try {
   if (!b) return bfail(GENCD_EINVAL, "batch handle is NULL");
   GENCD_TRY(enqueue_propose(b, false));
   std::vector<double> kv;
@@ -1808,8 +1818,9 @@ int gencd_batch_objective(gencd_batch* b, double* objective, double* kkt) {
     for (size_t q = 0; q < act.size(); ++q) objective[act[q]] = ob[q];
   return GENCD_OK;
 }
+GENCD_CATCH
 
-int gencd_batch_propose(gencd_batch* b, double* delta, double* phi, int32_t memory) {
+int gencd_batch_propose(gencd_batch* b, double* delta, double* phi, int32_t memory) try {
   if (!b || !delta || !phi) return bfail(GENCD_EINVAL, "NULL argument");
   GENCD_TRY(enqueue_propose(b, false));
   const size_t m = (size_t)b->S * b->k;
@@ -1828,6 +1839,7 @@ int gencd_batch_propose(gencd_batch* b, double* delta, double* phi, int32_t memo
   cudaFree(df);
   return rc;
 }
+GENCD_CATCH
 
 static int batch_path(gencd_batch* b, const gencd_path* path, gencd_path_solve* solves, double* w_out,
                       gencd_result* out);

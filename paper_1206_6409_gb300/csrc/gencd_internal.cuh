@@ -29,6 +29,13 @@ namespace gencd {
 void set_error(const std::string& msg);
 const char* last_error();
 
+// No C++ exception crosses the C boundary: an entry point is a function try
+// block that ends in GENCD_CATCH.  caught() sets the message of the exception
+// being handled (host memory ran out) and returns GENCD_ENOMEM.
+int caught() noexcept;
+#define GENCD_CATCH                                                                           \
+  catch (...) { return ::gencd::caught(); }
+
 #define GENCD_CUDA_TRY(expr)                                                                  \
   do {                                                                                        \
     cudaError_t e_ = (expr);                                                                  \

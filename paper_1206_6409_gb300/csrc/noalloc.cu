@@ -268,7 +268,7 @@ extern "C" int gencd_propose_all_noalloc(int64_t n, int64_t k, int64_t nnz, cons
                                          const int32_t* row_idx, const double* val, const double* y,
                                          const double* z, const double* w, int32_t loss, double lambda,
                                          int32_t beta_mode, double* delta, double* phi, double* kkt,
-                                         void* stream) {
+                                         void* stream) try {
   set_error("");
   if (n < 1 || k < 1 || nnz < 0) return fail_plan("need n >= 1, k >= 1, nnz >= 0");
   if (k > kNoAllocMaxCols || nnz > kNoAllocMaxNnz)
@@ -312,3 +312,4 @@ extern "C" int gencd_propose_all_noalloc(int64_t n, int64_t k, int64_t nnz, cons
   GENCD_CUDA_TRY(cudaGetLastError());
   return GENCD_OK;
 }
+GENCD_CATCH

@@ -68,7 +68,7 @@ struct Server {
   double held = 0.0;      // estimates of the requests in flight
   int inflight = 0;       // slots loading or running
   int err = GENCD_OK;
-  std::string err_msg;
+  const char* err_msg = "";
   std::vector<Slot> slots;
   std::deque<int> started;  // slots the loader has started (handed to the stepper)
   cudaMemPool_t pool = nullptr;
@@ -174,17 +174,23 @@ bool load(Server* S, int i) {
   return true;
 }
 
-// admits requests into free slots in arrival order and loads them
-void loader(Server* S) {
-  if (!S->service && cudaSetDevice(S->device) != cudaSuccess) {
-    cudaGetLastError();
+// stops the loader and the stepper; the first error is the call's
+void stop(Server* S, int err, const char* msg) {
+  {
     std::lock_guard<std::mutex> g(S->mu);
     if (S->err == GENCD_OK) {
-      S->err = GENCD_ECUDA;
-      S->err_msg = "the loader thread could not select the device";
+      S->err = err;
+      S->err_msg = msg;
     }
-    S->cv.notify_all();
-    return;
+  }
+  S->cv.notify_all();
+}
+
+// admits requests into free slots in arrival order and loads them
+void load_requests(Server* S) {
+  if (!S->service && cudaSetDevice(S->device) != cudaSuccess) {
+    cudaGetLastError();
+    return stop(S, GENCD_ECUDA, "the loader thread could not select the device");
   }
   for (;;) {
     int i = -1;
@@ -230,6 +236,14 @@ void loader(Server* S) {
       S->slots[(size_t)i].state = kRunning;
       S->started.push_back(i);
     }
+  }
+}
+
+void loader(Server* S) {  // the thread: an exception ends the call
+  try {
+    load_requests(S);
+  } catch (...) {
+    stop(S, GENCD_ENOMEM, "host allocation failed in the loader thread");
   }
 }
 
@@ -320,11 +334,15 @@ int run(Server& S) {
   std::thread th;
   try {
     th = std::thread(loader, &S);
-  } catch (const std::exception& e) {  // no exception crosses the C ABI
+  } catch (const std::exception& e) {
     set_error(std::string("loader thread creation failed: ") + e.what());
     return GENCD_ENOMEM;
   }
-  stepper(&S);
+  try {
+    stepper(&S);
+  } catch (...) {  // the loader thread still runs
+    stop(&S, GENCD_ENOMEM, "host allocation failed");
+  }
   if (S.err != GENCD_OK) S.cv.notify_all();
   th.join();
   // a request the loader started after the stepper stopped on an error
@@ -402,7 +420,7 @@ void teardown(Server& S) {
 using namespace gencd;
 
 extern "C" int gencd_serve(const gencd_request* requests, int64_t nreq, const gencd_serve_params* params,
-                           gencd_response* out, double* const* w_out) {
+                           gencd_response* out, double* const* w_out) try {
   GENCD_TRY(check_stream(requests, nreq, params, out));
   std::memset(out, 0, sizeof(gencd_response) * (size_t)nreq);
   Server S;
@@ -421,14 +439,20 @@ extern "C" int gencd_serve(const gencd_request* requests, int64_t nreq, const ge
     return GENCD_ECUDA;
   }
   S.budget = (double)free_b * params->hbm_fraction;
-  int rc = setup(S, params->workers);
-  if (rc == GENCD_OK) rc = run(S);
+  int rc;
+  try {
+    rc = setup(S, params->workers);
+    if (rc == GENCD_OK) rc = run(S);
+  } catch (...) {
+    rc = caught();
+  }
   teardown(S);
   return rc;
 }
+GENCD_CATCH
 
 extern "C" int gencd_serve_dry_run(const gencd_request* requests, int64_t nreq, const gencd_serve_params* params,
-                                   double budget_bytes, const double* service_s, gencd_response* out) {
+                                   double budget_bytes, const double* service_s, gencd_response* out) try {
   GENCD_TRY(check_stream(requests, nreq, params, out));
   if (!(budget_bytes > 0.0) || (nreq > 0 && !service_s)) {
     set_error("budget_bytes must be > 0 and service_s given");
@@ -450,3 +474,4 @@ extern "C" int gencd_serve_dry_run(const gencd_request* requests, int64_t nreq, 
   GENCD_TRY(setup(S, params->workers));
   return run(S);
 }
+GENCD_CATCH
