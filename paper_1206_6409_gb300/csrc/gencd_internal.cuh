@@ -128,28 +128,23 @@ struct ProposePlan {
   // light columns
   int64_t nlight = 0, light_nnz = 0, light_ntiles = 0;
   int32_t* light_cols = nullptr;
-  int64_t* light_col_ptr = nullptr;
   int32_t* light_row = nullptr;
   void* light_val = nullptr;
   int32_t* light_tile_lc = nullptr;  // light column of each 256-entry tile's first entry
   uint8_t* lmask = nullptr;          // per 8 light entries: bit i = entry 8g + i starts a column
   // heavy columns
   int64_t nheavy = 0, entries = 0, npairs = 0;
-  int32_t* heavy_cols = nullptr;   // original column of heavy id h
   uint16_t* s_row = nullptr;       // slab-local row of each entry
   void* s_val = nullptr;           // value of each entry (padding: 0)
   uint8_t* pmask = nullptr;        // per 8 entries: bit i = entry 8g + i starts a pair (pairs in entry order)
   uint32_t* pair_col = nullptr;    // the column j of each pair (its run sums go to g_j)
   uint32_t* slab_off = nullptr;    // first entry of each slab (nslabs + 1)
-  // tiles of the entries, inside one slab each: of the row-slab kernel, and of
-  // the kernel that runs both passes (if there are light columns, FP32)
-  struct Tiles {
-    int64_t count = 0;
-    uint32_t* pair = nullptr;        // pair holding the tile's first entry
-    int32_t* slab = nullptr;
-    int32_t* slab_begin = nullptr;   // nslabs + 1
-    int32_t* cta_begin = nullptr;    // grid + 1
-  } tiles, fused;
+  // tiles of the entries, inside one slab each
+  int64_t ntiles = 0;
+  uint32_t* tile_pair = nullptr;        // pair holding the tile's first entry
+  int32_t* tile_slab = nullptr;
+  int32_t* slab_tile_begin = nullptr;   // nslabs + 1
+  int32_t* cta_tile_begin = nullptr;    // grid + 1
   int grid = 0;
   // both passes in one kernel (k_propose_fused) when fused_split > 0 (the
   // number of warps that start on the row slabs; 0: two kernels), chosen by

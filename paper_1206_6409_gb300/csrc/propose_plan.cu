@@ -52,7 +52,6 @@ constexpr int kSlabDepthF32 = 1;
 constexpr int kSlabDepthF64 = 0;
 constexpr int kSlabItemsF32 = 8;
 constexpr int kSlabItemsF64 = 16;
-constexpr int kFusedItems = 8;  // the kernel that runs both passes (FP32): entries per lane
 constexpr int kSlabPad = kSlabTile;  // slabs are padded to whole tiles
 constexpr int kSlabZeroSlot = 4;   // shared u slots past the slab (16 B); the first holds 0
 
@@ -614,8 +613,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   }
 }
 
-static SlabTiles tiles_of(const ProposePlan& P, const ProposePlan::Tiles& t) {
-  return SlabTiles{t.pair, t.slab, t.slab_begin, t.cta_begin, P.slab_off};
+static SlabTiles tiles_of(const ProposePlan& P) {
+  return SlabTiles{P.tile_pair, P.tile_slab, P.slab_tile_begin, P.cta_tile_begin, P.slab_off};
 }
 
 // the two streaming passes for one value storage SV (V compute type, U type
@@ -630,8 +629,8 @@ constexpr int kNumFusedSplits = 4;
 template <typename V, typename U, typename G, typename SV, int SW>
 static cudaError_t launch_fused(gencd_problem* p, const void* u_vec, size_t smem) {
   ProposePlan& P = p->plan;
-  return launch_overlapped(k_propose_fused<V, U, G, kFusedThreads, SW, 1, kFusedItems, SV>, P.grid, kFusedThreads, smem,
-                           launch_on(p), P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P, P.fused),
+  return launch_overlapped(k_propose_fused<V, U, G, kFusedThreads, SW, 1, kSlabItemsF32, SV>, P.grid, kFusedThreads, smem,
+                           launch_on(p), P.s_row, (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P),
                            P.light_row, (const SV*)P.light_val, P.lmask, P.light_tile_lc, P.light_cols,
                            P.light_nnz, P.light_ntiles, P.light_counter, (const U*)u_vec, p->n, P.slab_rows,
                            (G*)p->gnat, P.second);
@@ -677,7 +676,7 @@ static int launch_plan_passes(gencd_problem* p, const void* u_vec) {
     prof_begin(p, K_PROPOSE_SLABS, &e1);
     const cudaError_t err = launch_overlapped(
         k_propose_slabs<V, U, G, THREADS, DEPTH, ITEMS, SV>, P.grid, THREADS, smem, launch_on(p), P.s_row,
-        (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P, P.tiles), (const U*)u_vec, p->n, P.slab_rows,
+        (const SV*)P.s_val, P.pmask, P.pair_col, tiles_of(P), (const U*)u_vec, p->n, P.slab_rows,
         (G*)p->gnat, P.second);
     prof_end(p, e1);
     GENCD_CUDA_TRY(err);
@@ -693,13 +692,13 @@ static int set_slab_smem(const ProposePlan& P) {
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   if constexpr (sizeof(V) == 4) {
     if (P.light_counter) {
-      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 20, 1, kFusedItems, SV>,
+      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 20, 1, kSlabItemsF32, SV>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 24, 1, kFusedItems, SV>,
+      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 24, 1, kSlabItemsF32, SV>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 28, 1, kFusedItems, SV>,
+      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 28, 1, kSlabItemsF32, SV>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 31, 1, kFusedItems, SV>,
+      GENCD_CUDA_TRY(cudaFuncSetAttribute(k_propose_fused<V, U, G, kFusedThreads, 31, 1, kSlabItemsF32, SV>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     }
   }
@@ -1084,7 +1083,11 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
 
   // classify, number and offset the columns
   uint32_t *hid, *lid, *loff, *tmp;
+  int32_t* heavy_cols;     // original column of heavy id h
+  int64_t* light_col_ptr;  // of the light columns' copy
   Arena cols;
+  cols.add(&heavy_cols, k);
+  cols.add(&light_col_ptr, k + 1);
   cols.add(&hid, k + 1);
   cols.add(&lid, k + 1);
   cols.add(&loff, k + 1);
@@ -1112,9 +1115,7 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   P.light_ntiles = (P.light_nnz + kLightTile - 1) / kLightTile;
   const bool fusable = P.forms;
   Arena light;
-  light.add(&P.heavy_cols, P.nheavy);
   light.add(&P.light_cols, P.nlight);
-  light.add(&P.light_col_ptr, P.nlight + 1);
   light.add(&P.light_row, lpad);
   light.add((char**)&P.light_val, lpad * (int64_t)vsz);
   light.add(&P.light_tile_lc, P.light_ntiles + 1);
@@ -1124,7 +1125,7 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   GENCD_TRY(dev_alloc_bytes(p, &P.mem[0], light.bytes()));
   light.place(P.mem[0]);
   k_plan_columns<<<grid_for(k + 1, kThreads, g), kThreads, 0, st>>>(p->col_ptr, k, P.heavy_min, hid, lid, loff,
-                                                                     P.heavy_cols, P.light_cols, P.light_col_ptr);
+                                                                     heavy_cols, P.light_cols, light_col_ptr);
   GENCD_CUDA_TRY(cudaGetLastError());
   if (P.nlight > 0) {
     if (p->vmode == kValNone) {  // padding has no value to zero it: it gathers u[n] = 0 instead
@@ -1136,7 +1137,7 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
       GENCD_CUDA_TRY(cudaMemsetAsync((char*)P.light_val + vsz * P.light_nnz, 0, vsz * (lpad - P.light_nnz), st));
     }
     GENCD_CUDA_TRY(cudaMemsetAsync(P.lmask, 0, 4 * (size_t)lwords, st));
-    GENCD_TRY(launch_tile_map_of(p, P.light_col_ptr, P.nlight, P.light_ntiles, P.light_tile_lc, kLightTile));
+    GENCD_TRY(launch_tile_map_of(p, light_col_ptr, P.nlight, P.light_ntiles, P.light_tile_lc, kLightTile));
   }
   if (fusable) GENCD_CUDA_TRY(cudaMemsetAsync(P.light_counter, 0, 2 * sizeof(unsigned int), st));
 
@@ -1155,7 +1156,7 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   std::vector<int64_t> hb(R + 2, 0), hp(R + 1, 0);
   if (P.nheavy > 0) {
     k_plan_segments<<<grid_for(runs + 1, kThreads, p->num_sms * 32), kThreads, 0, st>>>(
-        p->col_ptr, p->row_idx, P.heavy_cols, P.nheavy, runs, R, P.slab_rows, seg, pos, pair);
+        p->col_ptr, p->row_idx, heavy_cols, P.nheavy, runs, R, P.slab_rows, seg, pos, pair);
     GENCD_TRY(exclusive_scan(p, pos, pos, runs + 1, rtmp));
     GENCD_TRY(exclusive_scan(p, pair, pair, runs + 1, rtmp));
     k_plan_slab_begins<<<1, kThreads, 0, st>>>(pos, pair, P.nheavy, R, slab_begin);
@@ -1166,13 +1167,11 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   P.npairs = hb[R + 1];
   for (int r = 0; r < R; ++r) hp[r + 1] = hp[r] + ((hb[r + 1] - hb[r] + kSlabPad - 1) / kSlabPad) * kSlabPad;
   P.entries = hp[R];
+  const int64_t tile = 32LL * (f64 ? kSlabItemsF64 : kSlabItemsF32);
   if (P.entries >= (int64_t(1) << 32)) return fail_plan("heavy entries exceed 2^32");
 
   if (P.nheavy > 0) {
-    // tiles of both sizes in use inside each slab, and contiguous runs of
-    // tiles per CTA
-    ProposePlan::Tiles* sets[2] = {&P.tiles, fusable ? &P.fused : nullptr};
-    const int64_t tile[2] = {32LL * (f64 ? kSlabItemsF64 : kSlabItemsF32), 32LL * kFusedItems};
+    // tiles inside each slab, and contiguous runs of tiles per CTA
     const int64_t mask_words = (P.entries + 31) / 32;  // start bits: one byte per 8 entries
     std::vector<uint32_t> off(R + 1);
     for (int r = 0; r <= R; ++r) off[r] = (uint32_t)hp[r];
@@ -1182,28 +1181,22 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
     slabs.add((uint32_t**)&P.pmask, mask_words);
     slabs.add(&P.pair_col, P.npairs);
     slabs.add(&P.slab_off, R + 1);
-    for (int i = 0; i < 2; ++i)
-      if (sets[i]) {
-        sets[i]->count = P.entries / tile[i];
-        slabs.add(&sets[i]->pair, sets[i]->count);
-        slabs.add(&sets[i]->slab, sets[i]->count);
-        slabs.add(&sets[i]->slab_begin, R + 1);
-        slabs.add(&sets[i]->cta_begin, P.grid + 1);
-      }
+    P.ntiles = P.entries / tile;
+    slabs.add(&P.tile_pair, P.ntiles);
+    slabs.add(&P.tile_slab, P.ntiles);
+    slabs.add(&P.slab_tile_begin, R + 1);
+    slabs.add(&P.cta_tile_begin, P.grid + 1);
     GENCD_TRY(dev_alloc_bytes(p, &P.mem[1], slabs.bytes()));
     slabs.place(P.mem[1]);
     GENCD_CUDA_TRY(cudaMemcpyAsync(pad_off, hp.data(), 8 * (R + 1), cudaMemcpyHostToDevice, st));
     GENCD_CUDA_TRY(cudaMemcpyAsync(P.slab_off, off.data(), 4 * (R + 1), cudaMemcpyHostToDevice, st));
     GENCD_CUDA_TRY(cudaMemsetAsync(P.pmask, 0, 4 * (size_t)mask_words, st));
-    std::vector<int32_t> tb(R + 1), ctb;  // pageable sources: read when the copy returns
-    for (int i = 0; i < 2; ++i)
-      if (sets[i]) {
-        for (int r = 0; r <= R; ++r) tb[r] = (int32_t)(hp[r] / tile[i]);
-        ctb = split_tiles(tb, P.grid, tile[i]);
-        GENCD_CUDA_TRY(cudaMemcpyAsync(sets[i]->slab_begin, tb.data(), 4 * (R + 1), cudaMemcpyHostToDevice, st));
-        GENCD_CUDA_TRY(cudaMemcpyAsync(sets[i]->cta_begin, ctb.data(), 4 * (P.grid + 1), cudaMemcpyHostToDevice, st));
-        GENCD_CUDA_TRY(cudaStreamSynchronize(st));
-      }
+    std::vector<int32_t> tb(R + 1);
+    for (int r = 0; r <= R; ++r) tb[r] = (int32_t)(hp[r] / tile);
+    const std::vector<int32_t> ctb = split_tiles(tb, P.grid, tile);
+    GENCD_CUDA_TRY(cudaMemcpyAsync(P.slab_tile_begin, tb.data(), 4 * (R + 1), cudaMemcpyHostToDevice, st));
+    GENCD_CUDA_TRY(cudaMemcpyAsync(P.cta_tile_begin, ctb.data(), 4 * (P.grid + 1), cudaMemcpyHostToDevice, st));
+    GENCD_CUDA_TRY(cudaStreamSynchronize(st));  // the host arrays go here
   }
   if (p->nnz > 0) {
     if (f64)
@@ -1218,11 +1211,8 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   }
   P.fused_split = 0;
   if (P.nheavy > 0) {
-    for (ProposePlan::Tiles* t : {&P.tiles, &P.fused})
-      if (t->count > 0)
-        k_plan_tiles<<<grid_for(t->count, kThreads, g), kThreads, 0, st>>>(t->slab_begin, pad_off, R, t->count,
-                                                                            P.entries / t->count, pair_start, P.npairs,
-                                                                            t->pair, t->slab);
+    k_plan_tiles<<<grid_for(P.ntiles, kThreads, g), kThreads, 0, st>>>(P.slab_tile_begin, pad_off, R, P.ntiles, tile,
+                                                                      pair_start, P.npairs, P.tile_pair, P.tile_slab);
     GENCD_CUDA_TRY(cudaGetLastError());
     // both passes may run in one kernel when there are light and heavy columns
     // (FP32 arithmetic: FP64 stages do not fit the fused kernel's registers);
