@@ -371,17 +371,22 @@ __device__ __forceinline__ int scan_round_f32(float* gacc, const float* w32,
 //
 // Bound: latency (a few dependent loads and block reductions per CTA), so
 // what counts is that every chunk is resident at once and that no thread
-// walks columns one after another: the launcher cuts to about 8 CTAs per SM.
+// walks columns one after another: the launcher cuts to the CTAs that an SM
+// holds, 8 with FP32's 32 registers a thread and 5 with FP64's 44.
 // Chunks of 4,096 columns, a thread walking its 16 columns serially, and a
 // second launch for the slots took 34.5 + 5.5 us on k = 100,000, B = 1 (25
 // CTAs), 44.7 + 5.7 us on k = 500,000, B = 16 and, in FP64, 62.5 + 4.1 us on
-// k = 400,000, B = 128; this takes 11.1, 11.0 and 21.7 us (ncu, cold caches).
-// One CTA per partition, the many-partitions form, is the same work as before
-// (15 us on k = 4,000,000, B = 1,024).  The active columns are queued: testing
-// and evaluating them in place, four per thread, serialised their loads of
-// beta_j (89 us on k = 4,000,000).
+// k = 400,000, B = 128; this takes 11.1, 11.0 and 20.1 us (ncu, cold caches; the
+// last cut to 8 a SM, in two waves, 25.4).  One CTA per partition, the
+// many-partitions form, takes 22.5 us on k = 4,000,000, B = 1,024 with two sums a
+// column (15 with one).  The active columns are queued: testing and evaluating
+// them in place, four per thread, serialised their loads of beta_j (89 us on k =
+// 4,000,000).
 template <typename G>
-__global__ void __launch_bounds__(kThreads)
+constexpr int kAcceptPerSm = sizeof(G) == 4 ? 8 : 5;
+
+template <typename G>
+__global__ void __launch_bounds__(kThreads, kAcceptPerSm<G>)
     k_accept_partitions(G* gacc, AcceptCols c, int64_t B, int per, int64_t chunk,
                         const int64_t* __restrict__ part_lo, int want_kkt, uint64_t* slot_m, int32_t* slot_j,
                         double* slot_x, unsigned int* slot_cnt, int32_t* list_j, double* list_d, uint64_t* list_m,
@@ -706,7 +711,7 @@ static int ensure_part_bounds(gencd_problem* p, int64_t B) {
 }
 
 // Chunk size of k_accept_partitions: the smallest of 256, 512, ... columns
-// that keeps the launch within 8 CTAs per SM (all resident at once); a
+// that keeps the launch within the CTAs that are resident at once; a
 // partition that fits one chunk is one CTA and needs no slots.
 int launch_finalize_accept(gencd_problem* p, int64_t B, bool want_kkt, bool apply) {
   uint64_t b64;
@@ -716,7 +721,7 @@ int launch_finalize_accept(gencd_problem* p, int64_t B, bool want_kkt, bool appl
   GENCD_TRY(ensure_part_bounds(p, B));
   const AcceptCols c{p->w, p->bj, p->ib, p->w32, p->bj32, p->ib32, p->col_val, p->plan.second, 1.0 / (double)p->n, p->lambda,
                      (float)(1.0 / (double)p->n), (float)p->lambda, b64, b32};
-  const int64_t resident = (int64_t)p->num_sms * 8;
+  const int64_t resident = (int64_t)p->num_sms * (f64 ? kAcceptPerSm<double> : kAcceptPerSm<float>);
   const int64_t most = (p->k + B - 1) / B;  // columns of the largest partition
   int64_t chunk = kThreads;
   while (chunk < most && B * ((most + chunk - 1) / chunk) > resident) chunk *= 2;
