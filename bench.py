@@ -782,7 +782,7 @@ def run_gencd(args):
         gb.gencd_set_propose_schedule(p.h, args.propose_split)
     split, tuned = gb.gencd_propose_schedule(p.h)
     schedule = {"fused_split": split, "candidates_ms": tuned,
-                "form": "separate light and slab kernels" if split == 0 else
+                "form": "a kernel each for the row slabs and the light columns, if any" if split == 0 else
                 f"one kernel, {split} of 32 warps per SM start on the row slabs"}
     for _ in range(args.warmup):
         p.iterate(1, sync=False)
@@ -816,8 +816,8 @@ def run_gencd(args):
     value = nnz_total / (ms / 1000.0)
 
     # roofline of the dominant kernel: the streaming propose's pass over X
-    # (k_propose_fused, or the two separate passes when the autotuner keeps
-    # them), with what it must move as its algorithmic bytes: the X stream
+    # (k_propose_fused, or the separate passes that run: k_propose_slabs,
+    # k_propose_light_runs or both), with what it must move as its algorithmic bytes: the X stream
     # (row index + stored value per non-zero; u is L2-resident) and the
     # gradient it writes (one g_j per column, FP32 or FP64); the family (every
     # kernel of the propose over all columns) counts a column pointer and an
@@ -831,7 +831,8 @@ def run_gencd(args):
     if prof["propose_fused"][2]:
         dom_name, (dom_ms, _, dom_n) = "k_propose_fused", prof["propose_fused"]
     else:
-        dom_name = "k_propose_light_runs + k_propose_slabs"
+        passes = {"propose_light": "k_propose_light_runs", "propose_slabs": "k_propose_slabs"}
+        dom_name = " + ".join(name for k, name in passes.items() if prof[k][2])
         dom_ms = prof["propose_light"][0] + prof["propose_slabs"][0]
         dom_n = max(prof["propose_light"][2], prof["propose_slabs"][2])
     achieved = x_bytes / (dom_ms / dom_n / 1000.0) / 1e9 if dom_n else None

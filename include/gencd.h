@@ -321,7 +321,8 @@ int gencd_profile_reset(gencd_problem* p);
 /*
  * Schedule of the streaming propose over all columns, chosen at create by the
  * library's autotuner (not in the paper): the row-slab pass over the heavy
- * columns and the light-column pass run as two kernels (*split = 0) or as one
+ * columns and the light-column pass run as kernels of their own (*split = 0; one
+ * of them alone where the columns are all heavy or all light) or as one
  * kernel whose first *split of 32 warps per SM start on the row slabs and the
  * rest on a shared pool of light tiles.  ms[0..nms) receives the autotuner's
  * mean time per invocation (ms) of the two kernels, then of the splits 20,
@@ -350,15 +351,17 @@ int gencd_set_propose_schedule(gencd_problem* p, int32_t split);
  * bounds the input: k <= 524,288 columns and nnz <= 33,554,432 non-zeros;
  * larger inputs, a non-finite or negative lambda return GENCD_EINVAL.  The
  * first call on each device looks up the scratch's device address
- * (cudaGetSymbolAddress); make that first call before capturing any stream.  All calls on a device share the scratch and
- * each clears what it accumulates into, so calls that overlap on the GPU
- * (no stream ordering between them) race.
+ * (cudaGetSymbolAddress); make that first call before capturing any stream.
+ * All calls on a device share the scratch and each clears what it accumulates
+ * into, so calls that overlap on the GPU (no stream ordering between them)
+ * race.
  *
  * Inputs (device memory of the current device, not re-validated: they must
  * satisfy the CSC rules of gencd_create): col_ptr int64[k+1], row_idx
  * int32[nnz], val double[nnz], y double[n], z = Xw double[n], w double[k];
  * loss, lambda >= 0, beta_mode as in gencd_params.  u = l'(y, z) is evaluated
- * into the scratch (n <= 524,288 and n <= nnz) or per non-zero.  Outputs (device): delta, phi double[k], kkt double[1].
+ * into the scratch (n <= 524,288 and n <= nnz) or per non-zero.  Outputs
+ * (device): delta, phi double[k], kkt double[1].
  * Work is enqueued on `stream`; the call returns without synchronising.
  */
 int gencd_propose_all_noalloc(int64_t n, int64_t k, int64_t nnz, const int64_t* col_ptr, const int32_t* row_idx,

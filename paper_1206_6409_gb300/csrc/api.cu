@@ -237,7 +237,6 @@ static int effective_B(const gencd_problem* p) {
   return (int)B;
 }
 
-// KKT violation (dscal[0]) and objective (dscal[1]) of the current state
 // KKT violation (dscal[0]), objective (dscal[1]) and, with gap, the duality
 // gap (dscal[9]) of the current state (the gap's conjugates cost FP64
 // transcendentals on every row: only where a gap is asked for)

@@ -764,8 +764,9 @@ __global__ void k_b_fill_col(const double* __restrict__ y, const uint8_t* __rest
 // Slots that a path starts, finishes or clears together, passed by value: one
 // launch for all of them, lanes over slots, whose values of a row or column
 // are contiguous.  A path of 32 chains of two solves on 4e6 non-zeros, 60 steps
-// of 32 slots, takes 9.3 ms; slot by slot, with five launches and six copies a
-// start and a copy and a wait for every w, it took 13.9.
+// of 32 slots, took 9.3 ms with them (before the step's launches overlapped); slot
+// by slot, with five launches and six copies a start and a copy and a wait for
+// every w, 13.9.  Its host copies vary: both with the overlap, 12.5 -> 9.2 to 9.6.
 struct SlotWave {
   int32_t m = 0;
   int16_t slot[kBatchMaxSlots];

@@ -226,12 +226,13 @@ constexpr int kRoundCols = kColsPerThread * kThreads;  // columns a CTA scans pe
 // processed packed (one active column per thread), so FP64 work is
 // proportional to the number of active columns, not to the warps that hold
 // one.  second: offset of a column's second sum (0: none).  scale (index-only
-// storage): each column's value, applied to its sum.  Returns the queue length; the queue holds (j, raw sum, w_j).
+// storage): each column's value, applied to its sum.  Returns the queue length;
+// the queue holds (j, raw sum, w_j).
 template <typename G>
 __device__ __forceinline__ int scan_round(G* gacc, const double* w, int64_t base,
                                           int64_t hi, uint64_t lnb64, uint32_t lnb32, int64_t second,
-                                          const float* __restrict__ scale, int* s_n, int64_t* s_j, double* s_g, double* s_w, double* delta,
-                                          double* phi) {
+                                          const float* __restrict__ scale, int* s_n, int64_t* s_j, double* s_g,
+                                          double* s_w, double* delta, double* phi) {
   G ga[kColsPerThread];
   double wv[kColsPerThread];
 #pragma unroll

@@ -12,6 +12,7 @@
 //    columns of one colour class share no row (Section 4.1), so each warp
 //    proposes its column and then writes z and u of its own rows with plain
 //    stores -- no atomics, no second pass.
+//  * k_update_refresh: both passes over a short list in one launch.
 //  * k_w_segments, k_scatter_segments: z = Xw from the columns with w_j != 0
 //    (a warm start is sparse); k_csr_spmv: z = Xw by rows, for a dense w.
 //  * k_fill_u: u from z for all rows.
@@ -178,10 +179,10 @@ __global__ void __launch_bounds__(kListThreads)
 
 // u_i = l'(y_i, z_i) on the rows of the applied columns, or on all rows when
 // the iteration touched at least n entries (one dense pass is cheaper then).
-// Neighbouring warps of the range lie on different SMs: the logistic
-// derivative takes some 50 FP64 operations, which an SM starts about two a
-// cycle, so few rows have to be spread over all of them (FP64, 100,000 rows:
-// 7.7 us, 12.1 with neighbouring warps in one CTA).
+// Neighbouring warps of the range lie on different SMs: in FP64 the logistic
+// derivative takes some 12 FP64 operations, which an SM starts about two a
+// cycle, so few rows have to be spread over all of them (100,000 rows: 7.8 us,
+// 9.5 with neighbouring warps in one CTA; ncu).
 template <typename U, bool SCAN>
 __global__ void __launch_bounds__(kListThreads)
     k_refresh_flat(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
@@ -666,7 +667,7 @@ int launch_update_refresh(gencd_problem* p, const int32_t* J, const double* d, i
 }
 
 // u on the rows of the list's applied columns, after z.  counted: the list's
-// counts are in the counters already (launch_update_list); else (Shotgun's
+// counts are in the counters already (launch_update_refresh); else (Shotgun's
 // fused step) they are added here.
 int launch_refresh_list(gencd_problem* p, const int32_t* J, int64_t m, bool counted) {
   if (m <= 0) return GENCD_OK;

@@ -36,8 +36,8 @@ constexpr int kSlabBytes = 192 * 1024;
 // Entries of a slab are stored in tiles of kSlabTile, in the order in which a
 // warp's lanes load them: a lane owns 16 consecutive entries (or 8, taking half
 // a tile at a time), and its v-th 16-byte vector lies next to the other lanes'
-// v-th ones, so every load of a warp is one contiguous 512 bytes whatever the
-// lane's share (slab_at, load_lane).
+// v-th ones, so a load of a warp is one contiguous 512 bytes with 16 entries a
+// lane and two runs of 256 with 8 (slab_at, load_lane).
 constexpr int kSlabTile = 512;
 // Shape of the row-slab kernel: threads, tiles of loads in flight beyond the
 // current one, entries per lane.  FP32 is bound by instructions and loads in
@@ -45,7 +45,9 @@ constexpr int kSlabTile = 512;
 // 768 / 1 / 16 92 and 512 / 1 / 16 112.  FP64 is bound by its pipe, and a lane's
 // 16 entries halve the additions that combine the lanes: 10 Thread-Greedy
 // iterations on 2e7 non-zeros take 1259 us with 768 / 0 / 16, 1284 with 512 / 1 /
-// 16, 1322 with 1024 / 0 / 8.
+// 16, 1322 with 1024 / 0 / 8.  768 threads leave 80 registers each, which the FP64
+// kernel exceeds by 14 words (56 bytes spilled a thread); with a tile in flight
+// it would spill more.
 constexpr int kSlabThreadsF32 = 1024;
 constexpr int kSlabThreadsF64 = 768;
 constexpr int kSlabDepthF32 = 1;
@@ -200,12 +202,12 @@ __device__ __forceinline__ V lane_suffix_sum(V x, uint32_t stops, int lane) {
 // bit i says "entry 8g + i starts a pair", and tile_pair[t] is the pair of the
 // tile's first entry.  A lane finds the pair of its first entry from a warp
 // prefix count of the start bits, so no pair table is searched.  Per lane:
-// runs that start and end inside the lane are stored; the run that continues
-// from the left (cont) and the run that leaves to the right (tail) are
-// combined across the warp by a segmented suffix sum, so only the tile's first
-// and last pairs take atomic adds.
-// one tile's loads for one lane: ITEMS rows and values, the start bits, and
-// the pair of the tile's first entry
+// runs that start and end inside the lane are added into g_j as they end; the
+// run that continues from the left (cont) and the run that leaves to the right
+// (tail) are combined across the warp by a segmented suffix sum, so a pair
+// takes one atomic add per tile it touches.
+// TileStage: one tile's loads for one lane: ITEMS rows and values, the start
+// bits, and the pair of the tile's first entry.
 template <typename SV, int ITEMS>
 struct TileStage {
   LaneLoad<SV, ITEMS> L;
@@ -456,7 +458,7 @@ __device__ __forceinline__ void light_tile(const LightStage<SV>& cur, int64_t t,
     if (lane >= d) incl += y;
   }
   uint32_t q = lc0 + (incl - cnt) + (lane > 0 ? (m & 1u) : 0u);
-  // columns this lane may write (and their scales), loaded early
+  // columns this lane may write, loaded early
   const bool lead = lane == 0 && active && !(m & 1u);
   const uint32_t ql = q + __popc(m & 0xfeu);
   const int32_t j0 = lead ? __ldg(light_cols + lc0) : 0;
@@ -468,7 +470,7 @@ __device__ __forceinline__ void light_tile(const LightStage<SV>& cur, int64_t t,
 #pragma unroll
     // gathers of u through L2 without allocating in L1 (no reuse to keep)
     for (int i = 0; i < 8; ++i) uu[i] = load_l2(u + r[i]);  // padding rows are 0, values 0
-    // first run, last run and the whole columns between (see k_propose_slabs)
+    // first run, last run and the whole columns between (see slab_pass)
     const uint32_t inner = m & 0xfeu;
     const int bf = inner ? __ffs(inner) - 1 : 8;
     V acc = V(0), first = V(0);
@@ -542,8 +544,8 @@ __global__ void __launch_bounds__(kThreads, 3)
 }
 
 // The light tiles as a shared pool: warps take kLightChunk tiles at a time
-// from a global counter (reset to 0 by k_pairs_to_gacc after every launch),
-// the next tile's loads in flight while one is summed.
+// from a global counter (reset by the last warp of k_propose_fused), the next
+// tile's loads in flight while one is summed.
 constexpr int kLightChunk = 4;
 
 template <typename V, typename U, typename G, typename SV>
@@ -1056,7 +1058,10 @@ static int build_plan_impl(gencd_problem* p, Scratch& S) {
   // column's sums are added one after another, and two chains half as long keep
   // the error of short columns below that of the light pass, which adds in a
   // tree (columns of 30 over 21 slabs: 7.56e-8 of the norm with two, 8.74e-8 with
-  // one, 7.52e-8 as light columns; Zipf columns in all 6.25e-8, 6.77e-8, 6.52e-8)
+  // one, 7.52e-8 as light columns; Zipf columns in all 6.25e-8, 6.77e-8, 6.52e-8).
+  // A run of one entry rounds its product once more than a lane's chain does:
+  // uniform columns of 3 over 2 to 12 slabs 3.9e-8 to 4.2e-8 (light 3.7e-8), of 6
+  // 4.6e-8 to 5.0e-8 (4.7e-8), of 12 and more as the light pass or less.
   P.second = !f64 && P.nslabs >= 8 ? k : 0;
   P.heavy_min = 1;
   P.forms = false;

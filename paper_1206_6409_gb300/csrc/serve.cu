@@ -17,8 +17,9 @@
 //  - the calling thread is the stepper: it polls every running slot's last
 //    enqueued work (an event), and when it has completed takes the solve's
 //    next decision and enqueues its next iterations (gencd_solve's loop, one
-//    step at a time: solve_advance), so the kernels of all requests in
-//    flight overlap on the device while no host thread waits on one solve.
+//    step at a time: solve_advance, which does not wait), so the kernels of all
+//    requests in flight overlap on the device while no host thread waits on
+//    one solve.
 #include <algorithm>
 #include <chrono>
 #include <cmath>

@@ -1050,6 +1050,35 @@ def test_propose_with_light_and_heavy_columns(gb, precision):
             assert_steps_close(sp, z, w, lam, J, d, f, d_cpu, f_cpu, TOL["f64" if precision == "f64" else "f32"])
 
 
+@pytest.mark.parametrize("slabs", [1, 2, 4, 7, 8])
+@pytest.mark.parametrize("per_col", [3, 12, 100])
+def test_fp32_sums_of_short_columns_keep_their_error(gb, slabs, per_col):
+    # runs of few entries over 1 to 8 slabs (49,152 rows each), against 64 bits:
+    # each of a sum's L products and L - 1 additions is rounded by an independent
+    # c = 0.41 2^-24 of its value (rms), partial sums of i terms are sqrt(i) terms
+    # large, so the error is at most c sqrt(1 + L / 2) of the norm when the terms
+    # are added one after another (a lane's 8, then the lanes in a tree: 16 at
+    # most here); 1.3 for the values' spread
+    n, k = 49_152 * slabs - 100, 40_000
+    rng = np.random.default_rng(slabs)
+    counts = np.full(k, per_col, np.int64)
+    counts[5] = 20_000  # a heavy column beside them
+    col_ptr = np.zeros(k + 1, np.int64)
+    np.cumsum(counts, out=col_ptr[1:])
+    rows = workloads.synthetic._distinct_rows(n, counts, rng)
+    val = rng.lognormal(0.0, 1.0, rows.size).astype(np.float32).astype(np.float64)
+    y = rng.normal(size=n).astype(np.float32).astype(np.float64)
+    prob = workloads.Problem(n, k, col_ptr, rows, val, y, "squared", np.zeros(k), "short")
+    with gb.Problem(prob, precision="f32") as p:
+        p.set_lambda(0.0)
+        p.set_params(beta_mode=1)
+        d, _, _ = p.propose_all()  # lambda = 0, beta = 1, w = 0: delta = -g
+    g = np.add.reduceat(val * -y[rows], col_ptr[:-1]) / n
+    short = np.arange(k) != 5
+    err = np.linalg.norm((d + g)[short]) / np.linalg.norm(g[short])
+    assert err < 1.3 * 0.41 * 2.0**-24 * np.sqrt(1 + min(per_col, 16) / 2)
+
+
 @pytest.mark.parametrize("precision", ["f64", "f32"])
 @pytest.mark.parametrize("n,per_col,long,passes", [
     (300_000, 3, 0, "light"), (300_000, 3, 20_000, "slabs"),  # 7 slabs in FP32, 13 in FP64
