@@ -94,8 +94,9 @@ int gencd_batch_lambda_max(gencd_batch* b, int32_t held_out, double* lambda_max)
  * are ignored.  GENCD_EINVAL for another variant or a value out of range.
  * tol_gap > 0: gencd_batch_path also ends a solve when its duality gap
  * (include/gencd.h, gencd_duality_gap; the dual point's scale from the FP32
- * sums) is at most tol_gap * |P(w)|, checked when the solve's objective is
- * evaluated (every 8 checks). */
+ * sums, or from FP64 sums when the solve has stalled) is at most
+ * tol_gap * |P(w)|, checked when the solve's objective is evaluated (every 8
+ * checks). */
 int gencd_batch_set_params(gencd_batch* b, const gencd_params* params);
 
 /*

@@ -888,6 +888,26 @@ __global__ void k_b_objective(const double* __restrict__ y, const double* __rest
   }
 }
 
+// *out = max_j |X_j^T u_s| over slot s's training rows (bits), u from the FP64
+// fitted values and summed in FP64; a warp per column
+__global__ void k_b_absmax64(const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row,
+                             const float* __restrict__ val, const double* __restrict__ y,
+                             const uint8_t* __restrict__ fold, int nfolds, int loss, const double* __restrict__ tab,
+                             const double* __restrict__ z, int64_t k, int Sp, int s, int set,
+                             unsigned long long* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t j = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; j < k; j += nw) {  // warp-uniform
+    double g = 0.0;
+    for (int64_t t = col_ptr[j] + lane; t < col_ptr[j + 1]; t += 32) {
+      const int64_t i = row[t];
+      if (b_train(fold, i, set, nfolds)) g = fma((double)val[t], loss_deriv(loss, y[i], z[i * Sp + s], tab), g);
+    }
+    g = warp_sum(g);
+    if (lane == 0 && g != 0.0) atomicMax(out, (unsigned long long)__double_as_longlong(fabs(g)));
+  }
+}
+
 // parity hook: FP64 Eq. 7 / Eq. 9 of every (column, slot), slot-major output
 __global__ void k_b_propose(const float* __restrict__ G, const double* __restrict__ w, const double* __restrict__ bjs,
                             const double* __restrict__ ibs, int64_t k, SlotArgs sa, int Sp, double* __restrict__ delta,
@@ -1297,15 +1317,32 @@ static int wave_clear(gencd_batch* b, SlotWave v) {
   return wave_fill(b, v);
 }
 
+// max_j |g_js| of slot s's current state from FP64 sums, synchronising
+static int slot_gmax64(gencd_batch* b, int s, double* gmax) {
+  unsigned long long* out = reinterpret_cast<unsigned long long*>(b->obj_acc + 128);
+  const int set = b->h_set[s];
+  GENCD_CUDA_TRY(cudaMemsetAsync(out, 0, 8, b->st));
+  k_b_absmax64<<<grid_for(b->k * 32, kThreads, b->X->num_sms * 8), kThreads, 0, b->st>>>(
+      b->X->col_ptr, b->X->row_idx, (const float*)b->X->val, b->X->y, b->fold, b->nfolds, b->loss, b->X->ltab, b->z,
+      b->k, b->S, s, set, out);
+  GENCD_CUDA_TRY(cudaGetLastError());
+  double sum = 0.0;
+  GENCD_CUDA_TRY(cudaMemcpyAsync(&sum, out, 8, cudaMemcpyDeviceToHost, b->st));
+  GENCD_CUDA_TRY(cudaStreamSynchronize(b->st));
+  *gmax = b->set_rows[set] > 0 ? sum / (double)b->set_rows[set] : 0.0;
+  return GENCD_OK;
+}
+
 // objectives of the listed slots (FP64), synchronising; gap (nullable): their
-// duality gaps, which need the max |g_js| of the slots' current state (a
-// propose pass over the current state must have run since the last step)
+// duality gaps, which need the max |g_js| of the slots' current state: gmax64
+// (one per listed slot), or else the FP32 sums' (a propose pass over the
+// current state must have run since the last step)
 static int slot_objectives(gencd_batch* b, const std::vector<int32_t>& slots, std::vector<double>* obj,
-                           std::vector<double>* gap = nullptr) {
+                           std::vector<double>* gap = nullptr, const std::vector<double>* gmax64 = nullptr) {
   obj->assign(slots.size(), 0.0);
   if (gap) gap->assign(slots.size(), 0.0);
   std::vector<unsigned int> gbits;
-  if (gap) {
+  if (gap && !gmax64) {
     gbits.resize(b->S);
     GENCD_CUDA_TRY(cudaMemcpyAsync(gbits.data(), b->kkt_bits + b->S, 4 * b->S, cudaMemcpyDeviceToHost, b->st));
     GENCD_CUDA_TRY(cudaStreamSynchronize(b->st));
@@ -1323,10 +1360,10 @@ static int slot_objectives(gencd_batch* b, const std::vector<int32_t>& slots, st
     if (gap) {  // s = lambda / max(lambda, max_j |g_j|): the dual point s u is feasible
       for (int q = 0; q < m; ++q) {
         const int s = slots[q0 + q];
-        float gm;
-        std::memcpy(&gm, &gbits[s], 4);
-        const double lam = b->h_lam[s];
-        scale[q] = (double)gm > lam ? lam / (double)gm : 1.0;
+        float g32 = 0.0f;
+        if (!gmax64) std::memcpy(&g32, &gbits[s], 4);
+        const double lam = b->h_lam[s], gm = gmax64 ? (*gmax64)[q0 + q] : (double)g32;
+        scale[q] = gm > lam ? lam / gm : 1.0;
       }
       GENCD_CUDA_TRY(cudaMemcpyAsync(b->obj_acc + 96, scale.data(), sizeof(double) * 32, cudaMemcpyHostToDevice,
                                      b->st));
@@ -1555,7 +1592,7 @@ static int create_batch(gencd_batch* b, const uint8_t* fold, int32_t memory) {
   GENCD_TRY(balloc(&b->kkt_bits, 2 * S));  // KKT and max |g| per slot
   GENCD_TRY(balloc(&b->ctr, 2));
   GENCD_CUDA_TRY(cudaMemsetAsync(b->ctr, 0, 16, st));
-  GENCD_TRY(balloc(&b->obj_acc, 128));
+  GENCD_TRY(balloc(&b->obj_acc, 129));
   GENCD_TRY(balloc(&b->obj_list, 64));
   GENCD_TRY(balloc(&b->tmp_k, k));
   GENCD_TRY(balloc(&b->d_lam, 4 * (size_t)S));  // all six arrays (upload_slots)
@@ -2035,6 +2072,17 @@ static int batch_path(gencd_batch* b, const gencd_path* path, gencd_path_solve* 
           best_p[s] = P;
           stall[s] = 0;
         } else if (stall[s] >= stall_checks) {  // neither value improved for kStallIters iterations
+          if (gaps) {  // the FP32 sums' gap may stay above a tolerance that the state has long met
+            std::vector<double> g64(1), p64, gap64;
+            rc = slot_gmax64(b, s, &g64[0]);
+            if (rc == GENCD_OK) rc = slot_objectives(b, {s}, &p64, &gap64, &g64);
+            if (rc != GENCD_OK) break;
+            if (gap64[0] <= b->params.tol_gap * std::fabs(p64[0])) {
+              solves[slot_solve[s]].status = GENCD_OK;
+              retire.push_back(s);
+              continue;
+            }
+          }
           if (b->h_group[s] < b->B && kv[s] >= kStallKkt * b->h_lam[s]) {
             b->h_group[s] = std::min(b->B, 2 * b->h_group[s]);
             regroup = true;

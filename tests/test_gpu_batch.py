@@ -257,6 +257,27 @@ def test_every_update_schedule_keeps_z_equal_to_xw(gb, update_kind):
             assert obj[s] == pytest.approx(orc.objective(w), rel=1e-12)
 
 
+def test_path_solves_that_stall_at_the_rounding_level_end(gb):
+    # config 4 at 1/10 scale to a gap of 8e-7: one solve reaches a cycle at the
+    # rounding level of the FP32 sums (97 non-zeros, KKT 8e-7 lambda) where those
+    # put its gap at 8.3e-7 and FP64 sums at 6.7e-7; it ends there instead of
+    # running to the iteration cap
+    prob = workloads.config4("squared", seed=0, scale=0.1)
+    fold = workloads.cv_folds(prob.n, 5, seed=0)
+    with gb.Batch(prob, fold=fold, nfolds=5, slots=32) as b:
+        b.set_params(variant="thread_greedy", blocks=1024, check_every=5, max_iter=20_000, tol_kkt=0.0, tol_gap=8e-7)
+        lams = np.stack([workloads.lambda_grid(b.lambda_max(f), 32, 1e-2) for f in range(5)])
+        recs, W, tot = b.path(list(range(5)), lams, handoff=0.5, warm=True, want_w=True)
+    assert tot.status == 0, [(q // 32, q % 32) for q, r in enumerate(recs) if r["status"]]
+    sub = workloads.row_subset(prob, np.flatnonzero(fold != 3))
+    with gb.Problem(sub, precision="f64") as p:
+        for t in (18, 20, 23, 31):
+            p.set_lambda(lams[3, t])
+            p.set_w(W[3, t])
+            gap, P, _ = gb.gencd_duality_gap(p.h)
+            assert gap <= 1.3e-6 * P, t  # the FP32 sums' gap is accurate to about 5e-7
+
+
 def test_batch_path_to_a_duality_gap(gb):
     # solves that stop at a relative duality gap of 8e-7 (the dual point's
     # scale from FP32 sums, accurate to about 1e-6 relative) are certified by
