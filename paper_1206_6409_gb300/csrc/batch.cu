@@ -42,7 +42,7 @@ namespace gencd {
 constexpr int kBatchMaxSlots = 256;
 constexpr int kBatchMaxFolds = 31;
 constexpr int kSpmmThreads = 256;
-constexpr int kAcceptThreads = 1024;  // per partition: slots x column strides
+constexpr int kAcceptThreads[2] = {512, 1024};  // per partition: slots x column strides (accept_wide)
 constexpr int kObjChecks = 8;        // convergence checks between objective evaluations of a path solve
 constexpr int kStallIters = 500;     // iterations without progress taken as a stall (as gencd_solve)
 constexpr double kStallGain = 1e-2;  // a new lowest KKT value is 1% below the previous one
@@ -302,16 +302,18 @@ struct SlotArgs {
 // Thread-Greedy Accept for every slot of partition b = blockIdx.x.  Thread
 // (s, r) scans columns lo + r, lo + r + R, ... of the partition for slot s.
 // MODE 1: accept (acc_j = column or -1, acc_d = FP64 step) and KKT; MODE 0:
-// KKT only.
-template <int MODE>
-__global__ void __launch_bounds__(kAcceptThreads)
+// KKT only.  WIDE: 1,024 threads, four columns' loads in flight each, for
+// partitions of many columns; else 512, of whose partial results thread r = 0
+// reduces half as many (accept_wide).
+template <int MODE, int WIDE>
+__global__ void __launch_bounds__(kAcceptThreads[WIDE])
     k_b_accept(const float* G, const float* w32, const double* w,
                const float* __restrict__ bj32, const float* __restrict__ ib32, const double* __restrict__ bjs,
                const double* __restrict__ ibs, int64_t k, SlotArgs sa, const int64_t* __restrict__ part_lo, int Sp,
                int R, int32_t* acc_j, double* acc_d, double* acc_phi, unsigned int* kkt_bits) {
-  __shared__ uint32_t s_mag[kAcceptThreads];
-  __shared__ int32_t s_col[kAcceptThreads];
-  __shared__ float s_v[kAcceptThreads];
+  __shared__ uint32_t s_mag[kAcceptThreads[WIDE]];
+  __shared__ int32_t s_col[kAcceptThreads[WIDE]];
+  __shared__ float s_v[kAcceptThreads[WIDE]];
   pdl_trigger();
   pdl_wait();
   const int b = blockIdx.x;
@@ -326,7 +328,7 @@ __global__ void __launch_bounds__(kAcceptThreads)
     const float lam = sa.lam32[s], invn = sa.invn32[s];
     const float* bjv = bj32 + (int64_t)set * k;
     const float* ibv = ib32 + (int64_t)set * k;
-#pragma unroll 4
+#pragma unroll(WIDE ? 4 : 1)
     for (int64_t j = lo + r; j < hi; j += R) {
       const float g = G[j * Sp + s] * invn;
       const float wj = w32[j * Sp + s];
@@ -1087,7 +1089,14 @@ static int spmm_blocks_per_sm(int NC, int* blocks) {
   return bfail(GENCD_EINVAL, "slot count out of range");
 }
 
-static int accept_R(const gencd_batch* b) { return std::max(1, kAcceptThreads / b->S); }
+// 1,024 threads a partition when each of them then walks at least eight
+// columns.  A step of all slots takes, with 1,024 / 512 threads: 8 slots 97 / 106
+// us (3,125 columns a partition), 34 / 32 (625), 73 / 65 (390), 159 / 93 (49);
+// 32 slots 175 / 217 (3,125), 45 / 53 (625), 124 / 123 (390), 249 / 225 (49); 64
+// slots 253 / 351, 60 / 79, 170 / 178, 384 / 359.
+static int accept_wide(const gencd_batch* b) {
+  return b->k / b->B >= (int64_t)8 * std::max(1, kAcceptThreads[1] / b->S) ? 1 : 0;
+}
 
 // G = X^T U and the per-slot KKT maxima (MODE 0), or a whole step (MODE 1)
 static int enqueue_propose(gencd_batch* b, bool accept) {
@@ -1097,10 +1106,12 @@ static int enqueue_propose(gencd_batch* b, bool accept) {
   GENCD_CUDA_TRY(launch_overlapped(k_b_prep, dim3(grid_for(std::max<int64_t>(1, nb * b->S), kThreads, g)),
                                    dim3(kThreads), 0, b->st, b->bnd, nb, b->S, b->G, b->kkt_bits));
   GENCD_TRY(launch_spmm(b, b->spmm_kind, b->U, b->G));
-  const int R = accept_R(b);
-  GENCD_CUDA_TRY(launch_overlapped(accept ? k_b_accept<1> : k_b_accept<0>, dim3(b->B), dim3(b->S * R), 0, b->st, b->G,
-                                   b->w32, b->w, b->bj32, b->ib32, b->bj, b->ib, b->k, slot_args(b), b->part_lo, b->S,
-                                   R, b->acc_j, b->acc_d, b->acc_phi, b->kkt_bits));
+  const int wide = accept_wide(b), R = std::max(1, kAcceptThreads[wide] / b->S);
+  const auto kernel = accept ? (wide ? k_b_accept<1, 1> : k_b_accept<1, 0>)
+                             : (wide ? k_b_accept<0, 1> : k_b_accept<0, 0>);
+  GENCD_CUDA_TRY(launch_overlapped(kernel, dim3(b->B), dim3(b->S * R), 0, b->st, b->G, b->w32, b->w, b->bj32, b->ib32,
+                                   b->bj, b->ib, b->k, slot_args(b), b->part_lo, b->S, R, b->acc_j, b->acc_d,
+                                   b->acc_phi, b->kkt_bits));
   return GENCD_OK;
 }
 
