@@ -610,8 +610,7 @@ static int store_values(gencd_problem* p, int64_t* bad_out) {
   *bad_out = -1;
   if (p->vmode == kValPlain) return GENCD_OK;
   if (p->vmode == kValNone) GENCD_TRY(dev_alloc(p, &p->col_val, p->k));
-  unsigned long long* bad = nullptr;
-  GENCD_TRY(dev_alloc(p, &bad, 1));
+  unsigned long long* bad = p->flags;
   unsigned long long h = ~0ull;
   int rc = GENCD_OK;
   if (cudaMemcpyAsync(bad, &h, 8, cudaMemcpyHostToDevice, p->stream) != cudaSuccess) rc = GENCD_ECUDA;
@@ -626,7 +625,6 @@ static int store_values(gencd_problem* p, int64_t* bad_out) {
         cudaStreamSynchronize(p->stream) != cudaSuccess)
       rc = fail(GENCD_ECUDA, std::string("storage conversion: ") + cudaGetErrorString(cudaGetLastError()));
   }
-  dev_free(p, bad);
   p->prof.launches[K_SETUP] += 1;
   if (rc == GENCD_OK && h != ~0ull) *bad_out = (int64_t)h;
   return rc;
@@ -673,6 +671,7 @@ static int create_impl(gencd_problem* p, const int64_t* col_ptr, const int32_t* 
   a.add(&p->list_off, list_cap(k, nnz) + 2);
   a.add(&p->scan_tmp, scan_tmp_words(k + 2));
   a.add(&p->dscal, kScalars);
+  a.add(&p->flags, 4);
   a.add(&p->red, 3 * kRedBlocks);
   a.add(&p->ltab, kLogisticWords);
   GENCD_TRY(dev_alloc_bytes(p, &p->mem, a.bytes()));
@@ -1212,13 +1211,13 @@ int gencd_propose_at(gencd_problem* p, const int32_t* J, int64_t m, double* delt
                             memory == GENCD_DEVICE ? cudaMemcpyDeviceToHost : cudaMemcpyHostToHost));
   for (int64_t e = 0; e < m; ++e)
     if (hj[e] < 0 || hj[e] >= p->k) return fail(GENCD_EINVAL, "J[" + std::to_string(e) + "] out of range");
-  int32_t* dj = nullptr;
-  double *dd = nullptr, *df = nullptr;
+  // up to k columns: in the lists that every iteration writes anew
+  int32_t* dj = p->list_j;
+  double *dd = p->list_d, *df = p->phi;
   int rc = GENCD_OK;
-  if ((rc = dev_alloc(p, &dj, m)) || (rc = dev_alloc(p, &dd, m)) || (rc = dev_alloc(p, &df, m))) {
-    dev_free(p, dj);
-    dev_free(p, dd);
-    dev_free(p, df);
+  if (m > p->k && ((rc = dev_alloc(p, &dj, m)) || (rc = dev_alloc(p, &dd, m)) || (rc = dev_alloc(p, &df, m)))) {
+    if (dj != p->list_j) dev_free(p, dj);
+    if (dd != p->list_d) dev_free(p, dd);
     return rc;
   }
   if (cudaMemcpyAsync(dj, hj.data(), sizeof(int32_t) * m, cudaMemcpyHostToDevice, p->stream) != cudaSuccess)
@@ -1228,9 +1227,11 @@ int gencd_propose_at(gencd_problem* p, const int32_t* J, int64_t m, double* delt
                          cudaMemcpyAsync(phi, df, sizeof(double) * m, kind_out(memory), p->stream) != cudaSuccess ||
                          cudaStreamSynchronize(p->stream) != cudaSuccess))
     rc = fail(GENCD_ECUDA, std::string("propose_at: ") + cudaGetErrorString(cudaGetLastError()));
-  dev_free(p, dj);
-  dev_free(p, dd);
-  dev_free(p, df);
+  if (m > p->k) {
+    dev_free(p, dj);
+    dev_free(p, dd);
+    dev_free(p, df);
+  }
   return rc;
 }
 GENCD_CATCH
@@ -1296,8 +1297,7 @@ int gencd_set_colors(gencd_problem* p, const int32_t* colors, int64_t k, int32_t
   GENCD_TRY(build_csr(p));
   if (!p->color) GENCD_TRY(dev_alloc(p, &p->color, k));
   GENCD_CUDA_TRY(cudaMemcpyAsync(p->color, colors, sizeof(int32_t) * k, kind_in(memory), p->stream));
-  unsigned long long* chk = nullptr;
-  GENCD_TRY(dev_alloc(p, &chk, 2));
+  unsigned long long* chk = p->flags;
   GENCD_CUDA_TRY(cudaMemsetAsync(chk, 0xff, sizeof(unsigned long long), p->stream));
   GENCD_CUDA_TRY(cudaMemsetAsync(chk + 1, 0, sizeof(unsigned long long), p->stream));
   const int g = p->num_sms * 8;
@@ -1307,7 +1307,6 @@ int gencd_set_colors(gencd_problem* p, const int32_t* colors, int64_t k, int32_t
   unsigned long long h[2];
   GENCD_CUDA_TRY(cudaMemcpyAsync(h, chk, sizeof(h), cudaMemcpyDeviceToHost, p->stream));
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
-  dev_free(p, chk);
   int32_t mn = 0;
   {
     std::vector<int32_t> hc((size_t)k);

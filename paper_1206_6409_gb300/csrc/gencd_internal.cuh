@@ -246,6 +246,7 @@ struct gencd_problem {
   // sum of conjugates, [9] the duality gap P(w) - D, [10], [11] non-zeros and
   // segments of the columns that z = Xw scatters (int64)
   double* dscal = nullptr;
+  unsigned long long* flags = nullptr;  // what a check found (4; scratch of one call)
   double* red = nullptr;  // per-block partial sums (2 * kRedBlocks)
   double* hpin = nullptr; // pinned host memory: dscal's first kScalFit, then what z = Xw reports
   bool fit_open = false;  // whether the columns sufficed for z = Xw is in hpin once the stream gets there

@@ -739,8 +739,7 @@ int launch_tile_map(gencd_problem* p) {
 
 // validation entry used by the API: returns first bad column / row or -1
 int validate_input(gencd_problem* p, int64_t* bad_col, int64_t* bad_row, int* stage) {
-  unsigned long long* err = nullptr;
-  GENCD_TRY(dev_alloc_bytes(p, (void**)&err, 3 * sizeof(unsigned long long)));
+  unsigned long long* err = p->flags;
   GENCD_CUDA_TRY(cudaMemsetAsync(err, 0xff, 2 * sizeof(unsigned long long), p->stream));
   GENCD_CUDA_TRY(cudaMemsetAsync(err + 2, 0, sizeof(unsigned long long), p->stream));
   const int g = p->num_sms * 8;
@@ -751,7 +750,6 @@ int validate_input(gencd_problem* p, int64_t* bad_col, int64_t* bad_row, int* st
   *stage = 0;
   if (h[0] != ~0ull) {
     *bad_col = (int64_t)h[0];
-    dev_free(p, err);
     return GENCD_OK;
   }
   *stage = 1;
@@ -773,7 +771,6 @@ int validate_input(gencd_problem* p, int64_t* bad_col, int64_t* bad_row, int* st
   p->prof.launches[K_SETUP] += 4;
   GENCD_CUDA_TRY(cudaMemcpyAsync(h, err, sizeof(h), cudaMemcpyDeviceToHost, p->stream));
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
-  dev_free(p, err);
   *bad_col = h[0] == ~0ull ? -1 : (int64_t)h[0];
   *bad_row = h[1] == ~0ull ? -1 : (int64_t)h[1];
   return GENCD_OK;

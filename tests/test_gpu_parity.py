@@ -852,6 +852,30 @@ def test_accept_takes_each_partitions_best_column(gb, precision, k, B):
 
 
 @pytest.mark.parametrize("precision", ["f64", "f32"])
+def test_propose_at_longer_lists_and_between_iterations(gb, precision):
+    # up to k columns the call uses the iterations' lists, beyond (repeats) its
+    # own memory; between iterations it changes nothing of their course
+    prob = workloads.config1("logistic")
+    lam = 0.05 * oracle.Oracle(prob).lambda_max()
+    w = []
+    for ask in (False, True):
+        with gb.Problem(prob, precision=precision) as p:
+            p.set_lambda(lam)
+            p.set_params(variant="thread_greedy", blocks=64)
+            for _ in range(5):
+                p.iterate(1)
+                if ask:
+                    d, f = p.propose_at(np.arange(prob.k, dtype=np.int32))
+                    J = np.tile(np.arange(prob.k, dtype=np.int32), 3)[: 2 * prob.k + 7]
+                    d2, f2 = p.propose_at(J)
+                    np.testing.assert_array_equal(d2, d[J])
+                    np.testing.assert_array_equal(f2, f[J])
+            w.append(p.w())
+    # FP64 additions of an iteration land in any order
+    np.testing.assert_allclose(w[1], w[0], rtol=0, atol=(1e-12 if precision == "f64" else 1e-6) * np.abs(w[0]).max())
+
+
+@pytest.mark.parametrize("precision", ["f64", "f32"])
 @pytest.mark.parametrize("frac", [0.0, 0.002, 0.3, 0.5, 1.0])
 @pytest.mark.parametrize("large", [False, True])
 def test_set_w_fits_sparse_and_dense_coefficients(gb, precision, frac, large):
