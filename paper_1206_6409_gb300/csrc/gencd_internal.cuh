@@ -335,9 +335,7 @@ int launch_update_refresh(gencd_problem* p, const int32_t* J, const double* d, i
 int launch_refresh_list(gencd_problem* p, const int32_t* J, int64_t m, bool counted);    // u (after z)
 int launch_shotgun_step(gencd_problem* p, const int32_t* J, int64_t m, bool early);      // propose, w and z
 int launch_coloring_iter(gencd_problem* p, int64_t q, bool early);
-// out = X x (FP64), by rows; with total, only if *total > limit (on the device)
-int launch_csr_spmv(gencd_problem* p, const double* x, double* out, const unsigned long long* total = nullptr,
-                    unsigned long long limit = 0);
+int launch_csr_spmv(gencd_problem* p, const double* x, double* out);  // out = X x (FP64)
 // entries of list_j and list_off: a column of len non-zeros has ceil(len / kSegEntries) segments
 inline int64_t list_cap(int64_t k, int64_t nnz) { return k + (nnz > kFitRowsNnz ? nnz / kSegEntries : 0); }
 // z, u and w32 from p->w, without waiting.  When p->fit_open is then set, the

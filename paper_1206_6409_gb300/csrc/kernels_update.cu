@@ -13,7 +13,7 @@
 //    proposes its column and then writes z and u of its own rows with plain
 //    stores -- no atomics, no second pass.
 //  * k_update_refresh: both passes over a short list in one launch.
-//  * k_w_segments, k_scatter_segments: z = Xw from the columns with w_j != 0
+//  * k_w_segments, k_fit_segments: z = Xw from the columns with w_j != 0
 //    (a warm start is sparse); k_csr_spmv: z = Xw by rows, for a dense w.
 //  * k_fill_u: u from z for all rows.
 #include <algorithm>
@@ -419,12 +419,11 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
+// rows of X x, a warp each
 template <typename V>
-__global__ void __launch_bounds__(kThreads)
-    k_csr_spmv(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
-               const V* __restrict__ csr_val, const double* __restrict__ x, int64_t n,
-               double* __restrict__ out, const unsigned long long* __restrict__ total, unsigned long long limit) {
-  if (total && *total <= limit) return;
+__device__ __forceinline__ void sum_rows(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
+                                         const V* __restrict__ csr_val, const double* __restrict__ x, int64_t n,
+                                         double* __restrict__ out) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -435,6 +434,13 @@ __global__ void __launch_bounds__(kThreads)
     acc = warp_sum(acc);
     if (lane == 0) out[i] = acc;
   }
+}
+
+template <typename V>
+__global__ void __launch_bounds__(kThreads)
+    k_csr_spmv(const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
+               const V* __restrict__ csr_val, const double* __restrict__ x, int64_t n, double* __restrict__ out) {
+  sum_rows(row_ptr, col_idx, csr_val, x, n, out);
 }
 
 __global__ void k_mirror_w(const double* __restrict__ w, int64_t k, float* __restrict__ w32) {
@@ -504,17 +510,22 @@ __global__ void __launch_bounds__(kThreads)
   }
 }
 
-// pass 2: a warp per segment adds w_j X_ij into z (FP64 atomics); nothing when
-// the listed non-zeros exceed `limit`
+// pass 2: a warp per segment adds w_j X_ij into z (FP64 atomics).  When the listed
+// non-zeros exceed `limit`: z by rows if the row-major copy is there (row_ptr not
+// null), else nothing
 template <typename V>
 __global__ void __launch_bounds__(kThreads)
-    k_scatter_segments(const int32_t* __restrict__ seg_j, const uint32_t* __restrict__ seg_t,
-                       const unsigned long long* __restrict__ count, const unsigned long long* __restrict__ total,
-                       unsigned long long limit, const int64_t* __restrict__ col_ptr,
-                       const int32_t* __restrict__ row_idx, const V* __restrict__ val, const double* __restrict__ w,
-                       double* __restrict__ z) {
+    k_fit_segments(const int32_t* __restrict__ seg_j, const uint32_t* __restrict__ seg_t,
+                   const unsigned long long* __restrict__ count, const unsigned long long* __restrict__ total,
+                   unsigned long long limit, const int64_t* __restrict__ col_ptr, const int32_t* __restrict__ row_idx,
+                   const V* __restrict__ val, const double* __restrict__ w, const int64_t* __restrict__ row_ptr,
+                   const int32_t* __restrict__ col_idx, const V* __restrict__ csr_val, int64_t n,
+                   double* __restrict__ z) {
   const int64_t m = (int64_t)*count;
-  if (*total > limit) return;
+  if (*total > limit) {
+    if (row_ptr) sum_rows(row_ptr, col_idx, csr_val, w, n, z);
+    return;
+  }
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < m; g += nwarps) {
@@ -743,14 +754,13 @@ int launch_coloring_iter(gencd_problem* p, int64_t q, bool early) {
 // Sparse coefficients: their columns are scattered into z, which reads no more
 // of X than those columns and needs no row-major copy (whose build sorts every
 // non-zero).  Otherwise the rows are summed: once the row-major copy is there,
-// the device decides from the listed non-zeros which of the two launches does
-// the work; before that the host does, after a wait (finish_state_from_w), and
-// builds it.  The line
-// is drawn at 2/5 of the non-zeros: a call took, by columns with w_j != 0,
-// scattered / by rows, on 4.0e7 FP32 non-zeros 48 / 276 us at 0.5%, 84 / 276 at
-// 12.5%, 155 / 276 at 40%, 309 / 276 at 100%, and on 2.0e7 FP64 non-zeros 52 /
-// 123, 74 / 123, 116 / 123 and 164 / 123 us.  Deciding costs a dense w some 10 us
-// (287 and 131 us in all; 298 and 145 with the host deciding on every call).
+// the second launch takes one or the other by the listed non-zeros; before that
+// the host does, after a wait (finish_state_from_w), and builds it.  The line is
+// drawn at 2/5 of the non-zeros: a call took, by columns with w_j != 0, scattered
+// / by rows, on 4.0e7 FP32 non-zeros 48 / 276 us at 0.5%, 84 / 276 at 12.5%, 155 /
+// 276 at 40%, 309 / 276 at 100%, and on 2.0e7 FP64 non-zeros 52 / 123, 74 / 123,
+// 116 / 123 and 164 / 123 us.  The listing costs a dense w 6 to 8 us (284 and 128
+// us in all, 13 us on a million columns of 3 non-zeros).
 //
 // At most kFitRowsNnz non-zeros: always by rows.  Reading all of X takes no
 // longer there than listing w's segments, and the sums have a fixed order, so
@@ -783,17 +793,17 @@ int launch_state_from_w(gencd_problem* p) {
   k_w_segments<<<grid_for(std::max((p->k + 3) / 4, p->n), kThreads, g), kThreads, 0, p->stream>>>(
       p->w, p->w32, p->col_ptr, p->k, p->list_j, p->list_off, count, total, p->n, p->z);
   if (p->precision == GENCD_F64)
-    k_scatter_segments<double><<<g, kThreads, 0, p->stream>>>(p->list_j, p->list_off, count, total, limit, p->col_ptr,
-                                                              p->row_idx, (const double*)p->val, p->w, p->z);
+    k_fit_segments<double><<<g, kThreads, 0, p->stream>>>(p->list_j, p->list_off, count, total, limit, p->col_ptr,
+                                                          p->row_idx, (const double*)p->val, p->w, p->row_ptr,
+                                                          p->col_idx, (const double*)p->csr_val, p->n, p->z);
   else
-    k_scatter_segments<float><<<g, kThreads, 0, p->stream>>>(p->list_j, p->list_off, count, total, limit, p->col_ptr,
-                                                             p->row_idx, (const float*)p->val, p->w, p->z);
+    k_fit_segments<float><<<g, kThreads, 0, p->stream>>>(p->list_j, p->list_off, count, total, limit, p->col_ptr,
+                                                         p->row_idx, (const float*)p->val, p->w, p->row_ptr,
+                                                         p->col_idx, (const float*)p->csr_val, p->n, p->z);
   p->prof.launches[K_SETUP] += 2;
   GENCD_CUDA_TRY(cudaGetLastError());
-  const bool rows_too = p->row_ptr != nullptr;
-  if (rows_too) GENCD_TRY(launch_csr_spmv(p, p->w, p->z, total, limit));
   GENCD_TRY(launch_fill_u(p, total, host));
-  p->fit_open = !rows_too;
+  p->fit_open = p->row_ptr == nullptr;
   return GENCD_OK;
 }
 
@@ -805,16 +815,15 @@ int finish_state_from_w(gencd_problem* p) {
   return 1;
 }
 
-int launch_csr_spmv(gencd_problem* p, const double* x, double* out, const unsigned long long* total,
-                    unsigned long long limit) {
+int launch_csr_spmv(gencd_problem* p, const double* x, double* out) {
   if (p->n == 0) return GENCD_OK;
   const int grid = grid_for(p->n * 32, kThreads, p->num_sms * 8);
   if (p->precision == GENCD_F64)
     k_csr_spmv<double><<<grid, kThreads, 0, p->stream>>>(p->row_ptr, p->col_idx, (const double*)p->csr_val,
-                                                         x, p->n, out, total, limit);
+                                                         x, p->n, out);
   else
     k_csr_spmv<float><<<grid, kThreads, 0, p->stream>>>(p->row_ptr, p->col_idx, (const float*)p->csr_val,
-                                                        x, p->n, out, total, limit);
+                                                        x, p->n, out);
   p->prof.launches[K_SETUP] += 1;
   GENCD_CUDA_TRY(cudaGetLastError());
   return GENCD_OK;
