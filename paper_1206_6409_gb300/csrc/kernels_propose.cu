@@ -385,9 +385,14 @@ __device__ __forceinline__ int scan_round_f32(float* gacc, const float* w32,
 // 4,000,000).
 template <typename G>
 constexpr int kAcceptPerSm = sizeof(G) == 4 ? 8 : 5;
+// as a launch bound in FP64 only: FP32 has its 32 registers without one, and
+// asked for 8 CTAs the compiler leaves fewer loads in flight (25.5 us instead of
+// 22.5 on k = 4,000,000; asked for one, 52 registers and 27.0)
+template <typename G>
+constexpr int kAcceptBound = sizeof(G) == 4 ? 0 : kAcceptPerSm<G>;
 
 template <typename G>
-__global__ void __launch_bounds__(kThreads, kAcceptPerSm<G>)
+__global__ void __launch_bounds__(kThreads, kAcceptBound<G>)
     k_accept_partitions(G* gacc, AcceptCols c, int64_t B, int per, int64_t chunk,
                         const int64_t* __restrict__ part_lo, int want_kkt, uint64_t* slot_m, int32_t* slot_j,
                         double* slot_x, unsigned int* slot_cnt, int32_t* list_j, double* list_d, uint64_t* list_m,
