@@ -106,7 +106,9 @@ typedef struct {
                           full evaluation (gencd_duality_gap) is at most
                           tol_gap * |P(w)|, which bounds the relative objective
                           error (P(w) - P*) / P(w); every convergence check is
-                          then a full evaluation.  0 = off (default)            */
+                          then a full evaluation (FP32 arithmetic: of a solve
+                          that has stalled, with FP64 sums too).  0 = off
+                          (default)                                            */
 } gencd_params;
 
 typedef struct {

@@ -249,6 +249,37 @@ static int enqueue_evaluate(gencd_problem* p, bool gap = false) {
   return GENCD_OK;
 }
 
+// *out = max_j |gacc_j| / n as non-negative bits; gacc is zero again after it
+__global__ void k_sums_absmax(double* __restrict__ gacc, int64_t k, double inv_n, double* __restrict__ out) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  double m = 0.0;
+  for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < k; j += stride) {
+    const double g = fabs(gacc[j] * inv_n);
+    gacc[j] = 0.0;
+    m = g > m || g != g ? g : m;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double x = __shfl_xor_sync(0xffffffffu, m, o);
+    m = x > m || x != x ? x : m;
+  }
+  if ((threadIdx.x & 31) == 0) atomic_max_nonneg(out, m);
+}
+
+// The duality gap (dscal[9]) of an evaluated state again, its max_j |g_j| from
+// FP64 sums (FP32 arithmetic); the KKT value and the objective stay
+static int enqueue_fine_gap(gencd_problem* p) {
+  if (!p->u64) GENCD_TRY(dev_alloc(p, &p->u64, p->n));
+  GENCD_CUDA_TRY(cudaMemsetAsync(p->dscal + 7, 0, sizeof(double), p->stream));
+  GENCD_TRY(launch_fill_u64(p));
+  GENCD_TRY(launch_propose_all(p, p->u64, true));
+  k_sums_absmax<<<grid_for(p->k, kThreads, p->num_sms * 8), kThreads, 0, p->stream>>>(p->gacc, p->k, 1.0 / (double)p->n,
+                                                                                     p->dscal + 7);
+  p->prof.launches[K_SETUP] += 1;
+  GENCD_CUDA_TRY(cudaGetLastError());
+  return launch_objective(p, true);
+}
+
 static int read_scalars(gencd_problem* p) {
   GENCD_CUDA_TRY(cudaMemcpyAsync(p->hpin, p->dscal, kScalFit * sizeof(double), cudaMemcpyDeviceToHost, p->stream));
   GENCD_CUDA_TRY(cudaStreamSynchronize(p->stream));
@@ -561,7 +592,7 @@ __global__ void __launch_bounds__(kThreads)
 
 static void free_problem(gencd_problem* p) {
   if (!p) return;
-  void* bufs[] = {p->mem, p->w_start, p->top_buf, p->sort_tmp, p->row_ptr, p->col_idx, p->csr_val, p->color,
+  void* bufs[] = {p->mem, p->w_start, p->u64, p->top_buf, p->sort_tmp, p->row_ptr, p->col_idx, p->csr_val, p->color,
                   p->color_ptr, p->cols_by_color, p->slot_m, p->slot_d, p->slot_j, p->slot_cnt, p->part_lo, p->col_val,
                   p->block_lo, p->block_P};
   if (p->stream) cudaStreamSynchronize(p->stream);
@@ -845,6 +876,7 @@ int solve_advance(gencd_problem* p, SolveRun* S) {
     p->accept_group = std::min<int64_t>(S->B, 4 * p->accept_group);  // restart from the start state
     S->best_kkt = S->best_obj = HUGE_VAL;
     S->stall = 0;
+    S->fine = false;
     GENCD_CUDA_TRY(cudaMemcpyAsync(p->w, p->w_start, sizeof(double) * p->k, cudaMemcpyDeviceToDevice, p->stream));
     GENCD_TRY(launch_state_from_w(p));
     GENCD_TRY(solve_evaluate(p, S));
@@ -875,8 +907,12 @@ int solve_advance(gencd_problem* p, SolveRun* S) {
   // lowest values are kept from the solve's (re)start, so the phases of a
   // cycle do not pass for progress, and a solve whose objective keeps falling
   // is never touched.  Near the optimum both values stop improving at the
-  // rounding level of the FP32 sums, where fewer updates would not help.
-  if (S->backoff && p->accept_group < S->B) {
+  // rounding level of the FP32 sums, where fewer updates would not help, and the
+  // gap of those sums can stay above a tolerance that the state has long met:
+  // with tol_gap a stalled FP32 solve first has its gap taken with FP64 sums.
+  const bool group = S->backoff && p->accept_group < S->B;
+  const bool fine = a.tol_gap > 0.0 && p->precision == GENCD_F32;
+  if (group || fine) {
     bool progress = false;
     if (obj < S->best_obj * (1.0 - kObjGain)) {  // P >= 0 for both losses
       S->best_obj = obj;
@@ -889,8 +925,17 @@ int solve_advance(gencd_problem* p, SolveRun* S) {
     if (progress) {
       S->stall = 0;
     } else if (++S->stall >= std::max<int64_t>(1, (kStallIters + a.check_every - 1) / a.check_every)) {
-      if (kkt >= kStallKkt * p->lambda) p->accept_group = std::min<int64_t>(S->B, 2 * p->accept_group);
+      if (fine && !S->fine) {
+        S->fine = true;
+        GENCD_TRY(enqueue_fine_gap(p));
+        GENCD_TRY(read_scalars_async(p));
+        S->host_nnz += p->nnz;
+        p->stat_host_nnz += p->nnz;
+        return 1;
+      }
+      if (group && kkt >= kStallKkt * p->lambda) p->accept_group = std::min<int64_t>(S->B, 2 * p->accept_group);
       S->stall = 0;
+      S->fine = false;
     }
   }
   const double el = std::chrono::duration<double>(std::chrono::steady_clock::now() - S->t0).count();

@@ -216,6 +216,7 @@ struct gencd_problem {
   uint64_t* list_m = nullptr;   // candidate magnitude of each partition's accepted column (accept backoff)
   uint32_t* top_buf = nullptr;  // global top-|J'| Accept: sort keys and indices (6 k words)
   double* w_start = nullptr;    // w at the start of a solve (restarts of the accept backoff)
+  double* u64 = nullptr;        // FP32 mode: u in FP64 for the gap of a stalled solve (on first use)
   int64_t accept_group = 1;     // Thread-Greedy partitions merged per accept group (1: none)
   double* list_d = nullptr;
   uint32_t* list_off = nullptr;  // the listed columns' nnz | kApplied, or their exclusive prefix (k + 1)
@@ -330,6 +331,7 @@ int launch_inv_beta(gencd_problem* p);   // ib_j = 1 / beta_j for the current be
 // kernels_update.cu
 // u = l'(y, z); with report (pinned host memory), counts[0..1] are copied there and reset
 int launch_fill_u(gencd_problem* p, unsigned long long* counts = nullptr, unsigned long long* report = nullptr);
+int launch_fill_u64(gencd_problem* p);  // u64 = l'(y, z)
 int launch_apply_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m);   // w, list_off
 int launch_update_refresh(gencd_problem* p, const int32_t* J, const double* d, int64_t m);  // z and u (after w)
 int launch_refresh_list(gencd_problem* p, const int32_t* J, int64_t m, bool counted);    // u (after z)
@@ -377,6 +379,7 @@ struct SolveRun {
   // since the solve's (re)start, and the checks since either last improved
   double best_kkt = HUGE_VAL, best_obj = HUGE_VAL;
   int stall = 0;
+  bool fine = false;  // the gap last read is from FP64 sums (a stalled FP32 solve)
 };
 int solve_begin(gencd_problem* p, SolveRun* S);
 int solve_advance(gencd_problem* p, SolveRun* S);  // 1: more work enqueued, 0: done, < 0: error

@@ -610,6 +610,14 @@ int launch_fill_u(gencd_problem* p, unsigned long long* counts, unsigned long lo
   return GENCD_OK;
 }
 
+int launch_fill_u64(gencd_problem* p) {
+  k_fill_u<double><<<grid_for(p->n, kThreads, p->num_sms * 8), kThreads, 0, p->stream>>>(
+      p->y, p->z, p->n, p->loss, p->ltab, p->u64, nullptr, nullptr);
+  p->prof.launches[K_SETUP] += 1;
+  GENCD_CUDA_TRY(cudaGetLastError());
+  return GENCD_OK;
+}
+
 // w and list_off for the accepted entries of the list (J, d)
 int launch_apply_list(gencd_problem* p, const int32_t* J, const double* d, int64_t m) {
   if (m <= 0) return GENCD_OK;

@@ -101,6 +101,7 @@ double footprint(const gencd_request& r, int precision, const gencd_params& para
              + kAllowance;
   if (params.variant == GENCD_THREAD_GREEDY || params.variant == GENCD_TOP_GREEDY) b += 8.0 * k;  // backoff start
   if (params.variant == GENCD_TOP_GREEDY) b += 28.0 * k;  // sort keys, indices and scratch
+  if (params.tol_gap > 0.0 && precision != GENCD_F64) b += 8.0 * n;  // u in FP64 for a stalled solve's gap
   return b;
 }
 

@@ -927,6 +927,29 @@ def test_set_w_scatters_few_columns_of_many_segments(gb, precision):
             np.testing.assert_allclose(p.z(), orc.fitted(w), rtol=0, atol=1e-11 if precision == "f64" else 2e-5)
 
 
+def test_fp32_solves_to_a_gap_near_their_rounding_level_end(gb):
+    # two chains of 32 warm-started solves to a gap of 8e-7, which the FP32 sums
+    # barely resolve: a solve that stalls above it is decided by FP64 sums
+    # instead of running to the iteration cap
+    prob = workloads.config4("squared", seed=0, scale=0.1)
+    fold = workloads.cv_folds(prob.n, 5, seed=0)
+    for f in (3, 4):
+        sub = workloads.row_subset(prob, np.flatnonzero(fold != f))
+        with gb.Problem(sub, precision="f32") as p, gb.Problem(sub, precision="f64") as q:
+            for lam in workloads.lambda_grid(p.lambda_max(), 32, 1e-2):
+                p.set_lambda(lam)
+                p.set_params(variant="thread_greedy", blocks=1024, check_every=5, max_iter=20_000, tol_kkt=0.0,
+                             tol_gap=8e-7)
+                r = p.solve()
+                assert r.status == 0, (f, lam, r.as_dict())
+                q.set_lambda(lam)
+                q.set_w(p.w())
+                gap, P, _ = gb.gencd_duality_gap(q.h)
+                # FP32 sums of some hundred cancelling terms know max |g_j| to
+                # about 1.5e-6 of lambda, and lambda |w|_1 is up to 0.9 of P
+                assert gap <= (8e-7 + 1.5e-6) * P + 1e-300, (f, lam)
+
+
 @pytest.mark.parametrize("start", ["few", "dense", "grown"])
 def test_restarts_of_large_problems_start_from_their_w(gb, start):
     # 1.2e6 non-zeros (z = Xw from the columns): Thread-Greedy's first steps
